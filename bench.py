@@ -39,7 +39,7 @@ POPC_PER_SM_CLK = 16
 N_SMS = 152
 SM_MAX_MHZ = 2070.0
 # FP8 dense rate = 2 x BF16 dense (nominal 4.5 vs 2.25 PFLOP/s)
-FP8_OVER_BF16 = 2.0
+FP4_OVER_BF16 = 4.0
 
 
 def _env_int(name, default):
@@ -265,7 +265,7 @@ def measure_count_variants(epi, ctx, synth, flush, stream):
     with the POPC instruction, a byte lookup table in shared memory, and the
     binary tensor-core MMA (AND + POPC), each run twice (the second timed);
     paper work 3^k (W1 + W0) 32-bit word operations per combination, against
-    the POPC pipe's rate.  The FP8 tensor-core search of the same dataset is
+    the POPC pipe's rate.  The tensor-core search of the same dataset is
     timed beside them (it also scores and selects)."""
     import torch
     d, k, top_n = synth.make_workload("order3_2000snp_4000", n_snps=500)
@@ -281,7 +281,7 @@ def measure_count_variants(epi, ctx, synth, flush, stream):
         sums.add(r["checksum"])
         out[v] = dict(ms=r["ms"], word_ops_per_s=ops / (r["ms"] / 1e3), frac_of_popc_peak=ops / (r["ms"] / 1e3) / peak)
     m = time_search(epi, ctx, ds, k, top_n, "tc", 2, 1, flush, stream)
-    out["tc_fp8_search"] = dict(ms=m["t_ms"] / 2, word_ops_per_s=ops / (m["t_ms"] / 2 / 1e3),
+    out["tc_search"] = dict(ms=m["t_ms"] / 2, word_ops_per_s=ops / (m["t_ms"] / 2 / 1e3),
                                 note="whole search (count, score, top-N), paper work in the same units")
     ds.close()
     out["checksums_agree"] = len(sums) == 1
@@ -317,8 +317,8 @@ def measure_batch_full(epi, ctx, synth, peaks, tc_rate, stream):
         if key not in chosen:
             chosen[key] = epi.autotune(ds, k)
     tune_s = time.perf_counter() - t0
-    tc_peak = (2.0 * tc_rate[0]["mac_per_clk_sm"] * N_SMS * SM_MAX_MHZ * 1e6 if tc_rate
-               else FP8_OVER_BF16 * peaks["bf16"] * 1e12)
+    tc_peak = (2 * 2.0 * tc_rate[1]["mac_per_clk_sm"] * N_SMS * SM_MAX_MHZ * 1e6 if tc_rate
+               else FP4_OVER_BF16 * peaks["bf16"] * 1e12)
     popc_peak = N_SMS * POPC_PER_SM_CLK * SM_MAX_MHZ * 1e6
     work = 0
     ideal_s = 0.0
@@ -374,30 +374,33 @@ def measure_mlp_inference(epi, ctx, peaks):
     return out
 
 
-def comb_shift(d, k):
+def class_shift(d):
     """Class shift of the tensor path's combined-class variant, 0 where the
     separate-class variant runs (the rule include/epi.h states for
     EPI_TC_AUTO)."""
     m1, m0 = d.n_cases, d.n_samples - d.n_cases
-    if k != 3:
-        return 0
     p = 1
     while p < 15 and (1 << p) <= m0:
         p += 1
     return p if p <= 14 and m1 * (1 << p) + m0 < (1 << 23) else 0
 
 
+def comb_shift(d, k):
+    """The class shift of the order-3 headline's accumulator (0 at other
+    orders: their results are reported without it)."""
+    return class_shift(d) if k == 3 else 0
+
+
 def tc_executed_flops(d, k):
     """Multiply-adds the tensor-core counting kernel issues for a whole search,
     x 2.  The items are the M tiles of ppt prefixes that start in panel c
-    times the N tiles after c (the kernel's item table), each over the padded
-    K of both classes (128-individual stages).  Separate classes: N tiles of
-    64 last SNPs, every MMA M128 x N128.  Combined classes: N tiles of 128
-    last SNPs, the MMA's N cut to the columns below 2 n (steps of 16)."""
+    times the N tiles after c (the kernel's item table), each over both
+    classes padded to 128 individuals.  N tiles start at an even SNP and hold
+    120 last SNPs (combined classes) or 80 (separate classes); the MMA's N is
+    cut to the columns below 2 n (steps of 16)."""
     n = d.n_snps
     ppt = 1 if 3 ** (k - 1) > 32 else 4 * (32 // 3 ** (k - 1))
-    comb = comb_shift(d, k) != 0
-    kj = 128 if comb else 64
+    kj = 120 if class_shift(d) else 80
     cols = 0
     for c in range(k - 2, n - 1):
         t0 = -(-math.comb(c, k - 1) // ppt)
@@ -406,12 +409,12 @@ def tc_executed_flops(d, k):
             continue
         # the N tiles of an M tile whose first prefix lies in panel c
         per_m = 0
-        for u in range(-(-(n - 1 - c) // kj)):
-            j0 = c + 1 + u * kj
-            live = 2 * (n - j0)
-            per_m += min(2 * kj, -(-live // 16) * 16) if comb else 2 * kj
+        first = (c + 1) & ~1
+        for u in range(-(-(n - first) // kj)):
+            live = 2 * (n - first - u * kj)
+            per_m += min(2 * kj, -(-live // 16) * 16)
         cols += (t1 - t0) * per_m
-    kt = 32 * 4 * (-(-d.n_cases // 128) + -(-(d.n_samples - d.n_cases) // 128))
+    kt = 128 * (-(-d.n_cases // 128) + -(-(d.n_samples - d.n_cases) // 128))
     return 2.0 * cols * 128 * kt
 
 
@@ -424,24 +427,25 @@ def roofline(kind, d, k, kern_ms, peaks, tc_rate=None):
         flops = 2.0 * total * (3 ** k) * d.n_samples
         achieved = flops / (kern_ms / 1e3) / 1e12
         executed = tc_executed_flops(d, k) / (kern_ms / 1e3) / 1e12
-        fp8_conv = FP8_OVER_BF16 * peaks["bf16"]
-        comb = comb_shift(d, k) != 0
+        fp4_conv = FP4_OVER_BF16 * peaks["bf16"]
+        comb = class_shift(d) != 0
         if tc_rate:
-            # the measured rate of the kernel's own MMA, at the maximum SM clock
-            r = tc_rate[1 if comb else 0]
-            shape = "E5M2 M128 N256 K32" if comb else "E4M3 M128 N128 K32"
-            peak = 2.0 * r["mac_per_clk_sm"] * N_SMS * SM_MAX_MHZ * 1e6 / 1e12
-            note = (f"peak = measured FP8 {shape} tcgen05.mma rate, {r['mac_per_clk_sm']:.0f} "
+            # twice the measured rate of the FP8 MMA, at the maximum SM clock
+            # (kind::mxf4 retires 16384 multiply-adds per SM clock where the
+            # FP8 kinds retire 8192, both measured)
+            r = tc_rate[1]
+            peak = 2 * 2.0 * r["mac_per_clk_sm"] * N_SMS * SM_MAX_MHZ * 1e6 / 1e12
+            note = (f"peak = 2 x the measured FP8 tcgen05.mma rate, {r['mac_per_clk_sm']:.0f} "
                     f"MAC/clk/SM x 152 SMs x 2070 MHz (probe ran at {r['sm_mhz']:.0f} MHz: "
                     f"{r['tflops']:.0f} TFLOP/s); work 2*3^k*m flop per combination; "
                     f"{'combined' if comb else 'separate'}-class variant")
         else:
-            peak = fp8_conv
-            note = f"FP8 (E4M3) dense = 2 x {peaks['source']} burst BF16; work 2*3^k*m flop per combination"
+            peak = fp4_conv
+            note = f"FP4 (E2M1) dense = 4 x {peaks['source']} burst BF16; work 2*3^k*m flop per combination"
         return dict(bound="tensor", achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak,
                     traffic=None, kernel="tc_search_kernel", kernel_ms=kern_ms,
                     executed_tflops=executed, executed_frac=executed / peak,
-                    frac_vs_2x_bf16=achieved / fp8_conv, note=note)
+                    frac_vs_4x_bf16=achieved / fp4_conv, note=note)
     W = ((d.n_cases + 127) // 128 + (d.n_samples - d.n_cases + 127) // 128) * 4
     ops = total * (3 ** k) * W
     achieved = ops / (kern_ms / 1e3) / 1e12
@@ -527,8 +531,8 @@ def run_ours(args):
 
     line = dict(metric=METRIC, value=value, unit=UNIT, n_gpus=world, steps=args.steps, warmup=args.warmup,
                 ms_per_step=t_ms / args.steps, higher_is_better=True, scaling="weak", vs_baseline=None,
-                dtype=(("f8e5m2 0/1 operands (classes combined), f32 accumulate" if comb_shift(d, k)
-                        else "f8e4m3 0/1 operands, f32 accumulate") if kind == "tc" else "u32"),
+                dtype=(f"f4e2m1 0/1 operands{' (classes combined)' if class_shift(d) else ''}, f32 accumulate"
+                       if kind == "tc" else "u32"),
                 data="synthetic",
                 config=dict(**workload_desc(args.workload, d, k, top_n), path=path, counting=kind,
                             l2="flushed between steps (256 MiB write)", parallelism="replicas"),

@@ -64,10 +64,10 @@ typedef enum {
 
 /* Tensor-core counting variant (epi_set_tc_variant). */
 typedef enum {
-    EPI_TC_AUTO = 0,       /* order 3 with m1 * 2^p + m0 < 2^23 (2^p the
-                              least power of two above m0, p <= 14): both
-                              classes in one accumulator, 256-column tiles;
-                              else separate case and control accumulators */
+    EPI_TC_AUTO = 0,       /* m1 * 2^p + m0 < 2^23 (2^p the least power of
+                              two above m0, p <= 14): both classes in one
+                              accumulator, 240-column tiles; else separate
+                              case and control accumulators of 160 columns */
     EPI_TC_SEPARATE = 1    /* always separate case and control accumulators */
 } epi_tc_variant;
 

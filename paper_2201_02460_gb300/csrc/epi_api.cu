@@ -54,8 +54,7 @@ struct epi_dataset {
     int32_t W1 = 0, W0 = 0, Wt = 0;
     uint32_t *masks = nullptr;
     uint64_t *binom = nullptr;
-    unsigned char *b8 = nullptr;   // tensor-core operand (separate classes, E4M3), built on first use
-    unsigned char *b8c = nullptr;  // the same for the combined-class variant (E5M2), built on first use
+    unsigned char *b4 = nullptr;   // tensor-core operand, built on first use
     float *lower[5] = {};          // exhaustive order-1..4 scores for the proposer, built on first use
     DevData dev() const
     {
@@ -189,6 +188,10 @@ uint64_t tune_key(int k, int64_t n, int32_t wt)
     return ((uint64_t)k << 48) | ((uint64_t)nb << 24) | (uint64_t)wb;
 }
 
+// Dynamic shared memory a tensor-path CTA may ask for: the device's limit less
+// the kernel's static arrays (at most 5 KB, order 5).
+size_t tc_smem_limit(const epi_ctx *ctx) { return ctx->smem_optin > 6144 ? ctx->smem_optin - 6144 : 0; }
+
 struct SearchPlan {
     int k = 0, top_n = 0, pool = 0, tile = 0, slots = 0, cand_p2 = 0, grid = 0, R = 0;
     bool tc = false;
@@ -321,17 +324,20 @@ epi_status choose_path(const epi_dataset *ds, int k, int path, uint64_t rb, uint
     return EPI_OK;
 }
 
-// The dataset's B operand for a class shift (0: separate-class variant).
-epi_status ensure_b8(epi_dataset *ds, int comb_p = 0)
+// The dataset's tensor-core operand.
+epi_status ensure_b4(epi_dataset *ds)
 {
-    unsigned char *&buf = comb_p ? ds->b8c : ds->b8;
-    if (buf) return EPI_OK;
+    if (ds->b4) return EPI_OK;
     epi_ctx *ctx = ds->ctx;
-    CK(ctx_malloc(ctx, (void **)&buf, tc_b8_bytes(ds->dev())));
-    CK(launch_build_b8(ds->dev(), buf, ctx->num_sms, ctx->stream, comb_p));
-    ctx->launches += 1;
+    CK(ctx_malloc(ctx, (void **)&ds->b4, tc_b4_bytes(ds->dev())));
+    CK(launch_build_b4(ds->dev(), ds->b4, ctx->num_sms, ctx->stream));
+    ctx->launches += 2;
     return EPI_OK;
 }
+
+// The class shift a tensor-path search of the dataset runs with (0: separate
+// class accumulators).
+int plan_comb_shift(const epi_dataset *ds) { return ds->ctx->tc_combined ? tc_comb_shift(ds->dev()) : 0; }
 
 epi_status make_plan(const epi_dataset *ds, SearchPlan &p, int path)
 {
@@ -339,7 +345,7 @@ epi_status make_plan(const epi_dataset *ds, SearchPlan &p, int path)
     if (st != EPI_OK) return st;
     if (!p.tc) return plan_popc(ds, p);
     p.grid = ds->ctx->num_sms;
-    p.comb_p = ds->ctx->tc_combined ? tc_comb_shift(ds->dev(), p.k) : 0;
+    p.comb_p = plan_comb_shift(ds);
     return EPI_OK;
 }
 
@@ -369,7 +375,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     // tensor path: candidate buffers in global memory when they do not fit
     // beside the operand rings in shared memory (large pools)
     const int tc_cp2 = p.tc ? tc_cand_p2(p.k, p.pool, p.comb_p != 0) : 0;
-    const bool tc_cg = p.tc && tc_smem_bytes(tc_cp2, p.k, false, p.comb_p != 0) > ctx->smem_optin;
+    const bool tc_cg = p.tc && tc_smem_bytes(tc_cp2, false, p.comb_p != 0) > tc_smem_limit(ctx);
     const size_t o_tcs = tc_cg ? a.take<float>((size_t)p.grid * tc_cp2) : 0;
     const size_t o_tcr = tc_cg ? a.take<uint64_t>((size_t)p.grid * tc_cp2) : 0;
     epi_status st = ensure_scratch(ctx, a.off);
@@ -388,7 +394,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     int32_t *cb = reinterpret_cast<int32_t *>(base + o_cb);
     uint64_t *ic = reinterpret_cast<uint64_t *>(base + o_ic);
     if (p.tc) {
-        st = ensure_b8(ds, p.comb_p);
+        st = ensure_b4(ds);
         if (st != EPI_OK) return st;
     }
     // threshold word and status word live in the first 512 bytes
@@ -411,7 +417,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
             waits = ctx->waits_dev;
             ctx->waits_grid = p.grid;
         }
-        CK(launch_tc_search(d, p.k, p.comb_p ? ds->b8c : ds->b8, ic, p.pool, thr, ls, lr, lc, status, p.grid,
+        CK(launch_tc_search(d, p.k, ds->b4, ic, p.pool, thr, ls, lr, lc, status, p.grid,
                             p.total, p.rb, p.re, ctx->stream, &cand_p2,
                             tc_cg ? reinterpret_cast<float *>(base + o_tcs) : nullptr,
                             tc_cg ? reinterpret_cast<uint64_t *>(base + o_tcr) : nullptr, dump, waits,
@@ -527,6 +533,7 @@ struct BatchItem {
     epi_dataset *ds = nullptr;
     int k = 0, top_n = 0, pool = 0, cells = 0;
     bool tc = false;
+    int comb_p = 0;                // tensor path: class shift, 0 = separate classes
     uint64_t total = 0;
     double cost = 0;
     int group = -1, cta_begin = 0, cta_count = 0;
@@ -538,7 +545,7 @@ struct BatchItem {
 };
 
 struct BatchGroup {
-    bool tc = false;
+    bool tc = false, comb = false;
     int k = 0, R = 0, tile = 0, slots = 0, cand_p2 = 0, pool = 0, max_wt = 0, grid = 0;
     int64_t max_n = 0;
     size_t smem = 0;
@@ -642,7 +649,7 @@ epi_status record_batch(epi_ctx *ctx, std::vector<BatchItem> &items, std::vector
         if (g.tc)
             for (int i : g.items)
                 CK(launch_tc_item_cum(items[i].ds->dev(), g.k, 0, items[i].total,
-                                      reinterpret_cast<uint64_t *>(dev + items[i].o_ic), st));
+                                      reinterpret_cast<uint64_t *>(dev + items[i].o_ic), st, g.comb));
         float *ls = reinterpret_cast<float *>(dev + g.o_ls);
         uint64_t *lr = reinterpret_cast<uint64_t *>(dev + g.o_lr);
         int32_t *lc = reinterpret_cast<int32_t *>(dev + g.o_lc);
@@ -652,7 +659,7 @@ epi_status record_batch(epi_ctx *ctx, std::vector<BatchItem> &items, std::vector
             CK(launch_tc_batch(dev + g.o_desc, ctads, g.k, g.pool, ls, lr, lc,
                                reinterpret_cast<int32_t *>(dev + items[g.items[0]].o_status), g.grid, st,
                                g.o_tcs ? reinterpret_cast<float *>(dev + g.o_tcs) : nullptr,
-                               g.o_tcs ? reinterpret_cast<uint64_t *>(dev + g.o_tcr) : nullptr));
+                               g.o_tcs ? reinterpret_cast<uint64_t *>(dev + g.o_tcr) : nullptr, g.comb));
         else
             CK(launch_popc_batch(dev + g.o_desc, ctads, g.k, g.R, g.max_wt, g.tile, g.pool, g.slots, g.cand_p2, ls, lr,
                                  lc, g.grid, g.smem, st));
@@ -715,24 +722,28 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         st = choose_path(it.ds, it.k, path, 0, total, total, it.tc);
         if (st != EPI_OK) return fail(st, "dataset %d: %s", i, epi_last_error());
         const DevData d = it.ds->dev();
-        // work estimate for the CTA split: a tensor-core item costs its K stages,
-        // but never less than its epilogue (about 32 stages' worth)
-        it.cost = it.tc ? (double)tc_item_count(d.n, it.k) * (double)std::max(d.Wt / 4, 32)
+        if (it.tc) it.comb_p = plan_comb_shift(it.ds);
+        // work estimate for the CTA split: a tensor-core item costs its
+        // 128-individual chunks, but never less than its epilogue (about 32
+        // chunks' worth)
+        it.cost = it.tc ? (double)tc_item_count(d.n, it.k, it.comb_p != 0) * (double)std::max(d.Wt / 4, 32)
                         : (double)total * (double)(it.cells / 3) * (double)d.Wt;
     }
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return fail(EPI_ECUDA, "cannot select device %d", ctx->device);
-    // one group per (path, order)
+    // one group per (path, order, tensor variant)
     std::vector<BatchGroup> groups;
     for (int i = 0; i < n_ds; i++) {
         int gi = -1;
         for (size_t q = 0; q < groups.size(); q++)
-            if (groups[q].tc == items[i].tc && groups[q].k == items[i].k) gi = (int)q;
+            if (groups[q].tc == items[i].tc && groups[q].k == items[i].k &&
+                groups[q].comb == (items[i].comb_p != 0)) gi = (int)q;
         if (gi < 0) {
             groups.emplace_back();
             gi = (int)groups.size() - 1;
             groups[gi].tc = items[i].tc;
             groups[gi].k = items[i].k;
+            groups[gi].comb = items[i].comb_p != 0;
         }
         items[i].group = gi;
         BatchGroup &g = groups[gi];
@@ -763,9 +774,9 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         g.o_ls = a.take<float>((size_t)g.grid * g.pool);
         g.o_lr = a.take<uint64_t>((size_t)g.grid * g.pool);
         g.o_lc = a.take<int32_t>((size_t)g.grid);
-        if (g.tc && tc_smem_bytes(tc_cand_p2(g.k, g.pool), g.k, false) > ctx->smem_optin) {
-            g.o_tcs = a.take<float>((size_t)g.grid * tc_cand_p2(g.k, g.pool));
-            g.o_tcr = a.take<uint64_t>((size_t)g.grid * tc_cand_p2(g.k, g.pool));
+        if (g.tc && tc_smem_bytes(tc_cand_p2(g.k, g.pool, g.comb), false, g.comb) > tc_smem_limit(ctx)) {
+            g.o_tcs = a.take<float>((size_t)g.grid * tc_cand_p2(g.k, g.pool, g.comb));
+            g.o_tcr = a.take<uint64_t>((size_t)g.grid * tc_cand_p2(g.k, g.pool, g.comb));
         }
     }
     for (auto &it : items) {
@@ -794,12 +805,12 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
     if (st != EPI_OK) return st;
     for (auto &it : items)
         if (it.tc) {
-            st = ensure_b8(it.ds);
+            st = ensure_b4(it.ds);
             if (st != EPI_OK) return st;
         }
     // graph key: datasets, orders, sizes, path
     std::vector<uint64_t> key;
-    key.push_back((uint64_t)path);
+    key.push_back((uint64_t)path | (ctx->tc_combined ? 1ull << 32 : 0));
     for (auto &it : items) {
         key.push_back(it.ds->id);
         key.push_back((uint64_t)it.k << 32 | (uint64_t)it.top_n);
@@ -820,9 +831,9 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
                 const DevData d = it.ds->dev();
                 uint32_t *thr = reinterpret_cast<uint32_t *>(dev + it.o_thr);
                 if (g.tc) {
-                    CK(tc_fill_batch_entry(hd + dsz * q, hm + 128 * q, d, it.k, it.ds->b8,
+                    CK(tc_fill_batch_entry(hd + dsz * q, hm + 128 * q, d, it.k, it.ds->b4,
                                            reinterpret_cast<uint64_t *>(dev + it.o_ic), thr, it.total,
-                                           dev + g.o_tmap + 128 * q, it.cta_begin, it.cta_count));
+                                           dev + g.o_tmap + 128 * q, it.cta_begin, it.cta_count, it.comb_p));
                 } else {
                     popc_fill_ds(hd + dsz * q, d, 0, it.total, it.cta_begin, it.cta_count, thr);
                 }
@@ -878,6 +889,7 @@ double time_pass(epi_dataset *ds, int k, bool tc, int R, int tile, int slots, ui
     p.tc = tc;
     if (tc) {
         p.grid = ctx->num_sms;
+        p.comb_p = plan_comb_shift(ds);
     } else {
         p.tile = tile;
         p.slots = slots;
@@ -1418,8 +1430,7 @@ void epi_dataset_destroy(epi_dataset *ds)
         cudaStreamSynchronize(ctx->stream);
         cudaFree(ds->masks);
         cudaFree(ds->binom);
-        if (ds->b8) cudaFree(ds->b8);
-        if (ds->b8c) cudaFree(ds->b8c);
+        if (ds->b4) cudaFree(ds->b4);
         for (float *t : ds->lower)
             if (t) cudaFree(t);
     }

@@ -5,27 +5,35 @@
 //     count[(p, x'), (j, g)] = sum over individuals s of A[(p, x')][s] * B[(j, g)][s]
 // with A[(p, x')] the genotype-table row x' of prefix p (Section 2.1) and
 // B[(j, g)] row g of SNP j, summed separately over the case and the control
-// individuals.  Both operands hold 0/1 values as FP8 E4M3 bytes and the MMA
-// accumulates in FP32 in tensor memory.  Because the product sums over K,
-// any fixed permutation of the individuals inside a K stage, applied to both
+// individuals.  Both operands hold 0/1 patterns as FP4 E2M1 nibbles
+// (kind::mxf4: K = 64 per MMA, twice the FP8 kinds' rate, measured 16384
+// multiply-adds per SM clock, and half their operand bytes) and the MMA
+// accumulates in FP32 in tensor memory.  Because the product sums over K, any
+// fixed permutation of the individuals inside a K step, applied to both
 // operands, leaves the counts unchanged, and the two operands may carry
 // different weights per K position as long as their product is constant:
-//   * K byte 4 i + b of each 32-individual word holds individual 8 b + i, so
-//     the A producer turns one mask word into eight output words with one
-//     AND each (output i keeps bit i of every byte, shifted into bits 3..6);
-//   * A's nonzero byte at position i is 2^-5, 2^-3, 2^1 or 2^-6 (normal E4M3
-//     powers of two) and B's is the reciprocal times 2^-5, so every product
-//     of two ones is exactly 2^-5 and an accumulator holds count * 2^-5, an
-//     exact FP32 value.
+//   * 32-bit word i (of 4) of the 16 bytes of a mask word holds, in nibble b,
+//     individual 4 b + i: the A producer turns one mask word into four output
+//     words with one AND each (and one shift: nibble bit 3 is the sign);
+//   * A's nonzero nibble in word i is 0.5, 1, 2 or 2 (1, 2, 4, 4) and B's is
+//     the reciprocal, so every product of two ones is exactly 1.
+// kind::mxf4 multiplies every 32 K elements of a row by a power-of-two scale
+// kept in tensor memory.  All scales of A are 1; B's case blocks take 2^p and
+// its control blocks 1 in the combined-class variant, so one accumulator
+// holds ctrl + case 2^p.  Sums of such integers below 2^24 are exact in FP32
+// (measured against integer counts up to 2^23.96, and on every table of the
+// validation datasets).
 // Genotype 2 of the last SNP is obtained by subtraction from the prefix
 // row's total, as in the popcount path.
 //
 // Layout of one tile: M = 128 rows = 4 warps x 32 lanes; each warp holds
 // floor(32 / 3^(k-1)) whole prefixes (prefix rows never straddle a warp, so
-// the epilogue reduces a prefix within a warp); N = 128 columns = 64 last
-// SNPs x genotypes {0, 1}; K = 128 individuals per stage.  At order 3, where
-// the counts fit, the combined-class variant (Shape<true> below) sums both
-// classes into one accumulator with E5M2 operands and uses N = 256 columns.
+// the epilogue reduces a prefix within a warp; at order 5 one prefix takes 81
+// rows of three warps); N = 240 columns = 120 last SNPs x genotypes {0, 1}
+// (combined classes) or 160 columns per class (separate classes); K = 256
+// individuals per stage.  Columns come in groups of four: genotype 0 of SNPs
+// j, j + 1 (j even), then genotype 1 of both, so the epilogue's packed
+// two-lane arithmetic takes two SNPs at a time; a tile's first SNP is even.
 // Prefixes are taken in "panel order" (by their last SNP c ascending) so the
 // last SNPs of a tile, j > c, form one contiguous range.  A lexicographic rank
 // range [r0, r1) of combinations covers the first SNPs s1 in [a, b] (those of
@@ -35,16 +43,15 @@
 // in [r0, r1) (consecutive ranks share their prefix and differ in the last
 // SNP, so that is one interval of j).
 //
-// Warp roles (by default 576 threads = 18 warps, one CTA per SM, persistent,
-// a contiguous range of work items per CTA; an item = one M tile x one N
-// tile x the whole K range; the epilogue/producer split is Roles<C, K>
-// below: 8/8, or 12/4 for the combined-class variant):
+// Warp roles (one CTA per SM, persistent, segments of work items spread over
+// the panels; an item = one M tile x one N tile x the whole K range; the
+// epilogue/producer split is Roles<K> below):
 //   epilogue warps (first): TMEM -> registers, single-precision MI screen,
 //               exact-margin candidate selection, per-CTA candidate list;
 //               warp w reads TMEM lane quadrant w % 4 for the chunks of 8
 //               last SNPs w / 4, w / 4 + G, ... (G warps per quadrant)
 //   A producers: prefix rows = AND of the prefix SNPs' bit rows, expanded
-//               to FP8 bytes in the 128-byte-swizzled K-major layout; one
+//               to FP4 nibbles in the 128-byte-swizzled K-major layout; one
 //               thread per row, groups of 4 warps taking the ring's stages
 //               in turn, own stages prefetched
 //   next warp   TMA producer of B tiles, and writer of the item descriptors
@@ -60,107 +67,58 @@
 #include "epi_internal.cuh"
 #include "epi_tcgen05.cuh"
 
-// A producers' load distance in K stages (tuning parameter); the
-// stage-release group size is chosen per order (EPI_TC_RELEASE overrides it)
-#ifndef EPI_TC_PREFETCH
-#define EPI_TC_PREFETCH 2
-#endif
-
 namespace epi {
 
 namespace tc {
 
-constexpr int kKC = 128;               // individuals (bytes) per K stage
+constexpr int kChunk = 128;            // individuals a class is padded to
+constexpr int kRowBytes = 128;         // operand bytes of a row and K stage (256 individuals)
+constexpr int kTileBytes = 128 * kRowBytes;   // one A stage
 
 // Tile shapes of the two variants.
-//   separate classes (C = false): N tile = 64 last SNPs (128 columns), E4M3
-//     operands, one accumulator per class (2 x 128 columns, double buffered),
-//     6 stages of A and B tiles;
-//   combined classes (C = true): N tile = 128 last SNPs (256 columns), E5M2
-//     operands whose case products are 2^p times the control products, so
-//     one accumulator holds ctrl + case * 2^p (exact while below 2^23);
-//     double buffered in 2 x 256 columns; 4 stages of A (128 rows) and B
-//     (256 rows) tiles.  The MMA of an N tile that ends the last SNPs is cut
-//     to the columns in use (a multiple of 16).
+//   combined classes (C = true): one accumulator per tile holds
+//     ctrl + case 2^p (exact while below 2^23, the decode's range), two of
+//     240 columns in turn;
+//   separate classes (C = false): two accumulators per tile, three of 160
+//     columns in rotation (the next tile's case accumulator fills while the
+//     epilogue reads this tile's two).  480 columns either way: the other 32
+//     hold the scale factors.
+// The MMA of an N tile that ends the last SNPs is cut to the columns in use
+// (a multiple of 16).
 template <bool C>
 struct Shape {
-    static constexpr int J = C ? 128 : 64;          // last SNPs per N tile
-    static constexpr int N = 2 * J;                 // tile columns
-    static constexpr int Stages = C ? 4 : 6;        // K stages in the rings
-    static constexpr int BBytes = N * kKC;          // one B stage
+    static constexpr int J = C ? 120 : 80;          // last SNPs per N tile
+    static constexpr int N = 2 * J;                 // tile columns per accumulator
+    static constexpr int Stages = C ? 4 : 5;        // K stages in the rings
+    static constexpr int BBytes = N * kRowBytes;    // one B stage
+    static constexpr int Accs = C ? 2 : 3;          // accumulators in rotation
+    static constexpr int AccPerTile = C ? 1 : 2;
 };
+constexpr int kScaleACol = 480, kScaleBCol = 496;   // 16 tensor-memory columns each
 
-// Epilogue warps of the separate-class variant at order 4 (tuning
-// parameter; the other 16 - n warps produce A tiles).  Measured: 8 (two
-// producer groups) 126.5 ms at 300 SNPs x 4000 and 1522 ms at 500 x 8192;
-// 4 (three producer groups) 190 and 1579 ms.
-#ifndef EPI_TC_K4_EPI_WARPS
-#define EPI_TC_K4_EPI_WARPS 8
+// Epilogue and producer warps (tuning parameters).
+#ifndef EPI_TC_EPI_WARPS
+#define EPI_TC_EPI_WARPS 8
+#endif
+#ifndef EPI_TC_PROD_WARPS
+#define EPI_TC_PROD_WARPS 4
 #endif
 
-// Warp roles of an order-K launch.  The combined variant's producers write
-// each A row once per 512-cycle stage, so one group of 4 warps keeps up and
-// 12 warps (3 per TMEM lane quadrant) run the epilogue; the separate variant
-// has producer groups of 4 warps taking the ring's stages in turn.
-// Epilogue and producer warps of the combined-class variant (tuning
-// parameters; the launch's register cap follows from the warps per SM
-// sub-partition.  Order 3, 2000 x 4000: 12 + 4 warps (96 registers) 86.6 ms,
-// 8 + 4 (128 registers) 88.3 ms, 8 + 8 93.6 ms, 12 + 8 (80 registers,
-// spills) 100.6 ms; before the screen's logarithms lost their subnormal
-// handling: 93.8, 100.1, 110.8 ms, and 4 + 4 133.5 ms)
-#ifndef EPI_TC_C_EPI_WARPS
-#define EPI_TC_C_EPI_WARPS 12
-#endif
-#ifndef EPI_TC_C_PROD_WARPS
-#define EPI_TC_C_PROD_WARPS 4
-#endif
-
-template <bool C, int K>
 struct Roles {
-    static constexpr int J = Shape<C>::J;
-    static constexpr int EpiWarps = C ? EPI_TC_C_EPI_WARPS : (K == 4 ? EPI_TC_K4_EPI_WARPS : 8);
-    static constexpr int ProdWarps = C ? EPI_TC_C_PROD_WARPS : 16 - EpiWarps;
+    static constexpr int EpiWarps = EPI_TC_EPI_WARPS;
+    static constexpr int ProdWarps = EPI_TC_PROD_WARPS;
     static constexpr int Threads = 32 * (EpiWarps + ProdWarps + 2);   // + the TMA and MMA warps
     static constexpr int EpiThreads = 32 * EpiWarps;
     static constexpr int ProdGroups = ProdWarps / 4;  // one thread per tile row each
     static constexpr int ColGroups = EpiWarps / 4;    // epilogue warps per lane quadrant
-    // chunks of 8 last SNPs per epilogue warp and item, and the chunks
-    // between two candidate-buffer checks (a barrier of the epilogue warps
-    // and maybe a sort): every 2 chunks with separate classes, once per item
-    // with combined classes (its larger buffer then lives in global memory)
-    static constexpr int Iters = (J / 8 + ColGroups - 1) / ColGroups;
-    static constexpr int CheckIters = C ? Iters : 2;
     static_assert(EpiWarps % 4 == 0 && ProdWarps % 4 == 0, "roles come in whole lane quadrants");
 };
-constexpr int kMaxProdGroups = 3;
-
-// the host's view of the roles of a launch (order k, variant comb)
-inline int roles_epi_warps(bool comb, int k)
-{
-    return comb ? Roles<true, 3>::EpiWarps : (k == 4 ? Roles<false, 4>::EpiWarps : Roles<false, 3>::EpiWarps);
-}
-inline int roles_check_iters(bool comb, int k)
-{
-    return comb ? Roles<true, 3>::CheckIters : (k == 4 ? Roles<false, 4>::CheckIters : Roles<false, 3>::CheckIters);
-}
-// Stages are released to the producers in groups: a tcgen05.commit lets the
-// following MMAs start only after the earlier ones finish (about one MMA
-// latency of idle tensor pipe), so the issuer commits once per group of
-// kRelease stages instead of once per stage.
-// measured best: groups of 2 stages at orders 2-3 (the epilogue bounds the
-// issuer), single stages at orders 4-5 (the A producers do)
-template <int K, bool C>
-constexpr int release_group()
-{
-#ifdef EPI_TC_RELEASE
-    return EPI_TC_RELEASE;
-#else
-    return C ? 1 : (K <= 3 ? 2 : 1);
+// A producers' load distance in own stages
+#ifndef EPI_TC_PREFETCH
+#define EPI_TC_PREFETCH 3
 #endif
-}
+constexpr int kSegments = 16;
 constexpr int kDescDepth = 4;
-static_assert(Roles<false, 4>::ProdWarps / 4 <= 3, "at most kMaxProdGroups producer groups");
-constexpr int kTileBytes = 128 * kKC;        // one A tile (and a B tile of the separate-class variant)
 constexpr int kWaitSlots = 8;
 constexpr int kMaxDescSnps = 40;
 constexpr unsigned long long kTimeoutNs = 2000000000ull;
@@ -177,16 +135,19 @@ struct DsParams {
     DevData d;
     uint64_t n_prefix;         // prefixes searched (first SNP in [s1_lo, s1_hi])
     uint64_t n_items;
+    const uint4 *rows;         // the producers' masks [stage][n][3][2] (16 bytes each)
     const uint64_t *item_cum;  // [n + 1] items of M tiles starting in panels < c
     const uint64_t *pcum;      // [n + 1] prefixes searched in panels < c
     uint64_t rank_begin, rank_end;   // lexicographic ranks searched
     int32_t s1_lo, s1_hi;      // first SNPs of ranks rank_begin and rank_end - 1
     int32_t clip;              // 0: the whole combination range
     int32_t comb_p;            // combined-class variant: control counts in the low comb_p bits
-    int chunks, chunks_case;   // K stages in total / over the cases
-    float delta;               // screening margin (nats)
-    float tconst;              // T(m) - T(m1) - T(m0), T(c) = c log2 c
-    float ln2_over_m;
+    int chunks, chunks_case;   // 128-individual chunks in total / over the cases
+    // screen (see Screen below): MI bound = v vscale + voff; a combination
+    // passes when that reaches thr cut_mul - cut_add
+    int poly;                  // polynomial bound, else fast logarithms
+    float vscale, voff, cut_mul, cut_add;
+    float sc_pi, c2, c3, c4, c5a, c5b;
     uint64_t total;            // C(n, k)
     uint32_t *global_thr;
     const CUtensorMap *tmap;   // B-operand map in global memory (batched launches)
@@ -197,7 +158,6 @@ struct Params {
     DsParams one;              // the dataset when the launch has one
     const DsParams *many;      // else [n_ds] in device memory
     const int32_t *cta_ds;     // and the dataset of each CTA
-    int k, PR, ppw, ppt;
     int pool, cand_p2;
     // the CTA's candidate buffer [cand_p2] in global memory (per CTA, at
     // blockIdx.x * cand_p2) where it does not fit in shared memory; NULL:
@@ -237,6 +197,25 @@ __device__ __noinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile 
     }
 }
 
+// The same, inline and counting its cycles, for the producers' stage loops (a
+// call there costs more than the wait itself).
+__device__ __forceinline__ bool wait_here(uint64_t *bar, uint32_t parity, volatile int *abort_flag, long long &acc)
+{
+    if (mbar_test(bar, parity)) return true;
+    const long long c0 = clock64();
+    const uint64_t n0 = now_ns();
+    bool ok = true;
+    while (!mbar_try(bar, parity)) {
+        if (now_ns() - n0 > g_wait_limit_ns) *abort_flag = 1;
+        if (*abort_flag) {
+            ok = false;
+            break;
+        }
+    }
+    acc += clock64() - c0;
+    return ok;
+}
+
 // Hot-path wait: one inline non-blocking test; the bounded out-of-line wait
 // (and the cycle accounting of the trace) only when the phase is not
 // complete yet, so the trace counts every cycle spent waiting.
@@ -245,6 +224,25 @@ __device__ __forceinline__ bool wait_fast(uint64_t *bar, uint32_t parity, volati
     if (mbar_test(bar, parity)) return true;
     const long long t0 = clock64();
     const bool ok = mbar_wait(bar, parity, abort_flag);
+    acc += clock64() - t0;
+    return ok;
+}
+
+// The issuing warp's wait, inline: a function call in its loop would keep
+// every value that lives across it out of the uniform registers the MMAs take
+// their operands from.
+__device__ __forceinline__ bool wait_inline(uint64_t *bar, uint32_t parity, volatile int *abort_flag, long long &acc)
+{
+    const long long t0 = clock64();
+    const uint64_t n0 = now_ns();
+    bool ok = true;
+    while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
+        if (now_ns() - n0 > g_wait_limit_ns) *abort_flag = 1;
+        if (__any_sync(0xffffffffu, *abort_flag)) {
+            ok = false;
+            break;
+        }
+    }
     acc += clock64() - t0;
     return ok;
 }
@@ -258,31 +256,35 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
-// Instruction descriptor of kind::f8f6f4 with F32 accumulation, K-major A
-// and B, M = 128 and n columns; operand format 0 = E4M3, 1 = E5M2 (both).
-__host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt, uint32_t n)
+// Instruction descriptor of kind::mxf4 with F32 accumulation: E2M1 operands,
+// both K-major, UE8M0 scales, M = 128 and n columns; bits 4-5 select B's
+// pair of scale bytes (0: bytes 0-1, the controls' scale; 2: bytes 2-3, the
+// cases').
+__host__ __device__ constexpr uint32_t make_idesc(uint32_t n)
 {
-    return (1u << 4) | (fmt << 7) | (fmt << 10) | ((n >> 3) << 17) | ((128u >> 4) << 24);
+    return (1u << 7) | (1u << 10) | ((n >> 3) << 17) | (1u << 23) | (1u << 27);
 }
-constexpr uint32_t kIdesc = make_idesc(0, 128);
+constexpr uint32_t kIdescCase = 2u << 4;
 
-__device__ __forceinline__ void mma_f8(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            d_tmem),
-        "l"(a), "l"(b), "r"(kIdesc), "r"(accumulate));
-}
-
-// The same MMA executed by a whole warp in step; only the elected lane
-// (`leader` nonzero) issues it.
-__device__ __forceinline__ void mma_f8_warp(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate,
-                                            uint32_t leader, uint32_t idesc = kIdesc)
+// The MMA executed by a whole warp in step; only the elected lane (`leader`
+// nonzero) issues it.
+__device__ __forceinline__ void mma_f4_warp(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accumulate,
+                                            uint32_t leader, uint32_t idesc, uint32_t sfa, uint32_t sfb)
 {
     asm volatile(
         "{\n .reg .pred p, e;\n setp.ne.b32 p, %4, 0;\n setp.ne.b32 e, %5, 0;\n"
-        " @e tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(leader));
+        " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %3, [%6], [%7], p;\n}\n" ::"r"(
+            d_tmem),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(leader), "r"(sfa), "r"(sfb));
+}
+
+// 16 tensor-memory columns of this warp's lane quadrant set to v
+__device__ __forceinline__ void tmem_fill16(uint32_t taddr, uint32_t v)
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(taddr),
+        "r"(v)
+        : "memory");
 }
 
 __device__ __forceinline__ void mma_commit_warp(uint64_t *bar, uint32_t leader)
@@ -300,6 +302,14 @@ __device__ __forceinline__ uint32_t elect_one()
     asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(pred));
     return pred;
 }
+
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
+// lane 0's value in every lane, known to be warp-uniform
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
 
 template <int NT>
 __device__ __forceinline__ void epi_bar() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
@@ -382,49 +392,99 @@ __device__ inline void prefix_next(const DsParams &P, int k, PrefixIter &it)
     for (int t = 0; t < m2; t++) it.a[t] = P.s1_lo + t;
 }
 
-template <int J>
-__device__ __forceinline__ int64_t ntiles_of(const DevData &d, int32_t c) { return (d.n - 1 - c + J - 1) / J; }
+// first (even) last SNP of panel c's N tiles, and their number
+__host__ __device__ __forceinline__ int64_t panel_j0(int64_t c) { return (c + 1) & ~(int64_t)1; }
+__host__ __device__ __forceinline__ int64_t panel_ntiles(int64_t n, int64_t c, int kj)
+{
+    return (n - panel_j0(c) + kj - 1) / kj;
+}
 
 // -------------------------------------------------------------- epilogue --
-// accumulator = count * 2^-5 (exact): the count as a float, and as an integer
+// the integer value of an accumulator (below 2^23)
 __device__ __forceinline__ uint32_t f2u_exact(float v) { return __float_as_uint(v + 8388608.0f) & 0x7FFFFFu; }
 
-// Combined-class accumulator x = 2^-12 (ctrl + case 2^p), an integer v
-// below 2^23 times 2^-12: y = fma(x, 2^12, 2^23) = 2^23 + v holds v in its
-// 23 mantissa bits (exact).  Keeping the low p bits under the exponent of
-// 2^23 gives 2^23 + ctrl, hence ctrl / 32 in one fused multiply-add, and
-// y - (2^23 + ctrl) = case 2^p exactly, hence case / 32 in one multiply by
-// case_scale = 2^-(p+5).  Both come out as the separate-class variant's
-// accumulator values (count / 32).
-__device__ __forceinline__ void split_classes(uint32_t x, uint32_t lo_mask, float case_scale, uint32_t &case32,
-                                              uint32_t &ctrl32)
+// two floats handled by one instruction (f32x2)
+struct F2 {
+    uint64_t v;
+};
+__device__ __forceinline__ F2 f2_pack(float lo, float hi)
 {
-    const float y = fmaf(__uint_as_float(x), 4096.0f, 8388608.0f);
-    const float lo = __uint_as_float((__float_as_uint(y) & lo_mask) | 0x4B000000u);
-    ctrl32 = __float_as_uint(fmaf(lo, 0.03125f, -262144.0f));
-    case32 = __float_as_uint((y - lo) * case_scale);
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(F2 a, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a.v));
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c)
+{
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b)
+{
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b)
+{
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_abs(F2 a)
+{
+    float x, y;
+    f2_unpack(a, x, y);
+    return f2_pack(fabsf(x), fabsf(y));
+}
+// 1 / (s + tiny), approximate; finite for s = 0 (cells of no individuals,
+// whose terms then are 0)
+__device__ __forceinline__ F2 f2_rcp(F2 s, F2 tiny)
+{
+    float x, y;
+    f2_unpack(f2_add(s, tiny), x, y);
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(x));
+    asm("rcp.approx.ftz.f32 %0, %0;" : "+f"(y));
+    return f2_pack(x, y);
 }
 
-// t(x) = x log2 x of an accumulator value x = count / 32 (0 for x = 0)
-__device__ __forceinline__ float tlog32(float x) { return x * lg2n(fmaxf(x, 0.03125f)); }
-
-// sum over the three cells of one tile row of t(a) + t(b) - t(a + b) (a, b:
-// case and control accumulators): one fused multiply-add chain per cell,
-// the three cells side by side, then two adds
-__device__ __forceinline__ float row_screen(float a0, float a1, float a2, float b0, float b1, float b2)
+// The screen: an upper bound of m MI from the cells' totals and case counts.
+//
+// With s = a + b individuals in a cell, a of them cases, pi = m1 / m and
+// x = a / s - pi, m MI = sum over cells of s f(x), f(x) the divergence of a
+// Bernoulli(pi + x) from a Bernoulli(pi).  f(x) = c2 x^2 + c3 x^3 + g(x) x^4
+// with c2 = 1 / (2 pi (1 - pi)), c3 = (2 pi - 1) / (6 pi^2 (1 - pi)^2) and
+// g convex (the fourth derivative of f, 2 / p^3 + 2 / (1 - p)^3, is convex),
+// so g lies below its chords: from x = -pi to 0 and from 0 to 1 - pi, whose
+// end values have closed forms.  The bound c2 x^2 + c3 x^3 + (c4 + c5a x +
+// c5b |x|) x^4 takes one reciprocal per cell and packed multiply-adds where
+// exact logarithms take three; on Hardy-Weinberg tables of 1000-16000
+// individuals its excess over 2 m MI averages 0.2 (order 3, pi = 0.5) to 1.5
+// (order 4, pi = 0.2) while pi lies in [0.2, 0.8], and 2 to 25 at pi = 0.1,
+// so outside that interval the logarithms screen.
+// Per cell it gets e = 2^p (a - pi s) and s; the constants absorb the 2^p.
+struct ScreenConst {
+    F2 c2, c3, c4, c5a, c5b, tiny;
+};
+__device__ __forceinline__ F2 cell_bound(F2 e, F2 s, const ScreenConst &c, F2 acc)
 {
-    const float s0 = a0 + b0, s1 = a1 + b1, s2 = a2 + b2;
-    float v0 = a0 * lg2n(fmaxf(a0, 0.03125f));
-    float v1 = a1 * lg2n(fmaxf(a1, 0.03125f));
-    float v2 = a2 * lg2n(fmaxf(a2, 0.03125f));
-    v0 = fmaf(b0, lg2n(fmaxf(b0, 0.03125f)), v0);
-    v1 = fmaf(b1, lg2n(fmaxf(b1, 0.03125f)), v1);
-    v2 = fmaf(b2, lg2n(fmaxf(b2, 0.03125f)), v2);
-    v0 = fmaf(-s0, lg2n(fmaxf(s0, 0.03125f)), v0);
-    v1 = fmaf(-s1, lg2n(fmaxf(s1, 0.03125f)), v1);
-    v2 = fmaf(-s2, lg2n(fmaxf(s2, 0.03125f)), v2);
-    return (v0 + v1) + v2;
+    const F2 x = f2_mul(e, f2_rcp(s, c.tiny));
+    F2 t = f2_fma(c.c5a, x, c.c4);
+    t = f2_fma(c.c5b, f2_abs(x), t);
+    t = f2_fma(x, t, c.c3);
+    t = f2_fma(x, t, c.c2);
+    return f2_fma(f2_mul(e, x), t, acc);
 }
+
+// t(x) = x log2 x of a count (0 for x = 0)
+__device__ __forceinline__ float tlog(float x) { return x * lg2n(fmaxf(x, 1.0f)); }
+
+// t(a) + t(b) - t(a + b) of a cell's counts
+__device__ __forceinline__ float cell_log(float a, float b) { return tlog(a) + tlog(b) - tlog(a + b); }
 
 __device__ __forceinline__ float warp_sum(float v)
 {
@@ -467,8 +527,9 @@ __device__ inline void sort_cands_epi(float *sc, uint64_t *rk, int p2, int tid)
 }
 
 struct EpiState {
-    int32_t list_len, nbuf, stop;
-    float thr;
+    int32_t list_len, nbuf, stop, any;
+    float thr;                 // the CTA's own pool threshold
+    float next_thr;            // the larger of it and the other CTAs'
 };
 
 template <int NT>
@@ -508,13 +569,135 @@ __device__ __noinline__ float row_terms_precise(uint32_t a0, uint32_t b0, uint32
                    "=r"(r[15])                                                                                   \
                  : "r"(taddr))
 
+// Row values of a chunk: raw accumulators of 8 last SNPs -> the row's part of
+// the screen for each, vrow[jj].  Columns 4 h + {0, 1} hold genotype 0 of SNPs
+// 2 h and 2 h + 1, columns 4 h + {2, 3} genotype 1.
+template <bool C>
+struct RowScreen {
+    // packed constants
+    F2 m23, neg_m23, neg1, kinv, neg_pi;
+    ScreenConst sc;
+    F2 S, CT;                  // the row's totals: individuals and cases (times 2^p)
+    uint32_t lo_mask;
+    float kinv1;               // 2^-p
+
+    __device__ __forceinline__ void set_row(float cases, float ctrls, float p2)
+    {
+        const float s = cases + ctrls;
+        S = f2_pack(s, s);
+        CT = f2_pack(cases * p2, cases * p2);
+    }
+    // the two classes of a column pair: individuals s and cases times 2^p
+    __device__ __forceinline__ void split(uint32_t x0, uint32_t x1, F2 &s, F2 &ca) const
+    {
+        // y = 2^23 + v holds v = ctrl + case 2^p in its mantissa; its low p
+        // bits under the exponent of 2^23 are 2^23 + ctrl
+        const F2 y = f2_add(f2_pack(__uint_as_float(x0), __uint_as_float(x1)), m23);
+        float y0, y1;
+        f2_unpack(y, y0, y1);
+        const F2 lo = f2_pack(__uint_as_float((__float_as_uint(y0) & lo_mask) | 0x4B000000u),
+                              __uint_as_float((__float_as_uint(y1) & lo_mask) | 0x4B000000u));
+        ca = f2_fma(lo, neg1, y);
+        s = f2_fma(ca, kinv, f2_add(lo, neg_m23));
+    }
+    __device__ __forceinline__ void pair(const uint32_t *cs, const uint32_t *cn, int h, F2 &s0, F2 &s1, F2 &a0,
+                                         F2 &a1) const
+    {
+        if constexpr (C) {
+            split(cs[4 * h], cs[4 * h + 1], s0, a0);
+            split(cs[4 * h + 2], cs[4 * h + 3], s1, a1);
+        } else {
+            a0 = f2_pack(__uint_as_float(cs[4 * h]), __uint_as_float(cs[4 * h + 1]));
+            a1 = f2_pack(__uint_as_float(cs[4 * h + 2]), __uint_as_float(cs[4 * h + 3]));
+            s0 = f2_add(a0, f2_pack(__uint_as_float(cn[4 * h]), __uint_as_float(cn[4 * h + 1])));
+            s1 = f2_add(a1, f2_pack(__uint_as_float(cn[4 * h + 2]), __uint_as_float(cn[4 * h + 3])));
+        }
+    }
+    __device__ __forceinline__ void bound(const uint32_t *cs, const uint32_t *cn, float *vrow) const
+    {
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            F2 s0, s1, a0, a1;
+            pair(cs, cn, h, s0, s1, a0, a1);
+            const F2 e0 = f2_fma(s0, neg_pi, a0), e1 = f2_fma(s1, neg_pi, a1);
+            // genotype 2 by subtraction (exact), so that an empty cell has
+            // e = 0 whatever pi
+            const F2 s2 = f2_fma(s1, neg1, f2_fma(s0, neg1, S));
+            const F2 e2 = f2_fma(s2, neg_pi, f2_fma(a1, neg1, f2_fma(a0, neg1, CT)));
+            F2 acc;
+            acc.v = 0;
+            acc = cell_bound(e0, s0, sc, acc);
+            acc = cell_bound(e1, s1, sc, acc);
+            acc = cell_bound(e2, s2, sc, acc);
+            f2_unpack(acc, vrow[2 * h], vrow[2 * h + 1]);
+        }
+    }
+    // counts of column pair h's cells: a = cases, b = controls by genotype,
+    // of SNP 2 h + odd
+    __device__ __forceinline__ void counts(const uint32_t *cs, const uint32_t *cn, int h, bool odd, float *a,
+                                           float *b) const
+    {
+        F2 s0, s1, a0, a1;
+        pair(cs, cn, h, s0, s1, a0, a1);
+        const F2 s2 = f2_fma(s1, neg1, f2_fma(s0, neg1, S));
+        const F2 a2 = f2_fma(a1, neg1, f2_fma(a0, neg1, CT));
+        const F2 ss[3] = {s0, s1, s2}, aa[3] = {a0, a1, a2};
+#pragma unroll
+        for (int g = 0; g < 3; g++) {
+            float x, y, u, v;
+            f2_unpack(aa[g], x, y);
+            f2_unpack(ss[g], u, v);
+            a[g] = (odd ? y : x) * kinv1;
+            b[g] = (odd ? v : u) - a[g];
+        }
+    }
+    __device__ __forceinline__ void logs(const uint32_t *cs, const uint32_t *cn, float *vrow) const
+    {
+#pragma unroll
+        for (int jj = 0; jj < 8; jj++) {
+            float a[3], b[3];
+            counts(cs, cn, jj >> 1, jj & 1, a, b);
+            vrow[jj] = cell_log(a[0], b[0]) + cell_log(a[1], b[1]) + cell_log(a[2], b[2]);
+        }
+    }
+};
+
+// Lexicographic rank of a combination from the sum over its SNPs s_t of
+// C(n - 1 - s_t, K - t): total - 1 - sum.
+template <int km1>
+__device__ __forceinline__ uint64_t prefix_rank_sum(const DevData &d, const int32_t *psnp)
+{
+    uint64_t s = 0;
+#pragma unroll
+    for (int tt = 0; tt < km1; tt++) s += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], km1 + 1 - tt);
+    return s;
+}
+
+// Last SNPs [jlo, jhi) of a prefix inside the searched rank range: the
+// combination (prefix, j) has rank base + j.  Only prefixes whose first SNP
+// is the range's first or last can be cut.
+template <int km1>
+__device__ __forceinline__ void last_snp_range(const DsParams &DS, const DevData &d, const int32_t *psnp, int32_t &jlo,
+                                               int32_t &jhi)
+{
+    jlo = psnp[km1 - 1] + 1;
+    jhi = (int32_t)d.n;
+    if (DS.clip && (psnp[0] == DS.s1_lo || psnp[0] == DS.s1_hi)) {
+        const int64_t base = (int64_t)DS.total - (int64_t)prefix_rank_sum<km1>(d, psnp) - d.n;
+        int64_t lo64 = (int64_t)DS.rank_begin - base, hi64 = (int64_t)DS.rank_end - base;
+        lo64 = lo64 < (int64_t)jlo ? (int64_t)jlo : (lo64 > d.n ? d.n : lo64);
+        hi64 = hi64 > d.n ? d.n : (hi64 < lo64 ? lo64 : hi64);
+        jlo = (int32_t)lo64;
+        jhi = (int32_t)hi64;
+    }
+}
+
 template <int K, bool C>
-__global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(const __grid_constant__ CUtensorMap tmap_b,
+__global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                                                 const Params P)
 {
-    static_assert(!C || K == 3, "the combined-class variant serves order 3");
     using S = Shape<C>;
-    using R = Roles<C, K>;
+    using R = Roles;
     constexpr int kStages = S::Stages;
     constexpr int kJ = S::J;
     constexpr int kBBytes = S::BBytes;
@@ -523,7 +706,7 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
     // epilogue: the kQC chunks of 8 last SNPs of a lane quadrant go round-
     // robin to its kCG warps, kIters chunks each (the last may be empty)
     constexpr int kQC = kJ / 8;
-    constexpr int kIters = R::Iters;
+    constexpr int kIters = (kQC + kCG - 1) / kCG;
     constexpr int kPR = K == 2 ? 3 : (K == 3 ? 9 : (K == 4 ? 27 : 81));
     // order 5: one prefix per tile, its 81 rows over lane quadrants 0-2 (the
     // epilogue sums a combination across warps through shared memory)
@@ -533,56 +716,45 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
     constexpr int km1 = K - 1;
     constexpr int kWarpTma = kEpiWarps + kProdWarps;
     constexpr int kWarpMma = kWarpTma + 1;
-    // candidate-buffer checks (a barrier and maybe a sort) every kJcPerCheck
-    // chunks of 8 last SNPs; the buffer holds the pool and one interval
-    constexpr int kJcPerCheck = K == 2 ? 1 : R::CheckIters;
-    static_assert(kIters % kJcPerCheck == 0, "every item ends on a candidate-buffer check");
-    constexpr int kRelease = release_group<K, C>();
-    // orders 3-4: prefix sums through the shared transpose buffer
-    constexpr bool kTranspose = K == 3 || K == 4;
-    constexpr int kPairs = kWide ? 0 : kPPW * 8;              // (prefix, last SNP) pairs per warp and chunk
+    // (prefix, last SNP) pairs per warp and chunk; orders 4-5: 8 columns by 4
+    // lane parts of the rows
+    constexpr int kPairs = kPPW > 1 ? kPPW * 8 : 8;
     constexpr int kPairIters = (kPairs + 31) / 32;
 
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024 - (smem_u32(smem_raw) & 1023)) & 1023);
     unsigned char *stages_a = smem;
     unsigned char *stages_b = smem + kStages * kTileBytes;
+    // per epilogue warp, the row values of 8 last SNPs [lane][8] (transposed
+    // so that one lane sums one prefix's rows for one last SNP)
+    float *wsum = reinterpret_cast<float *>(stages_b + kStages * kBBytes);
+    uint32_t *tot = reinterpret_cast<uint32_t *>(wsum + kEpiWarps * 256);   // [2][128][kGroups][2 classes]
+    Desc *desc = reinterpret_cast<Desc *>(tot + 2 * 128 * kGroups * 2);
     float *sc;
     uint64_t *rk;
-    uint32_t *tot;                               // [2][128][kMaxProdGroups][2 classes]
     if (P.cand_score_g) {
         sc = P.cand_score_g + (size_t)blockIdx.x * P.cand_p2;
         rk = P.cand_rank_g + (size_t)blockIdx.x * P.cand_p2;
-        tot = reinterpret_cast<uint32_t *>(stages_b + kStages * kBBytes);
     } else {
-        sc = reinterpret_cast<float *>(stages_b + kStages * kBBytes);
-        rk = reinterpret_cast<uint64_t *>(sc + P.cand_p2);
-        tot = reinterpret_cast<uint32_t *>(rk + P.cand_p2);
+        rk = reinterpret_cast<uint64_t *>(desc + kDescDepth);
+        sc = reinterpret_cast<float *>(rk + P.cand_p2);
     }
-    Desc *desc = reinterpret_cast<Desc *>(tot + 2 * 128 * kMaxProdGroups * 2);
-    // orders 3-4: per epilogue warp, the row terms of 8 last SNPs [lane][8]
-    // (transposed so that one lane sums one prefix's rows for one last SNP)
-    unsigned char *after_desc = reinterpret_cast<unsigned char *>(desc + kDescDepth);
-    float *wsum = reinterpret_cast<float *>(after_desc + ((16 - (smem_u32(after_desc) & 15)) & 15));
 
-    // one "stage free" barrier per stage for both operands (the A and B rings
-    // advance together), released by one MMA commit
-    static_assert(kStages % kRelease == 0, "release groups tile the ring");
-    static_assert(kStages % kGroups == 0, "each producer group takes every kGroups-th ring slot");
-    // full_ab[s]: the A producer warps of the slot's parity and the TMA
-    // thread (with its bytes) have filled stage s of both operands
-    __shared__ __align__(8) uint64_t full_ab[kStages], empty_ab[kStages / kRelease];
-    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], tot_full[2];
+    // full_ab[s]: one group's producer warps and the TMA thread (with its
+    // bytes) have filled stage s of both operands; empty_ab[s]: the MMAs that
+    // read it are done (one commit per stage)
+    __shared__ __align__(8) uint64_t full_ab[kStages], empty_ab[kStages];
+    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[S::Accs], tot_full[2], tot_empty[2];
     __shared__ __align__(8) uint64_t desc_full[kDescDepth], desc_empty[kDescDepth], drain_bar;
     __shared__ uint32_t tmem_base_sh;
-    // combined variant: the MMA instruction descriptor of each item (its
-    // column count), written with the item's descriptor
+    // the MMA instruction descriptor of each item (its column count), written
+    // with the item's descriptor
     __shared__ uint32_t item_idesc[kDescDepth];
     __shared__ volatile int abort_flag;
     __shared__ EpiState ES;
-    // order 5: per-warp partial sums [jhalf][quadrant][last SNP of the chunk]
-    __shared__ float wred[2][4][8], wpre[2][4][8];
-    __shared__ int wflag[2][8];
+    // order 5: per-quadrant sums of the item's last SNPs, and their flags
+    __shared__ float wred[kWide ? 4 : 1][kWide ? kJ : 1], wpre[kWide ? 4 : 1][kWide ? kJ : 1];
+    __shared__ __align__(8) unsigned char wflag[kWide ? kJ : 1];
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
@@ -590,20 +762,28 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
     const DevData d = DS.d;
     const CUtensorMap *tmap = DS.tmap ? DS.tmap : &tmap_b;
 
-    const uint64_t cb = blockIdx.x - (uint64_t)DS.cta_begin, cn = (uint64_t)DS.cta_count;
-    const uint64_t it_b = (uint64_t)(((unsigned __int128)DS.n_items * cb) / cn);
-    const uint64_t it_e = (uint64_t)(((unsigned __int128)DS.n_items * (cb + 1)) / cn);
-    const int64_t n_my = (int64_t)(it_e - it_b);
+    const uint64_t cb = blockIdx.x - (uint64_t)DS.cta_begin, cn_ = (uint64_t)DS.cta_count;
+    // Items get cheaper along the panels (fewer last SNPs), so a CTA takes
+    // kSegments ranges spread over all of them: segment q of the dataset's
+    // kSegments cn goes to CTA q % cn.
+    auto segment_at = [&](uint64_t q) -> uint64_t {
+        return (uint64_t)(((unsigned __int128)DS.n_items * q) / (cn_ * kSegments));
+    };
+    int64_t n_my = 0;
+    for (int t = 0; t < kSegments; t++) n_my += (int64_t)(segment_at(cb + cn_ * t + 1) - segment_at(cb + cn_ * t));
+    const int chunks = DS.chunks, chunks_case = DS.chunks_case;
+    const int nst = (chunks + 1) >> 1;                // K stages of an item
 
     if (tid == 0) {
         for (int s = 0; s < kStages; s++) {
-            mbar_init(&full_ab[s], kProdWarps / kGroups + 1);   // one producer group + the TMA thread
-            if (s % kRelease == 0) mbar_init(&empty_ab[s / kRelease], 1);
+            mbar_init(&full_ab[s], 4 + 1);            // one producer group + the TMA thread
+            mbar_init(&empty_ab[s], 1);
         }
+        for (int b = 0; b < S::Accs; b++) mbar_init(&acc_empty[b], kEpiWarps);
         for (int b = 0; b < 2; b++) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], kEpiWarps);
             mbar_init(&tot_full[b], kProdWarps);
+            mbar_init(&tot_empty[b], kEpiWarps);
         }
         for (int q = 0; q < kDescDepth; q++) {
             mbar_init(&desc_full[q], 1);
@@ -612,7 +792,7 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
         g_wait_limit_ns = P.wait_ns ? P.wait_ns : kTimeoutNs;
-        ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.thr = -1.0f;
+        ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.any = 0; ES.thr = ES.next_thr = -1.0f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kWarpMma) {
@@ -625,25 +805,50 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_base_sh;
+    if (warp < 4) {
+        // scale factors (UE8M0, 127 = 1), the same in every byte pair's rows
+        // and columns, so their placement does not matter: A all 1; B bytes
+        // 0-1 the controls' 1, bytes 2-3 the cases' 2^p
+        const uint32_t q = tmem_base + ((uint32_t)(warp * 32) << 16);
+        const uint32_t cs = 127u + (uint32_t)DS.comb_p;
+        tmem_fill16(q + kScaleACol, 0x7F7F7F7Fu);
+        tmem_fill16(q + kScaleBCol, 0x00007F7Fu | (cs << 16) | (cs << 24));
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
 
     if (warp == kWarpTma) {
         // ------------------------------------------------ TMA + descriptors
         if (lane == 0 && n_my > 0) {
-            const uint64_t w0 = it_b;
-            int64_t lo = 0, hi = d.n - 1;
-            while (lo < hi) {
-                const int64_t mid = (lo + hi + 1) >> 1;
-                if (DS.item_cum[mid] <= w0) lo = mid;
-                else hi = mid - 1;
-            }
-            const int32_t c0 = (int32_t)lo;
-            const uint64_t off = w0 - DS.item_cum[c0];
-            const int64_t nt0 = ntiles_of<kJ>(d, c0);
-            const uint64_t tfirst = (DS.pcum[c0] + kPPT - 1) / kPPT;
-            const uint64_t t = tfirst + off / (uint64_t)nt0;
-            int64_t u = (int64_t)(off % (uint64_t)nt0);
+            // the segment's next item: M tile (prefix iterator) and N tile u
             PrefixIter it;
-            prefix_unrank(DS, K, t * (uint64_t)kPPT, it);
+            int64_t u = 0;
+            int seg = -1;
+            uint64_t seg_left = 0;
+            auto next_segment = [&]() {
+                uint64_t w0;
+                do {
+                    seg++;
+                    w0 = segment_at(cb + cn_ * seg);
+                    seg_left = segment_at(cb + cn_ * seg + 1) - w0;
+                } while (seg_left == 0);
+                int64_t lo = 0, hi = d.n - 1;
+                while (lo < hi) {
+                    const int64_t mid = (lo + hi + 1) >> 1;
+                    if (DS.item_cum[mid] <= w0) lo = mid;
+                    else hi = mid - 1;
+                }
+                const int32_t c0 = (int32_t)lo;
+                const uint64_t off = w0 - DS.item_cum[c0];
+                const int64_t nt0 = panel_ntiles(d.n, c0, kJ);
+                const uint64_t tfirst = (DS.pcum[c0] + kPPT - 1) / kPPT;
+                const uint64_t t = tfirst + off / (uint64_t)nt0;
+                u = (int64_t)(off % (uint64_t)nt0);
+                prefix_unrank(DS, K, t * (uint64_t)kPPT, it);
+            };
+            next_segment();
             int32_t tile_snp[kPPT * km1];
             int32_t nvalid = 0, cmin = it.c;
             auto fill_tile = [&]() {
@@ -662,91 +867,147 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
             };
             fill_tile();
             uint64_t g = 0;
+            int s = 0;
+            uint32_t ph = 0;
             long long w_tma = 0;
             for (int64_t i = 0; i < n_my && !abort_flag; i++) {
                 const int dq = (int)(i % kDescDepth);
                 const uint32_t ud = (uint32_t)(i / kDescDepth);
                 if (!mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag)) break;
                 Desc &D = desc[dq];
-                D.j0 = cmin + 1 + (int32_t)(u * kJ);
+                D.j0 = (int32_t)panel_j0(cmin) + (int32_t)(u * kJ);
                 D.nvalid = nvalid;
 #pragma unroll
                 for (int q = 0; q < kPPT * km1; q++) D.snp[q] = tile_snp[q];
-                if constexpr (C) {
+                {
                     // columns in use: 2 per last SNP below n, in steps of 16
                     const int32_t live = 2 * ((int32_t)d.n - D.j0);
                     const uint32_t ncol = live >= S::N ? (uint32_t)S::N : (uint32_t)((live + 15) & ~15);
-                    item_idesc[dq] = make_idesc(1, ncol);
+                    item_idesc[dq] = make_idesc(ncol);
                 }
                 mbar_arrive(&desc_full[dq]);
                 const int y = 2 * D.j0;
-                for (int kc = 0; kc < DS.chunks; kc++, g++) {
-                    const int s = (int)(g % kStages);
-                    const uint32_t us = (uint32_t)(g / kStages);
-                    if (!wait_fast(&empty_ab[s / kRelease], (us & 1) ^ 1, &abort_flag, w_tma)) break;
+                for (int kc = 0; kc < nst; kc++, g++) {
+                    if (!wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_tma)) break;
                     mbar_arrive_tx(&full_ab[s], (uint32_t)kBBytes);
-                    tma_load_2d(stages_b + s * kBBytes, tmap, kc * kKC, y, &full_ab[s]);
+                    tma_load_2d(stages_b + s * kBBytes, tmap, kc * kRowBytes, y, &full_ab[s]);
+                    if (++s == kStages) { s = 0; ph ^= 1; }
                 }
                 u++;
-                if (u == ntiles_of<kJ>(d, cmin)) {
+                if (--seg_left == 0) {
+                    if (i + 1 < n_my) {
+                        next_segment();
+                        fill_tile();
+                    }
+                } else if (u == panel_ntiles(d.n, cmin, kJ)) {
                     u = 0;
                     fill_tile();
                 }
             }
             if (P.waits) P.waits[blockIdx.x * kWaitSlots + 6] = (unsigned long long)w_tma;
-            for (int s = 0; s < kStages; s++) {
-                if (g > (uint64_t)s) {
-                    const uint64_t last = ((g - 1 - s) / kStages) * kStages + s;
+            for (int q = 0; q < kStages; q++) {
+                if (g > (uint64_t)q) {
+                    const uint64_t last = ((g - 1 - q) / kStages) * kStages + q;
                     const uint32_t us = (uint32_t)(last / kStages);
                     const uint64_t t0 = now_ns();
-                    while (!mbar_try(&full_ab[s], us & 1) && now_ns() - t0 < kTimeoutNs) {}
+                    while (!mbar_try(&full_ab[q], us & 1) && now_ns() - t0 < kTimeoutNs) {}
                 }
             }
         }
     } else if (warp == kWarpMma) {
         // ------------------------------------------------------------- MMA
         if (n_my > 0) {
-            // a lean issue loop run by the whole warp in step (warp-uniform
-            // values stay on the uniform datapath); one elected lane issues
-            // the MMAs and commits.  The tensor pipe is fed only as fast as
-            // this instruction stream runs, so stage descriptors are formed
-            // by one add and the ring position and phase are carried.
+            // The issue loop is run by the whole warp in step; one elected
+            // lane issues the MMAs and commits.  Only a few MMAs queue behind
+            // the running one, so the tensor pipe idles through whatever this
+            // instruction stream does between two MMAs: the next stage's
+            // barrier is tested and its operands' descriptors are formed
+            // between the MMAs of a stage (measured at order 4, 500 x 8192:
+            // testing after the last MMA left 290 cycles a stage exposed), and
+            // the class boundary of the separate variant has its own branch.
             const uint32_t leader = elect_one();
-            const uint64_t ad0 = sdesc(smem_u32(stages_a)), bd0 = sdesc(smem_u32(stages_b));
+            const uint32_t tb = uniform(tmem_base);
+            const uint64_t ad0 = sdesc(uniform(smem_u32(stages_a))), bd0 = sdesc(uniform(smem_u32(stages_b)));
             // stage strides in descriptor address units
             constexpr uint32_t kStageDescA = kTileBytes >> 4, kStageDescB = kBBytes >> 4;
+            const uint32_t sfa = tb + kScaleACol, sfb = tb + kScaleBCol;
+            const int u_chunks = (int)uniform((uint32_t)chunks), u_case = (int)uniform((uint32_t)chunks_case);
+            const int u_nst = (u_chunks + 1) >> 1;
+            const uint32_t u_items = uniform((uint32_t)n_my);
             int s = 0;
             uint32_t ph = 0;
-            const int chunks = DS.chunks, chunks_case = DS.chunks_case;
+            int ab = 0;                              // accumulator buffer and the phase of its uses
+            uint32_t aph = 0;
             long long w_a = 0, w_b = 0, w_acc = 0;
             const long long t_start = clock64();
-            for (int64_t i = 0; i < n_my && !abort_flag; i++) {
-                const int b = (int)(i & 1);
-                const uint32_t ub = (uint32_t)(i >> 1);
-                if (!wait_fast(&acc_empty[b], (ub & 1) ^ 1, &abort_flag, w_acc)) break;
+            auto next_acc = [&](uint32_t &col) -> bool {
+                if (!__all_sync(0xffffffffu, mbar_test(&acc_empty[ab], aph ^ 1)) &&
+                    !wait_inline(&acc_empty[ab], aph ^ 1, &abort_flag, w_acc))
+                    return false;
                 tc_fence_after();
-                // separate classes: case and control accumulators of 128
-                // columns each; combined: one accumulator of 256 columns
-                const uint32_t d_case = tmem_base + (uint32_t)(b * 256), d_ctrl = d_case + (C ? 0u : 128u);
-                uint32_t idesc = kIdesc;
+                col = tb + (uint32_t)(ab * S::N);
+                if (++ab == S::Accs) { ab = 0; aph ^= 1; }
+                return true;
+            };
+            bool ready = false;                      // stage s, phase ph is known to be full
+            for (uint32_t i = 0; i < u_items; i++) {
+                uint32_t dcol = 0, idesc = 0;
+                if (!next_acc(dcol)) break;
                 bool ok = true;
-                for (int kc = 0; kc < chunks; kc++) {
-                    if (!wait_fast(&full_ab[s], ph, &abort_flag, w_a)) { ok = false; break; }
+                for (int st = 0; st < u_nst; st++) {
+                    if (!__all_sync(0xffffffffu, ready)) {
+                        ok = wait_inline(&full_ab[s], ph, &abort_flag, w_a);
+                        if (!ok) break;
+                    }
                     tc_fence_after();
                     // the item's column count is in place once its first stage is full
-                    if (C && kc == 0) idesc = item_idesc[i % kDescDepth];
-                    const uint32_t dcol = kc < chunks_case ? d_case : d_ctrl;
-                    const uint32_t acc0 = (kc == 0 || (!C && kc == chunks_case)) ? 0u : 1u;
+                    if (st == 0) idesc = uniform(item_idesc[i % kDescDepth]);
                     const uint64_t ad = ad0 + (uint64_t)(s * kStageDescA), bd = bd0 + (uint64_t)(s * kStageDescB);
-                    mma_f8_warp(dcol, ad, bd, acc0, leader, idesc);
-#pragma unroll
-                    for (int kk = 1; kk < kKC / 32; kk++)
-                        mma_f8_warp(dcol, ad + 2 * kk, bd + 2 * kk, 1u, leader, idesc);
-                    if (s % kRelease == kRelease - 1) mma_commit_warp(&empty_ab[s / kRelease], leader);
+                    const int c = 2 * st;
+                    const bool second = c + 1 < u_chunks;
+                    uint64_t *const freed = &empty_ab[s];
                     if (++s == kStages) { s = 0; ph ^= 1; }
+                    if (!C && (c == u_case || c + 1 == u_case) && c > 0) {
+                        // the control accumulator starts in this stage
+                        if (c + 1 == u_case) {
+                            mma_f4_warp(dcol, ad, bd, 1u, leader, idesc, sfa, sfb);
+                            mma_f4_warp(dcol, ad + 2, bd + 2, 1u, leader, idesc, sfa, sfb);
+                            ok = next_acc(dcol);
+                            if (!ok) break;
+                            mma_f4_warp(dcol, ad + 4, bd + 4, 0u, leader, idesc, sfa, sfb);
+                        } else {
+                            ok = next_acc(dcol);
+                            if (!ok) break;
+                            mma_f4_warp(dcol, ad, bd, 0u, leader, idesc, sfa, sfb);
+                            mma_f4_warp(dcol, ad + 2, bd + 2, 1u, leader, idesc, sfa, sfb);
+                            if (second) mma_f4_warp(dcol, ad + 4, bd + 4, 1u, leader, idesc, sfa, sfb);
+                        }
+                        if (second) mma_f4_warp(dcol, ad + 6, bd + 6, 1u, leader, idesc, sfa, sfb);
+                        ready = mbar_test(&full_ab[s], ph);
+                    } else if (!C && c == 0 && u_case == 1) {
+                        // both classes within the first stage
+                        mma_f4_warp(dcol, ad, bd, 0u, leader, idesc, sfa, sfb);
+                        mma_f4_warp(dcol, ad + 2, bd + 2, 1u, leader, idesc, sfa, sfb);
+                        ok = next_acc(dcol);
+                        if (!ok) break;
+                        mma_f4_warp(dcol, ad + 4, bd + 4, 0u, leader, idesc, sfa, sfb);
+                        mma_f4_warp(dcol, ad + 6, bd + 6, 1u, leader, idesc, sfa, sfb);
+                        ready = mbar_test(&full_ab[s], ph);
+                    } else {
+                        const uint32_t id0 = C && c < u_case ? idesc | kIdescCase : idesc;
+                        const uint32_t id1 = C && c + 1 < u_case ? idesc | kIdescCase : idesc;
+                        mma_f4_warp(dcol, ad, bd, st ? 1u : 0u, leader, id0, sfa, sfb);
+                        mma_f4_warp(dcol, ad + 2, bd + 2, 1u, leader, id0, sfa, sfb);
+                        ready = mbar_test(&full_ab[s], ph);
+                        if (second) {
+                            mma_f4_warp(dcol, ad + 4, bd + 4, 1u, leader, id1, sfa, sfb);
+                            mma_f4_warp(dcol, ad + 6, bd + 6, 1u, leader, id1, sfa, sfb);
+                        }
+                    }
+                    mma_commit_warp(freed, leader);
                 }
                 if (!ok) break;
-                mma_commit_warp(&acc_full[b], leader);
+                mma_commit_warp(&acc_full[i & 1], leader);
             }
             if (P.waits && leader) {
                 unsigned long long *wp = P.waits + blockIdx.x * kWaitSlots;
@@ -762,15 +1023,19 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
         }
     } else if (warp >= kEpiWarps) {
         // ---------------------------------------------------- A producers
-        // Thread t owns tile row r = t % 128 in the ring slots of group
-        // t / 128 (with two groups they take alternate stages), and writes
-        // all 128 individuals of the row's stage: four mask words, each
-        // expanded to 32 bytes.
+        // Thread t owns tile row r = t % 128 in the stages of group t / 128
+        // (with two groups they take alternate stages), and writes all 256
+        // individuals of the row's stage: eight mask words, each expanded to
+        // 16 bytes.
         const int t = tid - kEpiThreads;     // 0 .. 32 kProdWarps - 1
         const int r = t & 127;
         const int grp = t >> 7;
         const int l = r & 31, w = r >> 5;
-        uint64_t g = 0;                      // stages of the CTA so far (both halves)
+        // 16-byte piece c of the row is stored at piece c ^ (r % 8): the row's
+        // address with r % 8 in the piece bits, xor c
+        const uint32_t arow0 = smem_u32(stages_a) + (uint32_t)(r * kRowBytes + ((r & 7) << 4));
+        const int64_t stage_stride = 6 * (d.n + 1);
+        uint64_t g = 0;                      // stages of the CTA so far (all groups)
         long long w_prod = 0, w_prod_acc = 0;
         for (int64_t i = 0; i < n_my; i++) {
             if (abort_flag) break;
@@ -778,101 +1043,75 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
             const uint32_t ud = (uint32_t)(i / kDescDepth);
             if (!mbar_wait(&desc_full[dq], ud & 1, &abort_flag)) break;
             const Desc &D = desc[dq];
+            // the row's SNP rows at stage 0; rows of no prefix read the zero
+            // rows kept past the last SNP
             const uint4 *rows[km1];
-            bool active = false;
+#pragma unroll
+            for (int tt = 0; tt < km1; tt++) rows[tt] = DS.rows + d.n * 6;
             if (kWide ? r < kPR : l < kPPW * kPR) {
                 const int p = kWide ? 0 : w * kPPW + l / kPR;
                 if (p < D.nvalid) {
-                    active = true;
                     int rem = kWide ? r : l % kPR, div = kPR / 3;
 #pragma unroll
                     for (int tt = 0; tt < km1; tt++) {
                         const int gg = rem / div;
                         rem -= gg * div;
                         div = div > 1 ? div / 3 : 1;
-                        rows[tt] = reinterpret_cast<const uint4 *>(d.masks + ((int64_t)D.snp[p * km1 + tt] * 3 + gg) * d.Wt);
+                        rows[tt] = DS.rows + (D.snp[p * km1 + tt] * 3 + gg) * 2;
                     }
                 }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&desc_empty[dq]);
-            uint32_t t1 = 0, t0 = 0;
+            uint32_t t1 = 0, ta = 0;             // individuals of the row: cases, all
             bool ok = true;
-            const int chunks = DS.chunks, chunks_case = DS.chunks_case;
-            // this group's first stage of the item and its number of stages
-            const int kc0 = (int)(((uint64_t)grp + kGroups - (g % kGroups)) % kGroups);
-            const int mine = (chunks - kc0 + kGroups - 1) / kGroups;
-            // the prefix SNPs' words of this row for the next kPf own stages
-            // (a register ring indexed statically: the loop is unrolled by
-            // kPf).  Up to order 3 they are kept as loaded and ANDed only
-            // when their stage is produced, so no instruction waits for a
-            // load issued for a later stage; at orders 4-5 the ring holds the
-            // AND (measured: the raw ring's registers spill there, 1586 vs
-            // 1527 ms at order 4, 500 x 8192, and 1548 ms with one own stage
-            // of prefetch; order 3 combined 94.6 -> 94.0 ms).  EPI_TC_RAW_HI
-            // (a prefetch distance) keeps the raw words at every order.
-#ifdef EPI_TC_RAW_HI
-            constexpr bool kKeepRaw = true;
-            constexpr int kPf = km1 <= 2 ? EPI_TC_PREFETCH : EPI_TC_RAW_HI;
-#else
-            constexpr bool kKeepRaw = km1 <= 2;
-            constexpr int kPf = EPI_TC_PREFETCH;
-#endif
-            constexpr int kRaw = kKeepRaw ? km1 : 1;     // words kept per own stage
-            uint4 ring[kPf][kRaw];
-            auto fetch = [&](int kc, uint4 *dst) {
-                if constexpr (kKeepRaw) {
+            // this group's first stage of the item
+            const int st0 = (int)(((uint64_t)grp + kGroups - (g % kGroups)) % kGroups);
+            // the prefix SNPs' words for the next own stage (chunk 2 st and,
+            // where it exists, 2 st + 1), kept as loaded and ANDed when their
+            // stage is produced, so no instruction waits for a load issued for
+            // a later stage
+            constexpr int kPf = K <= 4 ? EPI_TC_PREFETCH : 1;
+            uint4 ring[kPf][2][km1];
+            auto fetch = [&](int st, uint4 (*dst)[km1]) {
 #pragma unroll
-                    for (int tt = 0; tt < km1; tt++) dst[tt] = __ldg(rows[tt] + kc);
-                } else {
-                    uint4 a = __ldg(rows[0] + kc);
+                for (int hh = 0; hh < 2; hh++)
 #pragma unroll
-                    for (int tt = 1; tt < km1; tt++) {
-                        const uint4 v = __ldg(rows[tt] + kc);
-                        a.x &= v.x; a.y &= v.y; a.z &= v.z; a.w &= v.w;
-                    }
-                    dst[0] = a;
-                }
+                    for (int tt = 0; tt < km1; tt++) dst[hh][tt] = __ldg(rows[tt] + st * stage_stride + hh);
             };
 #pragma unroll
-            for (int u = 0; u < kPf; u++) {
-                if (active && u < mine) fetch(kc0 + kGroups * u, ring[u]);
-                else {
-#pragma unroll
-                    for (int tt = 0; tt < kRaw; tt++) ring[u][tt] = make_uint4(0, 0, 0, 0);
-                }
-            }
-            uint64_t gs = g + (uint64_t)kc0;                   // global stage of own stage m
+            for (int u = 0; u < kPf; u++) fetch(st0 + kGroups * u, ring[u]);
+            const uint64_t gs = g + (uint64_t)st0;             // global stage of the first own stage
             int s = (int)(gs % kStages);
             uint32_t ph = (uint32_t)((gs / kStages) & 1);
-            for (int mb = 0; mb < mine && ok; mb += kPf) {
+            for (int sb = st0; sb < nst && ok; sb += kGroups * kPf) {
 #pragma unroll
                 for (int u = 0; u < kPf; u++) {
-                    const int m = mb + u;
-                    if (m >= mine) break;
-                    const int kc = kc0 + kGroups * m;
-                    uint4 cur = ring[u][0];
+                    const int st = sb + kGroups * u;
+                    if (st >= nst) break;
+                    const uint32_t arow = arow0 + (uint32_t)(s * kTileBytes);
+                    if (!wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_prod)) { ok = false; break; }
 #pragma unroll
-                    for (int tt = 1; tt < kRaw; tt++) {
-                        cur.x &= ring[u][tt].x; cur.y &= ring[u][tt].y; cur.z &= ring[u][tt].z; cur.w &= ring[u][tt].w;
-                    }
-                    if (active && m + kPf < mine) fetch(kc + kGroups * kPf, ring[u]);
-                    if (!wait_fast(&empty_ab[s / kRelease], ph ^ 1, &abort_flag, w_prod)) { ok = false; break; }
-                    const uint32_t c4 = __popc(cur.x) + __popc(cur.y) + __popc(cur.z) + __popc(cur.w);
-                    if (kc < chunks_case) t1 += c4;
-                    else t0 += c4;
-                    unsigned char *arow = stages_a + s * kTileBytes + r * 128;
-                    const uint32_t wv4[4] = {cur.x, cur.y, cur.z, cur.w};
+                    for (int hh = 0; hh < 2; hh++) {
+                        uint4 cur = ring[u][hh][0];
 #pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        // output word i = bit i of every byte of the mask word
-                        const uint32_t wv = wv4[q];
-                        const uint32_t s4 = wv << 4, r4 = wv >> 4;
-                        const uint4 lo = make_uint4(s4 & 0x10101010u, s4 & 0x20202020u, s4 & 0x40404040u, wv & 0x08080808u);
-                        const uint4 hi = make_uint4(wv & 0x10101010u, wv & 0x20202020u, wv & 0x40404040u, r4 & 0x08080808u);
-                        *reinterpret_cast<uint4 *>(arow + (((2 * q) ^ (r & 7)) << 4)) = lo;
-                        *reinterpret_cast<uint4 *>(arow + (((2 * q + 1) ^ (r & 7)) << 4)) = hi;
+                        for (int tt = 1; tt < km1; tt++) {
+                            const uint4 v = ring[u][hh][tt];
+                            cur.x &= v.x; cur.y &= v.y; cur.z &= v.z; cur.w &= v.w;
+                        }
+                        const uint32_t wv4[4] = {cur.x, cur.y, cur.z, cur.w};
+                        const uint32_t c4 = __popc(wv4[0]) + __popc(wv4[1]) + __popc(wv4[2]) + __popc(wv4[3]);
+                        t1 += 2 * st + hh < chunks_case ? c4 : 0u;
+                        ta += c4;
+#pragma unroll
+                        for (int q = 0; q < 4; q++) {
+                            // output word i = bit i of every nibble of the mask word
+                            const uint32_t wv = wv4[q];
+                            st_shared_v4(arow ^ (uint32_t)((4 * hh + q) << 4), wv & 0x11111111u, wv & 0x22222222u,
+                                         wv & 0x44444444u, (wv >> 1) & 0x44444444u);
+                        }
                     }
+                    fetch(st + kGroups * kPf, ring[u]);
                     fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&full_ab[s]);
@@ -882,12 +1121,12 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
                 }
             }
             if (!ok) break;
-            g += (uint64_t)chunks;
+            g += (uint64_t)nst;
             const int b = (int)(i & 1);
             const uint32_t ub = (uint32_t)(i >> 1);
-            if (!wait_fast(&acc_empty[b], (ub & 1) ^ 1, &abort_flag, w_prod_acc)) break;
-            tot[((b * 128 + r) * kMaxProdGroups + grp) * 2 + 0] = t1;
-            tot[((b * 128 + r) * kMaxProdGroups + grp) * 2 + 1] = t0;
+            if (!wait_fast(&tot_empty[b], (ub & 1) ^ 1, &abort_flag, w_prod_acc)) break;
+            tot[((b * 128 + r) * kGroups + grp) * 2 + 0] = t1;
+            tot[((b * 128 + r) * kGroups + grp) * 2 + 1] = ta - t1;
             __syncwarp();
             if (lane == 0) mbar_arrive(&tot_full[b]);
         }
@@ -900,15 +1139,30 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
         const int quad = warp & 3;           // TMEM lane quadrant
         const int jhalf = warp >> 2;         // column group: chunks jhalf + kCG i of the quadrant
         const int r = quad * 32 + lane;      // tile row = TMEM lane
-        const int l = lane;
-        const int pos = kWide ? r : l % kPR;          // row of the prefix's table
-        const int pl = kWide ? 0 : l / kPR;
-        const bool lane_real = kWide ? r < kPR : l < kPPW * kPR;
+        const int pos = kWide ? r : lane % kPR;       // row of the prefix's table
+        const int pl = kWide ? 0 : lane / kPR;
+        const bool lane_real = kWide ? r < kPR : lane < kPPW * kPR;
         const MiConstF32 mc = make_mi_const(d.m, d.m1, d.m0);
-        const float vscale = 32.0f * DS.ln2_over_m, voff = DS.tconst * DS.ln2_over_m;
-        // combined classes: the decode's control-bit mask and 2^-(p+5)
-        const uint32_t lo_mask = (1u << (DS.comb_p & 31)) - 1u;
-        const float case_scale = __uint_as_float((uint32_t)(127 - 5 - DS.comb_p) << 23);
+        const float p2 = (float)(1u << DS.comb_p);
+        RowScreen<C> rs;
+        rs.m23 = f2_pack(8388608.0f, 8388608.0f);
+        rs.neg_m23 = f2_pack(-8388608.0f, -8388608.0f);
+        rs.neg1 = f2_pack(-1.0f, -1.0f);
+        rs.kinv1 = 1.0f / p2;
+        rs.kinv = f2_pack(rs.kinv1, rs.kinv1);
+        rs.neg_pi = f2_pack(-DS.sc_pi, -DS.sc_pi);
+        rs.lo_mask = (1u << DS.comb_p) - 1u;
+        rs.sc.c2 = f2_pack(DS.c2, DS.c2);
+        rs.sc.c3 = f2_pack(DS.c3, DS.c3);
+        rs.sc.c4 = f2_pack(DS.c4, DS.c4);
+        rs.sc.c5a = f2_pack(DS.c5a, DS.c5a);
+        rs.sc.c5b = f2_pack(DS.c5b, DS.c5b);
+        rs.sc.tiny = f2_pack(1e-30f, 1e-30f);
+        const float vscale = DS.vscale, voff = DS.voff;
+        const bool poly = DS.poly != 0;
+        float *wb = wsum + warp * 256;
+        int ab = 0;                          // first accumulator buffer of the item
+        float thr = -1.0f;                   // the threshold as of the last item's closing barrier
         long long w_epi = 0;
         for (int64_t i = 0; i < n_my; i++) {
             const int dq = (int)(i % kDescDepth);
@@ -920,256 +1174,254 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
             ok = ok && wait_fast(&tot_full[b], ub & 1, &abort_flag, w_epi);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
+            // this item's accumulators (case and control with separate classes)
+            const int ab1 = C ? ab : (ab + 1 == S::Accs ? 0 : ab + 1);
+            const uint32_t tq = tmem_base + ((uint32_t)(quad * 32) << 16);
+            const uint32_t ta_case = tq + (uint32_t)(ab * S::N), ta_ctrl = tq + (uint32_t)(ab1 * S::N);
+            const int ab_case = ab;
+            ab = ab1 + 1 == S::Accs ? 0 : ab1 + 1;
             const Desc &D = desc[dq];
             const int p = quad * kPPW + pl;
             const bool prow = ok && lane_real && p < D.nvalid;
-            const int32_t cpre = prow ? D.snp[p * km1 + km1 - 1] : 0x7fffffff;
             int32_t psnp[km1];
 #pragma unroll
             for (int tt = 0; tt < km1; tt++) psnp[tt] = prow ? D.snp[p * km1 + tt] : 0;
-            // last SNPs of this prefix inside the searched rank range: the
-            // combination (prefix, j) has rank base + j.  Only prefixes whose
-            // first SNP is the range's first or last can be cut.
-            int32_t jlo = cpre + 1, jhi = (int32_t)d.n;
-            if (prow && DS.clip && (psnp[0] == DS.s1_lo || psnp[0] == DS.s1_hi)) {
-                uint64_t sp = 0;
+            // the searched last SNPs of the prefixes whose (prefix, last SNP)
+            // pairs this lane sums: pair lane + 32 q is prefix (lane + 32 q) / 8
+            // of the warp and last SNP (lane + 32 q) % 8 of each chunk (at
+            // orders 4-5 the warp's only prefix, last SNP lane % 8)
+            int32_t plo[kPairIters], phi[kPairIters];
 #pragma unroll
-                for (int tt = 0; tt < km1; tt++) sp += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                const int64_t base = (int64_t)DS.total - (int64_t)sp - d.n;
-                int64_t lo64 = (int64_t)DS.rank_begin - base, hi64 = (int64_t)DS.rank_end - base;
-                lo64 = lo64 < (int64_t)jlo ? (int64_t)jlo : (lo64 > d.n ? d.n : lo64);
-                hi64 = hi64 > d.n ? d.n : (hi64 < lo64 ? lo64 : hi64);
-                jlo = (int32_t)lo64;
-                jhi = (int32_t)hi64;
-            }
-            // the same interval for the prefixes whose (prefix, last SNP)
-            // pairs this lane sums (orders 3-4): pair lane + 32 i is prefix
-            // (lane + 32 i) / 8 of the warp and last SNP (lane + 32 i) % 8 of
-            // each chunk
-            int32_t plo[kPairIters > 0 ? kPairIters : 1], phi[kPairIters > 0 ? kPairIters : 1];
-            if constexpr (kTranspose) {
+            for (int q = 0; q < kPairIters; q++) {
+                const int pp = kPPW > 1 ? (lane + 32 * q) >> 3 : 0;
+                const int pt = quad * kPPW + pp;
+                plo[q] = 1;
+                phi[q] = 0;                      // empty: no valid last SNP
+                if (ok && (kPPW <= 1 || pp < kPPW) && pt < D.nvalid) {
+                    int32_t qs[km1];
 #pragma unroll
-                for (int q = 0; q < kPairIters; q++) {
-                    const int pp = (lane + 32 * q) >> 3;
-                    const int pt = quad * kPPW + pp;
-                    plo[q] = 1;
-                    phi[q] = 0;                      // empty: no valid last SNP
-                    if (ok && pp < kPPW && pt < D.nvalid) {
-                        int32_t qs[km1];
-#pragma unroll
-                        for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
-                        plo[q] = qs[km1 - 1] + 1;
-                        phi[q] = (int32_t)d.n;
-                        if (DS.clip && (qs[0] == DS.s1_lo || qs[0] == DS.s1_hi)) {
-                            uint64_t sp = 0;
-#pragma unroll
-                            for (int tt = 0; tt < km1; tt++) sp += binom_at(d.binom, d.n, d.n - 1 - qs[tt], K - tt);
-                            const int64_t base = (int64_t)DS.total - (int64_t)sp - d.n;
-                            int64_t lo64 = (int64_t)DS.rank_begin - base, hi64 = (int64_t)DS.rank_end - base;
-                            lo64 = lo64 < (int64_t)plo[q] ? (int64_t)plo[q] : (lo64 > d.n ? d.n : lo64);
-                            hi64 = hi64 > d.n ? d.n : (hi64 < lo64 ? lo64 : hi64);
-                            plo[q] = (int32_t)lo64;
-                            phi[q] = (int32_t)hi64;
-                        }
-                    }
+                    for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
+                    last_snp_range<km1>(DS, d, qs, plo[q], phi[q]);
                 }
             }
-            uint32_t T1 = 0, T0 = 0;
+            {
+                uint32_t T1 = 0, T0 = 0;
 #pragma unroll
-            for (int gq = 0; gq < kGroups; gq++) {
-                T1 += tot[((b * 128 + r) * kMaxProdGroups + gq) * 2 + 0];
-                T0 += tot[((b * 128 + r) * kMaxProdGroups + gq) * 2 + 1];
+                for (int gq = 0; gq < kGroups; gq++) {
+                    T1 += tot[((b * 128 + r) * kGroups + gq) * 2 + 0];
+                    T0 += tot[((b * 128 + r) * kGroups + gq) * 2 + 1];
+                }
+                // rows of no prefix count nothing: their totals are 0
+                rs.set_row(u2f_exact(T1), u2f_exact(T0), p2);
             }
-            // row totals in accumulator units (count / 32, exact)
-            const float fT1 = u2f_exact(T1) * 0.03125f, fT0 = u2f_exact(T0) * 0.03125f;
-            if (tid == 0) {
-                const float gthr = __uint_as_float(*(volatile uint32_t *)DS.global_thr);
-                if (ES.list_len == P.pool || gthr > 0.0f) ES.thr = fmaxf(ES.thr, gthr);
-            }
-            epi_bar<kEpiThreads>();
-            float thr = ES.thr, cut = thr - DS.delta;
-            int list_len = ES.list_len;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&tot_empty[b]);
+            // the other CTAs' threshold, for the next item (loaded early)
+            const float gthr = tid == 0 ? __uint_as_float(*(volatile uint32_t *)DS.global_thr) : 0.0f;
+            const float cut = thr < 0.0f ? -1.0f : thr * DS.cut_mul - DS.cut_add;
+            const int list_len = ES.list_len;
+            const int32_t j0 = D.j0;
+            // before the item's closing barrier: the threshold the other CTAs
+            // have reached, and whether a role gave up
+            auto refresh = [&]() {
+                if (tid == 0) {
+                    if (ES.list_len == P.pool || gthr > 0.0f) ES.next_thr = fmaxf(ES.thr, gthr);
+                    ES.stop = abort_flag;
+                }
+            };
+            // one chunk's accumulators (queued): last SNPs j0 + 8 jcg ..
+            auto load_chunk = [&](int jcg, uint32_t *cs, uint32_t *cn) {
+                TMEM_LD16(ta_case + (uint32_t)(16 * jcg), cs);
+                if constexpr (!C) TMEM_LD16(ta_ctrl + (uint32_t)(16 * jcg), cn);
+            };
+            auto release_acc = [&]() {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&acc_empty[ab_case]);
+                    if constexpr (!C) mbar_arrive(&acc_empty[ab1]);
+                }
+            };
+            // validation: every table of the chunk, as counts
+            auto dump_chunk = [&](int jb, const uint32_t *cs, const uint32_t *cn) {
+                if (!prow) return;
+                int32_t jlo, jhi;
+                last_snp_range<km1>(DS, d, psnp, jlo, jhi);
 #pragma unroll 1
-            for (int jc = 0; jc < kIters; jc++) {
-                uint32_t cs[16], cn[16];
-                // this warp's chunk of the quadrant: last SNPs j0 .. j0 + 7
-                const int jcg = jhalf + kCG * jc;
-                const int32_t jb = D.j0 + 8 * jcg;   // the chunk's last SNPs are jb .. jb + 7
-                // a chunk past the quadrant's last one, or (orders 3-4) whose
-                // first last SNP is past the end (the last N tile of a panel),
-                // holds no combination, and its warp skips it (warp-uniform)
-                const bool live = ok && jcg < kQC && (!kTranspose || jb < (int32_t)d.n);
-                if (live) {
-                    // columns 2 (j - D.j0) + g of accumulator b; separate
-                    // classes: the control accumulator 128 columns on
-                    const uint32_t ta = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * 256 + 16 * jcg);
-                    if constexpr (C) {
-                        uint32_t cc[16];
-                        TMEM_LD16(ta, cc);
-                        tmem_wait_ld();
+                for (int jj = 0; jj < 8; jj++) {
+                    const int32_t j = jb + jj;
+                    if (j < jlo || j >= jhi) continue;
+                    float a[3] = {}, bb[3] = {};
 #pragma unroll
-                        for (int q = 0; q < 16; q++) split_classes(cc[q], lo_mask, case_scale, cs[q], cn[q]);
-                    } else {
-                        TMEM_LD16(ta, cs);
-                        TMEM_LD16(ta + 128, cn);
-                        tmem_wait_ld();
+                    for (int h = 0; h < 4; h++)
+                        if (h == jj >> 1) rs.counts(cs, cn, h, jj & 1, a, bb);
+                    constexpr int cells = kPR * 3;
+                    uint32_t *o = P.dump + (DS.total - 1 - prefix_rank_sum<km1>(d, psnp) - (uint64_t)(d.n - 1 - j)) *
+                                               2 * cells;
+#pragma unroll
+                    for (int g3 = 0; g3 < 3; g3++) {
+                        o[pos * 3 + g3] = f2u_exact(a[g3]);
+                        o[cells + pos * 3 + g3] = f2u_exact(bb[g3]);
                     }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < 16; q++) { cs[q] = 0; cn[q] = 0; }
                 }
-                if (jc == kIters - 1) {
-                    // every accumulator value is in registers: hand the
-                    // buffer back to the MMA issuer before the last scoring
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&acc_empty[b]);
+            };
+            // precise single-precision terms of this row for column jsel
+            auto row_precise = [&](const uint32_t *cs, const uint32_t *cn, int jsel) -> float {
+                float a[3] = {}, bb[3] = {};
+#pragma unroll
+                for (int h = 0; h < 4; h++)
+                    if (h == jsel >> 1) rs.counts(cs, cn, h, jsel & 1, a, bb);
+                return row_terms_precise(f2u_exact(a[0]), f2u_exact(bb[0]), f2u_exact(a[1]), f2u_exact(bb[1]),
+                                         f2u_exact(a[2]), f2u_exact(bb[2]), mc);
+            };
+            auto keep = [&](float score, int32_t j) {
+                if (score >= thr) {
+                    const int slot = list_len + atomicAdd(&ES.nbuf, 1);
+                    sc[slot] = score;
+                    rk[slot] = DS.total - 1 - prefix_rank_sum<km1>(d, psnp) - (uint64_t)(d.n - 1 - j);
                 }
-                if constexpr (kWide) {
-                    // screen sums of the chunk's 8 last SNPs: each warp sums
-                    // its rows, the quadrant-0 warp of the half adds the three
-                    float vs[8];
+            };
+            // 8 row values per lane -> transposed sums: the lane of pair
+            // (prefix pp, last SNP jj) adds rows pp kPR .. of column jj (all
+            // banks distinct); at orders 4-5 four lanes share a column
+            auto store_rows = [&](const float *vrow) {
+                reinterpret_cast<float4 *>(wb + lane * 8)[0] = make_float4(vrow[0], vrow[1], vrow[2], vrow[3]);
+                reinterpret_cast<float4 *>(wb + lane * 8)[1] = make_float4(vrow[4], vrow[5], vrow[6], vrow[7]);
+                __syncwarp();
+            };
+            auto column_sum = [&]() -> float {
+                constexpr int kPart = kWide ? 8 : 7;
+                const int part = lane >> 3;
+                float v = 0.0f, w2 = 0.0f;
 #pragma unroll
-                    for (int jj = 0; jj < 8; jj++) {
-                        const int32_t j = jb + jj;
-                        const float fa0 = __uint_as_float(cs[2 * jj]), fa1 = __uint_as_float(cs[2 * jj + 1]);
-                        const float fb0 = __uint_as_float(cn[2 * jj]), fb1 = __uint_as_float(cn[2 * jj + 1]);
-                        const float fa2 = fT1 - fa0 - fa1, fb2 = fT0 - fb0 - fb1;
-                        const bool valid = prow && j >= jlo && j < jhi;
-                        if (P.dump && valid) {
-                            uint64_t rs = 0;
-#pragma unroll
-                            for (int tt = 0; tt < km1; tt++) rs += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                            rs += binom_at(d.binom, d.n, d.n - 1 - j, 1);
-                            constexpr int cells = kPR * 3;
-                            uint32_t *o = P.dump + (DS.total - 1 - rs) * 2 * cells;
-                            o[pos * 3 + 0] = f2u_exact(32.0f * fa0); o[pos * 3 + 1] = f2u_exact(32.0f * fa1);
-                            o[pos * 3 + 2] = f2u_exact(32.0f * fa2);
-                            o[cells + pos * 3 + 0] = f2u_exact(32.0f * fb0);
-                            o[cells + pos * 3 + 1] = f2u_exact(32.0f * fb1);
-                            o[cells + pos * 3 + 2] = f2u_exact(32.0f * fb2);
-                        }
-                        float v = 0.0f;
-                        if (prow)
-                            v = (tlog32(fa0) + tlog32(fb0) - tlog32(fa0 + fb0)) +
-                                (tlog32(fa1) + tlog32(fb1) - tlog32(fa1 + fb1)) +
-                                (tlog32(fa2) + tlog32(fb2) - tlog32(fa2 + fb2));
-                        vs[jj] = warp_sum(v);
+                for (int rr = 0; rr < kPart; rr++) {
+                    const int row = part * kPart + rr;
+                    const float x = (kWide || row < kPR) ? wb[row * 8 + (lane & 7)] : 0.0f;
+                    if (rr & 1) w2 += x;
+                    else v += x;
+                }
+                v += w2;
+                v += __shfl_xor_sync(0xffffffffu, v, 8);
+                v += __shfl_xor_sync(0xffffffffu, v, 16);
+                return v;
+            };
+            if constexpr (kWide) {
+                // order 5: the item's sums of each quadrant's rows, then one
+                // pass over its last SNPs, then (rarely) the precise scores
+                // of the flagged ones
+#pragma unroll 1
+                for (int jcg = jhalf; jcg < kQC; jcg += kCG) {
+                    const int32_t jb = j0 + 8 * jcg;
+                    float v = 0.0f;
+                    if (ok && quad < 3 && jb < (int32_t)d.n) {
+                        uint32_t cs[16], cn[C ? 1 : 16];
+                        load_chunk(jcg, cs, cn);
+                        tmem_wait_ld();
+                        float vrow[8];
+                        if (poly) rs.bound(cs, cn, vrow);
+                        else rs.logs(cs, cn, vrow);
+                        if (P.dump) dump_chunk(jb, cs, cn);
+                        store_rows(vrow);
+                        v = column_sum();
+                        __syncwarp();
                     }
-                    if (lane == 0) {
-#pragma unroll
-                        for (int jj = 0; jj < 8; jj++) wred[jhalf][quad][jj] = vs[jj];
-                    }
-                    epi_bar<kEpiThreads>();
-                    if (quad == 0 && lane < 8) {
-                        const float tv = wred[jhalf][0][lane] + wred[jhalf][1][lane] + wred[jhalf][2][lane] +
-                                         wred[jhalf][3][lane];
-                        const int32_t j = jb + lane;
-                        const bool valid = prow && j >= jlo && j < jhi;
-                        wflag[jhalf][lane] = (valid && fmaf(tv, vscale, voff) >= cut) ? 1 : 0;
-                    }
-                    epi_bar<kEpiThreads>();
-                    int anyf = 0;
-#pragma unroll
-                    for (int q = 0; q < 16; q++) anyf |= wflag[q >> 3][q & 7];
-                    if (anyf) {
-                        // precise single-precision scores of the flagged sets
+                    if (lane < 8) wred[quad][8 * jcg + lane] = v;
+                }
+                epi_bar<kEpiThreads>();
+                bool any = false;
+                for (int q = tid; q < kJ; q += kEpiThreads) {
+                    const float tv = wred[0][q] + wred[1][q] + wred[2][q];
+                    const int32_t j = j0 + q;
+                    const bool f = phi[0] > 0 && j >= plo[0] && j < phi[0] && fmaf(tv, vscale, voff) >= cut;
+                    wflag[q] = f ? 1 : 0;
+                    any |= f;
+                }
+                if (any) ES.any = 1;
+                epi_bar<kEpiThreads>();
+                if (ES.any) {
+#pragma unroll 1
+                    for (int jcg = jhalf; jcg < kQC; jcg += kCG) {
+                        const unsigned long long fl = *reinterpret_cast<const unsigned long long *>(&wflag[8 * jcg]);
+                        if (!fl || quad == 3) continue;
+                        uint32_t cs[16], cn[C ? 1 : 16];
+                        load_chunk(jcg, cs, cn);
+                        tmem_wait_ld();
 #pragma unroll 1
                         for (int jj = 0; jj < 8; jj++) {
-                            if (!wflag[jhalf][jj]) continue;
-                            float e = 0.0f;
-                            if (prow) {
-                                const float fa0 = __uint_as_float(cs[2 * jj]), fa1 = __uint_as_float(cs[2 * jj + 1]);
-                                const float fb0 = __uint_as_float(cn[2 * jj]), fb1 = __uint_as_float(cn[2 * jj + 1]);
-                                e = row_terms_precise(f2u_exact(32.0f * fa0), f2u_exact(32.0f * fb0),
-                                                      f2u_exact(32.0f * fa1), f2u_exact(32.0f * fb1),
-                                                      f2u_exact(32.0f * (fT1 - fa0 - fa1)),
-                                                      f2u_exact(32.0f * (fT0 - fb0 - fb1)), mc);
-                            }
-                            e = warp_sum(e);
-                            if (lane == 0) wpre[jhalf][quad][jj] = e;
+                            if (!wflag[8 * jcg + jj]) continue;
+                            const float e = warp_sum(prow ? row_precise(cs, cn, jj) : 0.0f);
+                            if (lane == 0) wpre[quad][8 * jcg + jj] = e;
                         }
-                        epi_bar<kEpiThreads>();
-                        if (quad == 0 && lane < 8 && wflag[jhalf][lane]) {
-                            const float e = wpre[jhalf][0][lane] + wpre[jhalf][1][lane] + wpre[jhalf][2][lane] +
-                                            wpre[jhalf][3][lane];
-                            const float score = __fdiv_rn(e, mc.fm);
-                            if (score >= thr) {
-                                const int32_t j = jb + lane;
-                                uint64_t rk_sum = 0;
-#pragma unroll
-                                for (int tt = 0; tt < km1; tt++)
-                                    rk_sum += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                                rk_sum += binom_at(d.binom, d.n, d.n - 1 - j, 1);
-                                const int slot = list_len + atomicAdd(&ES.nbuf, 1);
-                                sc[slot] = score;
-                                rk[slot] = DS.total - 1 - rk_sum;
-                            }
-                        }
-                        epi_bar<kEpiThreads>();
                     }
-                } else if constexpr (kTranspose) {
-                  if (live) {
-                    // row terms of the chunk's 8 last SNPs, straight-line
+                }
+                release_acc();
+                if (ES.any) {
+                    epi_bar<kEpiThreads>();
+                    for (int q = tid; q < kJ; q += kEpiThreads) {
+                        if (!wflag[q]) continue;
+                        // every thread of the tile's one prefix knows its SNPs
+#pragma unroll
+                        for (int tt = 0; tt < km1; tt++) psnp[tt] = D.snp[tt];
+                        keep(__fdiv_rn(wpre[0][q] + wpre[1][q] + wpre[2][q], mc.fm), j0 + q);
+                    }
+                }
+                refresh();
+                epi_bar<kEpiThreads>();
+                if (tid == 0) ES.any = 0;
+            } else {
+                // this warp's chunks of the quadrant: those that hold a last
+                // SNP below n (all but in the last N tile of a panel)
+                const int live_chunks = ok ? min(kQC, ((int32_t)d.n - j0 + 7) >> 3) : 0;
+                const int mine = (live_chunks - jhalf + kCG - 1) / kCG;
+                uint32_t nx[16], ny[C ? 1 : 16];
+                if (mine > 0) load_chunk(jhalf, nx, ny);
+                else release_acc();
+#pragma unroll 1
+                for (int jc = 0; jc < mine; jc++) {
+                    const int jcg = jhalf + kCG * jc;
+                    const int32_t jb = j0 + 8 * jcg;
+                    uint32_t cs[16], cn[C ? 1 : 16];
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 16; q++) {
+                        cs[q] = nx[q];
+                        if constexpr (!C) cn[q] = ny[q];
+                    }
+                    // the next chunk's accumulators load while this one is
+                    // screened; once every value is in registers the buffer
+                    // goes back to the MMA issuer
+                    if (jc + 1 < mine) load_chunk(jcg + kCG, nx, ny);
+                    else release_acc();
                     float vrow[8];
-#pragma unroll
-                    for (int jj = 0; jj < 8; jj++) {
-                        // accumulator values x = count / 32 (exact); with
-                        // t(x) = x log2 x, T(32 x) = 32 t(x) + 160 x and the
-                        // linear parts cancel within a cell, so the screen
-                        // sums t over the raw values and scales once
-                        const float fa0 = __uint_as_float(cs[2 * jj]), fa1 = __uint_as_float(cs[2 * jj + 1]);
-                        const float fb0 = __uint_as_float(cn[2 * jj]), fb1 = __uint_as_float(cn[2 * jj + 1]);
-                        const float fa2 = fT1 - fa0 - fa1, fb2 = fT0 - fb0 - fb1;
-                        vrow[jj] = prow ? row_screen(fa0, fa1, fa2, fb0, fb1, fb2) : 0.0f;
-                    }
-                    if (P.dump) {
-                        // validation: every table of the chunk, as counts
-#pragma unroll
-                        for (int jj = 0; jj < 8; jj++) {
-                            const int32_t j = jb + jj;
-                            if (!(prow && j >= jlo && j < jhi)) continue;
-                            const float fa0 = __uint_as_float(cs[2 * jj]), fa1 = __uint_as_float(cs[2 * jj + 1]);
-                            const float fb0 = __uint_as_float(cn[2 * jj]), fb1 = __uint_as_float(cn[2 * jj + 1]);
-                            uint64_t rs = 0;
-#pragma unroll
-                            for (int tt = 0; tt < km1; tt++) rs += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                            rs += binom_at(d.binom, d.n, d.n - 1 - j, 1);
-                            constexpr int cells = kPR * 3;
-                            uint32_t *o = P.dump + (DS.total - 1 - rs) * 2 * cells;
-                            o[pos * 3 + 0] = f2u_exact(32.0f * fa0); o[pos * 3 + 1] = f2u_exact(32.0f * fa1);
-                            o[pos * 3 + 2] = f2u_exact(32.0f * (fT1 - fa0 - fa1));
-                            o[cells + pos * 3 + 0] = f2u_exact(32.0f * fb0);
-                            o[cells + pos * 3 + 1] = f2u_exact(32.0f * fb1);
-                            o[cells + pos * 3 + 2] = f2u_exact(32.0f * (fT0 - fb0 - fb1));
-                        }
-                    }
-                    // transpose: lane l's 8 values at [l][0..7]; the lane of
-                    // pair (prefix pp, last SNP jj) reads rows pp*kPR .. of
-                    // column jj (banks 8 (pp kPR + r) + jj: distinct over the
-                    // warp's pairs)
-                    float *wb = wsum + warp * 256;
-                    reinterpret_cast<float4 *>(wb + lane * 8)[0] = make_float4(vrow[0], vrow[1], vrow[2], vrow[3]);
-                    reinterpret_cast<float4 *>(wb + lane * 8)[1] = make_float4(vrow[4], vrow[5], vrow[6], vrow[7]);
-                    __syncwarp();
+                    if (poly) rs.bound(cs, cn, vrow);
+                    else rs.logs(cs, cn, vrow);
+                    if (P.dump) dump_chunk(jb, cs, cn);
+                    store_rows(vrow);
                     uint32_t cmask[kPairIters];
+                    if constexpr (kPPW > 1) {
 #pragma unroll
-                    for (int q = 0; q < kPairIters; q++) {
-                        const int pair = lane + 32 * q;
-                        bool cand = false;
-                        if (pair < kPairs) {
-                            const int pp = pair >> 3, jj = pair & 7;
-                            float v = 0.0f, w2 = 0.0f;
+                        for (int q = 0; q < kPairIters; q++) {
+                            const int pair = lane + 32 * q;
+                            bool cand = false;
+                            if (pair < kPairs) {
+                                const int pp = pair >> 3, jj = pair & 7;
+                                float v = 0.0f, w2 = 0.0f;
 #pragma unroll
-                            for (int rr = 0; rr < kPR; rr++) {
-                                if (rr & 1) w2 += wb[(pp * kPR + rr) * 8 + jj];
-                                else v += wb[(pp * kPR + rr) * 8 + jj];
+                                for (int rr = 0; rr < kPR; rr++) {
+                                    if (rr & 1) w2 += wb[(pp * kPR + rr) * 8 + jj];
+                                    else v += wb[(pp * kPR + rr) * 8 + jj];
+                                }
+                                v += w2;
+                                const int32_t j = jb + jj;
+                                cand = j >= plo[q] && j < phi[q] && fmaf(v, vscale, voff) >= cut;
                             }
-                            v += w2;
-                            const int32_t j = jb + jj;
-                            cand = j >= plo[q] && j < phi[q] && fmaf(v, vscale, voff) >= cut;
+                            cmask[q] = __ballot_sync(0xffffffffu, cand);
                         }
-                        cmask[q] = __ballot_sync(0xffffffffu, cand);
+                    } else {
+                        const float v = column_sum();
+                        const int32_t j = jb + (lane & 7);
+                        cmask[0] = __ballot_sync(0xffffffffu, lane < 8 && j >= plo[0] && j < phi[0] &&
+                                                                  fmaf(v, vscale, voff) >= cut);
                     }
                     __syncwarp();
                     // precise single-precision scores of the flagged pairs
@@ -1181,114 +1433,26 @@ __global__ void __launch_bounds__(Roles<C, K>::Threads, 1) tc_search_kernel(cons
                             const int pair = __ffs(cmask[q]) - 1 + 32 * q;
                             cmask[q] &= cmask[q] - 1;
                             const int pp = pair >> 3, jsel = pair & 7;
-                            uint32_t a0 = 0, a1 = 0, b0 = 0, b1 = 0;
-#pragma unroll
-                            for (int jj = 0; jj < 8; jj++)
-                                if (jj == jsel) { a0 = cs[2 * jj]; a1 = cs[2 * jj + 1]; b0 = cn[2 * jj]; b1 = cn[2 * jj + 1]; }
-                            const float fa0 = __uint_as_float(a0), fa1 = __uint_as_float(a1);
-                            const float fb0 = __uint_as_float(b0), fb1 = __uint_as_float(b1);
                             float e = 0.0f;
-                            if (lane_real && pl == pp)
-                                e = row_terms_precise(f2u_exact(32.0f * fa0), f2u_exact(32.0f * fb0),
-                                                      f2u_exact(32.0f * fa1), f2u_exact(32.0f * fb1),
-                                                      f2u_exact(32.0f * (fT1 - fa0 - fa1)),
-                                                      f2u_exact(32.0f * (fT0 - fb0 - fb1)), mc);
+                            if (lane_real && pl == pp) e = row_precise(cs, cn, jsel);
                             e = seg_sum<kPR>(e, pos);
-                            if (lane_real && pl == pp && pos == 0) {
-                                const float score = __fdiv_rn(e, mc.fm);
-                                if (score >= thr) {
-                                    const int32_t j = jb + jsel;
-                                    uint64_t rk_sum = 0;
-#pragma unroll
-                                    for (int tt = 0; tt < km1; tt++)
-                                        rk_sum += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                                    rk_sum += binom_at(d.binom, d.n, d.n - 1 - j, 1);
-                                    const int slot = list_len + atomicAdd(&ES.nbuf, 1);
-                                    sc[slot] = score;
-                                    rk[slot] = DS.total - 1 - rk_sum;
-                                }
-                            }
-                        }
-                    }
-                  }
-                } else {
-#pragma unroll
-                for (int jj = 0; jj < 8; jj++) {
-                    const int32_t j = jb + jj;
-                    // accumulator values x = count / 32 (exact); with
-                    // t(x) = x log2 x, T(32 x) = 32 t(x) + 160 x and the
-                    // linear parts cancel within a cell, so the screen sums
-                    // t over the raw values and scales once
-                    const float fa0 = __uint_as_float(cs[2 * jj]), fa1 = __uint_as_float(cs[2 * jj + 1]);
-                    const float fb0 = __uint_as_float(cn[2 * jj]), fb1 = __uint_as_float(cn[2 * jj + 1]);
-                    const float fa2 = fT1 - fa0 - fa1, fb2 = fT0 - fb0 - fb1;
-                    const bool valid = prow && j >= jlo && j < jhi;
-                    if (P.dump && valid) {
-                        const uint32_t a0 = f2u_exact(32.0f * fa0), a1 = f2u_exact(32.0f * fa1),
-                                       a2 = f2u_exact(32.0f * fa2);
-                        const uint32_t b0 = f2u_exact(32.0f * fb0), b1 = f2u_exact(32.0f * fb1),
-                                       b2 = f2u_exact(32.0f * fb2);
-                        uint64_t rs = 0;
-#pragma unroll
-                        for (int tt = 0; tt < km1; tt++) rs += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                        rs += binom_at(d.binom, d.n, d.n - 1 - j, 1);
-                        constexpr int cells = kPR * 3;
-                        uint32_t *o = P.dump + (DS.total - 1 - rs) * 2 * cells;
-                        o[pos * 3 + 0] = a0; o[pos * 3 + 1] = a1; o[pos * 3 + 2] = a2;
-                        o[cells + pos * 3 + 0] = b0; o[cells + pos * 3 + 1] = b1; o[cells + pos * 3 + 2] = b2;
-                    }
-                    float v = 0.0f;
-                    if (prow)
-                        v = (tlog32(fa0) + tlog32(fb0) - tlog32(fa0 + fb0)) +
-                            (tlog32(fa1) + tlog32(fb1) - tlog32(fa1 + fb1)) +
-                            (tlog32(fa2) + tlog32(fb2) - tlog32(fa2 + fb2));
-                    v = seg_sum<kPR>(v, pos);
-                    const float approx = fmaf(v, vscale, voff);
-                    const bool cand = valid && pos == 0 && approx >= cut;
-                    uint32_t seg_mask = __ballot_sync(0xffffffffu, cand);
-                    while (seg_mask) {
-                        const int leader = __ffs(seg_mask) - 1;
-                        seg_mask &= seg_mask - 1;
-                        float e = 0.0f;
-                        if (l / kPR == leader / kPR && lane_real)
-                            e = row_terms_precise(f2u_exact(32.0f * fa0), f2u_exact(32.0f * fb0),
-                                                  f2u_exact(32.0f * fa1), f2u_exact(32.0f * fb1),
-                                                  f2u_exact(32.0f * fa2), f2u_exact(32.0f * fb2), mc);
-                        e = seg_sum<kPR>(e, pos);
-                        if (l == leader) {
-                            const float score = __fdiv_rn(e, mc.fm);
-                            if (score >= thr) {
-                                uint64_t rk_sum = 0;
-#pragma unroll
-                                for (int tt = 0; tt < km1; tt++)
-                                    rk_sum += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], K - tt);
-                                rk_sum += binom_at(d.binom, d.n, d.n - 1 - j, 1);
-                                const int slot = list_len + atomicAdd(&ES.nbuf, 1);
-                                sc[slot] = score;
-                                rk[slot] = DS.total - 1 - rk_sum;
-                            }
+                            if (lane_real && pl == pp && pos == 0) keep(__fdiv_rn(e, mc.fm), jb + jsel);
                         }
                     }
                 }
-                }
-                if (jc % kJcPerCheck == kJcPerCheck - 1) {
-                    epi_bar<kEpiThreads>();
-                    // the next check interval adds at most kJcPerCheck chunks
-                    // of 8 last SNPs per column group and prefix of the tile:
-                    // sort and trim first if the buffer could not hold them
-                    if (ES.list_len + ES.nbuf + kJcPerCheck * 8 * kCG * kPPT > P.cand_p2)
-                        epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS.global_thr, tid);
-                    thr = ES.thr;
-                    cut = thr - DS.delta;
-                    list_len = ES.list_len;
-                }
+                refresh();
+                epi_bar<kEpiThreads>();
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&desc_empty[dq]);
-            epi_bar<kEpiThreads>();
-            if (tid == 0) ES.stop = abort_flag;
-            epi_bar<kEpiThreads>();
             if (ES.stop) break;
+            if (lane == 0) mbar_arrive(&desc_empty[dq]);
+            thr = ES.next_thr;
+            // the next item adds at most one candidate per last SNP and
+            // prefix: sort and trim first if the buffer could not hold them
+            if (ES.list_len + ES.nbuf + kJ * kPPT > P.cand_p2)
+                epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS.global_thr, tid);
+            // no candidate of the next item before every warp has read nbuf
+            epi_bar<kEpiThreads>();
+            thr = fmaxf(thr, ES.thr);
         }
         epi_bar<kEpiThreads>();
         if (ES.nbuf > 0) epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS.global_thr, tid);
@@ -1357,7 +1521,7 @@ __global__ void __launch_bounds__(1024) item_cum_kernel(DevData d, int k, int pp
         if (c < k - 2 || c > n - 2) return 0;
         const uint64_t t0 = (pcum[c] + ppt - 1) / ppt;
         const uint64_t t1 = (pcum[c + 1] + ppt - 1) / ppt;
-        return (t1 - t0) * (uint64_t)((n - 1 - c + kj - 1) / kj);
+        return (t1 - t0) * (uint64_t)panel_ntiles(n, c, kj);
     };
     s = 0;
     for (int64_t c = cb; c < ce; c++) s += items(c);
@@ -1369,35 +1533,41 @@ __global__ void __launch_bounds__(1024) item_cum_kernel(DevData d, int k, int pp
     if (threadIdx.x == 1023) cum[n] = all;
 }
 
-// B operand: row 2j+g (g = 0, 1) of SNP j, K byte 32 w + 4 i + b = individual
-// 32 w + 8 b + i (the A producer's order); where the genotype is g the byte
-// is a power of two, else 0.  The producer's A bytes by position i are 0x10,
-// 0x20, 0x40, 0x08 (twice), and B's are 0x38, 0x28, 0x08, 0x40:
-//   read as E4M3, A = 2^-5, 2^-3, 2^1, 2^-6 and B = 2^0, 2^-2, 2^-6, 2^1, so
-//   every product of two ones is 2^-5 (separate-class variant, case_shift 0);
-//   read as E5M2, A = 2^-11, 2^-7, 2^1, 2^-13 and B = 2^-1, 2^-5, 2^-13,
-//   2^1, so every product is 2^-12; the case words (w < W1) add p to B's
-//   exponent field (case_shift = 4 p, p <= 14 keeps it finite), making their
-//   products 2^(p-12) (combined-class variant).
-__global__ void build_b8_kernel(DevData d, unsigned char *__restrict__ b8, uint32_t case_shift)
+// B operand: rows 4 h + {0, 1} are genotype 0 of SNPs 2 h and 2 h + 1, rows
+// 4 h + {2, 3} genotype 1 (zero rows past the last SNP); the 16 bytes of mask
+// word w hold, in nibble b of 32-bit word i, individual 32 w + 4 b + i (the A
+// producer's order): 2, 1, 0.5 or 0.5 by i where the genotype is the row's.
+__global__ void build_b4_kernel(DevData d, uint4 *__restrict__ b4)
 {
-    const uint32_t bval[8] = {0x38u, 0x28u, 0x08u, 0x40u, 0x38u, 0x28u, 0x08u, 0x40u};
-    const int64_t Kt = (int64_t)d.Wt * 32;
-    const int64_t per_row = Kt / 16;
-    const int64_t total = 2 * d.n * per_row;
+    const int64_t total = 4 * ((d.n + 1) / 2) * d.Wt;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
          idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = idx / per_row;
-        const int64_t q = idx - row * per_row;            // 16-byte piece
-        const int64_t j = row >> 1;
-        const int g = (int)(row & 1);
-        const uint32_t word = d.masks[(j * 3 + g) * d.Wt + (q >> 1)];
-        const int i0 = (int)(q & 1) * 4;
-        const uint32_t add = (q >> 1) < d.W1 ? case_shift : 0u;
-        uint32_t o[4];
-#pragma unroll
-        for (int t = 0; t < 4; t++) o[t] = ((word >> (i0 + t)) & 0x01010101u) * (bval[i0 + t] + add);
-        reinterpret_cast<uint4 *>(b8)[idx] = make_uint4(o[0], o[1], o[2], o[3]);
+        const int64_t row = idx / d.Wt;
+        const int64_t w = idx - row * d.Wt;
+        const int64_t j = 2 * (row >> 2) + (row & 1);
+        const int g = (int)(row >> 1) & 1;
+        const uint32_t v = j < d.n ? d.masks[(j * 3 + g) * d.Wt + w] : 0u;
+        b4[idx] = make_uint4((v & 0x11111111u) << 2, v & 0x22222222u, (v & 0x44444444u) >> 2, (v >> 3) & 0x11111111u);
+    }
+}
+
+// The producers' masks: the 256 individuals of a K stage of every SNP's three
+// genotype rows side by side (96 bytes a SNP; zeros past the last word), so
+// the lanes of a warp, whose rows differ in genotype first, read one or two
+// cache lines per load instead of one per genotype.  One SNP of zeros follows
+// the last (rows of no prefix), and kRowsAhead unwritten stages the last one
+// (the producers' prefetch runs past it).
+constexpr int kRowsAhead = 2 * EPI_TC_PREFETCH * Roles::ProdGroups;
+__global__ void build_rows_kernel(DevData d, uint4 *__restrict__ rows)
+{
+    const int64_t nst = (d.Wt + 7) / 8;
+    const int64_t per = (d.n + 1) * 6;
+    const int64_t total = nst * per;
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t st = idx / per, q = idx - st * per;
+        const int64_t w = st * 8 + (q & 1) * 4;
+        rows[idx] = w < d.Wt && q < d.n * 6 ? *reinterpret_cast<const uint4 *>(d.masks + (q >> 1) * d.Wt + w) : make_uint4(0, 0, 0, 0);
     }
 }
 
@@ -1418,25 +1588,27 @@ static cudaError_t get_encode()
     return cudaSuccess;
 }
 
-size_t tc_b8_bytes(const DevData &d) { return (size_t)2 * d.n * d.Wt * 32; }
+// the B operand, then (256-byte aligned) the producers' masks
+static size_t tc_b_bytes(const DevData &d) { return ((size_t)4 * ((d.n + 1) / 2) * d.Wt * 16 + 255) & ~(size_t)255; }
+size_t tc_b4_bytes(const DevData &d) { return tc_b_bytes(d) + (size_t)((d.Wt + 7) / 8 + tc::kRowsAhead) * (d.n + 1) * 96; }
 
-cudaError_t launch_build_b8(const DevData &d, unsigned char *b8, int num_sms, cudaStream_t st, int comb_p)
+cudaError_t launch_build_b4(const DevData &d, unsigned char *b4, int num_sms, cudaStream_t st)
 {
-    const int64_t total = 2 * d.n * (int64_t)d.Wt * 2;
+    const int64_t total = 4 * ((d.n + 1) / 2) * (int64_t)d.Wt;
     int64_t blocks = (total + 255) / 256;
     if (blocks > (int64_t)num_sms * 16) blocks = (int64_t)num_sms * 16;
-    tc::build_b8_kernel<<<(unsigned)(blocks < 1 ? 1 : blocks), 256, 0, st>>>(d, b8, 4u * (uint32_t)comb_p);
+    if (blocks < 1) blocks = 1;
+    tc::build_b4_kernel<<<(unsigned)blocks, 256, 0, st>>>(d, reinterpret_cast<uint4 *>(b4));
+    tc::build_rows_kernel<<<(unsigned)blocks, 256, 0, st>>>(d, reinterpret_cast<uint4 *>(b4 + tc_b_bytes(d)));
     return cudaGetLastError();
 }
 
-// Class shift p of the combined-class variant for an order-k search of d, or
-// 0 where it does not apply: order 3 (at order 4 its single producer group
-// bounds it, measured slower than separate classes); the control count must
-// fit below 2^p and the accumulator value ctrl + case 2^p below 2^23 (the
-// decode's exact range; FP32 accumulation of such integers is exact).
-int tc_comb_shift(const DevData &d, int k)
+// Class shift p of the combined-class variant for a search of d, or 0 where
+// the separate-class variant runs: the control count must fit below 2^p and
+// the accumulator value ctrl + case 2^p below 2^23 (the decode's exact range;
+// FP32 accumulation of such integers is exact).
+int tc_comb_shift(const DevData &d)
 {
-    if (k != 3) return 0;
     int p = 1;
     while (p < 15 && (1ll << p) <= d.m0) p++;
     if (p > 14) return 0;
@@ -1444,6 +1616,7 @@ int tc_comb_shift(const DevData &d, int k)
     return p;
 }
 
+static int tc_tile_snps(bool comb) { return comb ? tc::Shape<true>::J : tc::Shape<false>::J; }
 static int tc_pr(int k) { return k == 2 ? 3 : (k == 3 ? 9 : (k == 4 ? 27 : 81)); }
 static int tc_ppt(int k) { return tc_pr(k) > 32 ? 1 : 4 * (32 / tc_pr(k)); }
 
@@ -1466,12 +1639,12 @@ uint64_t tc_item_count(int64_t n, int k, int64_t a, int64_t b, int kj)
         const uint64_t t0 = (pc + ppt - 1) / ppt;
         pc += cnt;
         const uint64_t t1 = (pc + ppt - 1) / ppt;
-        total += (t1 - t0) * (uint64_t)((n - 1 - c + kj - 1) / kj);
+        total += (t1 - t0) * (uint64_t)tc::panel_ntiles(n, c, kj);
     }
     return total;
 }
 
-uint64_t tc_item_count(int64_t n, int k) { return tc_item_count(n, k, 0, n - k, tc::Shape<false>::J); }
+uint64_t tc_item_count(int64_t n, int k, bool comb) { return tc_item_count(n, k, 0, n - k, tc_tile_snps(comb)); }
 
 // First SNP of the combination of lexicographic rank r: the largest s with
 // C(n, k) - C(n - s, k) <= r (the combinations starting below s come first).
@@ -1497,55 +1670,102 @@ uint64_t tc_range_work(int64_t n, int k, uint64_t rb, uint64_t re)
     return host_binom(n - a, k) - host_binom(n - b - 1, k);
 }
 
-int tc_prefixes_per_warp(int k)
-{
-    const int PR = k == 2 ? 3 : (k == 3 ? 9 : (k == 4 ? 27 : 81));
-    return PR <= 32 ? 32 / PR : 0;
-}
+// Candidate buffer entries: the pool plus one item's combinations, rounded up
+// to a power of two for the bitonic sort.
+int tc_cand_p2(int k, int pool, bool comb) { return next_pow2(pool + tc_tile_snps(comb) * tc_ppt(k)); }
 
-// Candidate buffer entries: the pool plus one check interval (2 chunks of 8
-// last SNPs, both halves, every prefix of the tile; order 2 checks every
-// chunk), rounded up to a power of two for the bitonic sort.
-int tc_cand_p2(int k, int pool, bool comb)
+size_t tc_smem_bytes(int cand_p2, bool cand_global, bool comb)
 {
-    const int groups = tc::roles_epi_warps(comb, k) / 4;
-    const int check = k == 2 ? 1 : tc::roles_check_iters(comb, k);
-    return next_pow2(pool + check * 8 * groups * tc_ppt(k));
-}
-
-size_t tc_smem_bytes(int cand_p2, int k, bool cand_global, bool comb)
-{
-    const size_t transpose =
-        (k == 3 || k == 4) ? (size_t)tc::roles_epi_warps(comb, k) * 256 * 4 + 16 : 0;
     const size_t rings = comb ? (size_t)tc::Shape<true>::Stages * (tc::kTileBytes + tc::Shape<true>::BBytes)
                               : (size_t)tc::Shape<false>::Stages * (tc::kTileBytes + tc::Shape<false>::BBytes);
-    return 1024 + rings + (cand_global ? 0 : (size_t)cand_p2 * 12) + 2 * 128 * tc::kMaxProdGroups * 2 * 4 +
-           tc::kDescDepth * sizeof(tc::Desc) + 64 + transpose;
+    return 1024 + rings + (cand_global ? 0 : (size_t)cand_p2 * 12) + 2 * 128 * tc::Roles::ProdGroups * 2 * 4 +
+           tc::kDescDepth * sizeof(tc::Desc) + (size_t)tc::Roles::EpiWarps * 256 * 4;
 }
 
-
-static cudaError_t encode_map(CUtensorMap *map, const DevData &d, const unsigned char *b8, bool comb)
+static cudaError_t encode_map(CUtensorMap *map, const DevData &d, const unsigned char *b4, bool comb)
 {
     cudaError_t e = get_encode();
     if (e != cudaSuccess) return e;
-    const int64_t Kt = (int64_t)d.Wt * 32;
-    cuuint64_t gdim[2] = {(cuuint64_t)Kt, (cuuint64_t)(2 * d.n)};
-    cuuint64_t gstride[1] = {(cuuint64_t)Kt};
-    cuuint32_t box[2] = {(cuuint32_t)tc::kKC, comb ? (cuuint32_t)tc::Shape<true>::N : (cuuint32_t)tc::Shape<false>::N};
+    const int64_t row = (int64_t)d.Wt * 16;
+    cuuint64_t gdim[2] = {(cuuint64_t)row, (cuuint64_t)(4 * ((d.n + 1) / 2))};
+    cuuint64_t gstride[1] = {(cuuint64_t)row};
+    cuuint32_t box[2] = {(cuuint32_t)tc::kRowBytes, (cuuint32_t)(2 * tc_tile_snps(comb))};
     cuuint32_t estr[2] = {1u, 1u};
-    CUresult cr = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<unsigned char *>(b8), gdim, gstride, box,
+    CUresult cr = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<unsigned char *>(b4), gdim, gstride, box,
                            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return cr == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// The screen's constants and margins (see cell_bound).
+static void fill_screen(tc::DsParams &D, const DevData &d, int k, int comb_p)
+{
+    const double u = 5.9604644775390625e-8, m = (double)d.m;
+    const double pi = (double)d.m1 / m;
+    const double p2 = (double)(1 << comb_p);
+    D.poly = pi >= 0.2 && pi <= 0.8;
+    if (!D.poly) {
+        // fast logarithms: m MI / ln 2 = T(m) - T(m1) - T(m0) + sum over cells
+        // of t(a) + t(b) - t(a + b), T = t on counts.  Margin: relative errors
+        // of the log2 approximation (2^-21) and of the float sums over the
+        // terms' magnitude T(m) + T(m1) + T(m0), doubled
+        auto T = [](double c) { return c > 0 ? c * log2(c) : 0.0; };
+        const int64_t cells = (int64_t)tc_pr(k) * 3;
+        const double mag = T(m) + T((double)d.m1) + T((double)d.m0);
+        D.vscale = (float)(0.6931471805599453 / m);
+        D.voff = (float)((T(m) - T((double)d.m1) - T((double)d.m0)) * 0.6931471805599453 / m);
+        D.cut_mul = 1.0f;
+        D.cut_add = (float)(2.0 * (4.0 * 4.76837158203125e-7 + (double)(2 * cells + 40) * u) * mag *
+                            0.6931471805599453 / m) + 1e-7f;
+        D.sc_pi = (float)(pi * p2);
+        D.c2 = D.c3 = D.c4 = D.c5a = D.c5b = 0.0f;
+        return;
+    }
+    const double v = pi * (1.0 - pi), q = 1.0 - pi;
+    const double c2 = 0.5 / v, c3 = (2.0 * pi - 1.0) / (6.0 * v * v);
+    // g at -pi (a cell without cases), 0 and 1 - pi (a cell without controls)
+    const double g0 = (-log(q) - c2 * pi * pi + c3 * pi * pi * pi) / (pi * pi * pi * pi);
+    const double gm = (2.0 / (pi * pi * pi) + 2.0 / (q * q * q)) / 24.0;
+    const double g1 = (-log(pi) - c2 * q * q - c3 * q * q * q) / (q * q * q * q);
+    const double slope_n = (g0 - gm) / pi, slope_p = (g1 - gm) / q;   // of g against |x|
+    const double c5a = 0.5 * (slope_p - slope_n), c5b = 0.5 * (slope_p + slope_n);
+    D.sc_pi = (float)(pi * p2);
+    D.c2 = (float)c2;
+    D.c3 = (float)(c3 / p2);
+    D.c4 = (float)(gm / (p2 * p2));
+    D.c5a = (float)(c5a / (p2 * p2 * p2));
+    D.c5b = (float)(c5b / (p2 * p2 * p2));
+    D.vscale = (float)(1.0 / (p2 * p2 * m));
+    D.voff = 0.0f;
+    // Rounding (u = 2^-24).  e: at most 2 u of the cell's individuals (pi and
+    // the fused product), so 2 u m over all cells, times the bound's slope; x: the
+    // reciprocal's and the product's 3 u relative, times the slope |x q'| / q;
+    // the polynomial's products and sums: 8 u of its terms' magnitudes, and
+    // its value's own 2 u; the sums over at most 81 rows, all terms positive:
+    // 40 u relative.  The ratios are evaluated on a grid and doubled.
+    double slope = 0.0, rel = 0.0;
+    for (int t = -32; t <= 32; t++) {
+        if (t == 0) continue;
+        const double x = t < 0 ? pi * t / 32.0 : q * t / 32.0, ax = fabs(x);
+        const double w = c2 + x * (c3 + x * (gm + c5a * x + c5b * ax));
+        const double mag = c2 + ax * (fabs(c3) + ax * (gm + (fabs(c5a) + fabs(c5b)) * ax));
+        const double dq = x * (2.0 * c2 + x * (3.0 * c3 + x * (4.0 * gm + 5.0 * (c5a * x + c5b * ax))));
+        slope = fmax(slope, fabs(dq));
+        rel = fmax(rel, (3.0 * fabs(dq) / (ax * w) + 8.0 * mag / w) * u);
+    }
+    // a precise score at the threshold exceeds MI by at most its own bound
+    D.cut_mul = (float)(1.0 - 2.0 * rel - 42.0 * u - f32_rel_bound(k, d.m));
+    D.cut_add = (float)(2.0 * slope * 2.0 * u) + 1e-9f;
 }
 
 // Per-dataset parameters (host side); the B-operand map goes to tmap_dev when
 // the launch is batched (nullptr: passed as a kernel parameter instead).
 static void fill_ds(tc::DsParams &D, const DevData &d, int k, uint64_t *item_cum, uint32_t *global_thr,
                     uint64_t total, uint64_t rb, uint64_t re, const CUtensorMap *tmap_dev, int cta_begin,
-                    int cta_count, int comb_p)
+                    int cta_count, int comb_p, const unsigned char *b4)
 {
     D.d = d;
+    D.rows = reinterpret_cast<const uint4 *>(b4 + tc_b_bytes(d));
     D.comb_p = comb_p;
     D.rank_begin = rb;
     D.rank_end = re;
@@ -1559,24 +1779,12 @@ static void fill_ds(tc::DsParams &D, const DevData &d, int k, uint64_t *item_cum
         else np += host_subsets_from(c, D.s1_lo, k - 2) - host_subsets_from(c, D.s1_hi + 1, k - 2);
     }
     D.n_prefix = np;
-    D.n_items = tc_item_count(d.n, k, D.s1_lo, D.s1_hi, comb_p ? tc::Shape<true>::J : tc::Shape<false>::J);
+    D.n_items = tc_item_count(d.n, k, D.s1_lo, D.s1_hi, tc_tile_snps(comb_p != 0));
     D.item_cum = item_cum;
     D.pcum = item_cum + d.n + 1;
-    const int64_t Kt = (int64_t)d.Wt * 32;
-    D.chunks = (int)(Kt / tc::kKC);
-    D.chunks_case = (int)((int64_t)d.W1 * 32 / tc::kKC);
-    auto T = [](double c) { return c > 0 ? c * log2(c) : 0.0; };
-    D.tconst = (float)(T((double)d.m) - T((double)d.m1) - T((double)d.m0));
-    D.ln2_over_m = (float)(0.6931471805599453 / (double)d.m);
-    // screening margin: relative errors of the log2 approximation (2^-21)
-    // and of the float sums over (T(m) + T(m1) + T(m0)), doubled
-    const int64_t cells = (int64_t)tc_pr(k) * 3;
-    // bound on the summed magnitudes of the screen's terms: with t(x) =
-    // T(32 x) / 32 - 5 x over accumulator values x = count / 32, 32 sum |t|
-    // <= sum T(c) + 5 sum c <= T(m) + T(m1) + T(m0) + 10 m
-    const double mag = T((double)d.m) + T((double)d.m1) + T((double)d.m0) + 10.0 * (double)d.m;
-    D.delta = (float)(2.0 * (4.0 * 4.76837158203125e-7 + (double)(2 * cells + 40) * 5.9604644775390625e-8) * mag *
-                      0.6931471805599453 / (double)d.m) + 1e-7f;
+    D.chunks = d.Wt * 32 / tc::kChunk;
+    D.chunks_case = d.W1 * 32 / tc::kChunk;
+    fill_screen(D, d, k, comb_p);
     D.total = total;
     D.global_thr = global_thr;
     D.tmap = tmap_dev;
@@ -1588,10 +1796,6 @@ static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint6
                         int32_t *status, uint32_t *dump, unsigned long long *waits, float *cand_g,
                         uint64_t *rank_g, bool comb)
 {
-    P.k = k;
-    P.PR = tc_pr(k);
-    P.ppw = P.PR > 32 ? 0 : 32 / P.PR;
-    P.ppt = tc_ppt(k);
     P.pool = pool;
     P.cand_p2 = tc_cand_p2(k, pool, comb);
     P.cand_score_g = cand_g;
@@ -1608,16 +1812,17 @@ static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint6
 static cudaError_t launch_kernel(const CUtensorMap &map, const tc::Params &P, int k, int grid, cudaStream_t st,
                                  bool comb)
 {
-    const size_t smem = tc_smem_bytes(P.cand_p2, k, P.cand_score_g != nullptr, comb);
-    auto kern = k == 2   ? tc::tc_search_kernel<2, false>
-                : k == 3 ? (comb ? tc::tc_search_kernel<3, true> : tc::tc_search_kernel<3, false>)
-                : k == 4 ? tc::tc_search_kernel<4, false>
-                         : tc::tc_search_kernel<5, false>;
+    const size_t smem = tc_smem_bytes(P.cand_p2, P.cand_score_g != nullptr, comb);
+    using Kernel = void (*)(const CUtensorMap, const tc::Params);
+    static const Kernel kernels[2][4] = {
+        {tc::tc_search_kernel<2, false>, tc::tc_search_kernel<3, false>, tc::tc_search_kernel<4, false>,
+         tc::tc_search_kernel<5, false>},
+        {tc::tc_search_kernel<2, true>, tc::tc_search_kernel<3, true>, tc::tc_search_kernel<4, true>,
+         tc::tc_search_kernel<5, true>}};
+    const Kernel kern = kernels[comb][k - 2];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int threads = comb ? tc::Roles<true, 3>::Threads
-                             : (k == 4 ? tc::Roles<false, 4>::Threads : tc::Roles<false, 3>::Threads);
-    kern<<<grid, threads, smem, st>>>(map, P);
+    kern<<<grid, tc::Roles::Threads, smem, st>>>(map, P);
     return cudaGetLastError();
 }
 
@@ -1625,19 +1830,18 @@ cudaError_t launch_tc_item_cum(const DevData &d, int k, uint64_t rb, uint64_t re
                                cudaStream_t st, bool comb)
 {
     const int32_t a = (int32_t)tc_first_snp(d.n, k, rb), b = (int32_t)tc_first_snp(d.n, k, re - 1);
-    const int kj = comb ? tc::Shape<true>::J : tc::Shape<false>::J;
-    tc::item_cum_kernel<<<1, 1024, 0, st>>>(d, k, tc_ppt(k), kj, a, b, item_cum + d.n + 1, item_cum);
+    tc::item_cum_kernel<<<1, 1024, 0, st>>>(d, k, tc_ppt(k), tc_tile_snps(comb), a, b, item_cum + d.n + 1, item_cum);
     return cudaGetLastError();
 }
 
-cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b8, uint64_t *item_cum, int pool,
+cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, uint64_t *item_cum, int pool,
                              uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                              int32_t *status, int grid, uint64_t total, uint64_t rb, uint64_t re, cudaStream_t st,
                              int *cand_p2_out, float *cand_g, uint64_t *rank_g, uint32_t *dump,
                              unsigned long long *waits, unsigned long long wait_ns, int comb_p)
 {
     tc::Params P;
-    fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p);
+    fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p, b4);
     P.many = nullptr;
     P.cta_ds = nullptr;
     fill_launch(P, k, pool, list_score, list_rank, list_count, status, dump, waits, cand_g, rank_g, comb_p != 0);
@@ -1646,34 +1850,34 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b8, u
     cudaError_t e = launch_tc_item_cum(d, k, rb, re, item_cum, st, comb_p != 0);
     if (e != cudaSuccess) return e;
     CUtensorMap map;
-    e = encode_map(&map, d, b8, comb_p != 0);
+    e = encode_map(&map, d, b4, comb_p != 0);
     if (e != cudaSuccess) return e;
     return launch_kernel(map, P, k, grid, st, comb_p != 0);
 }
 
 size_t tc_ds_bytes() { return sizeof(tc::DsParams); }
 
-cudaError_t tc_fill_batch_entry(void *ds_host, void *tmap_host, const DevData &d, int k, const unsigned char *b8,
+cudaError_t tc_fill_batch_entry(void *ds_host, void *tmap_host, const DevData &d, int k, const unsigned char *b4,
                                 uint64_t *item_cum, uint32_t *global_thr, uint64_t total, const void *tmap_dev,
-                                int cta_begin, int cta_count)
+                                int cta_begin, int cta_count, int comb_p)
 {
     fill_ds(*static_cast<tc::DsParams *>(ds_host), d, k, item_cum, global_thr, total, 0, total,
-            static_cast<const CUtensorMap *>(tmap_dev), cta_begin, cta_count, 0);
-    return encode_map(static_cast<CUtensorMap *>(tmap_host), d, b8, false);
+            static_cast<const CUtensorMap *>(tmap_dev), cta_begin, cta_count, comb_p, b4);
+    return encode_map(static_cast<CUtensorMap *>(tmap_host), d, b4, comb_p != 0);
 }
 
 cudaError_t launch_tc_batch(const void *ds_dev, const int32_t *cta_ds_dev, int k, int pool, float *list_score,
                             uint64_t *list_rank, int32_t *list_count, int32_t *status, int grid, cudaStream_t st,
-                            float *cand_g, uint64_t *rank_g)
+                            float *cand_g, uint64_t *rank_g, bool comb)
 {
     tc::Params P;
     P.one = tc::DsParams();
     P.many = static_cast<const tc::DsParams *>(ds_dev);
     P.cta_ds = cta_ds_dev;
-    fill_launch(P, k, pool, list_score, list_rank, list_count, status, nullptr, nullptr, cand_g, rank_g, false);
+    fill_launch(P, k, pool, list_score, list_rank, list_count, status, nullptr, nullptr, cand_g, rank_g, comb);
     CUtensorMap unused;
     memset(&unused, 0, sizeof(unused));
-    return launch_kernel(unused, P, k, grid, st, false);
+    return launch_kernel(unused, P, k, grid, st, comb);
 }
 
 }  // namespace epi
