@@ -41,6 +41,8 @@ struct epi_ctx {
     unsigned long long *waits_dev = nullptr;   // own buffer: per-role wait cycles of a profiled TC search
     int waits_grid = 0;                        // CTAs recorded in waits_dev (0: nothing recorded)
     bool destroy_requested = false;
+    void *result_host = nullptr;   // pinned staging of one search's results (at most kResultStaging bytes)
+    size_t result_host_bytes = 0;
     // test controls (epi_set_wait_limit, epi_inject_alloc_failure)
     unsigned long long wait_limit_ns = 0;   // tensor-core pipeline waits; 0 = the kernels' default
     int64_t fail_alloc_in = -1;             // device allocations until one fails; -1 = none
@@ -317,7 +319,12 @@ epi_status choose_path(const epi_dataset *ds, int k, int path, uint64_t rb, uint
         // automatic choice: the tensor path counts whole first-SNP blocks, so
         // it is taken for a rank range only when that adds at most as much
         // work again as the range itself
-        tc = ok && k >= 3 && (re - rb == total || tc_range_work(ds->n, k, rb, re) <= 2 * (re - rb));
+        tc = ok && (re - rb == total || tc_range_work(ds->n, k, rb, re) <= 2 * (re - rb));
+        // order 2: the popcount kernel starts faster, the tensor path counts
+        // faster; they meet near 2e8 combination words (1000 x 8192: 0.66 ms
+        // popcount, 0.54 tensor; 2000 x 2500: 0.61 and 0.72; 4000 x 2500:
+        // 1.48 and 0.90; 8000 x 8192: 22.1 and 1.5)
+        if (k == 2 && (double)(re - rb) * (double)ds->Wt < 2e8) tc = false;
         auto it = ds->ctx->tune.find(tune_key(k, ds->n, ds->Wt));
         if (ok && it != ds->ctx->tune.end() && it->second.path) tc = it->second.path == EPI_PATH_TC;
     }
@@ -349,9 +356,22 @@ epi_status make_plan(const epi_dataset *ds, SearchPlan &p, int path)
     return EPI_OK;
 }
 
-// Queues one search pass with the given plan; results land in device memory.
+// Where a search pass leaves its results when the caller gives no buffers:
+// in the scratch arena, records then tables in one piece; status and count
+// words in its first kHeadBytes.
+constexpr size_t kHeadBytes = 768, kHeadStatus = 256, kHeadCount = 512;
+struct ScratchOut {
+    bool counts = false;                // tables wanted
+    char *head = nullptr;               // kHeadBytes: status at kHeadStatus, record count at kHeadCount
+    char *results = nullptr;            // top_n records, then (256-byte aligned) tables
+    size_t counts_at = 0, bytes = 0;
+};
+
+// Queues one search pass with the given plan; results land in device memory
+// (the caller's, or with own != NULL the scratch arena).
 epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_result *out_dev, uint32_t *counts_dev,
-                        int32_t *n_out_dev, int32_t **status_dev_out, uint32_t *dump = nullptr)
+                        int32_t *n_out_dev, int32_t **status_dev_out, uint32_t *dump = nullptr,
+                        ScratchOut *own = nullptr)
 {
     epi_ctx *ctx = ds->ctx;
     (void)path;
@@ -359,6 +379,10 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     Arena a;
     const size_t o_thr = a.take<uint32_t>(1);
     const size_t o_status = a.take<int32_t>(1);
+    const size_t o_nout = a.take<int32_t>(1);
+    const size_t rec_bytes = ((size_t)p.top_n * sizeof(epi_result) + 255) & ~(size_t)255;
+    const size_t res_bytes = rec_bytes + (own && own->counts ? (size_t)p.top_n * 2 * cells * 4 : 0);
+    const size_t o_res = own ? a.take<char>(res_bytes) : 0;
     const size_t o_ls = a.take<float>((size_t)p.grid * p.pool);
     const size_t o_lr = a.take<uint64_t>((size_t)p.grid * p.pool);
     const size_t o_lc = a.take<int32_t>((size_t)p.grid);
@@ -397,8 +421,17 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
         st = ensure_b4(ds);
         if (st != EPI_OK) return st;
     }
-    // threshold word and status word live in the first 512 bytes
-    CK(cudaMemsetAsync(base, 0, 512, ctx->stream));
+    if (own) {
+        own->head = base;
+        own->results = base + o_res;
+        own->counts_at = rec_bytes;
+        own->bytes = res_bytes;
+        out_dev = reinterpret_cast<epi_result *>(base + o_res);
+        counts_dev = own->counts ? reinterpret_cast<uint32_t *>(base + o_res + rec_bytes) : nullptr;
+        n_out_dev = reinterpret_cast<int32_t *>(base + o_nout);
+    }
+    static_assert(kHeadStatus == 256 && kHeadCount == 512, "the arena's alignment");
+    CK(cudaMemsetAsync(base, 0, kHeadBytes, ctx->stream));
     const DevData d = ds->dev();
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (ctx->profiling) {
@@ -421,7 +454,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
                             p.total, p.rb, p.re, ctx->stream, &cand_p2,
                             tc_cg ? reinterpret_cast<float *>(base + o_tcs) : nullptr,
                             tc_cg ? reinterpret_cast<uint64_t *>(base + o_tcr) : nullptr, dump, waits,
-                            ctx->wait_limit_ns, p.comb_p));
+                            ctx->wait_limit_ns, p.comb_p, p.top_n));
         ctx->launches += 1;   // item table
     } else {
         CK(launch_popc_search(d, p.k, p.R, p.rb, p.re, p.tile, p.pool, p.slots, p.cand_p2, thr, ls, lr, lc, p.grid,
@@ -464,6 +497,7 @@ int initial_pool(int top_n)
 }
 
 constexpr int kMaxPool = 4096;
+constexpr size_t kResultStaging = (size_t)4 << 20;
 
 epi_status run_search_sync(epi_dataset *ds, int order, int top_n, int path, uint64_t rb, uint64_t re,
                            epi_result *out, uint32_t *counts, int *n_out)
@@ -484,36 +518,45 @@ epi_status run_search_sync(epi_dataset *ds, int order, int top_n, int path, uint
         p.k = order; p.top_n = top_n; p.pool = pool; p.rb = rb; p.re = re; p.total = total;
         st = make_plan(ds, p, path);
         if (st != EPI_OK) return st;
-        // device-side outputs of this pass (stream-ordered allocation)
-        const size_t rec_b = ((size_t)top_n * sizeof(epi_result) + 255) & ~(size_t)255;
-        const size_t cnt_b = ((size_t)top_n * 2 * cells * 4 + 255) & ~(size_t)255;
-        void *dout = nullptr;
-        CK(ctx_malloc_async(ctx, &dout, rec_b + cnt_b + 256, ctx->stream));
-        epi_result *out_dev = static_cast<epi_result *>(dout);
-        uint32_t *cnt_dev = reinterpret_cast<uint32_t *>(static_cast<char *>(dout) + rec_b);
-        int32_t *nout_dev = reinterpret_cast<int32_t *>(static_cast<char *>(dout) + rec_b + cnt_b);
+        ScratchOut so;
+        so.counts = counts != nullptr;
         int32_t *status_dev = nullptr;
-        st = queue_search(ds, p, path, out_dev, counts ? cnt_dev : nullptr, nout_dev, &status_dev);
-        if (st != EPI_OK) { cudaFreeAsync(dout, ctx->stream); return st; }
-        int32_t hst[2] = {0, 0};
-        CK(cudaMemcpyAsync(&hst[0], status_dev, 4, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaMemcpyAsync(&hst[1], nout_dev, 4, cudaMemcpyDeviceToHost, ctx->stream));
+        st = queue_search(ds, p, path, nullptr, nullptr, nullptr, &status_dev, nullptr, &so);
+        if (st != EPI_OK) return st;
+        // status, count, records and tables come back through one pinned
+        // buffer with one wait (a pageable copy waits by itself); large
+        // tables go straight to the caller
+        const size_t staged = so.bytes <= kResultStaging ? so.bytes : so.counts_at;
+        if (ctx->result_host_bytes < kHeadBytes + staged) {
+            if (ctx->result_host) cudaFreeHost(ctx->result_host);
+            ctx->result_host = nullptr;
+            ctx->result_host_bytes = 0;
+            CK(cudaMallocHost(&ctx->result_host, kHeadBytes + staged));
+            ctx->result_host_bytes = kHeadBytes + staged;
+        }
+        char *host = static_cast<char *>(ctx->result_host);
+        CK(cudaMemcpyAsync(host, so.head, kHeadBytes, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaMemcpyAsync(host + kHeadBytes, so.results, staged, cudaMemcpyDeviceToHost, ctx->stream));
         CK(cudaStreamSynchronize(ctx->stream));
-        if (hst[0] & ST_POOL_OVERFLOW) {
-            cudaFreeAsync(dout, ctx->stream);
+        int32_t status, n;
+        memcpy(&status, host + kHeadStatus, 4);
+        memcpy(&n, host + kHeadCount, 4);
+        if (status & ST_POOL_OVERFLOW) {
             if (pool >= kMaxPool)
                 return fail(EPI_EOVERFLOW, "candidate pool of %d cannot prove the exact top %d (ties)", pool, top_n);
             pool = std::min(pool * 4, kMaxPool);
             continue;
         }
-        if (hst[0] & ST_TIMEOUT) { cudaFreeAsync(dout, ctx->stream); return fail(EPI_ETIMEOUT, "device wait expired"); }
-        if (hst[0] != 0) { cudaFreeAsync(dout, ctx->stream); return fail(EPI_ECUDA, "device status 0x%x", hst[0]); }
-        const int n = hst[1];
-        CK(cudaMemcpyAsync(out, out_dev, (size_t)n * sizeof(epi_result), cudaMemcpyDeviceToHost, ctx->stream));
-        if (counts)
-            CK(cudaMemcpyAsync(counts, cnt_dev, (size_t)n * 2 * cells * 4, cudaMemcpyDeviceToHost, ctx->stream));
-        cudaFreeAsync(dout, ctx->stream);
-        CK(cudaStreamSynchronize(ctx->stream));
+        if (status & ST_TIMEOUT) return fail(EPI_ETIMEOUT, "device wait expired");
+        if (status != 0) return fail(EPI_ECUDA, "device status 0x%x", status);
+        const size_t table_bytes = (size_t)n * 2 * cells * 4;
+        if (counts && staged < so.bytes) {
+            CK(cudaMemcpyAsync(counts, so.results + so.counts_at, table_bytes, cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaStreamSynchronize(ctx->stream));
+        } else if (counts) {
+            memcpy(counts, host + kHeadBytes + so.counts_at, table_bytes);
+        }
+        memcpy(out, host + kHeadBytes, (size_t)n * sizeof(epi_result));
         *n_out = n;
         return EPI_OK;
     }
@@ -833,7 +876,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
                 if (g.tc) {
                     CK(tc_fill_batch_entry(hd + dsz * q, hm + 128 * q, d, it.k, it.ds->b4,
                                            reinterpret_cast<uint64_t *>(dev + it.o_ic), thr, it.total,
-                                           dev + g.o_tmap + 128 * q, it.cta_begin, it.cta_count, it.comb_p));
+                                           dev + g.o_tmap + 128 * q, it.cta_begin, it.cta_count, it.comb_p, it.top_n));
                 } else {
                     popc_fill_ds(hd + dsz * q, d, 0, it.total, it.cta_begin, it.cta_count, thr);
                 }
@@ -1320,6 +1363,7 @@ static void free_ctx(epi_ctx *ctx)
     if (ctx->batch_exec) cudaGraphExecDestroy(ctx->batch_exec);
     if (ctx->batch_dev) cudaFree(ctx->batch_dev);
     if (ctx->batch_host) cudaFreeHost(ctx->batch_host);
+    if (ctx->result_host) cudaFreeHost(ctx->result_host);
     if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
     delete ctx;
 }

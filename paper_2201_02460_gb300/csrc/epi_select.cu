@@ -1,7 +1,7 @@
 // Top-N retention (Section 2.4: only the combinations with the highest MI
 // are kept) made exact on the GPU:
-//   1. merge_lists: the per-CTA candidate lists of the search kernel are
-//      merged into one pool ordered by (single-precision score desc, rank asc);
+//   1. merge_level: the per-CTA candidate lists of the search kernel are
+//      merged, level by level, into one pool ordered by (single-precision score desc, rank asc);
 //   2. rescore: every pooled combination is recounted exactly (AND + POPC of
 //      its k genotype rows, Section 2.2) and scored in double precision;
 //   3. finalize: the pool is sorted by (double MI desc, lexicographic rank
@@ -14,66 +14,66 @@
 
 namespace epi {
 
-struct MergeState {
-    int32_t list_len, nbuf;
-    float thr;
-};
+// entries of a block's sort buffers (the sort works on at least two)
+__host__ __device__ inline int merge_entries(int group, int cap) { return next_pow2(group * cap < 2 ? 2 : group * cap); }
 
-__global__ void __launch_bounds__(1024) merge_lists_kernel(const float *__restrict__ ls, const uint64_t *__restrict__ lr,
-                                                           const int32_t *__restrict__ lc, int nlists, int stride,
-                                                           int pool, int cand_p2, float *__restrict__ out_s,
-                                                           uint64_t *__restrict__ out_r, int32_t *__restrict__ out_n,
-                                                           float floor)
+// One level of the merge: block b takes lists [b group, (b + 1) group) -- list
+// i at ls + i pitch with lc[i lstep] entries -- sorts their entries together
+// and keeps the best `pool`: in place as list b group of the next level, or
+// in out_* when this is the last level (one block).  A single block walking
+// all lists in rounds of 1024 took 124 us for 155 lists of 128 (its sorts are
+// serial); two levels of blocks take 2 x 5 us.
+__global__ void __launch_bounds__(1024) merge_level_kernel(float *__restrict__ ls, uint64_t *__restrict__ lr,
+                                                           int32_t *__restrict__ lc, int nlists, int64_t pitch,
+                                                           int lstep, int group, int cap, int pool,
+                                                           float *__restrict__ out_s, uint64_t *__restrict__ out_r,
+                                                           int32_t *__restrict__ out_n, float floor)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    const int entries = merge_entries(group, cap);
     uint64_t *rk = reinterpret_cast<uint64_t *>(smem);
-    float *sc = reinterpret_cast<float *>(rk + cand_p2);
-    __shared__ MergeState S;
-    if (threadIdx.x == 0) { S.list_len = 0; S.nbuf = 0; S.thr = floor; }
+    float *sc = reinterpret_cast<float *>(rk + entries);
+    __shared__ int32_t live_sh;
+    const int first = blockIdx.x * group;
+    const int lists = min(group, nlists - first);
+    if (threadIdx.x == 0) live_sh = 0;
     __syncthreads();
-    const int64_t total = (int64_t)nlists * stride;
-    for (int64_t base = 0; base < total; base += blockDim.x) {
-        const int64_t e = base + threadIdx.x;
-        if (e < total) {
-            const int l = (int)(e / stride);
-            const int i = (int)(e - (int64_t)l * stride);
-            if (i < lc[l]) {
-                const float s = ls[e];
-                if (s >= S.thr) {
-                    const int pos = S.list_len + atomicAdd(&S.nbuf, 1);
-                    sc[pos] = s;
-                    rk[pos] = lr[e];
-                }
+    for (int e = threadIdx.x; e < lists * cap; e += blockDim.x) {
+        const int l = e / cap, i = e - l * cap;
+        if (i < lc[(int64_t)(first + l) * lstep]) {
+            const int64_t at = (int64_t)(first + l) * pitch + i;
+            const float v = ls[at];
+            if (v >= floor) {
+                const int pos = atomicAdd(&live_sh, 1);
+                sc[pos] = v;
+                rk[pos] = lr[at];
             }
         }
-        __syncthreads();
-        const bool last = base + blockDim.x >= total;
-        if (S.nbuf > (int)blockDim.x || (last && S.nbuf > 0)) {
-            const int live = S.list_len + S.nbuf;
-            const int p2 = next_pow2(live < 2 ? 2 : live);
-            for (int i = live + threadIdx.x; i < p2; i += blockDim.x) { sc[i] = floor; rk[i] = ~0ull; }
-            __syncthreads();
-            block_sort_cands(sc, rk, p2);
-            if (threadIdx.x == 0) {
-                S.list_len = live < pool ? live : pool;
-                S.nbuf = 0;
-                if (S.list_len == pool) S.thr = sc[pool - 1];
-            }
-        }
-        __syncthreads();
     }
-    const int L = S.list_len;
-    for (int i = threadIdx.x; i < L; i += blockDim.x) { out_s[i] = sc[i]; out_r[i] = rk[i]; }
-    if (threadIdx.x == 0) *out_n = L;
+    __syncthreads();
+    const int live = live_sh;
+    const int p2 = next_pow2(live < 2 ? 2 : live);
+    for (int i = live + threadIdx.x; i < p2; i += blockDim.x) { sc[i] = floor; rk[i] = ~0ull; }
+    __syncthreads();
+    block_sort_cands(sc, rk, p2);
+    const int L = live < pool ? live : pool;
+    float *os = out_s ? out_s : ls + (int64_t)first * pitch;
+    uint64_t *orr = out_s ? out_r : lr + (int64_t)first * pitch;
+    for (int i = threadIdx.x; i < L; i += blockDim.x) { os[i] = sc[i]; orr[i] = rk[i]; }
+    if (threadIdx.x == 0) *(out_s ? out_n : lc + (int64_t)first * lstep) = L;
 }
 
-// Exact counts of one combination, cell x = sum_t g_t 3^(k-1-t); one thread
-// per (class, cell) pair.
+// Exact counts of one combination, cell x = sum_t g_t 3^(k-1-t): one thread
+// per (class, cell) pair, or, where those are fewer than the block's threads,
+// one warp per pair with the lanes along the words (an order-2 table has 18
+// pairs: one thread each walked its words alone).
 __device__ inline void count_cells(const DevData &d, int k, const int32_t *comb, uint32_t *out)
 {
     int cells = 1;
     for (int t = 0; t < k; t++) cells *= 3;
-    for (int idx = threadIdx.x; idx < 2 * cells; idx += blockDim.x) {
+    const bool by_warp = 2 * cells < (int)blockDim.x;
+    const int lane = by_warp ? threadIdx.x & 31 : 0, width = by_warp ? 32 : 1;
+    for (int idx = by_warp ? threadIdx.x >> 5 : threadIdx.x; idx < 2 * cells; idx += blockDim.x / width) {
         const int half = idx / cells;
         const int x = idx - half * cells;
         const uint32_t *rows[EPI_MAX_ORDER];
@@ -86,12 +86,40 @@ __device__ inline void count_cells(const DevData &d, int k, const int32_t *comb,
         }
         const int wb = half ? d.W1 : 0, we = half ? d.Wt : d.W1;
         uint32_t c = 0;
-        for (int w = wb; w < we; w++) {
+        for (int w = wb + lane; w < we; w += width) {
             uint32_t v = rows[0][w];
             for (int t = 1; t < k; t++) v &= rows[t][w];
             c += __popc(v);
         }
-        out[half * cells + x] = c;
+        if (by_warp) c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0) out[half * cells + x] = c;
+    }
+}
+
+// unrank_lex by one warp: each element's search probes 32 places at a time
+// (the binomials come from L2: a binary search waits for log2 n of them).
+__device__ inline void unrank_lex_warp(const uint64_t *tab, int64_t n, int k, uint64_t r, int32_t *out)
+{
+    const int lane = threadIdx.x & 31;
+    int64_t start = 0;
+    for (int t = 0; t < k; t++) {
+        const int rem = k - t;
+        const uint64_t total = binom_at(tab, n, n - start, rem);
+        const uint64_t x = total - r;
+        // smallest c in [start, n - rem] with C(n - 1 - c, rem) < x (true at n - rem)
+        int64_t lo = start, hi = n - rem;
+        while (lo < hi) {
+            const int64_t step = (hi - lo + 31) / 32;
+            const int64_t c = lo + lane * step < hi ? lo + lane * step : hi;
+            const uint32_t ok = __ballot_sync(0xffffffffu, binom_at(tab, n, n - 1 - c, rem) < x);
+            const int f = ok ? __ffs(ok) - 1 : 32;   // first probe that holds
+            const int64_t at = lo + f * step;
+            if (f > 0) lo += (f - 1) * step + 1;
+            hi = f < 32 && at < hi ? at : hi;
+        }
+        r -= total - binom_at(tab, n, n - lo, rem);
+        if (lane == 0) out[t] = (int32_t)lo;
+        start = lo + 1;
     }
 }
 
@@ -134,9 +162,10 @@ __global__ void __launch_bounds__(kRescoreThreads) rescore_kernel(DevData d, int
     if (c >= *cand_n) return;
     int cells = 1;
     for (int t = 0; t < k; t++) cells *= 3;
-    if (threadIdx.x == 0) {
-        unrank_lex(d.binom, d.n, k, cand_rank[c], comb);
-        for (int t = 0; t < k; t++) combs[(int64_t)c * k + t] = comb[t];
+    if (threadIdx.x < 32) {
+        unrank_lex_warp(d.binom, d.n, k, cand_rank[c], comb);
+        __syncwarp();
+        if (threadIdx.x < k) combs[(int64_t)c * k + threadIdx.x] = comb[threadIdx.x];
     }
     __syncthreads();
     uint32_t *ct = counts + (int64_t)c * 2 * cells;
@@ -296,18 +325,32 @@ cudaError_t launch_unrank(const DevData &d, int k, const uint64_t *ranks, int64_
     return cudaGetLastError();
 }
 
-size_t merge_smem_bytes(int cand_p2) { return (size_t)cand_p2 * 12; }
 size_t finalize_smem_bytes(int pool) { return (size_t)next_pow2(pool < 2 ? 2 : pool) * 20; }
 
-cudaError_t launch_merge(const float *ls, const uint64_t *lr, const int32_t *lc, int nlists, int stride, int pool,
-                         float *out_s, uint64_t *out_r, int32_t *out_n, cudaStream_t st, float floor)
+cudaError_t launch_merge(float *ls, uint64_t *lr, int32_t *lc, int nlists, int stride, int pool, float *out_s,
+                         uint64_t *out_r, int32_t *out_n, cudaStream_t st, float floor)
 {
-    const int cand_p2 = next_pow2(pool + 2 * 1024);
-    const size_t smem = merge_smem_bytes(cand_p2);
-    cudaError_t e = cudaFuncSetAttribute(merge_lists_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    merge_lists_kernel<<<1, 1024, smem, st>>>(ls, lr, lc, nlists, stride, pool, cand_p2, out_s, out_r, out_n, floor);
-    return cudaGetLastError();
+    // entries one block sorts: 4096 (48 KB), or twice the longest list
+    int cap = stride;
+    int64_t pitch = stride;
+    int lstep = 1;
+    for (int n = nlists;;) {
+        const int room = 2 * cap > 4096 ? 2 * cap : 4096;
+        const int group = n < room / cap ? n : room / cap;
+        const int blocks = (n + group - 1) / group;
+        const size_t smem = (size_t)merge_entries(group, cap) * 12;
+        cudaError_t e = cudaFuncSetAttribute(merge_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        const bool last = blocks == 1;
+        merge_level_kernel<<<blocks, 1024, smem, st>>>(ls, lr, lc, n, pitch, lstep, group, cap, pool,
+                                                       last ? out_s : nullptr, out_r, out_n, floor);
+        e = cudaGetLastError();
+        if (e != cudaSuccess || last) return e;
+        n = blocks;
+        pitch *= group;
+        lstep *= group;
+        cap = pool;
+    }
 }
 
 cudaError_t launch_rescore(const DevData &d, int k, int pool, const uint64_t *cand_r, const int32_t *cand_n,

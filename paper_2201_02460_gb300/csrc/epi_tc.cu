@@ -117,7 +117,6 @@ struct Roles {
 #ifndef EPI_TC_PREFETCH
 #define EPI_TC_PREFETCH 3
 #endif
-constexpr int kSegments = 16;
 constexpr int kDescDepth = 4;
 constexpr int kWaitSlots = 8;
 constexpr int kMaxDescSnps = 40;
@@ -142,6 +141,8 @@ struct DsParams {
     int32_t s1_lo, s1_hi;      // first SNPs of ranks rank_begin and rank_end - 1
     int32_t clip;              // 0: the whole combination range
     int32_t comb_p;            // combined-class variant: control counts in the low comb_p bits
+    int top_n;                 // records wanted (0: the pool alone sets the threshold)
+    float thr_mul;             // 1 - 4 f32_rel_bound: from a top_n-th best score to a safe threshold
     int chunks, chunks_case;   // 128-individual chunks in total / over the cases
     // screen (see Screen below): MI bound = v vscale + voff; a combination
     // passes when that reaches thr cut_mul - cut_add
@@ -334,7 +335,25 @@ __device__ __forceinline__ uint64_t subsets_from(const DevData &d, int64_t c, in
     return c - x >= m ? binom_at(d.binom, d.n, c - x, m) : 0;
 }
 
-// Lexicographic unranking of r among the m-subsets of [0, c) (m <= 3).
+// Largest x in [lo, hi] for which pred holds (true up to there, pred(lo)
+// taken as true), by the whole warp: 32 probes at a time, since each probe
+// waits for a load from L2.
+template <class F>
+__device__ __forceinline__ int64_t warp_last(int64_t lo, int64_t hi, F pred)
+{
+    const int lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t c = min(lo + (lane + 1) * step, hi);
+        const int n = __popc(__ballot_sync(0xffffffffu, pred(c)));   // the first n probes hold
+        hi = n < 32 ? min(lo + (n + 1) * step - 1, hi) : hi;
+        lo = min(lo + n * step, hi);
+    }
+    return lo;
+}
+
+// Lexicographic unranking of r among the m-subsets of [0, c) (m <= 3), by the
+// whole warp.
 __device__ inline void lex_unrank_below(const DevData &d, int64_t c, int m, uint64_t r, int32_t *out)
 {
     int64_t start = 0;
@@ -343,12 +362,9 @@ __device__ inline void lex_unrank_below(const DevData &d, int64_t c, int m, uint
         const uint64_t all = binom_at(d.binom, d.n, c - start, rem);
         // largest x in [start, c - rem] with fewer than r + 1 subsets whose
         // element i is below x
-        int64_t lo = start, hi = c - rem;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) >> 1;
-            if (all - binom_at(d.binom, d.n, c - mid, rem) <= r) lo = mid;
-            else hi = mid - 1;
-        }
+        const int64_t lo = warp_last(start, c - rem, [&](int64_t x) {
+            return all - binom_at(d.binom, d.n, c - x, rem) <= r;
+        });
         r -= all - binom_at(d.binom, d.n, c - lo, rem);
         out[i] = (int32_t)lo;
         start = lo + 1;
@@ -359,12 +375,7 @@ __device__ inline void prefix_unrank(const DsParams &P, int k, uint64_t q, Prefi
 {
     const DevData &d = P.d;
     // panel: largest c with pcum[c] <= q (a non-empty panel)
-    int64_t lo = 0, hi = d.n - 2;
-    while (lo < hi) {
-        const int64_t mid = (lo + hi + 1) >> 1;
-        if (P.pcum[mid] <= q) lo = mid;
-        else hi = mid - 1;
-    }
+    const int64_t lo = warp_last(0, d.n - 2, [&](int64_t x) { return P.pcum[x] <= q; });
     it.c = (int32_t)lo;
     it.q = q;
     const int m2 = k - 2;
@@ -533,7 +544,7 @@ struct EpiState {
 };
 
 template <int NT>
-__device__ inline void epi_flush(EpiState &S, float *sc, uint64_t *rk, int pool, uint32_t *global_thr, int tid)
+__device__ inline void epi_flush(EpiState &S, float *sc, uint64_t *rk, int pool, const DsParams &DS, int tid)
 {
     epi_bar<NT>();
     const int live = S.list_len + S.nbuf;
@@ -544,9 +555,14 @@ __device__ inline void epi_flush(EpiState &S, float *sc, uint64_t *rk, int pool,
     if (tid == 0) {
         S.list_len = live < pool ? live : pool;
         S.nbuf = 0;
-        if (S.list_len == pool) {
-            S.thr = sc[pool - 1];
-            atomicMax(global_thr, __float_as_uint(S.thr));
+        // at least top_n combinations score >= the top_n-th best: lowered by
+        // four times the score's error bound it is safe for the top N and
+        // still clears the final margin check
+        float t = S.list_len == pool ? sc[pool - 1] : -1.0f;
+        if (DS.top_n > 0 && live >= DS.top_n) t = fmaxf(t, sc[DS.top_n - 1] * DS.thr_mul);
+        if (t > S.thr) {
+            S.thr = t;
+            atomicMax(DS.global_thr, __float_as_uint(t));
         }
     }
     epi_bar<NT>();
@@ -764,13 +780,15 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
 
     const uint64_t cb = blockIdx.x - (uint64_t)DS.cta_begin, cn_ = (uint64_t)DS.cta_count;
     // Items get cheaper along the panels (fewer last SNPs), so a CTA takes
-    // kSegments ranges spread over all of them: segment q of the dataset's
-    // kSegments cn goes to CTA q % cn.
+    // several ranges spread over all of them (up to 16, of 8 items or more,
+    // since finding a range's first item takes microseconds): segment q of
+    // the dataset's segments x cn goes to CTA q % cn.
+    const int segments = (int)max((uint64_t)1, min((uint64_t)16, DS.n_items / (cn_ * 8)));
     auto segment_at = [&](uint64_t q) -> uint64_t {
-        return (uint64_t)(((unsigned __int128)DS.n_items * q) / (cn_ * kSegments));
+        return (uint64_t)(((unsigned __int128)DS.n_items * q) / (cn_ * segments));
     };
     int64_t n_my = 0;
-    for (int t = 0; t < kSegments; t++) n_my += (int64_t)(segment_at(cb + cn_ * t + 1) - segment_at(cb + cn_ * t));
+    for (int t = 0; t < segments; t++) n_my += (int64_t)(segment_at(cb + cn_ * t + 1) - segment_at(cb + cn_ * t));
     const int chunks = DS.chunks, chunks_case = DS.chunks_case;
     const int nst = (chunks + 1) >> 1;                // K stages of an item
 
@@ -821,7 +839,9 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
 
     if (warp == kWarpTma) {
         // ------------------------------------------------ TMA + descriptors
-        if (lane == 0 && n_my > 0) {
+        // the whole warp runs the loop (its searches probe with all lanes),
+        // lane 0 writes, arrives and issues the copies
+        if (n_my > 0) {
             // the segment's next item: M tile (prefix iterator) and N tile u
             PrefixIter it;
             int64_t u = 0;
@@ -834,12 +854,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     w0 = segment_at(cb + cn_ * seg);
                     seg_left = segment_at(cb + cn_ * seg + 1) - w0;
                 } while (seg_left == 0);
-                int64_t lo = 0, hi = d.n - 1;
-                while (lo < hi) {
-                    const int64_t mid = (lo + hi + 1) >> 1;
-                    if (DS.item_cum[mid] <= w0) lo = mid;
-                    else hi = mid - 1;
-                }
+                const int64_t lo = warp_last(0, d.n - 1, [&](int64_t x) { return DS.item_cum[x] <= w0; });
                 const int32_t c0 = (int32_t)lo;
                 const uint64_t off = w0 - DS.item_cum[c0];
                 const int64_t nt0 = panel_ntiles(d.n, c0, kJ);
@@ -870,27 +885,31 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             int s = 0;
             uint32_t ph = 0;
             long long w_tma = 0;
-            for (int64_t i = 0; i < n_my && !abort_flag; i++) {
+            for (int64_t i = 0; i < n_my; i++) {
                 const int dq = (int)(i % kDescDepth);
                 const uint32_t ud = (uint32_t)(i / kDescDepth);
-                if (!mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag)) break;
-                Desc &D = desc[dq];
-                D.j0 = (int32_t)panel_j0(cmin) + (int32_t)(u * kJ);
-                D.nvalid = nvalid;
+                if (!__all_sync(0xffffffffu, mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag))) break;
+                const int32_t tile_j0 = (int32_t)panel_j0(cmin) + (int32_t)(u * kJ);
+                if (lane == 0) {
+                    Desc &D = desc[dq];
+                    D.j0 = tile_j0;
+                    D.nvalid = nvalid;
 #pragma unroll
-                for (int q = 0; q < kPPT * km1; q++) D.snp[q] = tile_snp[q];
-                {
+                    for (int q = 0; q < kPPT * km1; q++) D.snp[q] = tile_snp[q];
                     // columns in use: 2 per last SNP below n, in steps of 16
-                    const int32_t live = 2 * ((int32_t)d.n - D.j0);
+                    const int32_t live = 2 * ((int32_t)d.n - tile_j0);
                     const uint32_t ncol = live >= S::N ? (uint32_t)S::N : (uint32_t)((live + 15) & ~15);
                     item_idesc[dq] = make_idesc(ncol);
+                    mbar_arrive(&desc_full[dq]);
                 }
-                mbar_arrive(&desc_full[dq]);
-                const int y = 2 * D.j0;
+                const int y = 2 * tile_j0;
                 for (int kc = 0; kc < nst; kc++, g++) {
-                    if (!wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_tma)) break;
-                    mbar_arrive_tx(&full_ab[s], (uint32_t)kBBytes);
-                    tma_load_2d(stages_b + s * kBBytes, tmap, kc * kRowBytes, y, &full_ab[s]);
+                    if (!__all_sync(0xffffffffu, wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_tma))) break;
+                    if (lane == 0) {
+                        mbar_arrive_tx(&full_ab[s], (uint32_t)kBBytes);
+                        tma_load_2d(stages_b + s * kBBytes, tmap, kc * kRowBytes, y, &full_ab[s]);
+                    }
+                    __syncwarp();
                     if (++s == kStages) { s = 0; ph ^= 1; }
                 }
                 u++;
@@ -904,7 +923,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     fill_tile();
                 }
             }
-            if (P.waits) P.waits[blockIdx.x * kWaitSlots + 6] = (unsigned long long)w_tma;
+            if (P.waits && lane == 0) P.waits[blockIdx.x * kWaitSlots + 6] = (unsigned long long)w_tma;
             for (int q = 0; q < kStages; q++) {
                 if (g > (uint64_t)q) {
                     const uint64_t last = ((g - 1 - q) / kStages) * kStages + q;
@@ -1218,14 +1237,14 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             if (lane == 0) mbar_arrive(&tot_empty[b]);
             // the other CTAs' threshold, for the next item (loaded early)
             const float gthr = tid == 0 ? __uint_as_float(*(volatile uint32_t *)DS.global_thr) : 0.0f;
-            const float cut = thr < 0.0f ? -1.0f : thr * DS.cut_mul - DS.cut_add;
-            const int list_len = ES.list_len;
+            float cut = thr * DS.cut_mul - DS.cut_add;
+            int list_len = ES.list_len;
             const int32_t j0 = D.j0;
             // before the item's closing barrier: the threshold the other CTAs
             // have reached, and whether a role gave up
             auto refresh = [&]() {
                 if (tid == 0) {
-                    if (ES.list_len == P.pool || gthr > 0.0f) ES.next_thr = fmaxf(ES.thr, gthr);
+                    ES.next_thr = gthr > 0.0f ? fmaxf(ES.thr, gthr) : ES.thr;
                     ES.stop = abort_flag;
                 }
             };
@@ -1274,13 +1293,22 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 return row_terms_precise(f2u_exact(a[0]), f2u_exact(bb[0]), f2u_exact(a[1]), f2u_exact(bb[1]),
                                          f2u_exact(a[2]), f2u_exact(bb[2]), mc);
             };
-            auto keep = [&](float score, int32_t j) {
+            // combination of tile prefix pt and last SNP j into the buffer
+            auto keep = [&](float score, int pt, int32_t j) {
                 if (score >= thr) {
+                    int32_t qs[km1];
+#pragma unroll
+                    for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
                     const int slot = list_len + atomicAdd(&ES.nbuf, 1);
                     sc[slot] = score;
-                    rk[slot] = DS.total - 1 - prefix_rank_sum<km1>(d, psnp) - (uint64_t)(d.n - 1 - j);
+                    rk[slot] = DS.total - 1 - prefix_rank_sum<km1>(d, qs) - (uint64_t)(d.n - 1 - j);
                 }
             };
+            // Without a threshold every combination needs its precise score:
+            // all prefixes of the warp at once, column by column (one flagged
+            // pair at a time, as below, the first items of a CTA took
+            // milliseconds at order 2), summed as the flagged ones are.
+            bool cold = thr < 0.0f;
             // 8 row values per lane -> transposed sums: the lane of pair
             // (prefix pp, last SNP jj) adds rows pp kPR .. of column jj (all
             // banks distinct); at orders 4-5 four lanes share a column
@@ -1317,22 +1345,39 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         uint32_t cs[16], cn[C ? 1 : 16];
                         load_chunk(jcg, cs, cn);
                         tmem_wait_ld();
-                        float vrow[8];
-                        if (poly) rs.bound(cs, cn, vrow);
-                        else rs.logs(cs, cn, vrow);
                         if (P.dump) dump_chunk(jb, cs, cn);
-                        store_rows(vrow);
-                        v = column_sum();
-                        __syncwarp();
+                        if (cold) {
+#pragma unroll 1
+                            for (int jj = 0; jj < 8; jj++) {
+                                const float e = warp_sum(prow ? row_precise(cs, cn, jj) : 0.0f);
+                                if (lane == jj) v = e;
+                            }
+                        } else {
+                            float vrow[8];
+                            if (poly) rs.bound(cs, cn, vrow);
+                            else rs.logs(cs, cn, vrow);
+                            store_rows(vrow);
+                            v = column_sum();
+                            __syncwarp();
+                        }
                     }
                     if (lane < 8) wred[quad][8 * jcg + lane] = v;
                 }
                 epi_bar<kEpiThreads>();
                 bool any = false;
+                // the tile's one prefix is every thread's
+                int32_t qs[km1], plo_any = 1, phi_any = 0;
+#pragma unroll
+                for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[tt];
+                if (ok) last_snp_range<km1>(DS, d, qs, plo_any, phi_any);
                 for (int q = tid; q < kJ; q += kEpiThreads) {
                     const float tv = wred[0][q] + wred[1][q] + wred[2][q];
                     const int32_t j = j0 + q;
-                    const bool f = phi[0] > 0 && j >= plo[0] && j < phi[0] && fmaf(tv, vscale, voff) >= cut;
+                    bool f = false;
+                    if (j >= plo_any && j < phi_any) {
+                        if (cold) keep(__fdiv_rn(tv, mc.fm), 0, j);
+                        else f = fmaf(tv, vscale, voff) >= cut;
+                    }
                     wflag[q] = f ? 1 : 0;
                     any |= f;
                 }
@@ -1359,10 +1404,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     epi_bar<kEpiThreads>();
                     for (int q = tid; q < kJ; q += kEpiThreads) {
                         if (!wflag[q]) continue;
-                        // every thread of the tile's one prefix knows its SNPs
-#pragma unroll
-                        for (int tt = 0; tt < km1; tt++) psnp[tt] = D.snp[tt];
-                        keep(__fdiv_rn(wpre[0][q] + wpre[1][q] + wpre[2][q], mc.fm), j0 + q);
+                        keep(__fdiv_rn(wpre[0][q] + wpre[1][q] + wpre[2][q], mc.fm), 0, j0 + q);
                     }
                 }
                 refresh();
@@ -1376,8 +1418,25 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 uint32_t nx[16], ny[C ? 1 : 16];
                 if (mine > 0) load_chunk(jhalf, nx, ny);
                 else release_acc();
+                // while there is no threshold the warps go chunk by chunk
+                // together, until enough combinations are scored to set one
+                // (kIters rounds for every warp, whatever its item or state: the
+                // rounds meet at barriers)
+                const int rounds = cold ? kIters : mine;
 #pragma unroll 1
-                for (int jc = 0; jc < mine; jc++) {
+                for (int jc = 0; jc < rounds; jc++) {
+                    if (cold && jc > 0) {
+                        epi_bar<kEpiThreads>();
+                        if (ES.nbuf > 0 && ES.list_len + ES.nbuf >= (DS.top_n > 0 ? DS.top_n : P.pool)) {
+                            epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
+                            thr = ES.thr;
+                            cut = thr * DS.cut_mul - DS.cut_add;
+                            list_len = ES.list_len;
+                            cold = thr < 0.0f;
+                        }
+                        epi_bar<kEpiThreads>();
+                    }
+                    if (jc >= mine) continue;
                     const int jcg = jhalf + kCG * jc;
                     const int32_t jb = j0 + 8 * jcg;
                     uint32_t cs[16], cn[C ? 1 : 16];
@@ -1392,10 +1451,20 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     // goes back to the MMA issuer
                     if (jc + 1 < mine) load_chunk(jcg + kCG, nx, ny);
                     else release_acc();
+                    if (P.dump) dump_chunk(jb, cs, cn);
+                    if (cold) {
+                        int32_t jlo = 1, jhi = 0;
+                        if (prow && pos == 0) last_snp_range<km1>(DS, d, psnp, jlo, jhi);
+#pragma unroll 1
+                        for (int jj = 0; jj < 8; jj++) {
+                            const float e = seg_sum<kPR>(prow ? row_precise(cs, cn, jj) : 0.0f, pos);
+                            if (jb + jj >= jlo && jb + jj < jhi) keep(__fdiv_rn(e, mc.fm), p, jb + jj);
+                        }
+                        continue;
+                    }
                     float vrow[8];
                     if (poly) rs.bound(cs, cn, vrow);
                     else rs.logs(cs, cn, vrow);
-                    if (P.dump) dump_chunk(jb, cs, cn);
                     store_rows(vrow);
                     uint32_t cmask[kPairIters];
                     if constexpr (kPPW > 1) {
@@ -1436,7 +1505,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                             float e = 0.0f;
                             if (lane_real && pl == pp) e = row_precise(cs, cn, jsel);
                             e = seg_sum<kPR>(e, pos);
-                            if (lane_real && pl == pp && pos == 0) keep(__fdiv_rn(e, mc.fm), jb + jsel);
+                            if (lane_real && pl == pp && pos == 0) keep(__fdiv_rn(e, mc.fm), p, jb + jsel);
                         }
                     }
                 }
@@ -1448,14 +1517,18 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             thr = ES.next_thr;
             // the next item adds at most one candidate per last SNP and
             // prefix: sort and trim first if the buffer could not hold them
-            if (ES.list_len + ES.nbuf + kJ * kPPT > P.cand_p2)
-                epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS.global_thr, tid);
+            // (and when a pool's worth is waiting: a better threshold keeps
+            // later ones out)
+            const int nbuf = ES.nbuf;
+            if (ES.list_len + nbuf + kJ * kPPT > P.cand_p2 || nbuf >= P.pool ||
+                (thr < 0.0f && DS.top_n > 0 && ES.list_len + nbuf >= DS.top_n))
+                epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
             // no candidate of the next item before every warp has read nbuf
             epi_bar<kEpiThreads>();
             thr = fmaxf(thr, ES.thr);
         }
         epi_bar<kEpiThreads>();
-        if (ES.nbuf > 0) epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS.global_thr, tid);
+        if (ES.nbuf > 0) epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
         const int L = ES.list_len;
         for (int q = tid; q < L; q += kEpiThreads) {
             P.list_score[(size_t)blockIdx.x * P.pool + q] = sc[q];
@@ -1762,11 +1835,13 @@ static void fill_screen(tc::DsParams &D, const DevData &d, int k, int comb_p)
 // the launch is batched (nullptr: passed as a kernel parameter instead).
 static void fill_ds(tc::DsParams &D, const DevData &d, int k, uint64_t *item_cum, uint32_t *global_thr,
                     uint64_t total, uint64_t rb, uint64_t re, const CUtensorMap *tmap_dev, int cta_begin,
-                    int cta_count, int comb_p, const unsigned char *b4)
+                    int cta_count, int comb_p, const unsigned char *b4, int top_n)
 {
     D.d = d;
     D.rows = reinterpret_cast<const uint4 *>(b4 + tc_b_bytes(d));
     D.comb_p = comb_p;
+    D.top_n = top_n;
+    D.thr_mul = (float)(1.0 - 4.0 * f32_rel_bound(k, d.m));
     D.rank_begin = rb;
     D.rank_end = re;
     D.s1_lo = (int32_t)tc_first_snp(d.n, k, rb);
@@ -1838,10 +1913,10 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
                              uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                              int32_t *status, int grid, uint64_t total, uint64_t rb, uint64_t re, cudaStream_t st,
                              int *cand_p2_out, float *cand_g, uint64_t *rank_g, uint32_t *dump,
-                             unsigned long long *waits, unsigned long long wait_ns, int comb_p)
+                             unsigned long long *waits, unsigned long long wait_ns, int comb_p, int top_n)
 {
     tc::Params P;
-    fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p, b4);
+    fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p, b4, top_n);
     P.many = nullptr;
     P.cta_ds = nullptr;
     fill_launch(P, k, pool, list_score, list_rank, list_count, status, dump, waits, cand_g, rank_g, comb_p != 0);
@@ -1859,10 +1934,10 @@ size_t tc_ds_bytes() { return sizeof(tc::DsParams); }
 
 cudaError_t tc_fill_batch_entry(void *ds_host, void *tmap_host, const DevData &d, int k, const unsigned char *b4,
                                 uint64_t *item_cum, uint32_t *global_thr, uint64_t total, const void *tmap_dev,
-                                int cta_begin, int cta_count, int comb_p)
+                                int cta_begin, int cta_count, int comb_p, int top_n)
 {
     fill_ds(*static_cast<tc::DsParams *>(ds_host), d, k, item_cum, global_thr, total, 0, total,
-            static_cast<const CUtensorMap *>(tmap_dev), cta_begin, cta_count, comb_p, b4);
+            static_cast<const CUtensorMap *>(tmap_dev), cta_begin, cta_count, comb_p, b4, top_n);
     return encode_map(static_cast<CUtensorMap *>(tmap_host), d, b4, comb_p != 0);
 }
 
