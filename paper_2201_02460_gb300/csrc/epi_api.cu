@@ -320,11 +320,10 @@ epi_status choose_path(const epi_dataset *ds, int k, int path, uint64_t rb, uint
         // it is taken for a rank range only when that adds at most as much
         // work again as the range itself
         tc = ok && (re - rb == total || tc_range_work(ds->n, k, rb, re) <= 2 * (re - rb));
-        // order 2: the popcount kernel starts faster, the tensor path counts
-        // faster; they meet near 2e8 combination words (1000 x 8192: 0.66 ms
-        // popcount, 0.54 tensor; 2000 x 2500: 0.61 and 0.72; 4000 x 2500:
-        // 1.48 and 0.90; 8000 x 8192: 22.1 and 1.5)
-        if (k == 2 && (double)(re - rb) * (double)ds->Wt < 2e8) tc = false;
+        // order 2 on few SNPs: the popcount kernel starts a little faster
+        // (60 SNPs: 125-132 us popcount, 129-147 tensor; 200 SNPs: 163-236
+        // and 126-161; 2000 x 2500: 493 and 158; 8000 x 8192: 22.0 and 1.1 ms)
+        if (k == 2 && ds->n < 100) tc = false;
         auto it = ds->ctx->tune.find(tune_key(k, ds->n, ds->Wt));
         if (ok && it != ds->ctx->tune.end() && it->second.path) tc = it->second.path == EPI_PATH_TC;
     }
@@ -380,6 +379,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     const size_t o_thr = a.take<uint32_t>(1);
     const size_t o_status = a.take<int32_t>(1);
     const size_t o_nout = a.take<int32_t>(1);
+    const size_t o_hist = p.tc ? a.take<uint32_t>(kTcHistBins) : 0;
     const size_t rec_bytes = ((size_t)p.top_n * sizeof(epi_result) + 255) & ~(size_t)255;
     const size_t res_bytes = rec_bytes + (own && own->counts ? (size_t)p.top_n * 2 * cells * 4 : 0);
     const size_t o_res = own ? a.take<char>(res_bytes) : 0;
@@ -431,7 +431,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
         n_out_dev = reinterpret_cast<int32_t *>(base + o_nout);
     }
     static_assert(kHeadStatus == 256 && kHeadCount == 512, "the arena's alignment");
-    CK(cudaMemsetAsync(base, 0, kHeadBytes, ctx->stream));
+    CK(cudaMemsetAsync(base, 0, p.tc ? o_hist + kTcHistBins * 4 : kHeadBytes, ctx->stream));
     const DevData d = ds->dev();
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (ctx->profiling) {
@@ -454,7 +454,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
                             p.total, p.rb, p.re, ctx->stream, &cand_p2,
                             tc_cg ? reinterpret_cast<float *>(base + o_tcs) : nullptr,
                             tc_cg ? reinterpret_cast<uint64_t *>(base + o_tcr) : nullptr, dump, waits,
-                            ctx->wait_limit_ns, p.comb_p, p.top_n));
+                            ctx->wait_limit_ns, p.comb_p, p.top_n, reinterpret_cast<uint32_t *>(base + o_hist)));
         ctx->launches += 1;   // item table
     } else {
         CK(launch_popc_search(d, p.k, p.R, p.rb, p.re, p.tile, p.pool, p.slots, p.cand_p2, thr, ls, lr, lc, p.grid,
@@ -463,7 +463,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
                               p.pair ? reinterpret_cast<uint32_t *>(base + o_sing) : nullptr, p.top_n));
     }
     if (ev1) CK(cudaEventRecord(ev1, ctx->stream));
-    CK(launch_merge(ls, lr, lc, p.grid, p.pool, p.pool, cs, cr, cn, ctx->stream));
+    CK(launch_merge(ls, lr, lc, p.grid, p.pool, p.pool, cs, cr, cn, ctx->stream, thr));
     CK(launch_rescore(d, p.k, p.pool, cr, cn, ct, mi, cb, ctx->stream));
     CK(launch_finalize(d, p.k, p.top_n, p.pool, cs, cr, cn, mi, cb, ct, thr, p.re - p.rb, out_dev, counts_dev,
                        n_out_dev, status, ctx->stream));
@@ -582,7 +582,7 @@ struct BatchItem {
     int group = -1, cta_begin = 0, cta_count = 0;
     // device offsets in the batch arena
     size_t o_thr = 0, o_status = 0, o_code = 0, o_nout = 0, o_cs = 0, o_cr = 0, o_cn = 0, o_ct = 0, o_mi = 0,
-           o_cb = 0, o_ic = 0, o_rec = 0, o_cnt = 0, o_ls = 0, o_lr = 0, o_lc = 0;
+           o_cb = 0, o_ic = 0, o_rec = 0, o_cnt = 0, o_ls = 0, o_lr = 0, o_lc = 0, o_hist = 0;
     // pinned host offsets of the copied-back results
     size_t h_rec = 0, h_cnt = 0, h_nout = 0, h_code = 0;
 };
@@ -682,12 +682,14 @@ epi_status ensure_batch_buffers(epi_ctx *ctx, size_t dev_bytes, size_t host_byte
 }
 
 // Records every step of the batched search on `st` (captured into a graph).
-epi_status record_batch(epi_ctx *ctx, std::vector<BatchItem> &items, std::vector<BatchGroup> &groups, cudaStream_t st)
+epi_status record_batch(epi_ctx *ctx, std::vector<BatchItem> &items, std::vector<BatchGroup> &groups,
+                        size_t zero_bytes, cudaStream_t st)
 {
     char *dev = static_cast<char *>(ctx->batch_dev);
     char *host = static_cast<char *>(ctx->batch_host);
-    // thresholds and status words of all datasets sit in one block at offset 0
-    CK(cudaMemsetAsync(dev, 0, items.size() * 256, st));
+    // thresholds, status words and histograms of all datasets sit in one
+    // block at offset 0
+    CK(cudaMemsetAsync(dev, 0, zero_bytes, st));
     for (auto &g : groups) {
         if (g.tc)
             for (int i : g.items)
@@ -726,7 +728,7 @@ epi_status record_batch(epi_ctx *ctx, std::vector<BatchItem> &items, std::vector
         uint32_t *cnt = reinterpret_cast<uint32_t *>(dev + it.o_cnt);
         int32_t *nout = reinterpret_cast<int32_t *>(dev + it.o_nout);
         int32_t *code = reinterpret_cast<int32_t *>(dev + it.o_code);
-        CK(launch_merge(ls, lr, lc, it.cta_count, g.pool, it.pool, cs, cr, cn, st));
+        CK(launch_merge(ls, lr, lc, it.cta_count, g.pool, it.pool, cs, cr, cn, st, thr));
         CK(launch_rescore(d, it.k, it.pool, cr, cn, ct, mi, cb, st));
         CK(launch_finalize(d, it.k, it.top_n, it.pool, cs, cr, cn, mi, cb, ct, thr, it.total, rec, cnt, nout, status,
                            st));
@@ -810,6 +812,10 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         it.o_code = base + 8;
         it.o_nout = base + 12;
     }
+    // score histograms next, zeroed with them
+    for (auto &it : items)
+        if (it.tc) it.o_hist = a.take<uint32_t>(kTcHistBins);
+    const size_t zero_bytes = a.off;
     for (auto &g : groups) {
         g.o_desc = a.take<char>((g.tc ? tc_ds_bytes() : popc_ds_bytes()) * g.items.size());
         g.o_tmap = a.take<char>((size_t)128 * g.items.size());
@@ -876,7 +882,8 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
                 if (g.tc) {
                     CK(tc_fill_batch_entry(hd + dsz * q, hm + 128 * q, d, it.k, it.ds->b4,
                                            reinterpret_cast<uint64_t *>(dev + it.o_ic), thr, it.total,
-                                           dev + g.o_tmap + 128 * q, it.cta_begin, it.cta_count, it.comb_p, it.top_n));
+                                           dev + g.o_tmap + 128 * q, it.cta_begin, it.cta_count, it.comb_p, it.top_n,
+                                           reinterpret_cast<uint32_t *>(dev + it.o_hist)));
                 } else {
                     popc_fill_ds(hd + dsz * q, d, 0, it.total, it.cta_begin, it.cta_count, thr);
                 }
@@ -890,7 +897,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         CK(cudaStreamSynchronize(ctx->stream));
         cudaGraph_t graph = nullptr;
         CK(cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
-        epi_status rs = record_batch(ctx, items, groups, ctx->capture_stream);
+        epi_status rs = record_batch(ctx, items, groups, zero_bytes, ctx->capture_stream);
         cudaError_t ec = cudaStreamEndCapture(ctx->capture_stream, &graph);
         if (rs != EPI_OK) { if (graph) cudaGraphDestroy(graph); return rs; }
         if (ec != cudaSuccess) return fail(EPI_ECUDA, "graph capture: %s", cudaGetErrorString(ec));

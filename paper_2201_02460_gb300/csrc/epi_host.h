@@ -86,7 +86,9 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
                              int32_t *status, int grid, uint64_t total, uint64_t rb, uint64_t re, cudaStream_t st,
                              int *cand_p2_out, float *cand_g, uint64_t *rank_g, uint32_t *dump = nullptr,
                              unsigned long long *waits = nullptr, unsigned long long wait_ns = 0, int comb_p = 0,
-                             int top_n = 0);
+                             int top_n = 0, uint32_t *hist = nullptr);
+// words of a search's score histogram (hist above: zeroed; NULL: none)
+constexpr int kTcHistBins = 2048;
 constexpr int kTcWaitSlots = 8;
 // batched tensor-core launches: per-dataset descriptors and B-operand maps
 // (128-byte CUtensorMap, 64-byte aligned) live in device memory
@@ -95,7 +97,7 @@ cudaError_t launch_tc_item_cum(const DevData &d, int k, uint64_t rb, uint64_t re
                                cudaStream_t st, bool comb);
 cudaError_t tc_fill_batch_entry(void *ds_host, void *tmap_host, const DevData &d, int k, const unsigned char *b4,
                                 uint64_t *item_cum, uint32_t *global_thr, uint64_t total, const void *tmap_dev,
-                                int cta_begin, int cta_count, int comb_p, int top_n);
+                                int cta_begin, int cta_count, int comb_p, int top_n, uint32_t *hist);
 cudaError_t launch_tc_batch(const void *ds_dev, const int32_t *cta_ds_dev, int k, int pool, float *list_score,
                             uint64_t *list_rank, int32_t *list_count, int32_t *status, int grid, cudaStream_t st,
                             float *cand_g, uint64_t *rank_g, bool comb);
@@ -152,9 +154,10 @@ cudaError_t launch_topk(const float *scores, const uint8_t *keep, int64_t count,
 
 // epi_select.cu
 // floor: below every score to merge (the search's scores are >= 0)
-// (the lists are overwritten; pool <= stride)
+// (the lists are overwritten; pool <= stride); thr: NULL, or the bits of a
+// threshold below which entries need not be kept
 cudaError_t launch_merge(float *ls, uint64_t *lr, int32_t *lc, int nlists, int stride, int pool, float *out_s,
-                         uint64_t *out_r, int32_t *out_n, cudaStream_t st, float floor = -1.0f);
+                         uint64_t *out_r, int32_t *out_n, cudaStream_t st, const uint32_t *thr, float floor = -1.0f);
 cudaError_t launch_rescore(const DevData &d, int k, int pool, const uint64_t *cand_r, const int32_t *cand_n,
                            uint32_t *counts, double *mi64, int32_t *combs, cudaStream_t st);
 cudaError_t launch_finalize(const DevData &d, int k, int top_n, int pool, const float *cand_s, const uint64_t *cand_r,

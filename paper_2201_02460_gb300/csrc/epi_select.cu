@@ -14,36 +14,53 @@
 
 namespace epi {
 
-// entries of a block's sort buffers (the sort works on at least two)
-__host__ __device__ inline int merge_entries(int group, int cap) { return next_pow2(group * cap < 2 ? 2 : group * cap); }
+// Shared memory of a merge block: its entries, and the pool's best of them.
+__host__ __device__ inline int merge_entries(int group, int cap, int pool)
+{
+    const int e = group * cap < 2 ? 2 : group * cap;
+    return next_pow2(e) + (pool < 2 ? 2 : pool);
+}
+
+// float bits in an order-preserving unsigned form
+__device__ __forceinline__ uint32_t order_bits(float f)
+{
+    const uint32_t u = __float_as_uint(f);
+    return u & 0x80000000u ? ~u : u | 0x80000000u;
+}
 
 // One level of the merge: block b takes lists [b group, (b + 1) group) -- list
-// i at ls + i pitch with lc[i lstep] entries -- sorts their entries together
-// and keeps the best `pool`: in place as list b group of the next level, or
-// in out_* when this is the last level (one block).  A single block walking
-// all lists in rounds of 1024 took 124 us for 155 lists of 128 (its sorts are
-// serial); two levels of blocks take 2 x 5 us.
+// i at ls + i pitch with lc[i lstep] entries -- and keeps the best `pool` of
+// their entries: in place as list b group of the next level, or sorted in
+// out_* when this is the last level (one block).  The cut is found by a radix
+// select over the scores (four 8-bit passes), and the last level sorts by
+// counting, for each entry kept, the better ones; entries below the search's
+// threshold are dropped on loading.  (One block that sorted 1024 entries at a
+// time took 124 us for 155 lists of 128, two levels of 4096-entry bitonic
+// sorts 2 x 45.)
 __global__ void __launch_bounds__(1024) merge_level_kernel(float *__restrict__ ls, uint64_t *__restrict__ lr,
                                                            int32_t *__restrict__ lc, int nlists, int64_t pitch,
                                                            int lstep, int group, int cap, int pool,
                                                            float *__restrict__ out_s, uint64_t *__restrict__ out_r,
-                                                           int32_t *__restrict__ out_n, float floor)
+                                                           int32_t *__restrict__ out_n,
+                                                           const uint32_t *__restrict__ thr, float floor)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int entries = merge_entries(group, cap);
+    const int entries = merge_entries(group, cap, pool);
     uint64_t *rk = reinterpret_cast<uint64_t *>(smem);
     float *sc = reinterpret_cast<float *>(rk + entries);
-    __shared__ int32_t live_sh;
+    __shared__ int32_t live_sh, kept_sh, need_sh;
+    __shared__ uint32_t hist[256], digit_sh;
     const int first = blockIdx.x * group;
     const int lists = min(group, nlists - first);
-    if (threadIdx.x == 0) live_sh = 0;
+    if (threadIdx.x == 0) { live_sh = 0; kept_sh = 0; need_sh = pool; }
     __syncthreads();
+    const float cut = thr ? fmaxf(floor, __uint_as_float(*thr)) : floor;
     for (int e = threadIdx.x; e < lists * cap; e += blockDim.x) {
         const int l = e / cap, i = e - l * cap;
         if (i < lc[(int64_t)(first + l) * lstep]) {
             const int64_t at = (int64_t)(first + l) * pitch + i;
             const float v = ls[at];
-            if (v >= floor) {
+            if (v >= cut) {
                 const int pos = atomicAdd(&live_sh, 1);
                 sc[pos] = v;
                 rk[pos] = lr[at];
@@ -52,15 +69,85 @@ __global__ void __launch_bounds__(1024) merge_level_kernel(float *__restrict__ l
     }
     __syncthreads();
     const int live = live_sh;
-    const int p2 = next_pow2(live < 2 ? 2 : live);
-    for (int i = live + threadIdx.x; i < p2; i += blockDim.x) { sc[i] = floor; rk[i] = ~0ull; }
-    __syncthreads();
-    block_sort_cands(sc, rk, p2);
-    const int L = live < pool ? live : pool;
-    float *os = out_s ? out_s : ls + (int64_t)first * pitch;
-    uint64_t *orr = out_s ? out_r : lr + (int64_t)first * pitch;
-    for (int i = threadIdx.x; i < L; i += blockDim.x) { os[i] = sc[i]; orr[i] = rk[i]; }
-    if (threadIdx.x == 0) *(out_s ? out_n : lc + (int64_t)first * lstep) = L;
+    float *ks = sc;                                  // the kept entries
+    uint64_t *kr = rk;
+    int L = live;
+    if (live > pool) {
+        // the pool-th largest score, digit by digit
+        uint32_t prefix = 0, mask = 0;
+        for (int shift = 24; shift >= 0; shift -= 8) {
+            if (threadIdx.x < 256) hist[threadIdx.x] = 0;
+            __syncthreads();
+            for (int i = threadIdx.x; i < live; i += blockDim.x) {
+                const uint32_t u = order_bits(sc[i]);
+                if ((u & mask) == prefix) atomicAdd(&hist[(u >> shift) & 255u], 1u);
+            }
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                // 8 bins a lane, from the top
+                const int lane = threadIdx.x, hi = 255 - 8 * lane;
+                int sum = 0;
+                for (int q = 0; q < 8; q++) sum += (int)hist[hi - q];
+                int inc = sum;
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int o = __shfl_up_sync(0xffffffffu, inc, off);
+                    if (lane >= off) inc += o;
+                }
+                const int need = need_sh;
+                __syncwarp();
+                int before = inc - sum;
+                if (before < need && inc >= need) {
+                    int q = 0;
+                    while (before + (int)hist[hi - q] < need) before += (int)hist[hi - q++];
+                    digit_sh = (uint32_t)(hi - q);
+                    need_sh = need - before;
+                }
+            }
+            __syncthreads();
+            prefix |= digit_sh << shift;
+            mask |= 255u << shift;
+            __syncthreads();
+        }
+        // every entry above the cut, and of those at it the need_sh best by
+        // rank (usually all of them)
+        ks = sc + entries - pool;
+        kr = rk + entries - pool;
+        const int need = need_sh;
+        for (int i = threadIdx.x; i < live; i += blockDim.x) {
+            const uint32_t u = order_bits(sc[i]);
+            bool keep = u > prefix;
+            if (u == prefix) {
+                int better = 0;
+                const uint64_t r = rk[i];
+                for (int q = 0; q < live; q++) better += order_bits(sc[q]) == prefix && rk[q] < r;
+                keep = better < need;
+            }
+            if (keep) {
+                const int pos = atomicAdd(&kept_sh, 1);
+                ks[pos] = sc[i];
+                kr[pos] = rk[i];
+            }
+        }
+        __syncthreads();
+        L = pool;
+    }
+    if (out_s) {
+        for (int i = threadIdx.x; i < L; i += blockDim.x) {
+            const float v = ks[i];
+            const uint64_t r = kr[i];
+            int pos = 0;
+            for (int q = 0; q < L; q++) pos += cand_better(ks[q], kr[q], v, r);
+            out_s[pos] = v;
+            out_r[pos] = r;
+        }
+        if (threadIdx.x == 0) *out_n = L;
+    } else {
+        for (int i = threadIdx.x; i < L; i += blockDim.x) {
+            ls[(int64_t)first * pitch + i] = ks[i];
+            lr[(int64_t)first * pitch + i] = kr[i];
+        }
+        if (threadIdx.x == 0) lc[(int64_t)first * lstep] = L;
+    }
 }
 
 // Exact counts of one combination, cell x = sum_t g_t 3^(k-1-t): one thread
@@ -328,9 +415,9 @@ cudaError_t launch_unrank(const DevData &d, int k, const uint64_t *ranks, int64_
 size_t finalize_smem_bytes(int pool) { return (size_t)next_pow2(pool < 2 ? 2 : pool) * 20; }
 
 cudaError_t launch_merge(float *ls, uint64_t *lr, int32_t *lc, int nlists, int stride, int pool, float *out_s,
-                         uint64_t *out_r, int32_t *out_n, cudaStream_t st, float floor)
+                         uint64_t *out_r, int32_t *out_n, cudaStream_t st, const uint32_t *thr, float floor)
 {
-    // entries one block sorts: 4096 (48 KB), or twice the longest list
+    // entries one block takes: 4096, or twice the longest list
     int cap = stride;
     int64_t pitch = stride;
     int lstep = 1;
@@ -338,12 +425,12 @@ cudaError_t launch_merge(float *ls, uint64_t *lr, int32_t *lc, int nlists, int s
         const int room = 2 * cap > 4096 ? 2 * cap : 4096;
         const int group = n < room / cap ? n : room / cap;
         const int blocks = (n + group - 1) / group;
-        const size_t smem = (size_t)merge_entries(group, cap) * 12;
+        const size_t smem = (size_t)merge_entries(group, cap, pool) * 12;
         cudaError_t e = cudaFuncSetAttribute(merge_level_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         const bool last = blocks == 1;
         merge_level_kernel<<<blocks, 1024, smem, st>>>(ls, lr, lc, n, pitch, lstep, group, cap, pool,
-                                                       last ? out_s : nullptr, out_r, out_n, floor);
+                                                       last ? out_s : nullptr, out_r, out_n, thr, floor);
         e = cudaGetLastError();
         if (e != cudaSuccess || last) return e;
         n = blocks;

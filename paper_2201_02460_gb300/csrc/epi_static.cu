@@ -228,7 +228,7 @@ extern "C" epi_status epi_search_static(const uint8_t *geno_dev, const uint8_t *
     e = cudaGetLastError();
     if (e == cudaSuccess)
         e = launch_popc_search(d, k, R, 0, total, tile, pool, slots, cand_p2, thr, ls, lr, lc, grid, smem, st);
-    if (e == cudaSuccess) e = launch_merge(ls, lr, lc, grid, pool, pool, cs, cr, cn, st);
+    if (e == cudaSuccess) e = launch_merge(ls, lr, lc, grid, pool, pool, cs, cr, cn, st, thr);
     if (e == cudaSuccess) e = launch_rescore(d, k, pool, cr, cn, ct, mi, cb, st);
     if (e == cudaSuccess)
         e = launch_finalize(d, k, top_n, pool, cs, cr, cn, mi, cb, ct, thr, total, out_dev, counts_dev, n_out_dev,

@@ -151,6 +151,7 @@ struct DsParams {
     float sc_pi, c2, c3, c4, c5a, c5b;
     uint64_t total;            // C(n, k)
     uint32_t *global_thr;
+    uint32_t *hist;            // [kTcHistBins] scores of the combinations kept so far, by value
     const CUtensorMap *tmap;   // B-operand map in global memory (batched launches)
     int32_t cta_begin, cta_count;
 };
@@ -541,7 +542,61 @@ struct EpiState {
     int32_t list_len, nbuf, stop, any;
     float thr;                 // the CTA's own pool threshold
     float next_thr;            // the larger of it and the other CTAs'
+    int32_t seen;              // kept combinations at the last look at the histogram
 };
+
+// Histogram of the precise scores of every combination any CTA has kept (each
+// is kept once): the bins are the scores' leading 16 bits (relative width
+// 2^-7) from 2^-16 up.  Its top_n-th best, lowered by four times the score's
+// error bound, is a threshold for all CTAs: after the first columns of every
+// CTA it comes from 152 times as many combinations as the CTA's own list, so
+// few of the later ones are scored precisely (searches with the thresholds of
+// the CTAs' own lists and with this: order 2, 6007 x 5003: 2.27 and 0.52 ms;
+// order 3, 300 x 2500: 0.69 and 0.38 ms).
+constexpr uint32_t kHistFirst = 0x3780u;   // 2^-16 >> 16
+__device__ __forceinline__ int hist_bin(float score)
+{
+    const int b = (int)(__float_as_uint(score) >> 16) - (int)kHistFirst + 1;
+    return b < 0 ? 0 : (b >= kTcHistBins ? kTcHistBins - 1 : b);
+}
+// the threshold the histogram gives, or -1 (all threads of the epilogue; tmp:
+// NT / 32 + 2 words of shared memory)
+template <int NT>
+__device__ inline float hist_threshold(const uint32_t *hist, int top_n, uint32_t *tmp, int tid)
+{
+    constexpr int kPer = kTcHistBins / NT;
+    static_assert(kPer * NT == kTcHistBins && kPer % 4 == 0, "whole vectors per thread");
+    const int lane = tid & 31, warp = tid >> 5;
+    const int top = kTcHistBins - kPer * (tid + 1);     // this thread's lowest bin (thread 0 has the highest)
+    uint32_t c[kPer], sum = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; q += 4) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(hist + top + q));
+        c[q] = v.x; c[q + 1] = v.y; c[q + 2] = v.z; c[q + 3] = v.w;
+        sum += v.x + v.y + v.z + v.w;
+    }
+    uint32_t inc = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xffffffffu, inc, off);
+        if (lane >= off) inc += o;
+    }
+    if (tid == 0) tmp[NT / 32] = 0;
+    if (lane == 31) tmp[warp] = inc;
+    epi_bar<NT>();
+    uint32_t before = inc - sum;
+    for (int w = 0; w < warp; w++) before += tmp[w];
+    const uint32_t need = (uint32_t)top_n;
+    if (before < need && before + sum >= need) {
+        int b = kPer;
+        while (before < need) before += c[--b];
+        b += top;
+        tmp[NT / 32] = b > 0 ? (uint32_t)(b - 1 + (int)kHistFirst) << 16 : 0u;
+    }
+    epi_bar<NT>();
+    const float t = __uint_as_float(tmp[NT / 32]);
+    return t > 0.0f ? t : -1.0f;
+}
 
 template <int NT>
 __device__ inline void epi_flush(EpiState &S, float *sc, uint64_t *rk, int pool, const DsParams &DS, int tid)
@@ -768,6 +823,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
     __shared__ uint32_t item_idesc[kDescDepth];
     __shared__ volatile int abort_flag;
     __shared__ EpiState ES;
+    __shared__ uint32_t hist_tmp[kEpiWarps + 1];
     // order 5: per-quadrant sums of the item's last SNPs, and their flags
     __shared__ float wred[kWide ? 4 : 1][kWide ? kJ : 1], wpre[kWide ? 4 : 1][kWide ? kJ : 1];
     __shared__ __align__(8) unsigned char wflag[kWide ? kJ : 1];
@@ -810,7 +866,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
         g_wait_limit_ns = P.wait_ns ? P.wait_ns : kTimeoutNs;
-        ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.any = 0; ES.thr = ES.next_thr = -1.0f;
+        ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.any = 0; ES.seen = 0; ES.thr = ES.next_thr = -1.0f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kWarpMma) {
@@ -1300,9 +1356,28 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
 #pragma unroll
                     for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
                     const int slot = list_len + atomicAdd(&ES.nbuf, 1);
+                    if (DS.top_n > 0) atomicAdd(DS.hist + hist_bin(score), 1u);
                     sc[slot] = score;
                     rk[slot] = DS.total - 1 - prefix_rank_sum<km1>(d, qs) - (uint64_t)(d.n - 1 - j);
                 }
+            };
+            // the threshold of everything kept so far, by all CTAs
+            auto share_threshold = [&]() {
+                epi_bar<kEpiThreads>();
+                const int kept = ES.list_len + ES.nbuf;
+                if (DS.top_n > 0) {
+                    __threadfence();
+                    const float t = hist_threshold<kEpiThreads>(DS.hist, DS.top_n, hist_tmp, tid) * DS.thr_mul;
+                    if (tid == 0) {
+                        ES.seen = kept;
+                        if (t > ES.thr) {
+                            ES.thr = t;
+                            atomicMax(DS.global_thr, __float_as_uint(t));
+                        }
+                    }
+                }
+                epi_bar<kEpiThreads>();
+                thr = fmaxf(thr, ES.thr);
             };
             // Without a threshold every combination needs its precise score:
             // all prefixes of the warp at once, column by column (one flagged
@@ -1426,15 +1501,9 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
 #pragma unroll 1
                 for (int jc = 0; jc < rounds; jc++) {
                     if (cold && jc > 0) {
-                        epi_bar<kEpiThreads>();
-                        if (ES.nbuf > 0 && ES.list_len + ES.nbuf >= (DS.top_n > 0 ? DS.top_n : P.pool)) {
-                            epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
-                            thr = ES.thr;
-                            cut = thr * DS.cut_mul - DS.cut_add;
-                            list_len = ES.list_len;
-                            cold = thr < 0.0f;
-                        }
-                        epi_bar<kEpiThreads>();
+                        share_threshold();
+                        cut = thr * DS.cut_mul - DS.cut_add;
+                        cold = thr < 0.0f;
                     }
                     if (jc >= mine) continue;
                     const int jcg = jhalf + kCG * jc;
@@ -1517,17 +1586,39 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             thr = ES.next_thr;
             // the next item adds at most one candidate per last SNP and
             // prefix: sort and trim first if the buffer could not hold them
-            // (and when a pool's worth is waiting: a better threshold keeps
-            // later ones out)
-            const int nbuf = ES.nbuf;
-            if (ES.list_len + nbuf + kJ * kPPT > P.cand_p2 || nbuf >= P.pool ||
-                (thr < 0.0f && DS.top_n > 0 && ES.list_len + nbuf >= DS.top_n))
-                epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
-            // no candidate of the next item before every warp has read nbuf
+            const int kept = ES.list_len + ES.nbuf;
+            const bool grew = kept != ES.seen;
+            // no candidate of the next item before every warp has read these
             epi_bar<kEpiThreads>();
-            thr = fmaxf(thr, ES.thr);
+            if (kept + kJ * kPPT > P.cand_p2) {
+                epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
+                thr = fmaxf(thr, ES.thr);
+            }
+            if (grew) share_threshold();
         }
         epi_bar<kEpiThreads>();
+        {
+            // what the other CTAs' threshold has passed meanwhile need not be
+            // sorted: compact the rest (any order) to the front
+            const float gthr = __uint_as_float(*(volatile uint32_t *)DS.global_thr);
+            const int kept = ES.list_len + ES.nbuf;
+            epi_bar<kEpiThreads>();
+            if (tid == 0) ES.nbuf = 0;
+            for (int q0 = 0; q0 < kept; q0 += kEpiThreads) {
+                const int q = q0 + tid;
+                const float v = q < kept ? sc[q] : -1.0f;
+                const uint64_t rv = q < kept ? rk[q] : 0;
+                epi_bar<kEpiThreads>();
+                if (q < kept && v >= gthr) {
+                    const int at = atomicAdd(&ES.nbuf, 1);
+                    sc[at] = v;
+                    rk[at] = rv;
+                }
+                epi_bar<kEpiThreads>();
+            }
+            if (tid == 0) ES.list_len = 0;
+            epi_bar<kEpiThreads>();
+        }
         if (ES.nbuf > 0) epi_flush<kEpiThreads>(ES, sc, rk, P.pool, DS, tid);
         const int L = ES.list_len;
         for (int q = tid; q < L; q += kEpiThreads) {
@@ -1835,12 +1926,13 @@ static void fill_screen(tc::DsParams &D, const DevData &d, int k, int comb_p)
 // the launch is batched (nullptr: passed as a kernel parameter instead).
 static void fill_ds(tc::DsParams &D, const DevData &d, int k, uint64_t *item_cum, uint32_t *global_thr,
                     uint64_t total, uint64_t rb, uint64_t re, const CUtensorMap *tmap_dev, int cta_begin,
-                    int cta_count, int comb_p, const unsigned char *b4, int top_n)
+                    int cta_count, int comb_p, const unsigned char *b4, int top_n, uint32_t *hist)
 {
     D.d = d;
     D.rows = reinterpret_cast<const uint4 *>(b4 + tc_b_bytes(d));
     D.comb_p = comb_p;
-    D.top_n = top_n;
+    D.top_n = hist ? top_n : 0;
+    D.hist = hist;
     D.thr_mul = (float)(1.0 - 4.0 * f32_rel_bound(k, d.m));
     D.rank_begin = rb;
     D.rank_end = re;
@@ -1913,10 +2005,10 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
                              uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                              int32_t *status, int grid, uint64_t total, uint64_t rb, uint64_t re, cudaStream_t st,
                              int *cand_p2_out, float *cand_g, uint64_t *rank_g, uint32_t *dump,
-                             unsigned long long *waits, unsigned long long wait_ns, int comb_p, int top_n)
+                             unsigned long long *waits, unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist)
 {
     tc::Params P;
-    fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p, b4, top_n);
+    fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p, b4, top_n, hist);
     P.many = nullptr;
     P.cta_ds = nullptr;
     fill_launch(P, k, pool, list_score, list_rank, list_count, status, dump, waits, cand_g, rank_g, comb_p != 0);
@@ -1934,10 +2026,10 @@ size_t tc_ds_bytes() { return sizeof(tc::DsParams); }
 
 cudaError_t tc_fill_batch_entry(void *ds_host, void *tmap_host, const DevData &d, int k, const unsigned char *b4,
                                 uint64_t *item_cum, uint32_t *global_thr, uint64_t total, const void *tmap_dev,
-                                int cta_begin, int cta_count, int comb_p, int top_n)
+                                int cta_begin, int cta_count, int comb_p, int top_n, uint32_t *hist)
 {
     fill_ds(*static_cast<tc::DsParams *>(ds_host), d, k, item_cum, global_thr, total, 0, total,
-            static_cast<const CUtensorMap *>(tmap_dev), cta_begin, cta_count, comb_p, b4, top_n);
+            static_cast<const CUtensorMap *>(tmap_dev), cta_begin, cta_count, comb_p, b4, top_n, hist);
     return encode_map(static_cast<CUtensorMap *>(tmap_host), d, b4, comb_p != 0);
 }
 

@@ -306,7 +306,7 @@ cudaError_t launch_topk(const float *scores, const uint8_t *keep, int64_t count,
     gather_kernel<<<(int)((k + 255) / 256), 256, 0, st>>>(scores, sel_i, out_n, sel_s);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_merge(sel_s, sel_i, out_n, 1, (int)k, (int)k, out_s, out_i, out_n, st, -INFINITY);
+    return launch_merge(sel_s, sel_i, out_n, 1, (int)k, (int)k, out_s, out_i, out_n, st, nullptr, -INFINITY);
 }
 
 }  // namespace epi
