@@ -78,6 +78,14 @@ uint64_t tc_range_work(int64_t n, int k, uint64_t rb, uint64_t re);
 // with that buffer in shared memory or (cand_global) in a global buffer
 int tc_cand_p2(int k, int pool, bool comb);
 size_t tc_smem_bytes(int cand_p2, bool cand_global, bool comb);
+// collect (ranks != NULL): instead of the best, every combination scoring at
+// least thr: its rank goes to ranks[0 .. cap), *n counts them
+struct TcCollect {
+    uint64_t *ranks = nullptr;
+    unsigned long long *n = nullptr;
+    uint64_t cap = 0;
+    float thr = 0.0f;
+};
 // item_cum: device [2][n + 1] (item and prefix tables); ranks [rb, re);
 // cand_g / rank_g: NULL, or [grid][tc_cand_p2] global candidate buffers;
 // comb_p: 0 = separate-class variant, else the combined-class variant's shift
@@ -86,7 +94,7 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
                              int32_t *status, int grid, uint64_t total, uint64_t rb, uint64_t re, cudaStream_t st,
                              int *cand_p2_out, float *cand_g, uint64_t *rank_g, uint32_t *dump = nullptr,
                              unsigned long long *waits = nullptr, unsigned long long wait_ns = 0, int comb_p = 0,
-                             int top_n = 0, uint32_t *hist = nullptr);
+                             int top_n = 0, uint32_t *hist = nullptr, TcCollect collect = TcCollect{});
 // words of a search's score histogram (hist above: zeroed; NULL: none)
 constexpr int kTcHistBins = 2048;
 constexpr int kTcWaitSlots = 8;

@@ -170,6 +170,7 @@ struct Params {
     uint64_t *list_rank;
     int32_t *list_count;
     int32_t *status;
+    TcCollect collect;            // ranks != NULL: every combination at or above its threshold instead of the best
     unsigned long long wait_ns;   // limit of the pipeline waits (0: kTimeoutNs)
     uint32_t *dump;            // optional: every table, [rank][2][3^k] (validation)
     unsigned long long *waits; // optional: [grid][8] cycles spent waiting, per role (tracing)
@@ -866,7 +867,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
         g_wait_limit_ns = P.wait_ns ? P.wait_ns : kTimeoutNs;
-        ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.any = 0; ES.seen = 0; ES.thr = ES.next_thr = -1.0f;
+        ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.any = 0; ES.seen = 0;
+        ES.thr = ES.next_thr = P.collect.ranks ? P.collect.thr : -1.0f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kWarpMma) {
@@ -1237,7 +1239,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         const bool poly = DS.poly != 0;
         float *wb = wsum + warp * 256;
         int ab = 0;                          // first accumulator buffer of the item
-        float thr = -1.0f;                   // the threshold as of the last item's closing barrier
+        float thr = ES.thr;                  // the threshold as of the last item's closing barrier
         long long w_epi = 0;
         for (int64_t i = 0; i < n_my; i++) {
             const int dq = (int)(i % kDescDepth);
@@ -1301,6 +1303,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             auto refresh = [&]() {
                 if (tid == 0) {
                     ES.next_thr = gthr > 0.0f ? fmaxf(ES.thr, gthr) : ES.thr;
+                    // more than the caller's array holds: give up
+                    if (P.collect.ranks && *(volatile unsigned long long *)P.collect.n > P.collect.cap) abort_flag = 1;
                     ES.stop = abort_flag;
                 }
             };
@@ -1355,10 +1359,16 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     int32_t qs[km1];
 #pragma unroll
                     for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
+                    const uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, qs) - (uint64_t)(d.n - 1 - j);
+                    if (P.collect.ranks) {
+                        const unsigned long long at = atomicAdd(P.collect.n, 1ull);
+                        if (at < P.collect.cap) P.collect.ranks[at] = rank;
+                        return;
+                    }
                     const int slot = list_len + atomicAdd(&ES.nbuf, 1);
                     if (DS.top_n > 0) atomicAdd(DS.hist + hist_bin(score), 1u);
                     sc[slot] = score;
-                    rk[slot] = DS.total - 1 - prefix_rank_sum<km1>(d, qs) - (uint64_t)(d.n - 1 - j);
+                    rk[slot] = rank;
                 }
             };
             // the threshold of everything kept so far, by all CTAs
@@ -2005,7 +2015,8 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
                              uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                              int32_t *status, int grid, uint64_t total, uint64_t rb, uint64_t re, cudaStream_t st,
                              int *cand_p2_out, float *cand_g, uint64_t *rank_g, uint32_t *dump,
-                             unsigned long long *waits, unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist)
+                             unsigned long long *waits, unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist,
+                             TcCollect collect)
 {
     tc::Params P;
     fill_ds(P.one, d, k, item_cum, global_thr, total, rb, re, nullptr, 0, grid, comb_p, b4, top_n, hist);
@@ -2013,6 +2024,7 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
     P.cta_ds = nullptr;
     fill_launch(P, k, pool, list_score, list_rank, list_count, status, dump, waits, cand_g, rank_g, comb_p != 0);
     P.wait_ns = wait_ns;
+    P.collect = collect;
     *cand_p2_out = P.cand_p2;
     cudaError_t e = launch_tc_item_cum(d, k, rb, re, item_cum, st, comb_p != 0);
     if (e != cudaSuccess) return e;
