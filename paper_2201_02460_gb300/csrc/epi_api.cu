@@ -198,6 +198,7 @@ struct SearchPlan {
     int k = 0, top_n = 0, pool = 0, tile = 0, slots = 0, cand_p2 = 0, grid = 0, R = 0;
     bool tc = false;
     int comb_p = 0;                // tensor path: class shift of the combined-class variant, 0 = separate classes
+    bool tc_pair = false;          // tensor path: pair tiles (orders 4-5)
     bool global_prefix = false;    // popcount path: prefix tables in a global buffer (orders 7-8)
     bool pair = false;             // popcount path: the (k-2)-prefix kernel (orders 6-8)
     float *all_scores = nullptr;   // optional: every combination's score (popcount path)
@@ -352,6 +353,7 @@ epi_status make_plan(const epi_dataset *ds, SearchPlan &p, int path)
     if (!p.tc) return plan_popc(ds, p);
     p.grid = ds->ctx->num_sms;
     p.comb_p = plan_comb_shift(ds);
+    p.tc_pair = p.rb == 0 && p.re == p.total && tc_pair_applies(ds->dev(), p.k, p.comb_p != 0);
     return EPI_OK;
 }
 
@@ -398,11 +400,21 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     const size_t o_sing = p.pair ? a.take<uint32_t>((size_t)p.grid * popc_pair_sing_words(p.k, ds->n)) : 0;
     // tensor path: candidate buffers in global memory when they do not fit
     // beside the operand rings in shared memory (large pools)
-    const int tc_cp2 = p.tc ? tc_cand_p2(p.k, p.pool, p.comb_p != 0) : 0;
-    const bool tc_cg = p.tc && tc_smem_bytes(tc_cp2, false, p.comb_p != 0) > tc_smem_limit(ctx);
+    const int tc_cp2 = p.tc ? tc_cand_p2(p.k, p.pool, p.comb_p != 0, p.tc_pair) : 0;
+    const bool tc_cg = p.tc && (p.tc_pair || tc_smem_bytes(tc_cp2, false, p.comb_p != 0) > tc_smem_limit(ctx));
+    const TcPairBytes pb = p.tc_pair ? tc_pair_bytes(ds->dev(), p.k, p.comb_p != 0) : TcPairBytes();
+    const size_t o_pt = p.tc_pair ? a.take<char>(pb.tables) : 0;
+    const size_t o_po = p.tc_pair ? a.take<char>(pb.operand) : 0;
+    const size_t o_ps = p.tc_pair ? a.take<char>(pb.singles) : 0;
     const size_t o_tcs = tc_cg ? a.take<float>((size_t)p.grid * tc_cp2) : 0;
     const size_t o_tcr = tc_cg ? a.take<uint64_t>((size_t)p.grid * tc_cp2) : 0;
     epi_status st = ensure_scratch(ctx, a.off);
+    if (st == EPI_ENOMEM && p.tc_pair) {
+        // no room for the pairs: the search without them
+        SearchPlan q = p;
+        q.tc_pair = false;
+        return queue_search(ds, q, path, out_dev, counts_dev, n_out_dev, status_dev_out, dump, own);
+    }
     if (st != EPI_OK) return st;
     char *base = static_cast<char *>(ctx->scratch);
     uint32_t *thr = reinterpret_cast<uint32_t *>(base + o_thr);
@@ -450,6 +462,16 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
             waits = ctx->waits_dev;
             ctx->waits_grid = p.grid;
         }
+        if (p.tc_pair) {
+            const TcPairWork ws{reinterpret_cast<unsigned char *>(base + o_po),
+                                reinterpret_cast<unsigned char *>(base + o_ps),
+                                reinterpret_cast<uint64_t *>(base + o_pt)};
+            CK(launch_tc_pair_search(d, p.k, ds->b4, ws, p.pool, thr, ls, lr, lc, status, p.grid, p.total, ctx->stream,
+                                     reinterpret_cast<float *>(base + o_tcs), reinterpret_cast<uint64_t *>(base + o_tcr),
+                                     dump, waits, ctx->wait_limit_ns, p.comb_p, p.top_n,
+                                     reinterpret_cast<uint32_t *>(base + o_hist), TcCollect{}));
+            ctx->launches += 3;
+        } else
         CK(launch_tc_search(d, p.k, ds->b4, ic, p.pool, thr, ls, lr, lc, status, p.grid,
                             p.total, p.rb, p.re, ctx->stream, &cand_p2,
                             tc_cg ? reinterpret_cast<float *>(base + o_tcs) : nullptr,

@@ -76,7 +76,7 @@ int64_t tc_first_snp(int64_t n, int k, uint64_t r);
 uint64_t tc_range_work(int64_t n, int k, uint64_t rb, uint64_t re);
 // entries of a CTA's candidate buffer for a pool; shared memory of one CTA
 // with that buffer in shared memory or (cand_global) in a global buffer
-int tc_cand_p2(int k, int pool, bool comb);
+int tc_cand_p2(int k, int pool, bool comb, bool pair = false);
 size_t tc_smem_bytes(int cand_p2, bool cand_global, bool comb);
 // collect (ranks != NULL): instead of the best, every combination scoring at
 // least thr: its rank goes to ranks[0 .. cap), *n counts them
@@ -97,6 +97,22 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
                              int top_n = 0, uint32_t *hist = nullptr, TcCollect collect = TcCollect{});
 // words of a search's score histogram (hist above: zeroed; NULL: none)
 constexpr int kTcHistBins = 2048;
+// pair tiles (orders 4-5, whole searches): their work space and whether they
+// apply; ws.tables: device [5][n + 1]; cand_g / rank_g: [grid][tc_cand_p2]
+struct TcPairBytes {
+    size_t operand = 0, singles = 0, tables = 0;
+};
+struct TcPairWork {
+    unsigned char *operand = nullptr, *singles = nullptr;
+    uint64_t *tables = nullptr;
+};
+TcPairBytes tc_pair_bytes(const DevData &d, int k, bool comb);
+bool tc_pair_applies(const DevData &d, int k, bool comb);
+cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *b4, const TcPairWork &ws, int pool,
+                                  uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
+                                  int32_t *status, int grid, uint64_t total, cudaStream_t st, float *cand_g,
+                                  uint64_t *rank_g, uint32_t *dump, unsigned long long *waits,
+                                  unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist, TcCollect collect);
 constexpr int kTcWaitSlots = 8;
 // batched tensor-core launches: per-dataset descriptors and B-operand maps
 // (128-byte CUtensorMap, 64-byte aligned) live in device memory

@@ -124,8 +124,11 @@ constexpr unsigned long long kTimeoutNs = 2000000000ull;
 
 struct Desc {
     int32_t j0;          // first last-SNP of the N tile
+    int32_t j1;          // pair tiles: the SNP before it
     int32_t nvalid;      // real prefixes in the M tile
-    int32_t snp[kMaxDescSnps];   // prefix p occupies snp[p*(k-1) .. p*(k-1)+k-2]
+    int32_t pad;
+    uint64_t single[kMaxDescSnps];   // prefix p's place in the single-count table (groups)
+    int32_t snp[kMaxDescSnps];   // prefix p occupies snp[p*(k-1) .. p*(k-1)+k-2] (k - 2 SNPs each with pairs)
 };
 
 // One dataset of a launch; a batched launch covers several datasets of the
@@ -137,6 +140,13 @@ struct DsParams {
     const uint4 *rows;         // the producers' masks [stage][n][3][2] (16 bytes each)
     const uint64_t *item_cum;  // [n + 1] items of M tiles starting in panels < c
     const uint64_t *pcum;      // [n + 1] prefixes searched in panels < c
+    // pair tiles and the single counts behind them (see the pair section
+    // below): [n + 1] groups of singles in panels < c; items and operand rows
+    // of the pairs whose first SNP is below j1
+    const uint64_t *scum;
+    const uint64_t *brow;
+    float4 *singles;
+    int store;                 // 1: write the single counts instead of scoring
     uint64_t rank_begin, rank_end;   // lexicographic ranks searched
     int32_t s1_lo, s1_hi;      // first SNPs of ranks rank_begin and rank_end - 1
     int32_t clip;              // 0: the whole combination range
@@ -411,6 +421,28 @@ __host__ __device__ __forceinline__ int64_t panel_ntiles(int64_t n, int64_t c, i
 {
     return (n - panel_j0(c) + kj - 1) / kj;
 }
+
+// ------------------------------------------------------------------ pairs --
+// Pair tiles (orders 4-5, whole searches): the last TWO SNPs move to the B
+// side.  A tile's rows are (k-2)-prefixes (9 or 27 rows each, 12 or 4 of them)
+// and its columns the four joint genotypes (g1, g2 in {0, 1}) of a SNP j1 with
+// 60 (or 40) SNPs j2 > j1, an operand built once per search.  A combination
+// then takes 128 / 12 x 4 multiply-adds per individual instead of 128 / 4 x 2
+// (order 4; order 5: 128 instead of 256), tiles keep all their columns (the
+// pairs (j1, j2) of one j1 are many more than the SNPs after a prefix), and
+// an A tile serves twice the combinations, which the producers need most.
+// The remaining cells of a row follow from its counts with one of the two
+// SNPs (the single counts: the same product one order lower, stored by a first
+// pass as raw accumulators) and its total:
+//     n[g1][2] = n[g1][*] - n[g1][0] - n[g1][1], n[2][g2] likewise, and
+//     n[2][2] = n[*][*] - n[0][*] - n[1][*] - n[2][0] - n[2][1].
+// Singles table: panel c holds its prefixes in order, each
+// single_groups(n, c) groups of two SNPs (from the even panel_j0(c)), a group
+// the prefix's rows side by side, a row one float4 per accumulator: genotype 0
+// of both SNPs, genotype 1 of both.
+__host__ __device__ __forceinline__ int64_t single_groups(int64_t n, int64_t c) { return (n - panel_j0(c) + 1) / 2; }
+// operand rows of j1's pairs: 8 per group of two SNPs from the even panel_j0(j1)
+__host__ __device__ __forceinline__ int64_t pair_rows(int64_t n, int64_t j1) { return 8 * single_groups(n, j1); }
 
 // -------------------------------------------------------------- epilogue --
 // the integer value of an accumulator (below 2^23)
@@ -723,6 +755,89 @@ struct RowScreen {
             b[g] = (odd ? v : u) - a[g];
         }
     }
+    // --- pair tiles: U0, U1 this row's counts with j1's genotypes 0 and 1,
+    // V its count with genotype 2 (individuals .s, cases times 2^p .c)
+    struct Cnt {
+        F2 s, c;
+    };
+    Cnt U0, U1, V;
+    __device__ __forceinline__ Cnt raw2(uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1) const
+    {
+        Cnt r;
+        if constexpr (C) {
+            split(x0, x1, r.s, r.c);
+        } else {
+            r.c = f2_pack(__uint_as_float(x0), __uint_as_float(x1));
+            r.s = f2_add(r.c, f2_pack(__uint_as_float(y0), __uint_as_float(y1)));
+        }
+        return r;
+    }
+    __device__ __forceinline__ Cnt minus2(Cnt a, Cnt b, Cnt d) const
+    {
+        return Cnt{f2_fma(d.s, neg1, f2_fma(b.s, neg1, a.s)), f2_fma(d.c, neg1, f2_fma(b.c, neg1, a.c))};
+    }
+    // the nine cells (3 g1 + g2) of two SNPs j2: accumulator columns in pairs
+    // (00, 01, 10, 11), s0 / s1 the single counts with them
+    __device__ __forceinline__ void nine(const uint32_t *cs, const uint32_t *cn, const float4 &a, const float4 &b,
+                                         Cnt *n) const
+    {
+        n[0] = raw2(cs[0], cs[1], cn[C ? 0 : 0], cn[C ? 0 : 1]);
+        n[1] = raw2(cs[2], cs[3], cn[C ? 0 : 2], cn[C ? 0 : 3]);
+        n[3] = raw2(cs[4], cs[5], cn[C ? 0 : 4], cn[C ? 0 : 5]);
+        n[4] = raw2(cs[6], cs[7], cn[C ? 0 : 6], cn[C ? 0 : 7]);
+        const Cnt t0 = raw2(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(b.x), __float_as_uint(b.y));
+        const Cnt t1 = raw2(__float_as_uint(a.z), __float_as_uint(a.w), __float_as_uint(b.z), __float_as_uint(b.w));
+        n[2] = minus2(U0, n[0], n[1]);
+        n[5] = minus2(U1, n[3], n[4]);
+        n[6] = minus2(t0, n[0], n[3]);
+        n[7] = minus2(t1, n[1], n[4]);
+        n[8] = minus2(V, n[6], n[7]);
+    }
+    __device__ __forceinline__ void pair_bound(const uint32_t *cs, const uint32_t *cn, const float4 &a, const float4 &b,
+                                               float &v0, float &v1) const
+    {
+        Cnt n[9];
+        nine(cs, cn, a, b, n);
+        F2 acc;
+        acc.v = 0;
+#pragma unroll
+        for (int x = 0; x < 9; x++) acc = cell_bound(f2_fma(n[x].s, neg_pi, n[x].c), n[x].s, sc, acc);
+        f2_unpack(acc, v0, v1);
+    }
+    // counts of one of the two SNPs' nine cells
+    __device__ __forceinline__ void pair_counts(const uint32_t *cs, const uint32_t *cn, const float4 &a,
+                                                const float4 &b, bool odd, float *ca, float *co) const
+    {
+        Cnt n[9];
+        nine(cs, cn, a, b, n);
+#pragma unroll
+        for (int x = 0; x < 9; x++) {
+            float c0, c1, s0, s1;
+            f2_unpack(n[x].c, c0, c1);
+            f2_unpack(n[x].s, s0, s1);
+            ca[x] = (odd ? c1 : c0) * kinv1;
+            co[x] = (odd ? s1 : s0) - ca[x];
+        }
+    }
+    __device__ __forceinline__ float pair_log(const uint32_t *cs, const uint32_t *cn, const float4 &a, const float4 &b,
+                                              bool odd) const
+    {
+        float ca[9], co[9], v = 0.0f;
+        pair_counts(cs, cn, a, b, odd, ca, co);
+#pragma unroll
+        for (int x = 0; x < 9; x++) v += cell_log(ca[x], co[x]);
+        return v;
+    }
+    // this item's j1: its group's float4s and whether it is the odd SNP
+    __device__ __forceinline__ void set_first(const float4 &a, const float4 &b, bool odd)
+    {
+        const uint32_t x0 = __float_as_uint(odd ? a.y : a.x), x1 = __float_as_uint(odd ? a.w : a.z);
+        const uint32_t y0 = __float_as_uint(odd ? b.y : b.x), y1 = __float_as_uint(odd ? b.w : b.z);
+        U0 = raw2(x0, x0, y0, y0);
+        U1 = raw2(x1, x1, y1, y1);
+        const Cnt all{S, CT};
+        V = minus2(all, U0, U1);
+    }
     __device__ __forceinline__ void logs(const uint32_t *cs, const uint32_t *cn, float *vrow) const
     {
 #pragma unroll
@@ -737,11 +852,11 @@ struct RowScreen {
 // Lexicographic rank of a combination from the sum over its SNPs s_t of
 // C(n - 1 - s_t, K - t): total - 1 - sum.
 template <int km1>
-__device__ __forceinline__ uint64_t prefix_rank_sum(const DevData &d, const int32_t *psnp)
+__device__ __forceinline__ uint64_t prefix_rank_sum(const DevData &d, const int32_t *psnp, int k = km1 + 1)
 {
     uint64_t s = 0;
 #pragma unroll
-    for (int tt = 0; tt < km1; tt++) s += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], km1 + 1 - tt);
+    for (int tt = 0; tt < km1; tt++) s += binom_at(d.binom, d.n, d.n - 1 - psnp[tt], k - tt);
     return s;
 }
 
@@ -764,33 +879,36 @@ __device__ __forceinline__ void last_snp_range(const DsParams &DS, const DevData
     }
 }
 
-template <int K, bool C>
+template <int K, bool C, bool PAIR>
 __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                                                 const Params P)
 {
     using S = Shape<C>;
     using R = Roles;
     constexpr int kStages = S::Stages;
-    constexpr int kJ = S::J;
+    constexpr int kJ = PAIR ? S::N / 4 : S::J;      // last SNPs per N tile
+    constexpr int kColsPerSnp = S::N / kJ;
     constexpr int kBBytes = S::BBytes;
     constexpr int kEpiWarps = R::EpiWarps, kProdWarps = R::ProdWarps, kEpiThreads = R::EpiThreads;
     constexpr int kGroups = R::ProdGroups, kCG = R::ColGroups;
     // epilogue: the kQC chunks of 8 last SNPs of a lane quadrant go round-
     // robin to its kCG warps, kIters chunks each (the last may be empty)
-    constexpr int kQC = kJ / 8;
+    // (pair tiles: chunks of 4 last SNPs, 16 columns)
+    constexpr int kCS = PAIR ? 4 : 8;
+    constexpr int kQC = kJ / kCS;
     constexpr int kIters = (kQC + kCG - 1) / kCG;
-    constexpr int kPR = K == 2 ? 3 : (K == 3 ? 9 : (K == 4 ? 27 : 81));
+    constexpr int km1 = PAIR ? K - 2 : K - 1;       // prefix SNPs
+    constexpr int kPR = km1 == 1 ? 3 : (km1 == 2 ? 9 : (km1 == 3 ? 27 : 81));
     // order 5: one prefix per tile, its 81 rows over lane quadrants 0-2 (the
     // epilogue sums a combination across warps through shared memory)
     constexpr bool kWide = kPR > 32;
     constexpr int kPPW = kWide ? 0 : 32 / kPR;
     constexpr int kPPT = kWide ? 1 : 4 * kPPW;
-    constexpr int km1 = K - 1;
     constexpr int kWarpTma = kEpiWarps + kProdWarps;
     constexpr int kWarpMma = kWarpTma + 1;
     // (prefix, last SNP) pairs per warp and chunk; orders 4-5: 8 columns by 4
     // lane parts of the rows
-    constexpr int kPairs = kPPW > 1 ? kPPW * 8 : 8;
+    constexpr int kPairs = (kPPW > 1 ? kPPW : 1) * kCS;
     constexpr int kPairIters = (kPairs + 31) / 32;
 
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -905,6 +1023,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             int64_t u = 0;
             int seg = -1;
             uint64_t seg_left = 0;
+            int32_t j1 = 0, row0 = 0;            // pair tiles: first SNP, its first operand row,
+            uint64_t mt = 0, mtiles = 0;         // and the M tile among those of j1
             auto next_segment = [&]() {
                 uint64_t w0;
                 do {
@@ -915,27 +1035,49 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 const int64_t lo = warp_last(0, d.n - 1, [&](int64_t x) { return DS.item_cum[x] <= w0; });
                 const int32_t c0 = (int32_t)lo;
                 const uint64_t off = w0 - DS.item_cum[c0];
-                const int64_t nt0 = panel_ntiles(d.n, c0, kJ);
-                const uint64_t tfirst = (DS.pcum[c0] + kPPT - 1) / kPPT;
-                const uint64_t t = tfirst + off / (uint64_t)nt0;
-                u = (int64_t)(off % (uint64_t)nt0);
-                prefix_unrank(DS, K, t * (uint64_t)kPPT, it);
+                if constexpr (PAIR) {
+                    // M tiles within N tiles within j1
+                    j1 = c0;
+                    mtiles = (DS.pcum[j1] + kPPT - 1) / kPPT;
+                    u = (int64_t)(off / mtiles);
+                    mt = off % mtiles;
+                    row0 = (int32_t)DS.brow[j1];
+                    prefix_unrank(DS, K - 1, mt * (uint64_t)kPPT, it);
+                } else {
+                    const int64_t nt0 = panel_ntiles(d.n, c0, kJ);
+                    const uint64_t tfirst = (DS.pcum[c0] + kPPT - 1) / kPPT;
+                    const uint64_t t = tfirst + off / (uint64_t)nt0;
+                    u = (int64_t)(off % (uint64_t)nt0);
+                    prefix_unrank(DS, K, t * (uint64_t)kPPT, it);
+                }
             };
             next_segment();
             int32_t tile_snp[kPPT * km1];
             int32_t nvalid = 0, cmin = it.c;
+            // place of this lane's prefixes (lane, lane + 32) in the singles
+            uint64_t single[2] = {0, 0};
             auto fill_tile = [&]() {
                 nvalid = 0;
                 cmin = it.c;
+                int32_t my_c[2] = {-1, -1};
+                uint64_t my_q[2] = {0, 0};
 #pragma unroll
                 for (int p = 0; p < kPPT; p++) {
                     if (it.q < DS.n_prefix) {
 #pragma unroll
                         for (int s2 = 0; s2 < km1 - 1; s2++) tile_snp[p * km1 + s2] = it.a[s2];
                         tile_snp[p * km1 + km1 - 1] = it.c;
+                        if (lane == (p & 31)) { my_c[p >> 5] = it.c; my_q[p >> 5] = it.q; }
                         nvalid++;
-                        prefix_next(DS, K, it);
+                        prefix_next(DS, km1 + 1, it);
                     }
+                }
+                if (DS.singles) {
+#pragma unroll
+                    for (int h = 0; h < 2; h++)
+                        if (my_c[h] >= 0)
+                            single[h] = DS.scum[my_c[h]] +
+                                        (my_q[h] - DS.pcum[my_c[h]]) * (uint64_t)single_groups(d.n, my_c[h]);
                 }
             };
             fill_tile();
@@ -947,20 +1089,26 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 const int dq = (int)(i % kDescDepth);
                 const uint32_t ud = (uint32_t)(i / kDescDepth);
                 if (!__all_sync(0xffffffffu, mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag))) break;
-                const int32_t tile_j0 = (int32_t)panel_j0(cmin) + (int32_t)(u * kJ);
+                const int32_t tile_j0 = (int32_t)panel_j0(PAIR ? j1 : cmin) + (int32_t)(u * kJ);
+                if (DS.singles) {
+                    if (lane < kPPT) desc[dq].single[lane] = single[0];
+                    if (lane + 32 < kPPT) desc[dq].single[lane + 32] = single[1];
+                    __syncwarp();
+                }
                 if (lane == 0) {
                     Desc &D = desc[dq];
                     D.j0 = tile_j0;
+                    D.j1 = j1;
                     D.nvalid = nvalid;
 #pragma unroll
                     for (int q = 0; q < kPPT * km1; q++) D.snp[q] = tile_snp[q];
-                    // columns in use: 2 per last SNP below n, in steps of 16
-                    const int32_t live = 2 * ((int32_t)d.n - tile_j0);
+                    // columns in use: 2 (4) per last SNP below n, in steps of 16
+                    const int32_t live = kColsPerSnp * ((int32_t)d.n - tile_j0);
                     const uint32_t ncol = live >= S::N ? (uint32_t)S::N : (uint32_t)((live + 15) & ~15);
                     item_idesc[dq] = make_idesc(ncol);
                     mbar_arrive(&desc_full[dq]);
                 }
-                const int y = 2 * tile_j0;
+                const int y = PAIR ? row0 + (int)(u * S::N) : 2 * tile_j0;
                 for (int kc = 0; kc < nst; kc++, g++) {
                     if (!__all_sync(0xffffffffu, wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_tma))) break;
                     if (lane == 0) {
@@ -969,6 +1117,32 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     }
                     __syncwarp();
                     if (++s == kStages) { s = 0; ph ^= 1; }
+                }
+                if constexpr (PAIR) {
+                    if (--seg_left == 0) {
+                        if (i + 1 < n_my) {
+                            next_segment();
+                            fill_tile();
+                        }
+                        continue;
+                    }
+                    if (++mt == mtiles) {
+                        // next N tile of j1, or the first of the next SNP:
+                        // from the first prefix again
+                        mt = 0;
+                        if (++u == panel_ntiles(d.n, j1, kJ)) {
+                            u = 0;
+                            j1++;
+                            mtiles = (DS.pcum[j1] + kPPT - 1) / kPPT;
+                            row0 = (int32_t)DS.brow[j1];
+                        }
+                        it.q = 0;
+                        it.c = km1 - 1;
+#pragma unroll
+                        for (int t = 0; t < km1 - 1; t++) it.a[t] = t;
+                    }
+                    fill_tile();
+                    continue;
                 }
                 u++;
                 if (--seg_left == 0) {
@@ -1270,7 +1444,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             int32_t plo[kPairIters], phi[kPairIters];
 #pragma unroll
             for (int q = 0; q < kPairIters; q++) {
-                const int pp = kPPW > 1 ? (lane + 32 * q) >> 3 : 0;
+                const int pp = kPPW > 1 ? (lane + 32 * q) / kCS : 0;
                 const int pt = quad * kPPW + pp;
                 plo[q] = 1;
                 phi[q] = 0;                      // empty: no valid last SNP
@@ -1278,7 +1452,12 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     int32_t qs[km1];
 #pragma unroll
                     for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
-                    last_snp_range<km1>(DS, d, qs, plo[q], phi[q]);
+                    if constexpr (PAIR) {
+                        // (prefix, j1) is a prefix of the combination
+                        if (qs[km1 - 1] < D.j1) { plo[q] = D.j1 + 1; phi[q] = (int32_t)d.n; }
+                    } else {
+                        last_snp_range<km1>(DS, d, qs, plo[q], phi[q]);
+                    }
                 }
             }
             {
@@ -1359,7 +1538,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     int32_t qs[km1];
 #pragma unroll
                     for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
-                    const uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, qs) - (uint64_t)(d.n - 1 - j);
+                    uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, qs, K) - (uint64_t)(d.n - 1 - j);
+                    if constexpr (PAIR) rank -= binom_at(d.binom, d.n, d.n - 1 - D.j1, 2);
                     if (P.collect.ranks) {
                         const unsigned long long at = atomicAdd(P.collect.n, 1ull);
                         if (at < P.collect.cap) P.collect.ranks[at] = rank;
@@ -1393,7 +1573,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             // all prefixes of the warp at once, column by column (one flagged
             // pair at a time, as below, the first items of a CTA took
             // milliseconds at order 2), summed as the flagged ones are.
-            bool cold = thr < 0.0f;
+            bool cold = thr < 0.0f && !DS.store;
             // 8 row values per lane -> transposed sums: the lane of pair
             // (prefix pp, last SNP jj) adds rows pp kPR .. of column jj (all
             // banks distinct); at orders 4-5 four lanes share a column
@@ -1495,6 +1675,156 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 refresh();
                 epi_bar<kEpiThreads>();
                 if (tid == 0) ES.any = 0;
+            } else if constexpr (PAIR) {
+                // Chunks of 4 last SNPs (16 columns): two groups of two, each
+                // 8 columns and one float4 (two with separate classes) of
+                // single counts per row, loaded one chunk ahead
+                constexpr int kAcc = C ? 1 : 2;
+                const int live_chunks = ok ? min(kQC, ((int32_t)d.n - j0 + 3) >> 2) : 0;
+                const int mine = (live_chunks - jhalf + kCG - 1) / kCG;
+                const bool row_in = prow && psnp[km1 - 1] < D.j1;
+                // rows outside read one place of the table (their values are dropped)
+                const int32_t base = row_in ? (int32_t)panel_j0(psnp[km1 - 1]) : 0;
+                const float4 *sp = DS.singles + (row_in ? (D.single[p] * kPR + pos) * kAcc : 0);
+                const int64_t gstep = row_in ? (int64_t)kPR * kAcc : 0;
+                auto load_singles = [&](int32_t j, float4 *a, float4 *b) {
+                    const float4 *q = sp + (int64_t)((j - base) >> 1) * gstep;
+                    a[0] = __ldg(q);
+                    if constexpr (!C) b[0] = __ldg(q + 1);
+                    a[1] = __ldg(q + gstep);
+                    if constexpr (!C) b[1] = __ldg(q + gstep + 1);
+                };
+                float4 na[2], nb[2];
+                {
+                    float4 fa, fb;
+                    const float4 *q = sp + (int64_t)((D.j1 - base) >> 1) * gstep;
+                    fa = __ldg(q);
+                    fb = C ? fa : __ldg(q + 1);
+                    if (mine > 0) load_singles(j0 + kCS * jhalf, na, nb);
+                    rs.set_first(fa, fb, ((D.j1 - base) & 1) != 0);
+                }
+                if (mine <= 0) release_acc();
+                const int rounds = cold ? kIters : mine;
+#pragma unroll 1
+                for (int jc = 0; jc < rounds; jc++) {
+                    if (cold && jc > 0) {
+                        share_threshold();
+                        cut = thr * DS.cut_mul - DS.cut_add;
+                        cold = thr < 0.0f;
+                    }
+                    if (jc >= mine) continue;
+                    const int jcg = jhalf + kCG * jc;
+                    const int32_t jb = j0 + kCS * jcg;
+                    uint32_t cs[16], cn[C ? 1 : 16];
+                    load_chunk(jcg, cs, cn);
+                    float4 a[2], b[2];
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        a[h] = na[h];
+                        b[h] = C ? na[h] : nb[h];
+                    }
+                    if (jc + 1 < mine) load_singles(jb + kCS * kCG, na, nb);
+                    tmem_wait_ld();
+                    if (jc + 1 == mine) release_acc();
+                    if (P.dump && row_in) {
+#pragma unroll 1
+                        for (int jj = 0; jj < kCS; jj++) {
+                            const int32_t j = jb + jj;
+                            if (j <= D.j1 || j >= (int32_t)d.n) continue;
+                            float ca[9], co[9];
+                            if (jj < 2) rs.pair_counts(cs, cn, a[0], b[0], jj & 1, ca, co);
+                            else rs.pair_counts(cs + 8, cn + (C ? 0 : 8), a[1], b[1], jj & 1, ca, co);
+                            constexpr int cells = kPR * 9;
+                            const uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, psnp, K) -
+                                                  binom_at(d.binom, d.n, d.n - 1 - D.j1, 2) - (uint64_t)(d.n - 1 - j);
+                            uint32_t *o = P.dump + rank * 2 * cells;
+#pragma unroll
+                            for (int x = 0; x < 9; x++) {
+                                o[pos * 9 + x] = f2u_exact(ca[x]);
+                                o[cells + pos * 9 + x] = f2u_exact(co[x]);
+                            }
+                        }
+                    }
+                    // precise terms of this row for column jsel
+                    auto precise = [&](int jsel) -> float {
+                        float ca[9], co[9];
+                        if (jsel < 2) rs.pair_counts(cs, cn, a[0], b[0], jsel & 1, ca, co);
+                        else rs.pair_counts(cs + 8, cn + (C ? 0 : 8), a[1], b[1], jsel & 1, ca, co);
+                        float e = 0.0f;
+#pragma unroll
+                        for (int x = 0; x < 9; x += 3)
+                            e += row_terms_precise(f2u_exact(ca[x]), f2u_exact(co[x]), f2u_exact(ca[x + 1]),
+                                                   f2u_exact(co[x + 1]), f2u_exact(ca[x + 2]), f2u_exact(co[x + 2]), mc);
+                        return e;
+                    };
+                    if (cold) {
+#pragma unroll 1
+                        for (int jj = 0; jj < kCS; jj++) {
+                            const float e = seg_sum<kPR>(row_in ? precise(jj) : 0.0f, pos);
+                            if (row_in && pos == 0 && jb + jj > D.j1 && jb + jj < (int32_t)d.n)
+                                keep(__fdiv_rn(e, mc.fm), p, jb + jj);
+                        }
+                        continue;
+                    }
+                    float vrow[4];
+                    if (poly) {
+                        rs.pair_bound(cs, cn, a[0], b[0], vrow[0], vrow[1]);
+                        rs.pair_bound(cs + 8, cn + (C ? 0 : 8), a[1], b[1], vrow[2], vrow[3]);
+                    } else {
+                        vrow[0] = rs.pair_log(cs, cn, a[0], b[0], false);
+                        vrow[1] = rs.pair_log(cs, cn, a[0], b[0], true);
+                        vrow[2] = rs.pair_log(cs + 8, cn + (C ? 0 : 8), a[1], b[1], false);
+                        vrow[3] = rs.pair_log(cs + 8, cn + (C ? 0 : 8), a[1], b[1], true);
+                    }
+                    reinterpret_cast<float4 *>(wb)[lane] = row_in ? make_float4(vrow[0], vrow[1], vrow[2], vrow[3])
+                                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    __syncwarp();
+                    uint32_t cmask[kPairIters];
+                    if constexpr (kPPW > 1) {
+#pragma unroll
+                        for (int q = 0; q < kPairIters; q++) {
+                            const int pair = lane + 32 * q;
+                            bool cand = false;
+                            if (pair < kPairs) {
+                                const int pp = pair / kCS, jj = pair % kCS;
+                                float v = 0.0f, w2 = 0.0f;
+#pragma unroll
+                                for (int rr = 0; rr < kPR; rr++) {
+                                    if (rr & 1) w2 += wb[(pp * kPR + rr) * kCS + jj];
+                                    else v += wb[(pp * kPR + rr) * kCS + jj];
+                                }
+                                v += w2;
+                                const int32_t j = jb + jj;
+                                cand = j >= plo[q] && j < phi[q] && fmaf(v, vscale, voff) >= cut;
+                            }
+                            cmask[q] = __ballot_sync(0xffffffffu, cand);
+                        }
+                    } else {
+                        // one prefix: 8 lanes share a column (4 rows each)
+                        float v = 0.0f;
+#pragma unroll
+                        for (int rr = 0; rr < 4; rr++) v += wb[((lane >> 2) * 4 + rr) * kCS + (lane & 3)];
+                        v += __shfl_xor_sync(0xffffffffu, v, 4);
+                        v += __shfl_xor_sync(0xffffffffu, v, 8);
+                        v += __shfl_xor_sync(0xffffffffu, v, 16);
+                        const int32_t j = jb + (lane & 3);
+                        cmask[0] = __ballot_sync(0xffffffffu, lane < 4 && j >= plo[0] && j < phi[0] &&
+                                                                  fmaf(v, vscale, voff) >= cut);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < kPairIters; q++) {
+                        while (cmask[q]) {
+                            const int pair = __ffs(cmask[q]) - 1 + 32 * q;
+                            cmask[q] &= cmask[q] - 1;
+                            const int pp = pair / kCS, jsel = pair % kCS;
+                            const float e = seg_sum<kPR>(row_in && pl == pp ? precise(jsel) : 0.0f, pos);
+                            if (row_in && pl == pp && pos == 0) keep(__fdiv_rn(e, mc.fm), p, jb + jsel);
+                        }
+                    }
+                }
+                refresh();
+                epi_bar<kEpiThreads>();
             } else {
                 // this warp's chunks of the quadrant: those that hold a last
                 // SNP below n (all but in the last N tile of a panel)
@@ -1531,6 +1861,26 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     if (jc + 1 < mine) load_chunk(jcg + kCG, nx, ny);
                     else release_acc();
                     if (P.dump) dump_chunk(jb, cs, cn);
+                    if (DS.store) {
+                        // the raw accumulators of this row, two SNPs at a time
+                        if (prow) {
+                            constexpr int kAcc = C ? 1 : 2;
+                            const int32_t base = (int32_t)panel_j0(psnp[km1 - 1]);
+                            const int32_t top = base + 2 * (int32_t)single_groups(d.n, psnp[km1 - 1]);
+#pragma unroll
+                            for (int h = 0; h < 4; h++) {
+                                const int32_t j = jb + 2 * h;
+                                if (j < base || j >= top) continue;
+                                float4 *o = DS.singles + ((D.single[p] + (uint64_t)((j - base) >> 1)) * kPR + pos) * kAcc;
+                                o[0] = make_float4(__uint_as_float(cs[4 * h]), __uint_as_float(cs[4 * h + 1]),
+                                                   __uint_as_float(cs[4 * h + 2]), __uint_as_float(cs[4 * h + 3]));
+                                if constexpr (!C)
+                                    o[1] = make_float4(__uint_as_float(cn[4 * h]), __uint_as_float(cn[4 * h + 1]),
+                                                       __uint_as_float(cn[4 * h + 2]), __uint_as_float(cn[4 * h + 3]));
+                            }
+                        }
+                        continue;
+                    }
                     if (cold) {
                         int32_t jlo = 1, jhi = 0;
                         if (prow && pos == 0) last_snp_range<km1>(DS, d, psnp, jlo, jhi);
@@ -1725,6 +2075,52 @@ __global__ void build_b4_kernel(DevData d, uint4 *__restrict__ b4)
     }
 }
 
+// Tables of a pair search over the (kp)-prefixes of pcum: groups of singles
+// per panel, items and operand rows per first SNP j1 of the pairs (exclusive
+// prefix sums).  One block.
+__global__ void __launch_bounds__(1024) pair_tables_kernel(DevData d, int kp, int ppt, int kj, const uint64_t *pcum,
+                                                           uint64_t *scum, uint64_t *icum, uint64_t *brow)
+{
+    __shared__ uint64_t part[1024];
+    const int64_t n = d.n;
+    const int64_t per = (n + 1023) / 1024;
+    const int64_t cb = (int64_t)threadIdx.x * per, ce = min(n, cb + per);
+    auto scan = [&](auto value, uint64_t *out) {
+        uint64_t s = 0, run = 0, all = 0;
+        for (int64_t c = cb; c < ce; c++) s += value(c);
+        block_exclusive_scan(part, s, run, all);
+        for (int64_t c = cb; c < ce; c++) {
+            out[c] = run;
+            run += value(c);
+        }
+        if (threadIdx.x == 1023) out[n] = all;
+    };
+    scan([&](int64_t c) -> uint64_t { return (pcum[c + 1] - pcum[c]) * (uint64_t)single_groups(n, c); }, scum);
+    scan([&](int64_t j) -> uint64_t {
+        return j < kp || j > n - 2 ? 0 : (pcum[j] + ppt - 1) / ppt * (uint64_t)panel_ntiles(n, j, kj);
+    }, icum);
+    scan([&](int64_t j) -> uint64_t { return j > n - 2 ? 0 : (uint64_t)pair_rows(n, j); }, brow);
+}
+
+// Pair operand: of j1 = blockIdx.y, rows 8 h + 4 g1 + 2 g2 + odd are the
+// individuals with genotype g1 at j1 and g2 at j2 = panel_j0(j1) + 2 h + odd
+// (zeros where j2 <= j1 or past the last SNP), expanded as the B operand is.
+__global__ void build_pairs_kernel(DevData d, const uint64_t *__restrict__ brow, uint4 *__restrict__ out)
+{
+    const int64_t j1 = blockIdx.y;
+    const int64_t rows = pair_rows(d.n, j1), j0 = panel_j0(j1);
+    uint4 *o = out + brow[j1] * d.Wt;
+    const int64_t total = rows * d.Wt;
+    for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
+         idx += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t row = idx / d.Wt, w = idx - row * d.Wt;
+        const int64_t j2 = j0 + 2 * (row >> 3) + (row & 1);
+        const int g1 = (int)(row >> 2) & 1, g2 = (int)(row >> 1) & 1;
+        const uint32_t v = j2 > j1 && j2 < d.n ? d.masks[(j1 * 3 + g1) * d.Wt + w] & d.masks[(j2 * 3 + g2) * d.Wt + w] : 0u;
+        o[idx] = make_uint4((v & 0x11111111u) << 2, v & 0x22222222u, (v & 0x44444444u) >> 2, (v >> 3) & 0x11111111u);
+    }
+}
+
 // The producers' masks: the 256 individuals of a K stage of every SNP's three
 // genotype rows side by side (96 bytes a SNP; zeros past the last word), so
 // the lanes of a warp, whose rows differ in genotype first, read one or two
@@ -1790,6 +2186,9 @@ int tc_comb_shift(const DevData &d)
     return p;
 }
 
+#ifndef EPI_TC_PAIR_MIN_N
+#define EPI_TC_PAIR_MIN_N 32
+#endif
 static int tc_tile_snps(bool comb) { return comb ? tc::Shape<true>::J : tc::Shape<false>::J; }
 static int tc_pr(int k) { return k == 2 ? 3 : (k == 3 ? 9 : (k == 4 ? 27 : 81)); }
 static int tc_ppt(int k) { return tc_pr(k) > 32 ? 1 : 4 * (32 / tc_pr(k)); }
@@ -1846,7 +2245,44 @@ uint64_t tc_range_work(int64_t n, int k, uint64_t rb, uint64_t re)
 
 // Candidate buffer entries: the pool plus one item's combinations, rounded up
 // to a power of two for the bitonic sort.
-int tc_cand_p2(int k, int pool, bool comb) { return next_pow2(pool + tc_tile_snps(comb) * tc_ppt(k)); }
+int tc_cand_p2(int k, int pool, bool comb, bool pair)
+{
+    return next_pow2(pool + (pair ? tc_tile_snps(comb) / 2 * tc_ppt(k - 1) : tc_tile_snps(comb) * tc_ppt(k)));
+}
+
+// Groups of the single-count table of a pair search, and operand rows.
+static uint64_t pair_single_groups(int64_t n, int kp)
+{
+    uint64_t g = 0;
+    for (int64_t c = kp - 1; c <= n - 2; c++) g += host_binom(c, kp - 1) * (uint64_t)tc::single_groups(n, c);
+    return g;
+}
+
+static uint64_t pair_operand_rows(int64_t n)
+{
+    uint64_t r = 0;
+    for (int64_t j = 0; j <= n - 2; j++) r += (uint64_t)tc::pair_rows(n, j);
+    return r;
+}
+
+TcPairBytes tc_pair_bytes(const DevData &d, int k, bool comb)
+{
+    TcPairBytes b;
+    b.operand = (size_t)pair_operand_rows(d.n) * d.Wt * 16;
+    // one group more: the chunk that ends a prefix's groups may read past them
+    b.singles = ((size_t)pair_single_groups(d.n, k - 2) + 4) * tc_pr(k - 1) * (comb ? 16 : 32);
+    b.tables = (size_t)5 * (d.n + 1) * 8;
+    return b;
+}
+
+// Whether a whole order-k search takes pair tiles: orders 4 and 5 on enough
+// SNPs, with the operand and the single counts within 16 GiB.
+bool tc_pair_applies(const DevData &d, int k, bool comb)
+{
+    if ((k != 4 && k != 5) || d.n < EPI_TC_PAIR_MIN_N || d.n > 16384) return false;
+    const TcPairBytes b = tc_pair_bytes(d, k, comb);
+    return b.operand + b.singles <= ((size_t)16 << 30);
+}
 
 size_t tc_smem_bytes(int cand_p2, bool cand_global, bool comb)
 {
@@ -1856,12 +2292,14 @@ size_t tc_smem_bytes(int cand_p2, bool cand_global, bool comb)
            tc::kDescDepth * sizeof(tc::Desc) + (size_t)tc::Roles::EpiWarps * 256 * 4;
 }
 
-static cudaError_t encode_map(CUtensorMap *map, const DevData &d, const unsigned char *b4, bool comb)
+// B operand of `rows` rows (0: the dataset's own)
+static cudaError_t encode_map(CUtensorMap *map, const DevData &d, const unsigned char *b4, bool comb,
+                              uint64_t rows = 0)
 {
     cudaError_t e = get_encode();
     if (e != cudaSuccess) return e;
     const int64_t row = (int64_t)d.Wt * 16;
-    cuuint64_t gdim[2] = {(cuuint64_t)row, (cuuint64_t)(4 * ((d.n + 1) / 2))};
+    cuuint64_t gdim[2] = {(cuuint64_t)row, rows ? (cuuint64_t)rows : (cuuint64_t)(4 * ((d.n + 1) / 2))};
     cuuint64_t gstride[1] = {(cuuint64_t)row};
     cuuint32_t box[2] = {(cuuint32_t)tc::kRowBytes, (cuuint32_t)(2 * tc_tile_snps(comb))};
     cuuint32_t estr[2] = {1u, 1u};
@@ -1959,6 +2397,9 @@ static void fill_ds(tc::DsParams &D, const DevData &d, int k, uint64_t *item_cum
     D.n_items = tc_item_count(d.n, k, D.s1_lo, D.s1_hi, tc_tile_snps(comb_p != 0));
     D.item_cum = item_cum;
     D.pcum = item_cum + d.n + 1;
+    D.scum = D.brow = nullptr;
+    D.singles = nullptr;
+    D.store = 0;
     D.chunks = d.Wt * 32 / tc::kChunk;
     D.chunks_case = d.W1 * 32 / tc::kChunk;
     fill_screen(D, d, k, comb_p);
@@ -1971,10 +2412,10 @@ static void fill_ds(tc::DsParams &D, const DevData &d, int k, uint64_t *item_cum
 
 static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint64_t *list_rank, int32_t *list_count,
                         int32_t *status, uint32_t *dump, unsigned long long *waits, float *cand_g,
-                        uint64_t *rank_g, bool comb)
+                        uint64_t *rank_g, bool comb, bool pair = false)
 {
     P.pool = pool;
-    P.cand_p2 = tc_cand_p2(k, pool, comb);
+    P.cand_p2 = tc_cand_p2(k, pool, comb, pair);
     P.cand_score_g = cand_g;
     P.cand_rank_g = rank_g;
     P.wait_ns = 0;
@@ -1987,16 +2428,19 @@ static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint6
 }
 
 static cudaError_t launch_kernel(const CUtensorMap &map, const tc::Params &P, int k, int grid, cudaStream_t st,
-                                 bool comb)
+                                 bool comb, bool pair = false)
 {
     const size_t smem = tc_smem_bytes(P.cand_p2, P.cand_score_g != nullptr, comb);
     using Kernel = void (*)(const CUtensorMap, const tc::Params);
     static const Kernel kernels[2][4] = {
-        {tc::tc_search_kernel<2, false>, tc::tc_search_kernel<3, false>, tc::tc_search_kernel<4, false>,
-         tc::tc_search_kernel<5, false>},
-        {tc::tc_search_kernel<2, true>, tc::tc_search_kernel<3, true>, tc::tc_search_kernel<4, true>,
-         tc::tc_search_kernel<5, true>}};
-    const Kernel kern = kernels[comb][k - 2];
+        {tc::tc_search_kernel<2, false, false>, tc::tc_search_kernel<3, false, false>,
+         tc::tc_search_kernel<4, false, false>, tc::tc_search_kernel<5, false, false>},
+        {tc::tc_search_kernel<2, true, false>, tc::tc_search_kernel<3, true, false>,
+         tc::tc_search_kernel<4, true, false>, tc::tc_search_kernel<5, true, false>}};
+    static const Kernel pair_kernels[2][2] = {
+        {tc::tc_search_kernel<4, false, true>, tc::tc_search_kernel<5, false, true>},
+        {tc::tc_search_kernel<4, true, true>, tc::tc_search_kernel<5, true, true>}};
+    const Kernel kern = pair ? pair_kernels[comb][k - 4] : kernels[comb][k - 2];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, tc::Roles::Threads, smem, st>>>(map, P);
@@ -2032,6 +2476,60 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
     e = encode_map(&map, d, b4, comb_p != 0);
     if (e != cudaSuccess) return e;
     return launch_kernel(map, P, k, grid, st, comb_p != 0);
+}
+
+// The same search with pair tiles (whole range): ws holds tc_pair_bytes of
+// operand, singles and tables.
+cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *b4, const TcPairWork &ws, int pool,
+                                  uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
+                                  int32_t *status, int grid, uint64_t total, cudaStream_t st, float *cand_g,
+                                  uint64_t *rank_g, uint32_t *dump, unsigned long long *waits,
+                                  unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist, TcCollect collect)
+{
+    const bool comb = comb_p != 0;
+    const int kp = k - 2;                       // prefix SNPs: the tiles of an order-(k-1) search
+    const int kj = tc_tile_snps(comb) / 2;
+    uint64_t *cum1 = ws.tables, *pcum = cum1 + d.n + 1, *scum = pcum + d.n + 1, *icum = scum + d.n + 1,
+             *brow = icum + d.n + 1;
+    const uint64_t total1 = host_binom(d.n, k - 1);
+    cudaError_t e = launch_tc_item_cum(d, k - 1, 0, total1, cum1, st, comb);
+    if (e != cudaSuccess) return e;
+    tc::pair_tables_kernel<<<1, 1024, 0, st>>>(d, kp, tc_ppt(k - 1), kj, pcum, scum, icum, brow);
+    tc::build_pairs_kernel<<<dim3(16, (unsigned)(d.n - 1)), 256, 0, st>>>(d, brow, reinterpret_cast<uint4 *>(ws.operand));
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // the single counts: an order-(k-1) pass that stores its accumulators
+    tc::Params P;
+    CUtensorMap map;
+    fill_ds(P.one, d, k - 1, cum1, global_thr, total1, 0, total1, nullptr, 0, grid, comb_p, b4, 0, nullptr);
+    P.one.singles = reinterpret_cast<float4 *>(ws.singles);
+    P.one.scum = scum;
+    P.one.store = 1;
+    P.many = nullptr;
+    P.cta_ds = nullptr;
+    fill_launch(P, k - 1, 32, list_score, list_rank, list_count, status, nullptr, nullptr, cand_g, rank_g, comb);
+    P.wait_ns = wait_ns;
+    e = encode_map(&map, d, b4, comb);
+    if (e == cudaSuccess) e = launch_kernel(map, P, k - 1, grid, st, comb);
+    if (e != cudaSuccess) return e;
+    // the pairs
+    fill_ds(P.one, d, k, icum, global_thr, total, 0, total, nullptr, 0, grid, comb_p, b4, top_n, hist);
+    P.one.singles = reinterpret_cast<float4 *>(ws.singles);
+    P.one.scum = scum;
+    P.one.brow = brow;
+    P.one.pcum = pcum;
+    P.one.s1_hi = (int32_t)(d.n - k + 1);        // the prefixes as the order-(k-1) pass lists them
+    P.one.n_prefix = 0;
+    for (int64_t c = kp - 1; c <= d.n - 2; c++) P.one.n_prefix += host_binom(c, kp - 1);
+    P.one.n_items = 0;
+    for (int64_t j = kp; j <= d.n - 2; j++)
+        P.one.n_items += (host_binom(j, kp) + tc_ppt(k - 1) - 1) / tc_ppt(k - 1) * (uint64_t)tc::panel_ntiles(d.n, j, kj);
+    fill_launch(P, k, pool, list_score, list_rank, list_count, status, dump, waits, cand_g, rank_g, comb, true);
+    P.wait_ns = wait_ns;
+    P.collect = collect;
+    e = encode_map(&map, d, ws.operand, comb, pair_operand_rows(d.n));
+    if (e != cudaSuccess) return e;
+    return launch_kernel(map, P, k, grid, st, comb, true);
 }
 
 size_t tc_ds_bytes() { return sizeof(tc::DsParams); }
