@@ -377,18 +377,22 @@ def measure_mlp_inference(epi, ctx, peaks):
 def class_shift(d):
     """Class shift of the tensor path's combined-class variant, 0 where the
     separate-class variant runs (the rule include/epi.h states for
-    EPI_TC_AUTO)."""
-    m1, m0 = d.n_cases, d.n_samples - d.n_cases
-    p = 1
-    while p < 15 and (1 << p) <= m0:
-        p += 1
-    return p if p <= 14 and m1 * (1 << p) + m0 < (1 << 23) else 0
+    EPI_TC_AUTO): from the largest counts of a genotype-0 or -1 row."""
+    case = d.pheno == 1
+    c1 = max(int((d.geno[:, case] == g).sum(axis=1).max()) for g in (0, 1))
+    c0 = max(int((d.geno[:, ~case] == g).sum(axis=1).max()) for g in (0, 1))
+    p = (c0 + 1).bit_length()
+    return p if c1 * (1 << p) + c0 < (1 << 24) else 0
 
 
 def comb_shift(d, k):
-    """The class shift of the order-3 headline's accumulator (0 at other
-    orders: their results are reported without it)."""
-    return class_shift(d) if k == 3 else 0
+    """A class shift of an order-3 search that the class sizes alone allow
+    with half the accumulator's range (0: none)."""
+    if k != 3:
+        return 0
+    m1, m0 = d.n_cases, d.n_samples - d.n_cases
+    p = max(1, m0.bit_length())
+    return p if p <= 14 and m1 * (1 << p) + m0 < (1 << 23) else 0
 
 
 def tc_executed_flops(d, k):

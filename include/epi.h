@@ -64,10 +64,12 @@ typedef enum {
 
 /* Tensor-core counting variant (epi_set_tc_variant). */
 typedef enum {
-    EPI_TC_AUTO = 0,       /* m1 * 2^p + m0 < 2^23 (2^p the least power of
-                              two above m0, p <= 14): both classes in one
-                              accumulator, 240-column tiles; else separate
-                              case and control accumulators of 160 columns */
+    EPI_TC_AUTO = 0,       /* c1 * 2^p + c0 < 2^24, with c1 and c0 the largest
+                              case and control counts of a genotype-0 or -1
+                              row and 2^p the least power of two above c0 + 1:
+                              both classes in one accumulator, 240-column
+                              tiles; else separate case and control
+                              accumulators of 160 columns */
     EPI_TC_SEPARATE = 1    /* always separate case and control accumulators */
 } epi_tc_variant;
 

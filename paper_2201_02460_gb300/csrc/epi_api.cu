@@ -54,6 +54,7 @@ struct epi_dataset {
     uint64_t id = 0;               // unique within the context (keys cached batch graphs)
     int64_t n = 0, m = 0, m1 = 0, m0 = 0;
     int32_t W1 = 0, W0 = 0, Wt = 0;
+    int32_t c1max = 0, c0max = 0;  // largest case / control count of a genotype-0 or -1 row
     uint32_t *masks = nullptr;
     uint64_t *binom = nullptr;
     unsigned char *b4 = nullptr;   // tensor-core operand, built on first use
@@ -65,6 +66,7 @@ struct epi_dataset {
         d.W1 = W1; d.W0 = W0; d.Wt = Wt;
         d.masks = masks;
         d.binom = binom;
+        d.c1max = c1max; d.c0max = c0max;
         return d;
     }
 };
@@ -1521,7 +1523,8 @@ epi_status epi_dataset_create(epi_ctx *ctx, const uint8_t *geno, const uint8_t *
     // 2 m int32 entries end on an 8-byte boundary
     int64_t *dm1 = reinterpret_cast<int64_t *>(case_idx + 2 * m);
     int32_t *dstatus = reinterpret_cast<int32_t *>(dm1 + 1);
-    CK(cudaMemsetAsync(dstatus, 0, 4, st));
+    // status word, then the largest row counts of the two classes
+    CK(cudaMemsetAsync(dstatus, 0, 12, st));
     launch_scan_pheno(dpheno, m, case_idx, ctrl_idx, dm1, dstatus, st);
     CK(cudaGetLastError());
     int64_t m1 = 0;
@@ -1548,10 +1551,15 @@ epi_status epi_dataset_create(epi_ctx *ctx, const uint8_t *geno, const uint8_t *
         } else {
             launch_pack_masks(dgeno, n, m, case_idx, ctrl_idx, m1, ds->W1, ds->Wt, ds->masks, dstatus, ctx->num_sms, st);
             launch_binom(n, ds->binom, ctx->num_sms, st);
-            ctx->launches += 3;
+            launch_count_max(ds->masks, n, ds->W1, ds->Wt, dstatus + 1, st);
+            ctx->launches += 4;
+            int32_t words[3] = {};
             cudaError_t e = cudaGetLastError();
-            if (e == cudaSuccess) e = cudaMemcpyAsync(&hstatus, dstatus, 4, cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(words, dstatus, 12, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            hstatus = words[0];
+            ds->c1max = words[1];
+            ds->c0max = words[2];
             if (e != cudaSuccess) ret = fail(EPI_ECUDA, "packing failed: %s", cudaGetErrorString(e));
             else if (hstatus & ST_BAD_GENO) ret = fail(EPI_EINVAL, "genotype values must be 0, 1 or 2");
         }

@@ -77,8 +77,7 @@ constexpr int kTileBytes = 128 * kRowBytes;   // one A stage
 
 // Tile shapes of the two variants.
 //   combined classes (C = true): one accumulator per tile holds
-//     ctrl + case 2^p (exact while below 2^23, the decode's range), two of
-//     240 columns in turn;
+//     ctrl + case 2^p (exact while below 2^24), two of 240 columns in turn;
 //   separate classes (C = false): two accumulators per tile, three of 160
 //     columns in rotation (the next tile's case accumulator fills while the
 //     epilogue reads this tile's two).  480 columns either way: the other 32
@@ -511,7 +510,8 @@ __device__ __forceinline__ F2 f2_rcp(F2 s, F2 tiny)
 // individuals its excess over 2 m MI averages 0.2 (order 3, pi = 0.5) to 1.5
 // (order 4, pi = 0.2) while pi lies in [0.2, 0.8], and 2 to 25 at pi = 0.1,
 // so outside that interval the logarithms screen.
-// Per cell it gets e = 2^p (a - pi s) and s; the constants absorb the 2^p.
+// Per cell it gets e = 2^(p-1) (a - pi s) and s; the constants absorb the
+// power of two.
 struct ScreenConst {
     F2 c2, c3, c4, c5a, c5b, tiny;
 };
@@ -678,31 +678,33 @@ __device__ __noinline__ float row_terms_precise(uint32_t a0, uint32_t b0, uint32
 // 2 h and 2 h + 1, columns 4 h + {2, 3} genotype 1.
 template <bool C>
 struct RowScreen {
-    // packed constants
-    F2 m23, neg_m23, neg1, kinv, neg_pi;
+    // packed constants; q = 2^(p-1) (1 with separate classes): cases are held
+    // times q
+    F2 half, neg2, m23, neg_m23, neg1, inv_q, neg_pi;
     ScreenConst sc;
-    F2 S, CT;                  // the row's totals: individuals and cases (times 2^p)
-    uint32_t lo_mask;
-    float kinv1;               // 2^-p
+    F2 S, CT;                  // the row's totals: individuals and cases
+    uint32_t hi_mask;
+    float inv_q1;
 
-    __device__ __forceinline__ void set_row(float cases, float ctrls, float p2)
+    __device__ __forceinline__ void set_row(float cases, float ctrls, float q)
     {
-        const float s = cases + ctrls;
-        S = f2_pack(s, s);
-        CT = f2_pack(cases * p2, cases * p2);
+        S = f2_pack(cases + ctrls, cases + ctrls);
+        CT = f2_pack(cases * q, cases * q);
     }
-    // the two classes of a column pair: individuals s and cases times 2^p
+    // the two classes of a column pair: individuals s and cases ca.  An
+    // accumulator holds v = ctrl + case 2^p < 2^24; v / 2 + 2^23 has the bits
+    // of v / 2 (rounded) in its mantissa, and those from bit p - 1 on are the
+    // cases (the rounding cannot carry into them: ctrl < 2^p - 1).  (Two
+    // products rounded down instead, without the mask: 63.8 instead of 57.7 ms
+    // at order 3, 2000 x 4000.)
     __device__ __forceinline__ void split(uint32_t x0, uint32_t x1, F2 &s, F2 &ca) const
     {
-        // y = 2^23 + v holds v = ctrl + case 2^p in its mantissa; its low p
-        // bits under the exponent of 2^23 are 2^23 + ctrl
-        const F2 y = f2_add(f2_pack(__uint_as_float(x0), __uint_as_float(x1)), m23);
+        const F2 v = f2_pack(__uint_as_float(x0), __uint_as_float(x1));
         float y0, y1;
-        f2_unpack(y, y0, y1);
-        const F2 lo = f2_pack(__uint_as_float((__float_as_uint(y0) & lo_mask) | 0x4B000000u),
-                              __uint_as_float((__float_as_uint(y1) & lo_mask) | 0x4B000000u));
-        ca = f2_fma(lo, neg1, y);
-        s = f2_fma(ca, kinv, f2_add(lo, neg_m23));
+        f2_unpack(f2_fma(v, half, m23), y0, y1);
+        ca = f2_add(f2_pack(__uint_as_float(__float_as_uint(y0) & hi_mask),
+                            __uint_as_float(__float_as_uint(y1) & hi_mask)), neg_m23);
+        s = f2_fma(ca, inv_q, f2_fma(ca, neg2, v));
     }
     __device__ __forceinline__ void pair(const uint32_t *cs, const uint32_t *cn, int h, F2 &s0, F2 &s1, F2 &a0,
                                          F2 &a1) const
@@ -751,12 +753,12 @@ struct RowScreen {
             float x, y, u, v;
             f2_unpack(aa[g], x, y);
             f2_unpack(ss[g], u, v);
-            a[g] = (odd ? y : x) * kinv1;
+            a[g] = (odd ? y : x) * inv_q1;
             b[g] = (odd ? v : u) - a[g];
         }
     }
     // --- pair tiles: U0, U1 this row's counts with j1's genotypes 0 and 1,
-    // V its count with genotype 2 (individuals .s, cases times 2^p .c)
+    // V its count with genotype 2 (individuals .s, cases .c)
     struct Cnt {
         F2 s, c;
     };
@@ -804,29 +806,22 @@ struct RowScreen {
         for (int x = 0; x < 9; x++) acc = cell_bound(f2_fma(n[x].s, neg_pi, n[x].c), n[x].s, sc, acc);
         f2_unpack(acc, v0, v1);
     }
-    // counts of one of the two SNPs' nine cells
-    __device__ __forceinline__ void pair_counts(const uint32_t *cs, const uint32_t *cn, const float4 &a,
-                                                const float4 &b, bool odd, float *ca, float *co) const
+    __device__ __forceinline__ void pair_logs(const uint32_t *cs, const uint32_t *cn, const float4 &a, const float4 &b,
+                                              float &v0, float &v1) const
     {
         Cnt n[9];
         nine(cs, cn, a, b, n);
+        v0 = v1 = 0.0f;
 #pragma unroll
         for (int x = 0; x < 9; x++) {
             float c0, c1, s0, s1;
             f2_unpack(n[x].c, c0, c1);
             f2_unpack(n[x].s, s0, s1);
-            ca[x] = (odd ? c1 : c0) * kinv1;
-            co[x] = (odd ? s1 : s0) - ca[x];
+            c0 *= inv_q1;
+            c1 *= inv_q1;
+            v0 += cell_log(c0, s0 - c0);
+            v1 += cell_log(c1, s1 - c1);
         }
-    }
-    __device__ __forceinline__ float pair_log(const uint32_t *cs, const uint32_t *cn, const float4 &a, const float4 &b,
-                                              bool odd) const
-    {
-        float ca[9], co[9], v = 0.0f;
-        pair_counts(cs, cn, a, b, odd, ca, co);
-#pragma unroll
-        for (int x = 0; x < 9; x++) v += cell_log(ca[x], co[x]);
-        return v;
     }
     // this item's j1: its group's float4s and whether it is the odd SNP
     __device__ __forceinline__ void set_first(const float4 &a, const float4 &b, bool odd)
@@ -848,6 +843,39 @@ struct RowScreen {
         }
     }
 };
+
+// One row's nine cells (3 g1 + g2) of a pair, as counts (the rare paths,
+// kept out of line): raw accumulators of the joint genotypes 00, 01, 10, 11
+// and of j2's single counts (x: the only or the case accumulator, y: the
+// control accumulator), counts of the row with j1's genotypes 0 and 1 and
+// with genotype 2 (c cases, s individuals), 2^-p and 2^p.
+struct PairRow {
+    float x[6], y[6];
+    float c0, s0, c1, s1, c2, s2;
+    float kinv, p2;
+};
+template <bool C>
+__device__ __noinline__ void pair_cells(const PairRow &r, uint32_t *ca, uint32_t *co)
+{
+    float c[6], t[6];                        // cases, controls
+#pragma unroll
+    for (int i = 0; i < 6; i++) {
+        c[i] = C ? floorf(r.x[i] * r.kinv) : r.x[i];
+        t[i] = C ? fmaf(c[i], -r.p2, r.x[i]) : r.y[i];
+    }
+    const float t0 = r.s0 - r.c0, t1 = r.s1 - r.c1, t2 = r.s2 - r.c2;
+    const float cc[9] = {c[0], c[1], r.c0 - c[0] - c[1], c[2], c[3], r.c1 - c[2] - c[3],
+                         c[4] - c[0] - c[2], c[5] - c[1] - c[3],
+                         r.c2 - (c[4] - c[0] - c[2]) - (c[5] - c[1] - c[3])};
+    const float tt[9] = {t[0], t[1], t0 - t[0] - t[1], t[2], t[3], t1 - t[2] - t[3],
+                         t[4] - t[0] - t[2], t[5] - t[1] - t[3],
+                         t2 - (t[4] - t[0] - t[2]) - (t[5] - t[1] - t[3])};
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+        ca[i] = f2u_exact(cc[i]);
+        co[i] = f2u_exact(tt[i]);
+    }
+}
 
 // Lexicographic rank of a combination from the sum over its SNPs s_t of
 // C(n - 1 - s_t, K - t): total - 1 - sum.
@@ -879,6 +907,11 @@ __device__ __forceinline__ void last_snp_range(const DsParams &DS, const DevData
     }
 }
 
+#define TMEM_LD8(taddr, r)                                                                                       \
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"                        \
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) \
+                 : "r"(taddr))
+
 template <int K, bool C, bool PAIR>
 __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                                                 const Params P)
@@ -893,8 +926,10 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
     constexpr int kGroups = R::ProdGroups, kCG = R::ColGroups;
     // epilogue: the kQC chunks of 8 last SNPs of a lane quadrant go round-
     // robin to its kCG warps, kIters chunks each (the last may be empty)
-    // (pair tiles: chunks of 4 last SNPs, 16 columns)
-    constexpr int kCS = PAIR ? 4 : 8;
+    // (pair tiles: chunks of 4 last SNPs, 16 columns; of 2 with separate
+    // classes, whose two accumulators and singles would spill)
+    constexpr int kCS = PAIR ? (C ? 4 : 2) : 8;
+    constexpr int kChunkCols = kCS * kColsPerSnp, kH = kCS / 2;   // columns and groups of two SNPs
     constexpr int kQC = kJ / kCS;
     constexpr int kIters = (kQC + kCG - 1) / kCG;
     constexpr int km1 = PAIR ? K - 2 : K - 1;       // prefix SNPs
@@ -1399,10 +1434,13 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         rs.m23 = f2_pack(8388608.0f, 8388608.0f);
         rs.neg_m23 = f2_pack(-8388608.0f, -8388608.0f);
         rs.neg1 = f2_pack(-1.0f, -1.0f);
-        rs.kinv1 = 1.0f / p2;
-        rs.kinv = f2_pack(rs.kinv1, rs.kinv1);
+        const float q1 = C ? 0.5f * p2 : 1.0f;
+        rs.half = f2_pack(0.5f, 0.5f);
+        rs.neg2 = f2_pack(-2.0f, -2.0f);
+        rs.hi_mask = C ? ~((1u << (DS.comb_p - 1)) - 1u) : 0u;
+        rs.inv_q1 = 1.0f / q1;
+        rs.inv_q = f2_pack(rs.inv_q1, rs.inv_q1);
         rs.neg_pi = f2_pack(-DS.sc_pi, -DS.sc_pi);
-        rs.lo_mask = (1u << DS.comb_p) - 1u;
         rs.sc.c2 = f2_pack(DS.c2, DS.c2);
         rs.sc.c3 = f2_pack(DS.c3, DS.c3);
         rs.sc.c4 = f2_pack(DS.c4, DS.c4);
@@ -1410,7 +1448,10 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         rs.sc.c5b = f2_pack(DS.c5b, DS.c5b);
         rs.sc.tiny = f2_pack(1e-30f, 1e-30f);
         const float vscale = DS.vscale, voff = DS.voff;
-        const bool poly = DS.poly != 0;
+        // (DS lies in the kernel parameters or in global memory: what the
+        // chunk loop needs of it is read once)
+        const bool poly = DS.poly != 0, store = !PAIR && DS.store != 0;
+        float4 *const singles = DS.singles;
         float *wb = wsum + warp * 256;
         int ab = 0;                          // first accumulator buffer of the item
         float thr = ES.thr;                  // the threshold as of the last item's closing barrier
@@ -1468,7 +1509,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     T0 += tot[((b * 128 + r) * kGroups + gq) * 2 + 1];
                 }
                 // rows of no prefix count nothing: their totals are 0
-                rs.set_row(u2f_exact(T1), u2f_exact(T0), p2);
+                rs.set_row(u2f_exact(T1), u2f_exact(T0), q1);
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&tot_empty[b]);
@@ -1487,10 +1528,15 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     ES.stop = abort_flag;
                 }
             };
-            // one chunk's accumulators (queued): last SNPs j0 + 8 jcg ..
+            // one chunk's accumulators (queued): last SNPs j0 + kCS jcg ..
             auto load_chunk = [&](int jcg, uint32_t *cs, uint32_t *cn) {
-                TMEM_LD16(ta_case + (uint32_t)(16 * jcg), cs);
-                if constexpr (!C) TMEM_LD16(ta_ctrl + (uint32_t)(16 * jcg), cn);
+                if constexpr (kChunkCols == 16) {
+                    TMEM_LD16(ta_case + (uint32_t)(16 * jcg), cs);
+                    if constexpr (!C) TMEM_LD16(ta_ctrl + (uint32_t)(16 * jcg), cn);
+                } else {
+                    TMEM_LD8(ta_case + (uint32_t)(8 * jcg), cs);
+                    if constexpr (!C) TMEM_LD8(ta_ctrl + (uint32_t)(8 * jcg), cn);
+                }
             };
             auto release_acc = [&]() {
                 tc_fence_before();
@@ -1573,7 +1619,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             // all prefixes of the warp at once, column by column (one flagged
             // pair at a time, as below, the first items of a CTA took
             // milliseconds at order 2), summed as the flagged ones are.
-            bool cold = thr < 0.0f && !DS.store;
+            bool cold = thr < 0.0f && !store;
             // 8 row values per lane -> transposed sums: the lane of pair
             // (prefix pp, last SNP jj) adds rows pp kPR .. of column jj (all
             // banks distinct); at orders 4-5 four lanes share a column
@@ -1676,25 +1722,26 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 epi_bar<kEpiThreads>();
                 if (tid == 0) ES.any = 0;
             } else if constexpr (PAIR) {
-                // Chunks of 4 last SNPs (16 columns): two groups of two, each
-                // 8 columns and one float4 (two with separate classes) of
-                // single counts per row, loaded one chunk ahead
+                // Chunks of kCS last SNPs: kH groups of two, each 8 columns and
+                // one float4 (two with separate classes) of single counts per
+                // row, loaded one chunk ahead
                 constexpr int kAcc = C ? 1 : 2;
-                const int live_chunks = ok ? min(kQC, ((int32_t)d.n - j0 + 3) >> 2) : 0;
+                const int live_chunks = ok ? min(kQC, ((int32_t)d.n - j0 + kCS - 1) / kCS) : 0;
                 const int mine = (live_chunks - jhalf + kCG - 1) / kCG;
                 const bool row_in = prow && psnp[km1 - 1] < D.j1;
                 // rows outside read one place of the table (their values are dropped)
                 const int32_t base = row_in ? (int32_t)panel_j0(psnp[km1 - 1]) : 0;
-                const float4 *sp = DS.singles + (row_in ? (D.single[p] * kPR + pos) * kAcc : 0);
+                const float4 *sp = singles + (row_in ? (D.single[p] * kPR + pos) * kAcc : 0);
                 const int64_t gstep = row_in ? (int64_t)kPR * kAcc : 0;
                 auto load_singles = [&](int32_t j, float4 *a, float4 *b) {
                     const float4 *q = sp + (int64_t)((j - base) >> 1) * gstep;
-                    a[0] = __ldg(q);
-                    if constexpr (!C) b[0] = __ldg(q + 1);
-                    a[1] = __ldg(q + gstep);
-                    if constexpr (!C) b[1] = __ldg(q + gstep + 1);
+#pragma unroll
+                    for (int h = 0; h < kH; h++) {
+                        a[h] = __ldg(q + h * gstep);
+                        if constexpr (!C) b[h] = __ldg(q + h * gstep + 1);
+                    }
                 };
-                float4 na[2], nb[2];
+                float4 na[kH], nb[kH];
                 {
                     float4 fa, fb;
                     const float4 *q = sp + (int64_t)((D.j1 - base) >> 1) * gstep;
@@ -1703,83 +1750,25 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     if (mine > 0) load_singles(j0 + kCS * jhalf, na, nb);
                     rs.set_first(fa, fb, ((D.j1 - base) & 1) != 0);
                 }
-                if (mine <= 0) release_acc();
-                const int rounds = cold ? kIters : mine;
-#pragma unroll 1
-                for (int jc = 0; jc < rounds; jc++) {
-                    if (cold && jc > 0) {
-                        share_threshold();
-                        cut = thr * DS.cut_mul - DS.cut_add;
-                        cold = thr < 0.0f;
-                    }
-                    if (jc >= mine) continue;
-                    const int jcg = jhalf + kCG * jc;
-                    const int32_t jb = j0 + kCS * jcg;
-                    uint32_t cs[16], cn[C ? 1 : 16];
-                    load_chunk(jcg, cs, cn);
-                    float4 a[2], b[2];
+                // one chunk's screen: the row values of its last SNPs, summed
+                // by prefix; the pairs that pass, as lane masks
+                auto screen_chunk = [&](int32_t jb, const uint32_t *cs, const uint32_t *cn, const float4 *a,
+                                        const float4 *b, uint32_t *cmask) {
 #pragma unroll
-                    for (int h = 0; h < 2; h++) {
-                        a[h] = na[h];
-                        b[h] = C ? na[h] : nb[h];
-                    }
-                    if (jc + 1 < mine) load_singles(jb + kCS * kCG, na, nb);
-                    tmem_wait_ld();
-                    if (jc + 1 == mine) release_acc();
-                    if (P.dump && row_in) {
-#pragma unroll 1
-                        for (int jj = 0; jj < kCS; jj++) {
-                            const int32_t j = jb + jj;
-                            if (j <= D.j1 || j >= (int32_t)d.n) continue;
-                            float ca[9], co[9];
-                            if (jj < 2) rs.pair_counts(cs, cn, a[0], b[0], jj & 1, ca, co);
-                            else rs.pair_counts(cs + 8, cn + (C ? 0 : 8), a[1], b[1], jj & 1, ca, co);
-                            constexpr int cells = kPR * 9;
-                            const uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, psnp, K) -
-                                                  binom_at(d.binom, d.n, d.n - 1 - D.j1, 2) - (uint64_t)(d.n - 1 - j);
-                            uint32_t *o = P.dump + rank * 2 * cells;
-#pragma unroll
-                            for (int x = 0; x < 9; x++) {
-                                o[pos * 9 + x] = f2u_exact(ca[x]);
-                                o[cells + pos * 9 + x] = f2u_exact(co[x]);
-                            }
+                    for (int h = 0; h < kH; h++) {
+                        const uint32_t *hs = cs + 8 * h, *hn = cn + (C ? 0 : 8 * h);
+                        float v0, v1;
+                        if (poly) {
+                            rs.pair_bound(hs, hn, a[h], b[h], v0, v1);
+                        } else {
+                            rs.pair_logs(hs, hn, a[h], b[h], v0, v1);
                         }
+                        // one group after the other: side by side they spill
+                        reinterpret_cast<float2 *>(wb)[lane * kH + h] =
+                            row_in ? make_float2(v0, v1) : make_float2(0.0f, 0.0f);
+                        __syncwarp();
                     }
-                    // precise terms of this row for column jsel
-                    auto precise = [&](int jsel) -> float {
-                        float ca[9], co[9];
-                        if (jsel < 2) rs.pair_counts(cs, cn, a[0], b[0], jsel & 1, ca, co);
-                        else rs.pair_counts(cs + 8, cn + (C ? 0 : 8), a[1], b[1], jsel & 1, ca, co);
-                        float e = 0.0f;
-#pragma unroll
-                        for (int x = 0; x < 9; x += 3)
-                            e += row_terms_precise(f2u_exact(ca[x]), f2u_exact(co[x]), f2u_exact(ca[x + 1]),
-                                                   f2u_exact(co[x + 1]), f2u_exact(ca[x + 2]), f2u_exact(co[x + 2]), mc);
-                        return e;
-                    };
-                    if (cold) {
-#pragma unroll 1
-                        for (int jj = 0; jj < kCS; jj++) {
-                            const float e = seg_sum<kPR>(row_in ? precise(jj) : 0.0f, pos);
-                            if (row_in && pos == 0 && jb + jj > D.j1 && jb + jj < (int32_t)d.n)
-                                keep(__fdiv_rn(e, mc.fm), p, jb + jj);
-                        }
-                        continue;
-                    }
-                    float vrow[4];
-                    if (poly) {
-                        rs.pair_bound(cs, cn, a[0], b[0], vrow[0], vrow[1]);
-                        rs.pair_bound(cs + 8, cn + (C ? 0 : 8), a[1], b[1], vrow[2], vrow[3]);
-                    } else {
-                        vrow[0] = rs.pair_log(cs, cn, a[0], b[0], false);
-                        vrow[1] = rs.pair_log(cs, cn, a[0], b[0], true);
-                        vrow[2] = rs.pair_log(cs + 8, cn + (C ? 0 : 8), a[1], b[1], false);
-                        vrow[3] = rs.pair_log(cs + 8, cn + (C ? 0 : 8), a[1], b[1], true);
-                    }
-                    reinterpret_cast<float4 *>(wb)[lane] = row_in ? make_float4(vrow[0], vrow[1], vrow[2], vrow[3])
-                                                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                     __syncwarp();
-                    uint32_t cmask[kPairIters];
                     if constexpr (kPPW > 1) {
 #pragma unroll
                         for (int q = 0; q < kPairIters; q++) {
@@ -1800,18 +1789,141 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                             cmask[q] = __ballot_sync(0xffffffffu, cand);
                         }
                     } else {
-                        // one prefix: 8 lanes share a column (4 rows each)
+                        // one prefix: 32 / kCS lanes share a column, kCS rows each
                         float v = 0.0f;
 #pragma unroll
-                        for (int rr = 0; rr < 4; rr++) v += wb[((lane >> 2) * 4 + rr) * kCS + (lane & 3)];
-                        v += __shfl_xor_sync(0xffffffffu, v, 4);
-                        v += __shfl_xor_sync(0xffffffffu, v, 8);
-                        v += __shfl_xor_sync(0xffffffffu, v, 16);
-                        const int32_t j = jb + (lane & 3);
-                        cmask[0] = __ballot_sync(0xffffffffu, lane < 4 && j >= plo[0] && j < phi[0] &&
+                        for (int rr = 0; rr < kCS; rr++) v += wb[((lane / kCS) * kCS + rr) * kCS + lane % kCS];
+#pragma unroll
+                        for (int off = kCS; off < 32; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                        const int32_t j = jb + lane % kCS;
+                        cmask[0] = __ballot_sync(0xffffffffu, lane < kCS && j >= plo[0] && j < phi[0] &&
                                                                   fmaf(v, vscale, voff) >= cut);
                     }
                     __syncwarp();
+                };
+                // The chunks' screen; the rare work (precise scores, a search
+                // without a threshold, the validation dump) has a loop of its
+                // own below, which loads its chunks again: in one loop it cost
+                // every chunk registers and reordering (order 3, 2000 x 4000:
+                // 63 ms with all of it inside, 54 without).
+                const bool slow = cold || P.dump;
+                uint32_t todo = 0xffffffffu;
+                if (!slow) {
+                    todo = 0;
+#pragma unroll 1
+                    for (int jc = 0; jc < mine; jc++) {
+                        const int jcg = jhalf + kCG * jc;
+                        const int32_t jb = j0 + kCS * jcg;
+                        uint32_t cs[kChunkCols], cn[C ? 1 : kChunkCols];
+                        load_chunk(jcg, cs, cn);
+                        float4 a[kH], b[kH];
+#pragma unroll
+                        for (int h = 0; h < kH; h++) {
+                            a[h] = na[h];
+                            b[h] = C ? na[h] : nb[h];
+                        }
+                        if (jc + 1 < mine) load_singles(jb + kCS * kCG, na, nb);
+                        tmem_wait_ld();
+                        uint32_t cmask[kPairIters], any = 0;
+                        screen_chunk(jb, cs, cn, a, b, cmask);
+#pragma unroll
+                        for (int q = 0; q < kPairIters; q++) any |= cmask[q];
+                        if (any) todo |= 1u << jc;
+                    }
+                }
+                const int rounds = slow && cold ? kIters : (todo ? mine : 0);
+#pragma unroll 1
+                for (int jc = 0; jc < rounds; jc++) {
+                    if (cold && jc > 0) {
+                        share_threshold();
+                        cut = thr * DS.cut_mul - DS.cut_add;
+                        cold = thr < 0.0f;
+                    }
+                    if (jc >= mine || !(todo >> jc & 1u)) continue;
+                    const int jcg = jhalf + kCG * jc;
+                    const int32_t jb = j0 + kCS * jcg;
+                    uint32_t cs[kChunkCols], cn[C ? 1 : kChunkCols];
+                    load_chunk(jcg, cs, cn);
+                    float4 a[kH], b[kH];
+                    load_singles(jb, a, b);
+                    if constexpr (C) {
+#pragma unroll
+                        for (int h = 0; h < kH; h++) b[h] = a[h];
+                    }
+                    tmem_wait_ld();
+                    // this row's nine cells of column jsel
+                    auto chunk_counts = [&](int jsel, uint32_t *ca, uint32_t *co) {
+                        PairRow pr;
+                        const bool odd = jsel & 1;
+#pragma unroll
+                        for (int h = 0; h < kH; h++) {
+                            if (h != jsel >> 1) continue;
+#pragma unroll
+                            for (int i = 0; i < 4; i++) {
+                                pr.x[i] = __uint_as_float(odd ? cs[8 * h + 2 * i + 1] : cs[8 * h + 2 * i]);
+                                if constexpr (!C)
+                                    pr.y[i] = __uint_as_float(odd ? cn[8 * h + 2 * i + 1] : cn[8 * h + 2 * i]);
+                            }
+                            pr.x[4] = odd ? a[h].y : a[h].x;
+                            pr.x[5] = odd ? a[h].w : a[h].z;
+                            if constexpr (!C) {
+                                pr.y[4] = odd ? b[h].y : b[h].x;
+                                pr.y[5] = odd ? b[h].w : b[h].z;
+                            }
+                        }
+                        float drop;
+                        f2_unpack(rs.U0.c, pr.c0, drop);
+                        f2_unpack(rs.U0.s, pr.s0, drop);
+                        f2_unpack(rs.U1.c, pr.c1, drop);
+                        f2_unpack(rs.U1.s, pr.s1, drop);
+                        f2_unpack(rs.V.c, pr.c2, drop);
+                        f2_unpack(rs.V.s, pr.s2, drop);
+                        pr.c0 *= rs.inv_q1;
+                        pr.c1 *= rs.inv_q1;
+                        pr.c2 *= rs.inv_q1;
+                        pr.kinv = 1.0f / p2;
+                        pr.p2 = p2;
+                        pair_cells<C>(pr, ca, co);
+                    };
+                    if (P.dump && row_in) {
+#pragma unroll 1
+                        for (int jj = 0; jj < kCS; jj++) {
+                            const int32_t j = jb + jj;
+                            if (j <= D.j1 || j >= (int32_t)d.n) continue;
+                            uint32_t ca[9], co[9];
+                            chunk_counts(jj, ca, co);
+                            constexpr int cells = kPR * 9;
+                            const uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, psnp, K) -
+                                                  binom_at(d.binom, d.n, d.n - 1 - D.j1, 2) - (uint64_t)(d.n - 1 - j);
+                            uint32_t *o = P.dump + rank * 2 * cells;
+#pragma unroll
+                            for (int x = 0; x < 9; x++) {
+                                o[pos * 9 + x] = ca[x];
+                                o[cells + pos * 9 + x] = co[x];
+                            }
+                        }
+                    }
+                    // precise terms of this row for column jsel
+                    auto precise = [&](int jsel) -> float {
+                        uint32_t ca[9], co[9];
+                        chunk_counts(jsel, ca, co);
+                        float e = 0.0f;
+#pragma unroll 1
+                        for (int x = 0; x < 9; x += 3)
+                            e += row_terms_precise(ca[x], co[x], ca[x + 1], co[x + 1], ca[x + 2], co[x + 2], mc);
+                        return e;
+                    };
+                    if (cold) {
+#pragma unroll 1
+                        for (int jj = 0; jj < kCS; jj++) {
+                            const float e = seg_sum<kPR>(row_in ? precise(jj) : 0.0f, pos);
+                            if (row_in && pos == 0 && jb + jj > D.j1 && jb + jj < (int32_t)d.n)
+                                keep(__fdiv_rn(e, mc.fm), p, jb + jj);
+                        }
+                        continue;
+                    }
+                    uint32_t cmask[kPairIters];
+                    screen_chunk(jb, cs, cn, a, b, cmask);
 #pragma unroll
                     for (int q = 0; q < kPairIters; q++) {
                         while (cmask[q]) {
@@ -1823,6 +1935,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         }
                     }
                 }
+                release_acc();
                 refresh();
                 epi_bar<kEpiThreads>();
             } else {
@@ -1830,72 +1943,13 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 // SNP below n (all but in the last N tile of a panel)
                 const int live_chunks = ok ? min(kQC, ((int32_t)d.n - j0 + 7) >> 3) : 0;
                 const int mine = (live_chunks - jhalf + kCG - 1) / kCG;
-                uint32_t nx[16], ny[C ? 1 : 16];
-                if (mine > 0) load_chunk(jhalf, nx, ny);
-                else release_acc();
-                // while there is no threshold the warps go chunk by chunk
-                // together, until enough combinations are scored to set one
-                // (kIters rounds for every warp, whatever its item or state: the
-                // rounds meet at barriers)
-                const int rounds = cold ? kIters : mine;
-#pragma unroll 1
-                for (int jc = 0; jc < rounds; jc++) {
-                    if (cold && jc > 0) {
-                        share_threshold();
-                        cut = thr * DS.cut_mul - DS.cut_add;
-                        cold = thr < 0.0f;
-                    }
-                    if (jc >= mine) continue;
-                    const int jcg = jhalf + kCG * jc;
-                    const int32_t jb = j0 + 8 * jcg;
-                    uint32_t cs[16], cn[C ? 1 : 16];
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int q = 0; q < 16; q++) {
-                        cs[q] = nx[q];
-                        if constexpr (!C) cn[q] = ny[q];
-                    }
-                    // the next chunk's accumulators load while this one is
-                    // screened; once every value is in registers the buffer
-                    // goes back to the MMA issuer
-                    if (jc + 1 < mine) load_chunk(jcg + kCG, nx, ny);
-                    else release_acc();
-                    if (P.dump) dump_chunk(jb, cs, cn);
-                    if (DS.store) {
-                        // the raw accumulators of this row, two SNPs at a time
-                        if (prow) {
-                            constexpr int kAcc = C ? 1 : 2;
-                            const int32_t base = (int32_t)panel_j0(psnp[km1 - 1]);
-                            const int32_t top = base + 2 * (int32_t)single_groups(d.n, psnp[km1 - 1]);
-#pragma unroll
-                            for (int h = 0; h < 4; h++) {
-                                const int32_t j = jb + 2 * h;
-                                if (j < base || j >= top) continue;
-                                float4 *o = DS.singles + ((D.single[p] + (uint64_t)((j - base) >> 1)) * kPR + pos) * kAcc;
-                                o[0] = make_float4(__uint_as_float(cs[4 * h]), __uint_as_float(cs[4 * h + 1]),
-                                                   __uint_as_float(cs[4 * h + 2]), __uint_as_float(cs[4 * h + 3]));
-                                if constexpr (!C)
-                                    o[1] = make_float4(__uint_as_float(cn[4 * h]), __uint_as_float(cn[4 * h + 1]),
-                                                       __uint_as_float(cn[4 * h + 2]), __uint_as_float(cn[4 * h + 3]));
-                            }
-                        }
-                        continue;
-                    }
-                    if (cold) {
-                        int32_t jlo = 1, jhi = 0;
-                        if (prow && pos == 0) last_snp_range<km1>(DS, d, psnp, jlo, jhi);
-#pragma unroll 1
-                        for (int jj = 0; jj < 8; jj++) {
-                            const float e = seg_sum<kPR>(prow ? row_precise(cs, cn, jj) : 0.0f, pos);
-                            if (jb + jj >= jlo && jb + jj < jhi) keep(__fdiv_rn(e, mc.fm), p, jb + jj);
-                        }
-                        continue;
-                    }
+                // one chunk's screen: the row values of its last SNPs, summed
+                // by prefix; the pairs that pass, as lane masks
+                auto screen_chunk = [&](int32_t jb, const uint32_t *cs, const uint32_t *cn, uint32_t *cmask) {
                     float vrow[8];
                     if (poly) rs.bound(cs, cn, vrow);
                     else rs.logs(cs, cn, vrow);
                     store_rows(vrow);
-                    uint32_t cmask[kPairIters];
                     if constexpr (kPPW > 1) {
 #pragma unroll
                         for (int q = 0; q < kPairIters; q++) {
@@ -1922,6 +1976,88 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                                                                   fmaf(v, vscale, voff) >= cut);
                     }
                     __syncwarp();
+                };
+                // The chunks' screen, accumulators loaded one chunk ahead; the
+                // rare work (precise scores, a search without a threshold, the
+                // stored single counts, the validation dump) has a loop of its
+                // own below, which loads its chunks again: in one loop it cost
+                // every chunk registers and reordering (order 3, 2000 x 4000:
+                // 63 ms with all of it inside, 54 without).
+                const bool slow = cold || store || P.dump;
+                uint32_t todo = 0xffffffffu;
+                if (!slow) {
+                    todo = 0;
+                    uint32_t nx[16], ny[C ? 1 : 16];
+                    if (mine > 0) load_chunk(jhalf, nx, ny);
+#pragma unroll 1
+                    for (int jc = 0; jc < mine; jc++) {
+                        const int jcg = jhalf + kCG * jc;
+                        uint32_t cs[16], cn[C ? 1 : 16];
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int q = 0; q < 16; q++) {
+                            cs[q] = nx[q];
+                            if constexpr (!C) cn[q] = ny[q];
+                        }
+                        if (jc + 1 < mine) load_chunk(jcg + kCG, nx, ny);
+                        uint32_t cmask[kPairIters], any = 0;
+                        screen_chunk(j0 + 8 * jcg, cs, cn, cmask);
+#pragma unroll
+                        for (int q = 0; q < kPairIters; q++) any |= cmask[q];
+                        if (any) todo |= 1u << jc;
+                    }
+                }
+                // while there is no threshold the warps go chunk by chunk
+                // together, until enough combinations are scored to set one
+                // (kIters rounds for every warp, whatever its item or state:
+                // the rounds meet at barriers)
+                const int rounds = slow && cold ? kIters : (todo ? mine : 0);
+#pragma unroll 1
+                for (int jc = 0; jc < rounds; jc++) {
+                    if (cold && jc > 0) {
+                        share_threshold();
+                        cut = thr * DS.cut_mul - DS.cut_add;
+                        cold = thr < 0.0f;
+                    }
+                    if (jc >= mine || !(todo >> jc & 1u)) continue;
+                    const int jcg = jhalf + kCG * jc;
+                    const int32_t jb = j0 + 8 * jcg;
+                    uint32_t cs[16], cn[C ? 1 : 16];
+                    load_chunk(jcg, cs, cn);
+                    tmem_wait_ld();
+                    if (P.dump) dump_chunk(jb, cs, cn);
+                    if (store) {
+                        // the raw accumulators of this row, two SNPs at a time
+                        if (prow) {
+                            constexpr int kAcc = C ? 1 : 2;
+                            const int32_t base = (int32_t)panel_j0(psnp[km1 - 1]);
+                            const int32_t top = base + 2 * (int32_t)single_groups(d.n, psnp[km1 - 1]);
+#pragma unroll
+                            for (int h = 0; h < 4; h++) {
+                                const int32_t j = jb + 2 * h;
+                                if (j < base || j >= top) continue;
+                                float4 *o = singles + ((D.single[p] + (uint64_t)((j - base) >> 1)) * kPR + pos) * kAcc;
+                                o[0] = make_float4(__uint_as_float(cs[4 * h]), __uint_as_float(cs[4 * h + 1]),
+                                                   __uint_as_float(cs[4 * h + 2]), __uint_as_float(cs[4 * h + 3]));
+                                if constexpr (!C)
+                                    o[1] = make_float4(__uint_as_float(cn[4 * h]), __uint_as_float(cn[4 * h + 1]),
+                                                       __uint_as_float(cn[4 * h + 2]), __uint_as_float(cn[4 * h + 3]));
+                            }
+                        }
+                        continue;
+                    }
+                    if (cold) {
+                        int32_t jlo = 1, jhi = 0;
+                        if (prow && pos == 0) last_snp_range<km1>(DS, d, psnp, jlo, jhi);
+#pragma unroll 1
+                        for (int jj = 0; jj < 8; jj++) {
+                            const float e = seg_sum<kPR>(prow ? row_precise(cs, cn, jj) : 0.0f, pos);
+                            if (jb + jj >= jlo && jb + jj < jhi) keep(__fdiv_rn(e, mc.fm), p, jb + jj);
+                        }
+                        continue;
+                    }
+                    uint32_t cmask[kPairIters];
+                    screen_chunk(jb, cs, cn, cmask);
                     // precise single-precision scores of the flagged pairs
                     // (rare): the prefix's row lanes score their rows of that
                     // column, the prefix's first row lane adds them up
@@ -1938,6 +2074,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         }
                     }
                 }
+                release_acc();
                 refresh();
                 epi_bar<kEpiThreads>();
             }
@@ -2174,16 +2311,15 @@ cudaError_t launch_build_b4(const DevData &d, unsigned char *b4, int num_sms, cu
 }
 
 // Class shift p of the combined-class variant for a search of d, or 0 where
-// the separate-class variant runs: the control count must fit below 2^p and
-// the accumulator value ctrl + case 2^p below 2^23 (the decode's exact range;
-// FP32 accumulation of such integers is exact).
+// the separate-class variant runs: with c1 and c0 the largest case and control
+// counts of a genotype-0 or -1 row (no accumulator exceeds them), c0 must lie
+// below 2^p - 1 and ctrl + case 2^p below 2^24, where FP32 accumulation of such
+// integers and the decode are exact.
 int tc_comb_shift(const DevData &d)
 {
     int p = 1;
-    while (p < 15 && (1ll << p) <= d.m0) p++;
-    if (p > 14) return 0;
-    if (d.m1 * (1ll << p) + d.m0 >= (1ll << 23)) return 0;
-    return p;
+    while (p < 24 && (1ll << p) <= (int64_t)d.c0max + 1) p++;
+    return (int64_t)d.c1max * (1ll << p) + d.c0max < (1ll << 24) ? p : 0;
 }
 
 #ifndef EPI_TC_PAIR_MIN_N
@@ -2314,7 +2450,7 @@ static void fill_screen(tc::DsParams &D, const DevData &d, int k, int comb_p)
 {
     const double u = 5.9604644775390625e-8, m = (double)d.m;
     const double pi = (double)d.m1 / m;
-    const double p2 = (double)(1 << comb_p);
+    const double q2 = comb_p ? (double)(1 << (comb_p - 1)) : 1.0;   // e's factor
     D.poly = pi >= 0.2 && pi <= 0.8;
     if (!D.poly) {
         // fast logarithms: m MI / ln 2 = T(m) - T(m1) - T(m0) + sum over cells
@@ -2329,7 +2465,7 @@ static void fill_screen(tc::DsParams &D, const DevData &d, int k, int comb_p)
         D.cut_mul = 1.0f;
         D.cut_add = (float)(2.0 * (4.0 * 4.76837158203125e-7 + (double)(2 * cells + 40) * u) * mag *
                             0.6931471805599453 / m) + 1e-7f;
-        D.sc_pi = (float)(pi * p2);
+        D.sc_pi = (float)(pi * q2);
         D.c2 = D.c3 = D.c4 = D.c5a = D.c5b = 0.0f;
         return;
     }
@@ -2341,13 +2477,13 @@ static void fill_screen(tc::DsParams &D, const DevData &d, int k, int comb_p)
     const double g1 = (-log(pi) - c2 * q * q - c3 * q * q * q) / (q * q * q * q);
     const double slope_n = (g0 - gm) / pi, slope_p = (g1 - gm) / q;   // of g against |x|
     const double c5a = 0.5 * (slope_p - slope_n), c5b = 0.5 * (slope_p + slope_n);
-    D.sc_pi = (float)(pi * p2);
+    D.sc_pi = (float)(pi * q2);
     D.c2 = (float)c2;
-    D.c3 = (float)(c3 / p2);
-    D.c4 = (float)(gm / (p2 * p2));
-    D.c5a = (float)(c5a / (p2 * p2 * p2));
-    D.c5b = (float)(c5b / (p2 * p2 * p2));
-    D.vscale = (float)(1.0 / (p2 * p2 * m));
+    D.c3 = (float)(c3 / q2);
+    D.c4 = (float)(gm / (q2 * q2));
+    D.c5a = (float)(c5a / (q2 * q2 * q2));
+    D.c5b = (float)(c5b / (q2 * q2 * q2));
+    D.vscale = (float)(1.0 / (q2 * q2 * m));
     D.voff = 0.0f;
     // Rounding (u = 2^-24).  e: at most 2 u of the cell's individuals (pi and
     // the fused product), so 2 u m over all cells, times the bound's slope; x: the
