@@ -601,6 +601,7 @@ struct BatchItem {
     int k = 0, top_n = 0, pool = 0, cells = 0;
     bool tc = false;
     int comb_p = 0;                // tensor path: class shift, 0 = separate classes
+    bool alone = false;            // pair tiles: a search of its own, after the batch's launches
     uint64_t total = 0;
     double cost = 0;
     int group = -1, cta_begin = 0, cta_count = 0;
@@ -735,6 +736,7 @@ epi_status record_batch(epi_ctx *ctx, std::vector<BatchItem> &items, std::vector
         ctx->launches += 1;
     }
     for (auto &it : items) {
+        if (it.alone) continue;
         const BatchGroup &g = groups[it.group];
         const DevData d = it.ds->dev();
         float *ls = reinterpret_cast<float *>(dev + g.o_ls) + (size_t)it.cta_begin * g.pool;
@@ -792,6 +794,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         if (st != EPI_OK) return fail(st, "dataset %d: %s", i, epi_last_error());
         const DevData d = it.ds->dev();
         if (it.tc) it.comb_p = plan_comb_shift(it.ds);
+        it.alone = it.tc && tc_pair_applies(d, it.k, it.comb_p != 0);
         // work estimate for the CTA split: a tensor-core item costs its
         // 128-individual chunks, but never less than its epilogue (about 32
         // chunks' worth)
@@ -803,6 +806,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
     // one group per (path, order, tensor variant)
     std::vector<BatchGroup> groups;
     for (int i = 0; i < n_ds; i++) {
+        if (items[i].alone) continue;
         int gi = -1;
         for (size_t q = 0; q < groups.size(); q++)
             if (groups[q].tc == items[i].tc && groups[q].k == items[i].k &&
@@ -838,7 +842,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
     }
     // score histograms next, zeroed with them
     for (auto &it : items)
-        if (it.tc) it.o_hist = a.take<uint32_t>(kTcHistBins);
+        if (it.tc && !it.alone) it.o_hist = a.take<uint32_t>(kTcHistBins);
     const size_t zero_bytes = a.off;
     for (auto &g : groups) {
         g.o_desc = a.take<char>((g.tc ? tc_ds_bytes() : popc_ds_bytes()) * g.items.size());
@@ -853,6 +857,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         }
     }
     for (auto &it : items) {
+        if (it.alone) continue;
         it.o_cs = a.take<float>((size_t)it.pool);
         it.o_cr = a.take<uint64_t>((size_t)it.pool);
         it.o_cn = a.take<int32_t>(1);
@@ -865,6 +870,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
     }
     size_t hoff = 0;
     for (auto &it : items) {
+        if (it.alone) continue;
         it.h_rec = hoff; hoff = align_up(hoff + (size_t)it.top_n * sizeof(epi_result), 64);
         it.h_cnt = hoff; hoff = align_up(hoff + (size_t)it.top_n * 2 * it.cells * 4, 64);
         it.h_nout = hoff; hoff += 64;
@@ -877,7 +883,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
     epi_status st = ensure_batch_buffers(ctx, a.off, hdesc + 256);
     if (st != EPI_OK) return st;
     for (auto &it : items)
-        if (it.tc) {
+        if (it.tc && !it.alone) {
             st = ensure_b4(it.ds);
             if (st != EPI_OK) return st;
         }
@@ -890,7 +896,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
     }
     char *dev = static_cast<char *>(ctx->batch_dev);
     char *host = static_cast<char *>(ctx->batch_host);
-    if (!ctx->batch_exec || key != ctx->batch_key) {
+    if (!groups.empty() && (!ctx->batch_exec || key != ctx->batch_key)) {
         if (ctx->batch_exec) { cudaGraphExecDestroy(ctx->batch_exec); ctx->batch_exec = nullptr; }
         // descriptor tables, built once per graph
         size_t hp = hoff;
@@ -930,10 +936,20 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         if (ec != cudaSuccess) { ctx->batch_exec = nullptr; return fail(EPI_ECUDA, "graph instantiate: %s", cudaGetErrorString(ec)); }
         ctx->batch_key = key;
     }
-    CK(cudaGraphLaunch(ctx->batch_exec, ctx->stream));
+    if (!groups.empty()) CK(cudaGraphLaunch(ctx->batch_exec, ctx->stream));
+    // large order-4 and -5 studies fill the GPU by themselves and count with
+    // pair tiles (their work space belongs to one search at a time)
+    for (int i = 0; i < n_ds; i++) {
+        BatchItem &it = items[i];
+        if (!it.alone) continue;
+        st = run_search_sync(it.ds, it.k, it.top_n, EPI_PATH_TC, 0, it.total, outs[i], counts ? counts[i] : nullptr,
+                             &n_outs[i]);
+        if (st != EPI_OK) return fail(st, "dataset %d: %s", i, std::string(epi_last_error()).c_str());
+    }
     CK(cudaStreamSynchronize(ctx->stream));
     for (int i = 0; i < n_ds; i++) {
         BatchItem &it = items[i];
+        if (it.alone) continue;
         const int32_t code = *reinterpret_cast<int32_t *>(host + it.h_code);
         if (code == EPI_EOVERFLOW) {
             // ties at the pool boundary: this dataset alone, with the retrying search

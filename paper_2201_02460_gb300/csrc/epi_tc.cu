@@ -114,7 +114,7 @@ struct Roles {
 };
 // A producers' load distance in own stages
 #ifndef EPI_TC_PREFETCH
-#define EPI_TC_PREFETCH 3
+#define EPI_TC_PREFETCH 4
 #endif
 constexpr int kDescDepth = 4;
 constexpr int kWaitSlots = 8;
@@ -1116,14 +1116,12 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 }
             };
             fill_tile();
-            uint64_t g = 0;
-            int s = 0;
-            uint32_t ph = 0;
-            long long w_tma = 0;
-            for (int64_t i = 0; i < n_my; i++) {
+            // item i's descriptor, and the operand row its N tile starts at
+            int y_next = 0;
+            auto write_desc = [&](int64_t i) -> bool {
                 const int dq = (int)(i % kDescDepth);
                 const uint32_t ud = (uint32_t)(i / kDescDepth);
-                if (!__all_sync(0xffffffffu, mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag))) break;
+                if (!__all_sync(0xffffffffu, mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag))) return false;
                 const int32_t tile_j0 = (int32_t)panel_j0(PAIR ? j1 : cmin) + (int32_t)(u * kJ);
                 if (DS.singles) {
                     if (lane < kPPT) desc[dq].single[lane] = single[0];
@@ -1143,24 +1141,17 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     item_idesc[dq] = make_idesc(ncol);
                     mbar_arrive(&desc_full[dq]);
                 }
-                const int y = PAIR ? row0 + (int)(u * S::N) : 2 * tile_j0;
-                for (int kc = 0; kc < nst; kc++, g++) {
-                    if (!__all_sync(0xffffffffu, wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_tma))) break;
-                    if (lane == 0) {
-                        mbar_arrive_tx(&full_ab[s], (uint32_t)kBBytes);
-                        tma_load_2d(stages_b + s * kBBytes, tmap, kc * kRowBytes, y, &full_ab[s]);
-                    }
-                    __syncwarp();
-                    if (++s == kStages) { s = 0; ph ^= 1; }
+                y_next = PAIR ? row0 + (int)(u * S::N) : 2 * tile_j0;
+                return true;
+            };
+            // the tile after this one (there is one)
+            auto next_tile = [&]() {
+                if (--seg_left == 0) {
+                    next_segment();
+                    fill_tile();
+                    return;
                 }
                 if constexpr (PAIR) {
-                    if (--seg_left == 0) {
-                        if (i + 1 < n_my) {
-                            next_segment();
-                            fill_tile();
-                        }
-                        continue;
-                    }
                     if (++mt == mtiles) {
                         // next N tile of j1, or the first of the next SNP:
                         // from the first prefix again
@@ -1177,17 +1168,34 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         for (int t = 0; t < km1 - 1; t++) it.a[t] = t;
                     }
                     fill_tile();
-                    continue;
-                }
-                u++;
-                if (--seg_left == 0) {
-                    if (i + 1 < n_my) {
-                        next_segment();
-                        fill_tile();
-                    }
-                } else if (u == panel_ntiles(d.n, cmin, kJ)) {
+                } else if (++u == panel_ntiles(d.n, cmin, kJ)) {
                     u = 0;
                     fill_tile();
+                }
+            };
+            uint64_t g = 0;
+            int s = 0;
+            uint32_t ph = 0;
+            long long w_tma = 0;
+            bool on = write_desc(0);
+            for (int64_t i = 0; i < n_my && on; i++) {
+                const int y = y_next;
+                // the next item's descriptor before this one's loads, which
+                // wait for the ring: its producers start without a gap (the
+                // descriptor written after them: 48.5 ms at order 3,
+                // 2000 x 4000)
+                if (i + 1 < n_my) {
+                    next_tile();
+                    on = write_desc(i + 1);
+                }
+                for (int kc = 0; kc < nst; kc++, g++) {
+                    if (!__all_sync(0xffffffffu, wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_tma))) { on = false; break; }
+                    if (lane == 0) {
+                        mbar_arrive_tx(&full_ab[s], (uint32_t)kBBytes);
+                        tma_load_2d(stages_b + s * kBBytes, tmap, kc * kRowBytes, y, &full_ab[s]);
+                    }
+                    __syncwarp();
+                    if (++s == kStages) { s = 0; ph ^= 1; }
                 }
             }
             if (P.waits && lane == 0) P.waits[blockIdx.x * kWaitSlots + 6] = (unsigned long long)w_tma;
@@ -1357,7 +1365,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             // where it exists, 2 st + 1), kept as loaded and ANDed when their
             // stage is produced, so no instruction waits for a load issued for
             // a later stage
-            constexpr int kPf = K <= 4 ? EPI_TC_PREFETCH : 1;
+            constexpr int kPf = km1 <= 2 ? EPI_TC_PREFETCH : 2;
+            static_assert(kPf % 2 == 0, "stages are produced in twos");
             uint4 ring[kPf][2][km1];
             auto fetch = [&](int st, uint4 (*dst)[km1]) {
 #pragma unroll
@@ -1370,40 +1379,61 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             const uint64_t gs = g + (uint64_t)st0;             // global stage of the first own stage
             int s = (int)(gs % kStages);
             uint32_t ph = (uint32_t)((gs / kStages) & 1);
+            // one stage of this row from its words
+            auto produce = [&](int st, int slot, const uint4 (*w)[km1]) {
+                const uint32_t arow = arow0 + (uint32_t)(slot * kTileBytes);
+#pragma unroll
+                for (int hh = 0; hh < 2; hh++) {
+                    uint4 cur = w[hh][0];
+#pragma unroll
+                    for (int tt = 1; tt < km1; tt++) {
+                        const uint4 v = w[hh][tt];
+                        cur.x &= v.x; cur.y &= v.y; cur.z &= v.z; cur.w &= v.w;
+                    }
+                    const uint32_t wv4[4] = {cur.x, cur.y, cur.z, cur.w};
+                    const uint32_t c4 = __popc(wv4[0]) + __popc(wv4[1]) + __popc(wv4[2]) + __popc(wv4[3]);
+                    t1 += 2 * st + hh < chunks_case ? c4 : 0u;
+                    ta += c4;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        // output word i = bit i of every nibble of the mask word
+                        const uint32_t wv = wv4[q];
+                        st_shared_v4(arow ^ (uint32_t)((4 * hh + q) << 4), wv & 0x11111111u, wv & 0x22222222u,
+                                     wv & 0x44444444u, (wv >> 1) & 0x44444444u);
+                    }
+                }
+            };
+            // Two own stages at a time: the barrier tests, the proxy fence and
+            // the arrivals wait for shared memory (about 400 of 930 cycles a
+            // stage taken one by one, at order 4)
             for (int sb = st0; sb < nst && ok; sb += kGroups * kPf) {
 #pragma unroll
-                for (int u = 0; u < kPf; u++) {
+                for (int u = 0; u < kPf; u += 2) {
                     const int st = sb + kGroups * u;
                     if (st >= nst) break;
-                    const uint32_t arow = arow0 + (uint32_t)(s * kTileBytes);
-                    if (!wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_prod)) { ok = false; break; }
-#pragma unroll
-                    for (int hh = 0; hh < 2; hh++) {
-                        uint4 cur = ring[u][hh][0];
-#pragma unroll
-                        for (int tt = 1; tt < km1; tt++) {
-                            const uint4 v = ring[u][hh][tt];
-                            cur.x &= v.x; cur.y &= v.y; cur.z &= v.z; cur.w &= v.w;
-                        }
-                        const uint32_t wv4[4] = {cur.x, cur.y, cur.z, cur.w};
-                        const uint32_t c4 = __popc(wv4[0]) + __popc(wv4[1]) + __popc(wv4[2]) + __popc(wv4[3]);
-                        t1 += 2 * st + hh < chunks_case ? c4 : 0u;
-                        ta += c4;
-#pragma unroll
-                        for (int q = 0; q < 4; q++) {
-                            // output word i = bit i of every nibble of the mask word
-                            const uint32_t wv = wv4[q];
-                            st_shared_v4(arow ^ (uint32_t)((4 * hh + q) << 4), wv & 0x11111111u, wv & 0x22222222u,
-                                         wv & 0x44444444u, (wv >> 1) & 0x44444444u);
-                        }
+                    const bool two = st + kGroups < nst;
+                    int s2 = s + kGroups;
+                    uint32_t ph2 = ph;
+                    if (s2 >= kStages) { s2 -= kStages; ph2 ^= 1; }
+                    if (!wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_prod) ||
+                        (two && !wait_here(&empty_ab[s2], ph2 ^ 1, &abort_flag, w_prod))) {
+                        ok = false;
+                        break;
                     }
+                    produce(st, s, ring[u]);
+                    if (two) produce(st + kGroups, s2, ring[u + 1]);
                     fetch(st + kGroups * kPf, ring[u]);
+                    fetch(st + kGroups * (kPf + 1), ring[u + 1]);
                     fence_proxy_async();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(&full_ab[s]);
-                    // next own stage: kGroups global stages on
-                    s += kGroups;
-                    if (s >= kStages) { s -= kStages; ph ^= 1; }
+                    if (lane == 0) {
+                        mbar_arrive(&full_ab[s]);
+                        if (two) mbar_arrive(&full_ab[s2]);
+                    }
+                    // the next own stage: kGroups global stages on from the last
+                    s = two ? s2 + kGroups : s2;
+                    ph = ph2;
+                    if (two && s >= kStages) { s -= kStages; ph ^= 1; }
                 }
             }
             if (!ok) break;
@@ -2322,9 +2352,6 @@ int tc_comb_shift(const DevData &d)
     return (int64_t)d.c1max * (1ll << p) + d.c0max < (1ll << 24) ? p : 0;
 }
 
-#ifndef EPI_TC_PAIR_MIN_N
-#define EPI_TC_PAIR_MIN_N 32
-#endif
 static int tc_tile_snps(bool comb) { return comb ? tc::Shape<true>::J : tc::Shape<false>::J; }
 static int tc_pr(int k) { return k == 2 ? 3 : (k == 3 ? 9 : (k == 4 ? 27 : 81)); }
 static int tc_ppt(int k) { return tc_pr(k) > 32 ? 1 : 4 * (32 / tc_pr(k)); }
@@ -2412,10 +2439,13 @@ TcPairBytes tc_pair_bytes(const DevData &d, int k, bool comb)
 }
 
 // Whether a whole order-k search takes pair tiles: orders 4 and 5 on enough
-// SNPs, with the operand and the single counts within 16 GiB.
+// SNPs, with the operand and the single counts within 16 GiB.  The passes
+// before the search cost about 30 us (order 4 with and without pairs, 2500
+// individuals: 33 SNPs 207 and 191 us, 40 SNPs 214 and 263, 130 SNPs 1.8 and
+// 2.7 ms; order 5: 33 SNPs 0.58 and 2.7 ms, 60 SNPs 4.0 and 12.1).
 bool tc_pair_applies(const DevData &d, int k, bool comb)
 {
-    if ((k != 4 && k != 5) || d.n < EPI_TC_PAIR_MIN_N || d.n > 16384) return false;
+    if ((k != 4 && k != 5) || d.n < (k == 4 ? 40 : 24) || d.n > 16384) return false;
     const TcPairBytes b = tc_pair_bytes(d, k, comb);
     return b.operand + b.singles <= ((size_t)16 << 30);
 }
