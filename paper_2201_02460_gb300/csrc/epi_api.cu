@@ -1322,6 +1322,36 @@ epi_status epi_score_all(epi_dataset *ds, int order, float *out_dev)
     if (!g.ok) return fail(EPI_ECUDA, "cannot select device %d", ctx->device);
     if (!out_dev || !is_device_ptr(out_dev, ctx->device))
         return fail(EPI_EINVAL, "epi_score_all: out must be device memory of device %d", ctx->device);
+    const int comb_p = plan_comb_shift(ds);
+    if ((order == 3 || order == 4) && tc_applicable(ds, order, 0, total, total) &&
+        tc_scores_smem_bytes(ds->dev(), comb_p != 0) <= tc_smem_limit(ctx)) {
+        // the tensor path's counts, scored from a table of n ln n
+        Arena a;
+        const int grid = ctx->num_sms;
+        const size_t o_thr = a.take<uint32_t>(1);
+        const size_t o_status = a.take<int32_t>(1);
+        const size_t o_lc = a.take<int32_t>((size_t)grid);
+        const size_t o_ic = a.take<uint64_t>(2 * ((size_t)ds->n + 1));
+        const size_t o_tl = a.take<long long>((size_t)ds->m + 1);
+        st = ensure_scratch(ctx, a.off);
+        if (st != EPI_OK) return st;
+        st = ensure_b4(ds);
+        if (st != EPI_OK) return st;
+        char *base = static_cast<char *>(ctx->scratch);
+        CK(cudaMemsetAsync(base, 0, 512, ctx->stream));
+        CK(launch_tc_scores(ds->dev(), order, ds->b4, reinterpret_cast<uint64_t *>(base + o_ic),
+                            reinterpret_cast<long long *>(base + o_tl), out_dev,
+                            reinterpret_cast<uint32_t *>(base + o_thr), reinterpret_cast<int32_t *>(base + o_lc),
+                            reinterpret_cast<int32_t *>(base + o_status), grid, total, ctx->stream,
+                            ctx->wait_limit_ns, comb_p));
+        ctx->launches += 3;
+        int32_t bits = 0;
+        CK(cudaMemcpyAsync(&bits, base + o_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
+        CK(cudaStreamSynchronize(ctx->stream));
+        if (bits & ST_TIMEOUT) return fail(EPI_ETIMEOUT, "device wait expired");
+        if (bits) return fail(EPI_ECUDA, "device status 0x%x", bits);
+        return EPI_OK;
+    }
     SearchPlan p;
     p.k = order; p.top_n = 1; p.pool = initial_pool(1); p.rb = 0; p.re = total; p.total = total;
     p.all_scores = out_dev;

@@ -116,6 +116,12 @@ cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *
                                   int32_t *status, int grid, uint64_t total, cudaStream_t st, float *cand_g,
                                   uint64_t *rank_g, uint32_t *dump, unsigned long long *waits,
                                   unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist, TcCollect collect);
+// Every score of an order-3 or -4 dataset by rank (tlog: device [m + 1] work
+// space), where the shared memory suffices
+size_t tc_scores_smem_bytes(const DevData &d, bool comb);
+cudaError_t launch_tc_scores(const DevData &d, int k, const unsigned char *b4, uint64_t *item_cum, long long *tlog,
+                             float *scores, uint32_t *global_thr, int32_t *list_count, int32_t *status, int grid,
+                             uint64_t total, cudaStream_t st, unsigned long long wait_ns, int comb_p);
 constexpr int kTcWaitSlots = 8;
 // batched tensor-core launches: per-dataset descriptors and B-operand maps
 // (128-byte CUtensorMap, 64-byte aligned) live in device memory

@@ -179,6 +179,8 @@ struct Params {
     uint64_t *list_rank;
     int32_t *list_count;
     int32_t *status;
+    float *scores;                // orders 3-4: every combination's score, by rank (nothing is kept)
+    const long long *tlog;        // with scores: n ln n 2^46 for n = 0 .. m, rounded
     TcCollect collect;            // ranks != NULL: every combination at or above its threshold instead of the best
     unsigned long long wait_ns;   // limit of the pipeline waits (0: kTimeoutNs)
     uint32_t *dump;            // optional: every table, [rank][2][3^k] (validation)
@@ -955,6 +957,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
     float *wsum = reinterpret_cast<float *>(stages_b + kStages * kBBytes);
     uint32_t *tot = reinterpret_cast<uint32_t *>(wsum + kEpiWarps * 256);   // [2][128][kGroups][2 classes]
     Desc *desc = reinterpret_cast<Desc *>(tot + 2 * 128 * kGroups * 2);
+    // (or, when every score is wanted, the n ln n table: nothing is kept then)
+    long long *tlog = reinterpret_cast<long long *>(desc + kDescDepth);
     float *sc;
     uint64_t *rk;
     if (P.cand_score_g) {
@@ -1030,6 +1034,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    if (P.scores)
+        for (int q = tid; q <= (int)d.m; q += R::Threads) tlog[q] = P.tlog[q];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1481,6 +1487,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         // (DS lies in the kernel parameters or in global memory: what the
         // chunk loop needs of it is read once)
         const bool poly = DS.poly != 0, store = !PAIR && DS.store != 0;
+        const bool scoring = !PAIR && (K == 3 || K == 4) && P.scores;
         float4 *const singles = DS.singles;
         float *wb = wsum + warp * 256;
         int ab = 0;                          // first accumulator buffer of the item
@@ -1649,7 +1656,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             // all prefixes of the warp at once, column by column (one flagged
             // pair at a time, as below, the first items of a CTA took
             // milliseconds at order 2), summed as the flagged ones are.
-            bool cold = thr < 0.0f && !store;
+            bool cold = thr < 0.0f && !store && !scoring;
             // 8 row values per lane -> transposed sums: the lane of pair
             // (prefix pp, last SNP jj) adds rows pp kPR .. of column jj (all
             // banks distinct); at orders 4-5 four lanes share a column
@@ -2007,13 +2014,73 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     }
                     __syncwarp();
                 };
+                // Every score of a chunk: m MI = T(m) - T(m1) - T(m0) + sum over
+                // cells of T(a) + T(b) - T(a + b), T(c) = c ln c from a table
+                // in shared memory as integers of 2^-46, so the sum is exact
+                // and the score's error is the two roundings to float (the
+                // popcount path's per-term series takes ten times the
+                // instructions: order 4, 200 x 2000, 177 ms)
+                auto score_chunk = [&](int32_t jb, const uint32_t *cs, const uint32_t *cn) {
+                    long long *w64 = reinterpret_cast<long long *>(wb);
+                    const int pp = kPPW > 1 ? lane >> 2 : 0;
+                    const int pt = quad * kPPW + pp;
+                    const bool sums = kPPW > 1 ? pp < kPPW && pt < D.nvalid : lane < 4 && pt < D.nvalid;
+                    int64_t rank0 = 0;
+                    int32_t c = 0x7fffffff;
+                    if (sums) {
+                        int32_t qs[km1];
+#pragma unroll
+                        for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
+                        rank0 = (int64_t)(DS.total - prefix_rank_sum<km1>(d, qs)) - d.n;
+                        c = qs[km1 - 1];
+                    }
+                    const long long all = tlog[d.m] - tlog[d.m1] - tlog[d.m0];
+#pragma unroll
+                    for (int half = 0; half < 2; half++) {
+                        long long v[4];
+#pragma unroll
+                        for (int e = 0; e < 4; e++) {
+                            float a[3], bb[3];
+                            rs.counts(cs, cn, 2 * half + (e >> 1), e & 1, a, bb);
+                            long long t = 0;
+#pragma unroll
+                            for (int g3 = 0; g3 < 3; g3++) {
+                                const uint32_t ia = f2u_exact(a[g3]), ib = f2u_exact(bb[g3]);
+                                t += tlog[ia] + tlog[ib] - tlog[ia + ib];
+                            }
+                            v[e] = prow ? t : 0;
+                        }
+                        reinterpret_cast<longlong2 *>(w64)[lane * 2] = make_longlong2(v[0], v[1]);
+                        reinterpret_cast<longlong2 *>(w64)[lane * 2 + 1] = make_longlong2(v[2], v[3]);
+                        __syncwarp();
+                        long long sum = 0;
+                        if constexpr (kPPW > 1) {
+                            if (sums) {
+#pragma unroll
+                                for (int rr = 0; rr < kPR; rr++) sum += w64[(pp * kPR + rr) * 4 + (lane & 3)];
+                            }
+                        } else {
+#pragma unroll
+                            for (int rr = 0; rr < 4; rr++) sum += w64[((lane >> 2) * 4 + rr) * 4 + (lane & 3)];
+#pragma unroll
+                            for (int off = 4; off < 32; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+                        }
+                        const int32_t j = jb + 4 * half + (lane & 3);
+                        if (sums && j > c && j < (int32_t)d.n) {
+                            const long long t = sum + all;
+                            P.scores[rank0 + j] =
+                                __fdiv_rn(__ll2float_rn(t > 0 ? t : 0) * 1.4210854715202004e-14f, mc.fm);   // 2^-46
+                        }
+                        __syncwarp();
+                    }
+                };
                 // The chunks' screen, accumulators loaded one chunk ahead; the
                 // rare work (precise scores, a search without a threshold, the
                 // stored single counts, the validation dump) has a loop of its
                 // own below, which loads its chunks again: in one loop it cost
                 // every chunk registers and reordering (order 3, 2000 x 4000:
                 // 63 ms with all of it inside, 54 without).
-                const bool slow = cold || store || P.dump;
+                const bool slow = cold || store || scoring || P.dump;
                 uint32_t todo = 0xffffffffu;
                 if (!slow) {
                     todo = 0;
@@ -2056,6 +2123,12 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     load_chunk(jcg, cs, cn);
                     tmem_wait_ld();
                     if (P.dump) dump_chunk(jb, cs, cn);
+                    if constexpr (K == 3 || K == 4) {
+                        if (scoring) {
+                            score_chunk(jb, cs, cn);
+                            continue;
+                        }
+                    }
                     if (store) {
                         // the raw accumulators of this row, two SNPs at a time
                         if (prow) {
@@ -2286,6 +2359,12 @@ __global__ void build_pairs_kernel(DevData d, const uint64_t *__restrict__ brow,
         const uint32_t v = j2 > j1 && j2 < d.n ? d.masks[(j1 * 3 + g1) * d.Wt + w] & d.masks[(j2 * 3 + g2) * d.Wt + w] : 0u;
         o[idx] = make_uint4((v & 0x11111111u) << 2, v & 0x22222222u, (v & 0x44444444u) >> 2, (v >> 3) & 0x11111111u);
     }
+}
+
+__global__ void tlog_kernel(int64_t m, long long *__restrict__ out)
+{
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= m; c += (int64_t)gridDim.x * blockDim.x)
+        out[c] = c > 0 ? __double2ll_rn((double)c * log((double)c) * 70368744177664.0) : 0;   // 2^46
 }
 
 // The producers' masks: the 256 individuals of a K stage of every SNP's three
@@ -2585,6 +2664,8 @@ static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint6
     P.cand_score_g = cand_g;
     P.cand_rank_g = rank_g;
     P.wait_ns = 0;
+    P.scores = nullptr;
+    P.tlog = nullptr;
     P.list_score = list_score;
     P.list_rank = list_rank;
     P.list_count = list_count;
@@ -2596,7 +2677,8 @@ static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint6
 static cudaError_t launch_kernel(const CUtensorMap &map, const tc::Params &P, int k, int grid, cudaStream_t st,
                                  bool comb, bool pair = false)
 {
-    const size_t smem = tc_smem_bytes(P.cand_p2, P.cand_score_g != nullptr, comb);
+    const size_t smem = tc_smem_bytes(P.cand_p2, P.cand_score_g != nullptr, comb) +
+                        (P.scores ? (size_t)(P.one.d.m + 1) * 8 : 0);
     using Kernel = void (*)(const CUtensorMap, const tc::Params);
     static const Kernel kernels[2][4] = {
         {tc::tc_search_kernel<2, false, false>, tc::tc_search_kernel<3, false, false>,
@@ -2696,6 +2778,31 @@ cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *
     e = encode_map(&map, d, ws.operand, comb, pair_operand_rows(d.n));
     if (e != cudaSuccess) return e;
     return launch_kernel(map, P, k, grid, st, comb, true);
+}
+
+// shared memory of a pass that writes every score
+size_t tc_scores_smem_bytes(const DevData &d, bool comb) { return tc_smem_bytes(0, true, comb) + (size_t)(d.m + 1) * 8; }
+
+cudaError_t launch_tc_scores(const DevData &d, int k, const unsigned char *b4, uint64_t *item_cum, long long *tlog,
+                             float *scores, uint32_t *global_thr, int32_t *list_count, int32_t *status, int grid,
+                             uint64_t total, cudaStream_t st, unsigned long long wait_ns, int comb_p)
+{
+    tc::tlog_kernel<<<16, 256, 0, st>>>(d.m, tlog);
+    tc::Params P;
+    CUtensorMap map;
+    fill_ds(P.one, d, k, item_cum, global_thr, total, 0, total, nullptr, 0, grid, comb_p, b4, 0, nullptr);
+    P.many = nullptr;
+    P.cta_ds = nullptr;
+    // nothing is kept: any address will do for the candidate buffers
+    fill_launch(P, k, 32, nullptr, nullptr, list_count, status, nullptr, nullptr, reinterpret_cast<float *>(tlog),
+                reinterpret_cast<uint64_t *>(tlog), comb_p != 0);
+    P.scores = scores;
+    P.tlog = tlog;
+    P.wait_ns = wait_ns;
+    cudaError_t e = launch_tc_item_cum(d, k, 0, total, item_cum, st, comb_p != 0);
+    if (e == cudaSuccess) e = encode_map(&map, d, b4, comb_p != 0);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(map, P, k, grid, st, comb_p != 0);
 }
 
 size_t tc_ds_bytes() { return sizeof(tc::DsParams); }
