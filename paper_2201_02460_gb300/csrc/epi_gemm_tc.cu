@@ -9,9 +9,11 @@
 // transposed copies where a product needs one), FP32 accumulation in tensor
 // memory, and C in FP32.
 //
-// One CTA computes one 128 x NT tile of C over one slice of K: 128 threads
-// load 64-wide K chunks of A (128 rows) and B (NT rows) with 16-byte loads
-// into shared memory in the 128-byte swizzle (two stages), one thread issues
+// One CTA computes one 128 x NT tile of C over one slice of K: 256 threads
+// load 64-wide K chunks of A (128 rows) and B (NT rows) with 16-byte loads,
+// four of a thread in flight (at most four chunks a CTA here, so load latency
+// bounds the kernel: 8192 x 256 x 256 took 45 us with 128 threads and one load
+// at a time, 13 us so), into shared memory in the 128-byte swizzle (two stages), one thread issues
 // the MMAs (M128 x NT x K16, four per chunk) and commits each stage to an
 // mbarrier, so the loads of chunk c + 1 overlap the MMAs of chunk c.  Rows,
 // columns and K past the matrix edges enter as zeros.  With several K slices
@@ -31,7 +33,7 @@
 namespace epi {
 namespace gemmtc {
 
-constexpr int kThreads = 128;
+constexpr int kThreads = 256;
 constexpr int kM = 128;
 constexpr int kKC = 64;                              // K elements per chunk (128 bytes)
 constexpr unsigned long long kTimeoutNs = 2000000000ull;
@@ -77,22 +79,32 @@ __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity)
 __device__ __forceinline__ void load_chunk(unsigned char *dst, const __nv_bfloat16 *X, int64_t ld, int r0, int rows,
                                            int R, int k0, int K)
 {
-    for (int i = threadIdx.x; i < rows * 8; i += kThreads) {
-        const int r = i >> 3, c = i & 7;
-        const int row = r0 + r, k = k0 + 8 * c;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (row < R) {
-            const __nv_bfloat16 *src = X + (int64_t)row * ld + k;
-            if (k + 8 <= K) {
-                v = __ldg(reinterpret_cast<const uint4 *>(src));
-            } else if (k < K) {
-                uint16_t h[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                for (int e = 0; e < K - k; e++) h[e] = reinterpret_cast<const uint16_t *>(src)[e];
-                v = make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
-                               h[6] | (uint32_t)h[7] << 16);
+    // four loads before their stores
+    for (int i0 = threadIdx.x; i0 < rows * 8; i0 += 4 * kThreads) {
+        uint4 v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int i = i0 + q * kThreads;
+            const int r = i >> 3, c = i & 7;
+            const int row = r0 + r, k = k0 + 8 * c;
+            v[q] = make_uint4(0, 0, 0, 0);
+            if (i < rows * 8 && row < R) {
+                const __nv_bfloat16 *src = X + (int64_t)row * ld + k;
+                if (k + 8 <= K) {
+                    v[q] = __ldg(reinterpret_cast<const uint4 *>(src));
+                } else if (k < K) {
+                    uint16_t h[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+                    for (int e = 0; e < K - k; e++) h[e] = reinterpret_cast<const uint16_t *>(src)[e];
+                    v[q] = make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16,
+                                      h[4] | (uint32_t)h[5] << 16, h[6] | (uint32_t)h[7] << 16);
+                }
             }
         }
-        *reinterpret_cast<uint4 *>(dst + swz(r, c)) = v;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int i = i0 + q * kThreads;
+            if (i < rows * 8) *reinterpret_cast<uint4 *>(dst + swz(i >> 3, i & 7)) = v[q];
+        }
     }
 }
 
@@ -156,19 +168,32 @@ __global__ void __launch_bounds__(kThreads) gemm_kernel(const Args P)
     __syncthreads();
     tc_fence_after();
     const bool empty = c_end <= c_begin;
-    // thread t reads tile row t (TMEM lane t) in 32-column pieces
-    const int row = m0 + tid;
+    // thread t reads tile row t % 128 (a TMEM lane) in 32-column pieces, the
+    // two halves of the warps taking alternate pieces
+    const int lane_row = tid & 127;
+    const int row = m0 + lane_row;
     float *crow = P.C + (size_t)slice * P.M * P.ldc + (int64_t)row * P.ldc;
-    for (int cb = 0; cb < P.nt; cb += 32) {
+    const bool vec = (P.ldc & 3) == 0 && (P.N & 3) == 0;
+    for (int cb = 32 * (tid >> 7); cb < P.nt; cb += 64) {
         uint32_t v[32];
-        const uint32_t ta = tmem + ((uint32_t)((tid >> 5) * 32) << 16) + (uint32_t)cb;
+        const uint32_t ta = tmem + ((uint32_t)(lane_row & ~31) << 16) + (uint32_t)cb;
         TMEM_LD32(ta, v);
         tmem_wait_ld();
         if (row < P.M && !bad) {
 #pragma unroll
-            for (int q = 0; q < 32; q++) {
+            for (int q = 0; q < 32; q += 4) {
                 const int col = n0 + cb + q;
-                if (col < P.N) crow[col] = empty ? 0.0f : __uint_as_float(v[q]);
+                float4 o = make_float4(__uint_as_float(v[q]), __uint_as_float(v[q + 1]), __uint_as_float(v[q + 2]),
+                                       __uint_as_float(v[q + 3]));
+                if (empty) o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (vec) {
+                    if (col < P.N) *reinterpret_cast<float4 *>(crow + col) = o;
+                } else {
+                    if (col < P.N) crow[col] = o.x;
+                    if (col + 1 < P.N) crow[col + 1] = o.y;
+                    if (col + 2 < P.N) crow[col + 2] = o.z;
+                    if (col + 3 < P.N) crow[col + 3] = o.w;
+                }
             }
         }
     }
@@ -189,6 +214,7 @@ __global__ void sum_slices_kernel(const float *__restrict__ part, int slices, in
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int m = (int)(i / N), n = (int)(i - (int64_t)m * N);
         float s = 0.0f;
+#pragma unroll 8
         for (int q = 0; q < slices; q++) s += part[((int64_t)q * M + m) * ldp + n];
         float *o = C + (int64_t)m * ldc + n;
         *o = accumulate ? *o + s : s;

@@ -519,6 +519,246 @@ __global__ void transpose_bf16_kernel(const T *__restrict__ in, int64_t R, int C
     }
 }
 
+// ---------------------------------------------------------------------------
+// The parts of a training step beside its three hidden x hidden products,
+// fused for up to 32 inputs and 256 hidden units (a multiple of 32): one
+// thread per hidden unit, 32 rows at a time.  What bounds them is latency: a
+// gradient of 8192 rows x 30 inputs x 256 units moves 60 MB within L2, and as
+// 23 separate kernels (input, layer-1 product, bias, output product, loss,
+// outer products, transposes, masks and their sums) it took 404 us, launches
+// and single loads waited for.  Fused, with 16 rows' loads in flight, it takes
+// 152 us: these 11, 14, 11 and 8 us, three products of 13-15 us.  A block takes
+// row tiles blockIdx.x, blockIdx.x + gridDim.x, ...; its sums over the rows go
+// to part[block][FusedParts::total], added over the blocks in a fixed order.
+// ---------------------------------------------------------------------------
+constexpr int kFusedRows = 32, kFusedIn = 32;
+
+// a block's partial sums: dW1 as [in][h], then db1, db2, dW3 [h] each, db3, loss
+struct FusedParts {
+    int in, h;
+    __host__ __device__ int b1() const { return in * h; }
+    __host__ __device__ int b2() const { return b1() + h; }
+    __host__ __device__ int w3() const { return b2() + h; }
+    __host__ __device__ int b3() const { return w3() + h; }
+    __host__ __device__ int loss() const { return b3() + 1; }
+    __host__ __device__ int total() const { return loss() + 1; }
+};
+
+// normalised BF16 inputs of a row tile, as floats, padded to 32 columns
+__device__ __forceinline__ void stage_inputs(const float *__restrict__ X, int64_t r0, int64_t rows, int in,
+                                             const float *__restrict__ norm, float (*xs)[kFusedIn])
+{
+#pragma unroll 4
+    for (int e = threadIdx.x; e < kFusedRows * kFusedIn; e += blockDim.x) {
+        const int r = e / kFusedIn, f = e - r * kFusedIn;
+        const int fc = min(f, in - 1);
+        const float v = (X[min(r0 + r, rows - 1) * in + fc] - norm[fc]) * norm[in + fc];
+        xs[r][f] = f < in && r0 + r < rows ? __bfloat162float(__float2bfloat16(v)) : 0.0f;
+    }
+}
+
+// column j of 32 rows into the transposed operand: out[j][r0 .. r0 + 31], in
+// pieces of 8 rows below ld
+__device__ __forceinline__ void store_transposed(__nv_bfloat16 *__restrict__ out, int64_t ld, int j, int64_t r0,
+                                                 const uint32_t *pairs)
+{
+    uint4 *o = reinterpret_cast<uint4 *>(out + (int64_t)j * ld + r0);
+#pragma unroll
+    for (int q = 0; q < kFusedRows / 8; q++)
+        if (r0 + 8 * q < ld) o[q] = make_uint4(pairs[4 * q], pairs[4 * q + 1], pairs[4 * q + 2], pairs[4 * q + 3]);
+}
+
+__device__ __forceinline__ void put_bf16(uint32_t *pairs, int r, __nv_bfloat16 v)
+{
+    const uint32_t b = (uint32_t)__bfloat16_as_ushort(v);
+    if (r & 1) pairs[r >> 1] |= b << 16;
+    else pairs[r >> 1] = b;
+}
+
+// H1 = relu(X W1^T + b1) in BF16, row-major and transposed ([h][ldt])
+__global__ void __launch_bounds__(256) fused_layer1_kernel(const float *__restrict__ X, int64_t rows, int in, int h,
+                                                           const float *__restrict__ norm,
+                                                           const __nv_bfloat16 *__restrict__ W1,
+                                                           const float *__restrict__ b1, __nv_bfloat16 *__restrict__ H1,
+                                                           __nv_bfloat16 *__restrict__ H1t, int64_t ldt)
+{
+    __shared__ float xs[kFusedRows][kFusedIn];
+    const int j = threadIdx.x;
+    float w[kFusedIn];
+#pragma unroll
+    for (int f = 0; f < kFusedIn; f++) w[f] = f < in ? __bfloat162float(W1[(int64_t)j * in + f]) : 0.0f;
+    const float bias = b1[j];
+    for (int64_t r0 = (int64_t)blockIdx.x * kFusedRows; r0 < rows; r0 += (int64_t)gridDim.x * kFusedRows) {
+        __syncthreads();
+        stage_inputs(X, r0, rows, in, norm, xs);
+        __syncthreads();
+        uint32_t col[kFusedRows / 2];
+#pragma unroll
+        for (int r = 0; r < kFusedRows; r++) {
+            float z = 0.0f;
+#pragma unroll
+            for (int f = 0; f < kFusedIn; f += 4) {
+                const float4 x = *reinterpret_cast<const float4 *>(&xs[r][f]);
+                z = fmaf(x.x, w[f], z);
+                z = fmaf(x.y, w[f + 1], z);
+                z = fmaf(x.z, w[f + 2], z);
+                z = fmaf(x.w, w[f + 3], z);
+            }
+            const bool in_row = r0 + r < rows;
+            const __nv_bfloat16 v = __float2bfloat16(in_row ? fmaxf(z + bias, 0.0f) : 0.0f);
+            if (in_row) H1[(r0 + r) * h + j] = v;
+            put_bf16(col, r, v);
+        }
+        store_transposed(H1t, ldt, j, r0, col);
+    }
+}
+
+// From Z2 = H1 W2^T: H2 = relu(Z2 + b2) in BF16, the prediction, its error,
+// and dZ2 = dY W3 where H2 > 0, in BF16 row-major and transposed; partial sums
+// of dW3, db3, db2 and the squared error
+__global__ void __launch_bounds__(256) fused_output_kernel(const float *__restrict__ Z2, int64_t rows, int h,
+                                                           const float *__restrict__ b2,
+                                                           const __nv_bfloat16 *__restrict__ W3,
+                                                           const float *__restrict__ b3, const float *__restrict__ t,
+                                                           __nv_bfloat16 *__restrict__ dZb,
+                                                           __nv_bfloat16 *__restrict__ dZt, int64_t ldt,
+                                                           float *__restrict__ part, FusedParts at)
+{
+    __shared__ __nv_bfloat16 hs[kFusedRows][256 + 2];
+    __shared__ float w3s[256], dys[kFusedRows], es[kFusedRows];
+    const int j = threadIdx.x, lane = j & 31, warp = j >> 5, warps = blockDim.x >> 5;
+    const float bias = b2[j], w3 = __bfloat162float(W3[j]), out_bias = b3[0];
+    w3s[j] = w3;
+    float dw3 = 0.0f, db2 = 0.0f, db3 = 0.0f, loss = 0.0f;
+    for (int64_t r0 = (int64_t)blockIdx.x * kFusedRows; r0 < rows; r0 += (int64_t)gridDim.x * kFusedRows) {
+        __syncthreads();
+#pragma unroll 16
+        for (int r = 0; r < kFusedRows; r++) {
+            const float z = Z2[min(r0 + r, rows - 1) * h + j];
+            hs[r][j] = __float2bfloat16(r0 + r < rows ? fmaxf(z + bias, 0.0f) : 0.0f);
+        }
+        __syncthreads();
+        for (int r = warp; r < kFusedRows; r += warps) {
+            float y = 0.0f;
+            for (int q = lane; q < h; q += 32) y = fmaf(__bfloat162float(hs[r][q]), w3s[q], y);
+#pragma unroll
+            for (int off = 16; off; off >>= 1) y += __shfl_xor_sync(0xffffffffu, y, off);
+            if (lane == 0) {
+                const bool in_row = r0 + r < rows;
+                const float e = in_row ? y + out_bias - t[r0 + r] : 0.0f;
+                es[r] = e;
+                dys[r] = 2.0f * e / (float)rows;
+            }
+        }
+        __syncthreads();
+        uint32_t col[kFusedRows / 2];
+#pragma unroll
+        for (int r = 0; r < kFusedRows; r++) {
+            const float v = __bfloat162float(hs[r][j]), dy = dys[r];
+            dw3 = fmaf(v, dy, dw3);
+            const float dz = v > 0.0f ? dy * w3 : 0.0f;
+            db2 += dz;
+            const __nv_bfloat16 b = __float2bfloat16(dz);
+            if (r0 + r < rows) dZb[(r0 + r) * h + j] = b;
+            put_bf16(col, r, b);
+        }
+        store_transposed(dZt, ldt, j, r0, col);
+        if (warp == 0) {
+            float d = dys[lane], q = es[lane] * es[lane];
+#pragma unroll
+            for (int off = 16; off; off >>= 1) {
+                d += __shfl_xor_sync(0xffffffffu, d, off);
+                q += __shfl_xor_sync(0xffffffffu, q, off);
+            }
+            db3 += d;
+            loss += q;
+        }
+    }
+    float *o = part + (size_t)blockIdx.x * at.total();
+    o[at.b2() + j] = db2;
+    o[at.w3() + j] = dw3;
+    if (j == 0) {
+        o[at.b3()] = db3;
+        o[at.loss()] = loss / (float)rows;
+    }
+}
+
+// dZ1 = dH1 where H1 > 0; partial sums of dW1 = dZ1^T X and db1
+__global__ void __launch_bounds__(256) fused_grad1_kernel(const float *__restrict__ dH1,
+                                                          const __nv_bfloat16 *__restrict__ H1,
+                                                          const float *__restrict__ X, int64_t rows, int in, int h,
+                                                          const float *__restrict__ norm, float *__restrict__ part,
+                                                          FusedParts at)
+{
+    __shared__ float xs[kFusedRows][kFusedIn];
+    const int j = threadIdx.x;
+    float acc[kFusedIn], db1 = 0.0f;
+#pragma unroll
+    for (int f = 0; f < kFusedIn; f++) acc[f] = 0.0f;
+    for (int64_t r0 = (int64_t)blockIdx.x * kFusedRows; r0 < rows; r0 += (int64_t)gridDim.x * kFusedRows) {
+        __syncthreads();
+        stage_inputs(X, r0, rows, in, norm, xs);
+        __syncthreads();
+        // the loads of 16 rows in flight (rows past the end read the last one)
+        float dzs[16];
+#pragma unroll
+        for (int r = 0; r < kFusedRows; r++) {
+            if ((r & 15) == 0) {
+                __nv_bfloat16 hv[16];
+#pragma unroll
+                for (int q = 0; q < 16; q++) {
+                    const int64_t at_row = min(r0 + r + q, rows - 1) * h + j;
+                    hv[q] = H1[at_row];
+                    dzs[q] = dH1[at_row];
+                }
+#pragma unroll
+                for (int q = 0; q < 16; q++)
+                    if (r0 + r + q >= rows || !(__bfloat162float(hv[q]) > 0.0f)) dzs[q] = 0.0f;
+            }
+            const float dz = dzs[r & 15];
+            db1 += dz;
+#pragma unroll
+            for (int f = 0; f < kFusedIn; f += 4) {
+                const float4 x = *reinterpret_cast<const float4 *>(&xs[r][f]);
+                acc[f] = fmaf(dz, x.x, acc[f]);
+                acc[f + 1] = fmaf(dz, x.y, acc[f + 1]);
+                acc[f + 2] = fmaf(dz, x.z, acc[f + 2]);
+                acc[f + 3] = fmaf(dz, x.w, acc[f + 3]);
+            }
+        }
+    }
+    float *o = part + (size_t)blockIdx.x * at.total();
+#pragma unroll
+    for (int f = 0; f < kFusedIn; f++)
+        if (f < in) o[f * h + j] = acc[f];
+    o[at.b1() + j] = db1;
+}
+
+// the parts' sums over the blocks, in a fixed order, to their places in the
+// gradient (parameter offsets W1, b1, b2, W3, b3) and the loss
+__global__ void __launch_bounds__(256) fused_sum_kernel(const float *__restrict__ part, int blocks, FusedParts at,
+                                                        float *__restrict__ g, int64_t oW1, int64_t ob1, int64_t ob2,
+                                                        int64_t oW3, int64_t ob3, float *__restrict__ loss)
+{
+    __shared__ float sums[8][32];
+    const int e = blockIdx.x * 32 + (threadIdx.x & 31), grp = threadIdx.x >> 5;
+    float s = 0.0f;
+    if (e < at.total()) {
+#pragma unroll 4
+        for (int q = grp; q < blocks; q += 8) s += part[(size_t)q * at.total() + e];
+    }
+    sums[grp][threadIdx.x & 31] = s;
+    __syncthreads();
+    if (grp || e >= at.total()) return;
+    for (int q = 1; q < 8; q++) s += sums[q][threadIdx.x & 31];
+    if (e < at.b1()) g[oW1 + (int64_t)(e % at.h) * at.in + e / at.h] = s;
+    else if (e < at.b2()) g[ob1 + e - at.b1()] = s;
+    else if (e < at.w3()) g[ob2 + e - at.b2()] = s;
+    else if (e < at.b3()) g[oW3 + e - at.w3()] = s;
+    else if (e < at.loss()) g[ob3] = s;
+    else loss[0] = s;
+}
+
 // AdamW on the FP32 master weights; BF16 working copies refreshed
 __global__ void adamw_kernel(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m1,
                              float *__restrict__ m2, __nv_bfloat16 *__restrict__ wb, int64_t count, float lr, float b1,
@@ -636,11 +876,22 @@ struct Acts {
     __nv_bfloat16 *W2t;  // [h][h]   W2 transposed (BF16 working copy)
     float *part;         // split-K partial tiles of dW2
     float *opart;        // [slices][h][n_in + 1] partial sums of the batch reductions
+    float *fpart;        // [fused_blocks][FusedParts::total] the fused kernels' partial sums
 };
 
 // The three hidden x hidden products of a training step run on the tensor
 // cores (epi_gemm_tc.cu) when the hidden width allows 16-byte rows.
 bool train_tc(const epi_mlp *net);
+
+// The fused kernels beside them, where a thread per hidden unit serves: more
+// than 256 units make more than one block a row tile, more than 32 inputs do
+// not stay in a thread's registers (8192 rows x 30 x 256: 152 us fused, 404 us
+// separate; the separate kernels remain for those shapes).
+bool train_fused(const epi_mlp *net)
+{
+    return net->n_in <= learn::kFusedIn && net->hidden <= 256 && net->hidden % 32 == 0;
+}
+int fused_blocks(int64_t rows) { return (int)std::min<int64_t>((rows + learn::kFusedRows - 1) / learn::kFusedRows, 512); }
 
 epi_status ensure_acts(epi_mlp *net, int64_t B, Acts &a)
 {
@@ -653,6 +904,7 @@ epi_status ensure_acts(epi_mlp *net, int64_t B, Acts &a)
             b += (size_t)h * rp * 2 * 2 + (size_t)rows * h * 2 + (size_t)h * h * 2 +
                  gemm_tc_partial_floats(h, h, (int)std::min<int64_t>(rows, INT32_MAX), net->num_sms) * 4 + 5 * 256;
         b += (size_t)((rows + learn::kSliceRows - 1) / learn::kSliceRows) * h * (std::max(in, 1) + 1) * 4 + 256;
+        if (train_fused(net)) b += (size_t)fused_blocks(rows) * learn::FusedParts{in, h}.total() * 4 + 256;
         return b;
     };
     if (net->cap < B) {
@@ -684,6 +936,9 @@ epi_status ensure_acts(epi_mlp *net, int64_t B, Acts &a)
     }
     a.opart = reinterpret_cast<float *>(
         take((size_t)((B + learn::kSliceRows - 1) / learn::kSliceRows) * h * (std::max(in, 1) + 1) * 4));
+    a.fpart = train_fused(net) ? reinterpret_cast<float *>(
+                                     take((size_t)fused_blocks(B) * learn::FusedParts{in, h}.total() * 4))
+                               : nullptr;
     return EPI_OK;
 }
 
@@ -768,6 +1023,34 @@ epi_status backward(epi_mlp *net, const float *t, int64_t B, Acts &a)
         LCK(gemm(st, h, in, (int)B, dZ1, 1, h, a.X, in, 1, net->g + o.W1, in, 1, 0));
         learn::colsum_kernel<<<h, 256, 0, st>>>(dZ1, B, h, net->g + o.b1);
     }
+    return EPI_OK;
+}
+
+// Loss and gradients of a batch into a.loss and net->g.
+epi_status batch_gradients(epi_mlp *net, const float *X, const float *t, int64_t B, Acts &a)
+{
+    if (!train_fused(net)) {
+        const epi_status s = forward(net, X, B, a, a.Y, true);
+        return s == EPI_OK ? backward(net, t, B, a) : s;
+    }
+    const int in = net->n_in, h = net->hidden;
+    const Offs o = offsets(in, h);
+    const learn::FusedParts at{in, h};
+    cudaStream_t st = net->stream;
+    const int blocks = fused_blocks(B);
+    learn::fused_layer1_kernel<<<blocks, h, 0, st>>>(X, B, in, h, net->norm, net->wb + o.W1, net->w + o.b1, a.H1, a.H1t,
+                                                     a.Bp);
+    LCK(launch_gemm_tc(a.H1, h, net->wb + o.W2, h, a.Z2, h, (int)B, h, h, nullptr, net->status, net->num_sms, st));
+    learn::fused_output_kernel<<<blocks, h, 0, st>>>(a.Z2, B, h, net->w + o.b2, net->wb + o.W3, net->w + o.b3, t, a.dZb,
+                                                     a.dZt, a.Bp, a.fpart, at);
+    LCK(transpose_bf16(net->wb + o.W2, h, h, h, a.W2t, h, nullptr, st));
+    // dW2 = dZ2^T H1 (K = the batch, split over CTAs), dH1 = dZ2 W2
+    LCK(launch_gemm_tc(a.dZt, a.Bp, a.H1t, a.Bp, net->g + o.W2, h, h, h, (int)B, a.part, net->status, net->num_sms, st));
+    LCK(launch_gemm_tc(a.dZb, h, a.W2t, h, a.Z1, h, (int)B, h, h, nullptr, net->status, net->num_sms, st));
+    learn::fused_grad1_kernel<<<blocks, h, 0, st>>>(a.Z1, a.H1, X, B, in, h, net->norm, a.fpart, at);
+    learn::fused_sum_kernel<<<(at.total() + 31) / 32, 256, 0, st>>>(a.fpart, blocks, at, net->g, o.W1, o.b1, o.b2, o.W3,
+                                                                    o.b3, a.loss);
+    LCK(cudaGetLastError());
     return EPI_OK;
 }
 
@@ -920,8 +1203,7 @@ epi_status epi_mlp_gradients(epi_mlp *net, const float *X_dev, const float *t_de
     Acts a;
     epi_status s = ensure_acts(net, rows, a);
     if (s == EPI_OK) LCK(cudaMemsetAsync(net->status, 0, 4, net->stream));
-    if (s == EPI_OK) s = forward(net, X_dev, rows, a, a.Y, true);
-    if (s == EPI_OK) s = backward(net, t_dev, rows, a);
+    if (s == EPI_OK) s = batch_gradients(net, X_dev, t_dev, rows, a);
     if (s != EPI_OK) return s;
     int32_t hs = 0;
     if (grad_host) LCK(cudaMemcpyAsync(grad_host, net->g, (size_t)net->n_params * 4, cudaMemcpyDeviceToHost, net->stream));
@@ -939,8 +1221,7 @@ epi_status epi_mlp_train_step(epi_mlp *net, const float *X_dev, const float *t_d
     Acts a;
     epi_status s = ensure_acts(net, rows, a);
     if (s == EPI_OK) LCK(cudaMemsetAsync(net->status, 0, 4, net->stream));
-    if (s == EPI_OK) s = forward(net, X_dev, rows, a, a.Y, true);
-    if (s == EPI_OK) s = backward(net, t_dev, rows, a);
+    if (s == EPI_OK) s = batch_gradients(net, X_dev, t_dev, rows, a);
     if (s != EPI_OK) return s;
     net->step++;
     const float b1 = 0.9f, b2 = 0.999f;
