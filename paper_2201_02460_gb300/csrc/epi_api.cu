@@ -137,7 +137,10 @@ bool injected_alloc_failure(epi_ctx *ctx)
 cudaError_t ctx_malloc(epi_ctx *ctx, void **p, size_t bytes)
 {
     if (injected_alloc_failure(ctx)) return cudaErrorMemoryAllocation;
-    return cudaMalloc(p, bytes);
+    const cudaError_t e = cudaMalloc(p, bytes);
+    // a caller may go on without the memory: no launch check sees this error
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
 }
 
 cudaError_t ctx_malloc_async(epi_ctx *ctx, void **p, size_t bytes, cudaStream_t st)
@@ -348,9 +351,24 @@ epi_status ensure_b4(epi_dataset *ds)
 // class accumulators).
 int plan_comb_shift(const epi_dataset *ds) { return ds->ctx->tc_combined ? tc_comb_shift(ds->dev()) : 0; }
 
-epi_status make_plan(const epi_dataset *ds, SearchPlan &p, int path)
+// choose_path, with the operand an automatic choice of the tensor path needs;
+// where that does not fit in memory, the popcount path.
+epi_status take_path(epi_dataset *ds, int k, int path, uint64_t rb, uint64_t re, uint64_t total, bool &tc)
 {
-    epi_status st = choose_path(ds, p.k, path, p.rb, p.re, p.total, p.tc);
+    epi_status st = choose_path(ds, k, path, rb, re, total, tc);
+    if (st == EPI_OK && tc && path == EPI_PATH_AUTO) {
+        st = ensure_b4(ds);
+        if (st == EPI_ENOMEM) {
+            tc = false;
+            st = EPI_OK;
+        }
+    }
+    return st;
+}
+
+epi_status make_plan(epi_dataset *ds, SearchPlan &p, int path)
+{
+    epi_status st = take_path(ds, p.k, path, p.rb, p.re, p.total, p.tc);
     if (st != EPI_OK) return st;
     if (!p.tc) return plan_popc(ds, p);
     p.grid = ds->ctx->num_sms;
@@ -776,6 +794,8 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
 {
     if (!ctx || !dss || !orders || !top_ns || !outs || !n_outs) return fail(EPI_EINVAL, "NULL argument");
     if (n_ds < 1 || n_ds > 4096) return fail(EPI_EINVAL, "n_ds %d outside 1..4096", n_ds);
+    DeviceGuard guard(ctx->device);
+    if (!guard.ok) return fail(EPI_ECUDA, "cannot select device %d", ctx->device);
     std::vector<BatchItem> items((size_t)n_ds);
     for (int i = 0; i < n_ds; i++) {
         BatchItem &it = items[i];
@@ -790,7 +810,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         it.total = total;
         it.pool = initial_pool(it.top_n);
         it.cells = pow3i(it.k);
-        st = choose_path(it.ds, it.k, path, 0, total, total, it.tc);
+        st = take_path(it.ds, it.k, path, 0, total, total, it.tc);
         if (st != EPI_OK) return fail(st, "dataset %d: %s", i, epi_last_error());
         const DevData d = it.ds->dev();
         if (it.tc) it.comb_p = plan_comb_shift(it.ds);
@@ -801,8 +821,6 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         it.cost = it.tc ? (double)tc_item_count(d.n, it.k, it.comb_p != 0) * (double)std::max(d.Wt / 4, 32)
                         : (double)total * (double)(it.cells / 3) * (double)d.Wt;
     }
-    DeviceGuard guard(ctx->device);
-    if (!guard.ok) return fail(EPI_ECUDA, "cannot select device %d", ctx->device);
     // one group per (path, order, tensor variant)
     std::vector<BatchGroup> groups;
     for (int i = 0; i < n_ds; i++) {
@@ -1240,18 +1258,21 @@ epi_status epi_search_threshold(epi_dataset *ds, int order, double threshold, in
     // A threshold few combinations reach: the tensor path counts and screens
     // all of them and keeps the ranks that pass (order 3, 1000 x 4000, 104
     // found: 129 ms when the popcount path wrote every score, 9 ms so).  More
-    // than cand_cap of them, or a threshold that is no screen: every score.
+    // than cand_cap of them, a threshold that is no screen, or no room for the operand:
+    // every score.
     bool done = false;
     if (chunk == 0 && thr32 > 0.0f && tc_applicable(ds, order, 0, total, total)) {
         int32_t *status = nullptr;
         st = queue_collect(ds, order, total, thr32, cand, cand_cap, n_dev, &status);
-        if (st != EPI_OK) { cleanup(); return st; }
+        if (st != EPI_OK && st != EPI_ENOMEM) { cleanup(); return st; }
         unsigned long long nc = 0;
         int32_t bits = 0;
-        TCK(cudaMemcpyAsync(&nc, n_dev, 8, cudaMemcpyDeviceToHost, sm));
-        TCK(cudaMemcpyAsync(&bits, status, 4, cudaMemcpyDeviceToHost, sm));
-        TCK(cudaStreamSynchronize(sm));
-        done = nc <= cand_cap;
+        if (st == EPI_OK) {
+            TCK(cudaMemcpyAsync(&nc, n_dev, 8, cudaMemcpyDeviceToHost, sm));
+            TCK(cudaMemcpyAsync(&bits, status, 4, cudaMemcpyDeviceToHost, sm));
+            TCK(cudaStreamSynchronize(sm));
+            done = nc <= cand_cap;
+        }
         if (done && bits != 0) {
             cleanup();
             return bits & ST_TIMEOUT ? fail(EPI_ETIMEOUT, "device wait expired")
@@ -1334,23 +1355,24 @@ epi_status epi_score_all(epi_dataset *ds, int order, float *out_dev)
         const size_t o_ic = a.take<uint64_t>(2 * ((size_t)ds->n + 1));
         const size_t o_tl = a.take<long long>((size_t)ds->m + 1);
         st = ensure_scratch(ctx, a.off);
-        if (st != EPI_OK) return st;
-        st = ensure_b4(ds);
-        if (st != EPI_OK) return st;
-        char *base = static_cast<char *>(ctx->scratch);
-        CK(cudaMemsetAsync(base, 0, 512, ctx->stream));
-        CK(launch_tc_scores(ds->dev(), order, ds->b4, reinterpret_cast<uint64_t *>(base + o_ic),
-                            reinterpret_cast<long long *>(base + o_tl), out_dev,
-                            reinterpret_cast<uint32_t *>(base + o_thr), reinterpret_cast<int32_t *>(base + o_lc),
-                            reinterpret_cast<int32_t *>(base + o_status), grid, total, ctx->stream,
-                            ctx->wait_limit_ns, comb_p));
-        ctx->launches += 3;
-        int32_t bits = 0;
-        CK(cudaMemcpyAsync(&bits, base + o_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
-        CK(cudaStreamSynchronize(ctx->stream));
-        if (bits & ST_TIMEOUT) return fail(EPI_ETIMEOUT, "device wait expired");
-        if (bits) return fail(EPI_ECUDA, "device status 0x%x", bits);
-        return EPI_OK;
+        if (st == EPI_OK) st = ensure_b4(ds);
+        if (st == EPI_OK) {
+            char *base = static_cast<char *>(ctx->scratch);
+            CK(cudaMemsetAsync(base, 0, 512, ctx->stream));
+            CK(launch_tc_scores(ds->dev(), order, ds->b4, reinterpret_cast<uint64_t *>(base + o_ic),
+                                reinterpret_cast<long long *>(base + o_tl), out_dev,
+                                reinterpret_cast<uint32_t *>(base + o_thr), reinterpret_cast<int32_t *>(base + o_lc),
+                                reinterpret_cast<int32_t *>(base + o_status), grid, total, ctx->stream,
+                                ctx->wait_limit_ns, comb_p));
+            ctx->launches += 3;
+            int32_t bits = 0;
+            CK(cudaMemcpyAsync(&bits, base + o_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaStreamSynchronize(ctx->stream));
+            if (bits & ST_TIMEOUT) return fail(EPI_ETIMEOUT, "device wait expired");
+            if (bits) return fail(EPI_ECUDA, "device status 0x%x", bits);
+            return EPI_OK;
+        }
+        if (st != EPI_ENOMEM) return st;   // no room for the operand: the popcount path
     }
     SearchPlan p;
     p.k = order; p.top_n = 1; p.pool = initial_pool(1); p.rb = 0; p.re = total; p.total = total;

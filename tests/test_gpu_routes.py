@@ -34,6 +34,140 @@ def ctx(epi):
     return epi.Context(0)
 
 
+def _same(a, b):
+    """Two routes of one search: the same records, bit for bit."""
+    assert (a.rank == b.rank).all() and (a.combs == b.combs).all()
+    assert (a.mi == b.mi).all() and (a.counts == b.counts).all()
+
+
+# pair tiles start at 40 SNPs (order 4) and 24 (order 5); one SNP fewer takes
+# the other tiles.  Odd SNP and sample counts, one class small, both variants.
+@pytest.mark.parametrize("k,n,m,m1,variant", [
+    (4, 39, 300, 130, "auto"), (4, 40, 300, 130, "auto"), (4, 41, 257, 20, "auto"), (4, 42, 300, 130, "separate"),
+    (4, 75, 513, 256, "auto"), (5, 23, 270, 140, "auto"), (5, 24, 270, 140, "auto"), (5, 25, 129, 11, "separate"),
+    (5, 27, 1000, 900, "auto")])
+def test_pair_tiles(epi, ctx, k, n, m, m1, variant):
+    geno, pheno = random_data(n, m, seed=100 * k + n, m1=m1)
+    ds = epi.Dataset(ctx, geno, pheno)
+    ctx.set_tc_variant(variant)
+    try:
+        if math.comb(n, k) * 2 * 3 ** k * 4 < 1 << 30:
+            got = epi.debug_counts(ds, k)
+            combs = np.array(list(itertools.combinations(range(n), k)), dtype=np.uint32)
+            for i in range(0, len(combs), 50000):
+                assert (got[i:i + 50000] == epi.tables(ds, combs[i:i + 50000])).all()
+        _same(epi.search(ds, k, 50, path="tc"), epi.search(ds, k, 50, path="popc"))
+    finally:
+        ctx.set_tc_variant("auto")
+
+
+# the classes share an accumulator while c1 2^p + c0 < 2^24 with 2^p > c0 + 1
+# (c1, c0: the largest counts of a genotype): 4094 each is the last equal pair
+@pytest.mark.parametrize("m1,m0", [(4094, 4094), (4095, 4095), (4094, 4095), (3, 8190), (8190, 3)])
+@pytest.mark.parametrize("k,n", [(2, 12), (3, 12), (4, 40)])
+def test_class_shift_limit(epi, ctx, k, n, m1, m0):
+    geno, pheno = random_data(n, m1 + m0, seed=m1 + n, m1=m1)
+    geno[:4] = 0          # one cell of the first combinations holds everyone
+    ds = epi.Dataset(ctx, geno, pheno)
+    first = np.arange(k, dtype=np.uint32)[None]
+    assert epi.tables(ds, first)[0, :, 0].tolist() == O.tables(geno, pheno, first.astype(np.int32))[0, :, 0].tolist()
+    _same(epi.search(ds, k, 40, path="tc"), epi.search(ds, k, 40, path="popc"))
+    if k < 4:
+        combs = np.array(list(itertools.combinations(range(n), k)), dtype=np.uint32)
+        assert (epi.debug_counts(ds, k) == epi.tables(ds, combs)).all()
+
+
+# the automatic path of order 2 changes at 100 SNPs
+@pytest.mark.parametrize("n,m,m1", [(99, 333, None), (100, 333, None), (121, 64, 5), (241, 130, 125)])
+def test_order2_automatic_path(epi, ctx, n, m, m1):
+    geno, pheno = random_data(n, m, seed=n, m1=m1)
+    ds = epi.Dataset(ctx, geno, pheno)
+    r = epi.search(ds, 2, 64)
+    _same(r, epi.search(ds, 2, 64, path="popc"))
+    oc, om, _ = O.search(geno, pheno, 2, 64)
+    check_topn(r.combs, r.mi, oc, om)
+
+
+# merges: one entry, fewer combinations than asked for (990) and a few more (1035)
+@pytest.mark.parametrize("k,n,top_n", [(2, 120, 1), (2, 130, 2), (2, 45, 1024), (2, 46, 1024), (3, 40, 1000)])
+def test_merge_sizes(epi, ctx, k, n, top_n):
+    geno, pheno = random_data(n, 200, seed=top_n)
+    ds = epi.Dataset(ctx, geno, pheno)
+    a, b = epi.search(ds, k, top_n, path="tc"), epi.search(ds, k, top_n, path="popc")
+    assert len(a) == min(top_n, math.comb(n, k))
+    _same(a, b)
+
+
+# chunk 0 screens on the tensor cores, a chunk size takes every score
+@pytest.mark.parametrize("k,n,m,m1", [(2, 50, 200, None), (3, 33, 700, None), (3, 30, 129, 9), (4, 22, 300, 150),
+                                      (5, 15, 90, 50)])
+def test_threshold_routes(epi, ctx, k, n, m, m1):
+    geno, pheno = random_data(n, m, seed=k * n, m1=m1)
+    ds = epi.Dataset(ctx, geno, pheno)
+    best = epi.search(ds, k, 40)
+    # in the widest gap among the best scores; above the best there is nothing;
+    # below zero everything qualifies
+    cut = 1 + int(np.argmax(best.mi[:-1] - best.mi[1:]))
+    for thr, want in ((0.5 * float(best.mi[cut - 1] + best.mi[cut]), cut), (float(best.mi[0]) * 1.01, 0), (-1.0, math.comb(n, k))):
+        a, na = epi.search_threshold(ds, k, thr, 60)
+        b, nb = epi.search_threshold(ds, k, thr, 60, chunk=1000)
+        assert (na, nb) == (want, want) and len(a) == min(60, na)
+        _same(a, b)
+
+
+# whole tables of orders 3-4: counted on the tensor cores and scored in fixed
+# point, within the FP32 path's bound of the 64-bit score
+@pytest.mark.parametrize("k,n,m,m1", [(3, 3, 50, None), (3, 41, 257, 30), (3, 25, 2999, 1500), (4, 4, 64, 32),
+                                      (4, 23, 129, 100), (3, 20, 3500, 1700)])
+def test_whole_score_tables(epi, ctx, k, n, m, m1):
+    geno, pheno = random_data(n, m, seed=n + m, m1=m1)
+    geno[1] = 2           # a SNP with one genotype: empty cells
+    ds = epi.Dataset(ctx, geno, pheno)
+    got = epi.score_all(ds, k).cpu().numpy().astype(np.float64)
+    combs = np.array(list(itertools.combinations(range(n), k)), dtype=np.int32)
+    want = np.array([O.mi(x[0], x[1], m) for x in O.tables(geno, pheno, combs)])
+    assert (np.abs(got - want) <= F32_RTOL * np.abs(want) + 1e-9).all(), np.abs(got - want).max()
+
+
+# a study large enough for pair tiles is searched by itself within a batch
+@pytest.mark.parametrize("n_alone", [1, 2])
+def test_batch_with_studies_alone(epi, ctx, n_alone):
+    shapes = [(3, 30, 200), (2, 60, 150)] + [(4, 40 + i, 260) for i in range(n_alone)] + [(4, 20, 100)]
+    dss = [epi.Dataset(ctx, *random_data(n, m, seed=n)) for _, n, m in shapes]
+    orders = [k for k, _, _ in shapes]
+    for _ in range(2):
+        got = epi.search_batched(ctx, dss, orders, [20] * len(dss))
+        for r, ds, k in zip(got, dss, orders):
+            _same(r, epi.search(ds, k, 20, path="popc"))
+
+
+# without room for the tensor path's operand the automatic choice answers by
+# the popcount path
+@pytest.mark.parametrize("call", ["search", "threshold", "scores"])
+def test_no_room_for_the_operand(epi, call):
+    geno, pheno = random_data(110, 200, seed=5)
+    k = 2 if call == "search" else 3
+    want_ctx, ctx = epi.Context(0), epi.Context(0)
+
+    def run(c, ds):
+        if call == "search":
+            return epi.search(ds, k, 30)
+        if call == "threshold":
+            return epi.search_threshold(ds, k, 0.06, 100)[0]
+        return epi.score_all(ds, k).cpu().numpy()
+
+    a = run(want_ctx, epi.Dataset(want_ctx, geno, pheno))
+    ds = epi.Dataset(ctx, geno, pheno)
+    run(ctx, epi.Dataset(ctx, geno, pheno))   # the context's scratch is there
+    ctx.inject_alloc_failure(0)
+    b = run(ctx, ds)
+    ctx.inject_alloc_failure(-1)
+    if call == "scores":
+        np.testing.assert_allclose(a, b, rtol=2 * F32_RTOL, atol=2e-9)
+    else:
+        _same(a, b)
+
+
 # fused training kernels: rows around a tile and beyond one tile a block
 # (512 x 32), inputs and hidden units at the rule's edges; (33 inputs, 288
 # hidden units: the separate kernels).  Bounds as for the gradients of other
