@@ -205,7 +205,7 @@ struct SearchPlan {
     int comb_p = 0;                // tensor path: class shift of the combined-class variant, 0 = separate classes
     bool tc_pair = false;          // tensor path: pair tiles (orders 4-5)
     bool global_prefix = false;    // popcount path: prefix tables in a global buffer (orders 7-8)
-    bool pair = false;             // popcount path: the (k-2)-prefix kernel (orders 6-8)
+    bool hist = false;             // popcount path: the histogram kernel (orders 6-8)
     float *all_scores = nullptr;   // optional: every combination's score (popcount path)
     size_t smem = 0;
     uint64_t rb = 0, re = 0, total = 0;
@@ -288,14 +288,23 @@ epi_status plan_popc(const epi_dataset *ds, SearchPlan &p, int R_req = 0)
     if (best_score < 0)
         return fail(EPI_EUNSUPPORTED, "order %d with %lld samples: one prefix table does not fit in shared memory",
                     p.k, (long long)ds->m);
-    uint64_t grid = (uint64_t)ctx->num_sms * (uint64_t)p.grid;
-    // orders 6-8: the (k-2)-prefix kernel, one 1024-thread CTA per SM, its
-    // own number of waves
-    p.pair = popc_pair_applies(p.k, ds->Wt, p.pool, p.all_scores != nullptr);
-    if (p.pair) {
+    // orders 6-8: by histogram wherever it takes the sample; 100 best, against
+    // the kernels over words it replaced (a table of k - 2 or k - 1 SNPs):
+    //   order 6   14 x  200  0.30 and 0.86 ms    40 x  2048  17.9 and  30.1 ms
+    //   order 7   12 x  300  0.47 and 1.31 ms    26 x  2048   3.8 and  17.8 ms
+    //   order 7   22 x 6000   3.5 and 15.9 ms    20 x 16000   4.8 and  53.5 ms
+    //   order 8   11 x  200  0.75 and 1.80 ms    23 x  2048   3.3 and  37.1 ms
+    //   order 8   18 x 5000   1.8 and 55.0 ms    17 x 16000   2.7 and 152.9 ms
+    // A forced launch shape is one of the word kernels', and what they refuse
+    // for its size stays refused.
+    p.hist = !R_req && hist_applies(ds->dev(), p.k, p.pool);
+    if (p.hist) {
         p.global_prefix = false;
-        grid = (uint64_t)popc_pair_grid(ctx->num_sms, p.k, ds->n);
+        p.grid = (int)std::max<uint64_t>(1, std::min<uint64_t>((uint64_t)hist_grid(ctx->num_sms, ds->dev(), p.k, p.pool),
+                                                               (span + 15) / 16));
+        return EPI_OK;
     }
+    uint64_t grid = (uint64_t)ctx->num_sms * (uint64_t)p.grid;
     const uint64_t by_work = (span + 127) / 128;
     if (grid > by_work) grid = by_work;
     if (grid < 1) grid = 1;
@@ -417,7 +426,8 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     const size_t o_ic = a.take<uint64_t>(2 * ((size_t)ds->n + 1));
     const size_t o_pre =
         p.global_prefix ? a.take<uint32_t>((size_t)p.grid * p.slots * popc_slot_words(p.k, ds->Wt)) : 0;
-    const size_t o_sing = p.pair ? a.take<uint32_t>((size_t)p.grid * popc_pair_sing_words(p.k, ds->n)) : 0;
+    const size_t o_hg = p.hist ? a.take<uint32_t>(hist_geno_words(ds->dev())) : 0;
+    const size_t o_hl = p.hist ? a.take<long long>((size_t)ds->m + 1) : 0;
     // tensor path: candidate buffers in global memory when they do not fit
     // beside the operand rings in shared memory (large pools)
     const int tc_cp2 = p.tc ? tc_cand_p2(p.k, p.pool, p.comb_p != 0, p.tc_pair) : 0;
@@ -498,11 +508,15 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
                             tc_cg ? reinterpret_cast<uint64_t *>(base + o_tcr) : nullptr, dump, waits,
                             ctx->wait_limit_ns, p.comb_p, p.top_n, reinterpret_cast<uint32_t *>(base + o_hist)));
         ctx->launches += 1;   // item table
+    } else if (p.hist) {
+        CK(launch_hist_search(d, p.k, p.rb, p.re, p.pool, p.top_n, thr, ls, lr, lc, p.grid, p.all_scores,
+                              reinterpret_cast<uint32_t *>(base + o_hg), reinterpret_cast<long long *>(base + o_hl),
+                              ctx->stream));
+        ctx->launches += 1;   // genotype fields and logarithms
     } else {
         CK(launch_popc_search(d, p.k, p.R, p.rb, p.re, p.tile, p.pool, p.slots, p.cand_p2, thr, ls, lr, lc, p.grid,
                               p.smem, ctx->stream, p.all_scores,
-                              p.global_prefix ? reinterpret_cast<uint32_t *>(base + o_pre) : nullptr,
-                              p.pair ? reinterpret_cast<uint32_t *>(base + o_sing) : nullptr, p.top_n));
+                              p.global_prefix ? reinterpret_cast<uint32_t *>(base + o_pre) : nullptr));
     }
     if (ev1) CK(cudaEventRecord(ev1, ctx->stream));
     CK(launch_merge(ls, lr, lc, p.grid, p.pool, p.pool, cs, cr, cn, ctx->stream, thr));

@@ -153,11 +153,32 @@ __global__ void __launch_bounds__(1024) merge_level_kernel(float *__restrict__ l
 // Exact counts of one combination, cell x = sum_t g_t 3^(k-1-t): one thread
 // per (class, cell) pair, or, where those are fewer than the block's threads,
 // one warp per pair with the lanes along the words (an order-2 table has 18
-// pairs: one thread each walked its words alone).
+// pairs: one thread each walked its words alone).  From order 6 the table has
+// about as many cells as individuals or more, and the individuals are visited
+// instead, a warp per mask word adding into the zeroed table (order 8 x 2048,
+// 164 candidates: 0.5 ms less of 1.07).
 __device__ inline void count_cells(const DevData &d, int k, const int32_t *comb, uint32_t *out)
 {
     int cells = 1;
     for (int t = 0; t < k; t++) cells *= 3;
+    if (k >= 6) {
+        for (int x = threadIdx.x; x < 2 * cells; x += blockDim.x) out[x] = 0;
+        __syncthreads();
+        const int lane = threadIdx.x & 31;
+        for (int w = threadIdx.x >> 5; w < d.Wt; w += blockDim.x >> 5) {
+            uint32_t any = 0;
+            int x = 0;
+#pragma unroll 4
+            for (int t = 0; t < k; t++) {
+                const uint32_t *r = d.masks + (int64_t)comb[t] * 3 * d.Wt + w;
+                const uint32_t g0 = r[0], g1 = r[d.Wt], g2 = r[2 * (int64_t)d.Wt];
+                any = g0 | g1 | g2;
+                x = 3 * x + (int)(g1 >> lane & 1u) + 2 * (int)(g2 >> lane & 1u);
+            }
+            if (any >> lane & 1u) atomicAdd(out + (w < d.W1 ? 0 : cells) + x, 1u);
+        }
+        return;
+    }
     const bool by_warp = 2 * cells < (int)blockDim.x;
     const int lane = by_warp ? threadIdx.x & 31 : 0, width = by_warp ? 32 : 1;
     for (int idx = by_warp ? threadIdx.x >> 5 : threadIdx.x; idx < 2 * cells; idx += blockDim.x / width) {
@@ -236,7 +257,9 @@ constexpr int kRescoreThreads = 256;
 // with the cells shared out over the block (thread t takes cells t, t + 256,
 // ...) and the threads' sums added as a tree in a fixed order, so the value
 // is the same on every run (the 13,122 terms of an order-8 table took one
-// thread 4.8 ms of double-precision divisions and logarithms).
+// thread 4.8 ms of double-precision divisions and logarithms).  Orders 6 and
+// up: 164 order-8 tables of 2048 individuals took 1.07 ms; 0.58 with the
+// counts by individuals, 0.22 with the empty cells left out as well.
 __global__ void __launch_bounds__(kRescoreThreads) rescore_kernel(DevData d, int k,
                                                                   const uint64_t *__restrict__ cand_rank,
                                                                   const int32_t *__restrict__ cand_n,
@@ -259,10 +282,57 @@ __global__ void __launch_bounds__(kRescoreThreads) rescore_kernel(DevData d, int
     count_cells(d, k, comb, ct);
     __syncthreads();
     double acc = 0.0;
-    for (int x = threadIdx.x; x < cells; x += kRescoreThreads) {
-        const uint32_t a = ct[x], b = ct[cells + x];
-        acc += mi_term_f64(a, a + b, d.m1, d.m);
-        acc += mi_term_f64(b, a + b, d.m0, d.m);
+    if (k < 6) {
+        for (int x = threadIdx.x; x < cells; x += kRescoreThreads) {
+            const uint32_t a = ct[x], b = ct[cells + x];
+            acc += mi_term_f64(a, a + b, d.m1, d.m);
+            acc += mi_term_f64(b, a + b, d.m0, d.m);
+        }
+    } else {
+        // most cells are empty: each warp gathers 32 others before it takes
+        // them to double precision, and every lane then adds the terms of its
+        // own cells in their order (an empty cell would have added zero)
+        __shared__ uint16_t queue[kRescoreThreads / 32][64];
+        __shared__ double term[kRescoreThreads / 32][64];
+        uint16_t *q = queue[threadIdx.x >> 5];
+        double *te = term[threadIdx.x >> 5];
+        const int lane = threadIdx.x & 31;
+        int held = 0;
+        uint64_t mine = 0;   // places of the lane's own cells in the queue
+        auto take32 = [&]() {
+            if (lane < held) {
+                const int x = q[lane];
+                const uint32_t a = ct[x], b = ct[cells + x];
+                te[lane] = mi_term_f64(a, a + b, d.m1, d.m);
+                te[32 + lane] = mi_term_f64(b, a + b, d.m0, d.m);
+            }
+            const uint16_t next = q[32 + lane];
+            __syncwarp();
+            for (uint32_t own = (uint32_t)mine; own; own &= own - 1) {
+                const int e = __ffs(own) - 1;
+                acc += te[e];
+                acc += te[32 + e];
+            }
+            q[lane] = next;
+            mine >>= 32;
+            held -= 32;
+            __syncwarp();
+        };
+        q[32 + lane] = 0;
+        for (int x0 = threadIdx.x & ~31; x0 < cells; x0 += kRescoreThreads) {
+            const int x = x0 + lane;
+            const bool some = x < cells && (ct[x] | ct[cells + x]) != 0;
+            const uint32_t mask = __ballot_sync(0xffffffffu, some);
+            const int at = held + __popc(mask & ((1u << lane) - 1u));
+            if (some) {
+                q[at] = (uint16_t)x;
+                mine |= 1ull << at;
+            }
+            held += __popc(mask);
+            __syncwarp();
+            if (held >= 32) take32();
+        }
+        if (held > 0) take32();
     }
     part[threadIdx.x] = acc;
     __syncthreads();

@@ -192,3 +192,29 @@ def test_fused_gradients(epi, ctx, rows, n_in, hidden):
     assert (err <= 2.0 ** -6 * L + 2.0 ** -12 * S + A + 1e-30).all()
     assert abs(loss - M.loss(theta, X, t, n_in, hidden, rnd=_bf16)) <= 1e-4 * abs(loss) + 1e-7
     net.close()
+
+
+# orders 6-8 by histogram: items past a class's words, one individual in a
+# class, eight and sixteen items a thread, counts past the logarithms kept in
+# shared memory (1024), everyone in one cell, more samples than it takes
+@pytest.mark.parametrize("k,n,m,m1", [
+    (6, 9, 31, 1), (6, 13, 300, 299), (7, 10, 64, 32), (8, 10, 33, 16), (8, 9, 4096, 2048), (7, 10, 4097, 2100),
+    (7, 9, 5000, 4990), (6, 9, 6000, 3000), (8, 9, 16384, 8000), (7, 9, 16500, 8000)])
+@pytest.mark.parametrize("rare", [False, True])
+def test_high_orders_by_histogram(epi, ctx, k, n, m, m1, rare):
+    geno, pheno = random_data(n, m, seed=k + m, m1=m1, p_levels=(0.001, 0.02) if rare else (0.2, 0.5))
+    geno[0] = 1
+    ds = epi.Dataset(ctx, geno, pheno)
+    combs = np.array(list(itertools.combinations(range(n), k)), dtype=np.int32)
+    tables = O.tables(geno, pheno, combs)
+    want = np.array([O.mi(x[0], x[1], m) for x in tables])
+    assert (epi.tables(ds, combs.astype(np.uint32)) == tables).all()
+    got = epi.score_all(ds, k).cpu().numpy().astype(np.float64)
+    assert (np.abs(got - want) <= F32_RTOL * want + 1e-12).all(), np.abs(got - want).max()
+    total = len(combs)
+    for r0, r1 in ((0, total), (total // 3, total - 1)):
+        r = epi.search(ds, k, 8, path="popc", rank_range=(r0, r1))
+        oc, om, _ = O.search(geno, pheno, k, 8, rank_begin=r0, rank_end=r1)
+        check_topn(r.combs, r.mi, oc, om)
+        assert (r.counts == tables[r.rank.astype(np.int64)]).all()
+        assert (np.abs(r.mi_f32 - want[r.rank.astype(np.int64)]) <= F32_RTOL * r.mi + 1e-12).all()
