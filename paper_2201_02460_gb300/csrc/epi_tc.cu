@@ -533,22 +533,32 @@ __device__ __forceinline__ float tlog(float x) { return x * lg2n(fmaxf(x, 1.0f))
 // t(a) + t(b) - t(a + b) of a cell's counts
 __device__ __forceinline__ float cell_log(float a, float b) { return tlog(a) + tlog(b) - tlog(a + b); }
 
-__device__ __forceinline__ float warp_sum(float v)
+// Compensated sums of the precise scores' terms, over the warp and over a
+// prefix's PR row lanes (with plain sums order 2 was 1.5e-7 off 64 bits, and
+// 3.6e-8 on the popcount path, whose sum is compensated).
+__device__ __forceinline__ float warp_sum(SumF32 v)
 {
 #pragma unroll
-    for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
+    for (int off = 16; off; off >>= 1) {
+        const float s = __shfl_xor_sync(0xffffffffu, v.s, off), c = __shfl_xor_sync(0xffffffffu, v.c, off);
+        v.add(s);
+        v.c += c;
+    }
+    return v.value();
 }
 
 template <int PR>
-__device__ __forceinline__ float seg_sum(float v, int pos)
+__device__ __forceinline__ float seg_sum(SumF32 v, int pos)
 {
 #pragma unroll
     for (int off = 1; off < PR; off <<= 1) {
-        const float o = __shfl_down_sync(0xffffffffu, v, off);
-        if ((pos & (2 * off - 1)) == 0 && pos + off < PR) v += o;
+        const float s = __shfl_down_sync(0xffffffffu, v.s, off), c = __shfl_down_sync(0xffffffffu, v.c, off);
+        if ((pos & (2 * off - 1)) == 0 && pos + off < PR) {
+            v.add(s);
+            v.c += c;
+        }
     }
-    return v;
+    return v.value();
 }
 
 template <int NT>
@@ -661,10 +671,14 @@ __device__ inline void epi_flush(EpiState &S, float *sc, uint64_t *rk, int pool,
 // ---------------------------------------------------------------- kernel --
 // Precise single-precision terms of one tile row's three cells (the rare
 // candidate path, kept out of line).
-__device__ __noinline__ float row_terms_precise(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, uint32_t a2,
-                                                uint32_t b2, const MiConstF32 mc)
+__device__ __noinline__ SumF32 row_terms_precise(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, uint32_t a2,
+                                                 uint32_t b2, const MiConstF32 mc)
 {
-    return cell_terms_f32(a0, b0, mc) + cell_terms_f32(a1, b1, mc) + cell_terms_f32(a2, b2, mc);
+    SumF32 v;
+    v.add(cell_terms_f32(a0, b0, mc));
+    v.add(cell_terms_f32(a1, b1, mc));
+    v.add(cell_terms_f32(a2, b2, mc));
+    return v;
 }
 
 #define TMEM_LD16(taddr, r)                                                                                      \
@@ -1607,7 +1621,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 }
             };
             // precise single-precision terms of this row for column jsel
-            auto row_precise = [&](const uint32_t *cs, const uint32_t *cn, int jsel) -> float {
+            auto row_precise = [&](const uint32_t *cs, const uint32_t *cn, int jsel) -> SumF32 {
                 float a[3] = {}, bb[3] = {};
 #pragma unroll
                 for (int h = 0; h < 4; h++)
@@ -1697,7 +1711,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         if (cold) {
 #pragma unroll 1
                             for (int jj = 0; jj < 8; jj++) {
-                                const float e = warp_sum(prow ? row_precise(cs, cn, jj) : 0.0f);
+                                const float e = warp_sum(prow ? row_precise(cs, cn, jj) : SumF32());
                                 if (lane == jj) v = e;
                             }
                         } else {
@@ -1742,7 +1756,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
 #pragma unroll 1
                         for (int jj = 0; jj < 8; jj++) {
                             if (!wflag[8 * jcg + jj]) continue;
-                            const float e = warp_sum(prow ? row_precise(cs, cn, jj) : 0.0f);
+                            const float e = warp_sum(prow ? row_precise(cs, cn, jj) : SumF32());
                             if (lane == 0) wpre[quad][8 * jcg + jj] = e;
                         }
                     }
@@ -1941,19 +1955,23 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         }
                     }
                     // precise terms of this row for column jsel
-                    auto precise = [&](int jsel) -> float {
+                    auto precise = [&](int jsel) -> SumF32 {
                         uint32_t ca[9], co[9];
                         chunk_counts(jsel, ca, co);
-                        float e = 0.0f;
+                        SumF32 e;
 #pragma unroll 1
-                        for (int x = 0; x < 9; x += 3)
-                            e += row_terms_precise(ca[x], co[x], ca[x + 1], co[x + 1], ca[x + 2], co[x + 2], mc);
+                        for (int x = 0; x < 9; x += 3) {
+                            const SumF32 r =
+                                row_terms_precise(ca[x], co[x], ca[x + 1], co[x + 1], ca[x + 2], co[x + 2], mc);
+                            e.add(r.s);
+                            e.c += r.c;
+                        }
                         return e;
                     };
                     if (cold) {
 #pragma unroll 1
                         for (int jj = 0; jj < kCS; jj++) {
-                            const float e = seg_sum<kPR>(row_in ? precise(jj) : 0.0f, pos);
+                            const float e = seg_sum<kPR>(row_in ? precise(jj) : SumF32(), pos);
                             if (row_in && pos == 0 && jb + jj > D.j1 && jb + jj < (int32_t)d.n)
                                 keep(__fdiv_rn(e, mc.fm), p, jb + jj);
                         }
@@ -1967,7 +1985,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                             const int pair = __ffs(cmask[q]) - 1 + 32 * q;
                             cmask[q] &= cmask[q] - 1;
                             const int pp = pair / kCS, jsel = pair % kCS;
-                            const float e = seg_sum<kPR>(row_in && pl == pp ? precise(jsel) : 0.0f, pos);
+                            const float e = seg_sum<kPR>(row_in && pl == pp ? precise(jsel) : SumF32(), pos);
                             if (row_in && pl == pp && pos == 0) keep(__fdiv_rn(e, mc.fm), p, jb + jsel);
                         }
                     }
@@ -2154,7 +2172,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                         if (prow && pos == 0) last_snp_range<km1>(DS, d, psnp, jlo, jhi);
 #pragma unroll 1
                         for (int jj = 0; jj < 8; jj++) {
-                            const float e = seg_sum<kPR>(prow ? row_precise(cs, cn, jj) : 0.0f, pos);
+                            const float e = seg_sum<kPR>(prow ? row_precise(cs, cn, jj) : SumF32(), pos);
                             if (jb + jj >= jlo && jb + jj < jhi) keep(__fdiv_rn(e, mc.fm), p, jb + jj);
                         }
                         continue;
@@ -2170,9 +2188,9 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                             const int pair = __ffs(cmask[q]) - 1 + 32 * q;
                             cmask[q] &= cmask[q] - 1;
                             const int pp = pair >> 3, jsel = pair & 7;
-                            float e = 0.0f;
-                            if (lane_real && pl == pp) e = row_precise(cs, cn, jsel);
-                            e = seg_sum<kPR>(e, pos);
+                            SumF32 rv;
+                            if (lane_real && pl == pp) rv = row_precise(cs, cn, jsel);
+                            const float e = seg_sum<kPR>(rv, pos);
                             if (lane_real && pl == pp && pos == 0) keep(__fdiv_rn(e, mc.fm), p, jb + jsel);
                         }
                     }
