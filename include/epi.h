@@ -459,10 +459,11 @@ epi_status epi_set_wait_limit(epi_ctx *ctx, uint64_t limit_ns);
 epi_status epi_inject_alloc_failure(epi_ctx *ctx, int64_t after);
 epi_status epi_set_tc_variant(epi_ctx *ctx, int variant);
 
-/* Rate of the tensor pipe for an MMA the tensor-core counting path issues
- * (tcgen05.mma kind::f8f6f4, operands in shared memory, FP32 accumulation):
- * shape 0 = M128 N128 K32 with E4M3 operands (separate-class variant),
- * shape 1 = M128 N256 K32 with E5M2 operands (combined-class variant);
+/* Rate of the tensor pipe for FP8 MMAs (tcgen05.mma kind::f8f6f4, operands in
+ * shared memory, FP32 accumulation; the FP4 MMAs of the counting path retire
+ * twice the multiply-adds per clock):
+ * shape 0 = M128 N128 K32 with E4M3 operands,
+ * shape 1 = M128 N256 K32 with E5M2 operands;
  * EPI_EINVAL for other shapes.  One CTA per SM issues `stages` (32..2^32)
  * groups of four such MMAs back to back from one thread, with no other work.
  * The paper has no counterpart; this is the roofline's denominator.

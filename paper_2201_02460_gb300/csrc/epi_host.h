@@ -137,7 +137,7 @@ cudaError_t launch_tc_batch(const void *ds_dev, const int32_t *cta_ds_dev, int k
                             uint64_t *list_rank, int32_t *list_count, int32_t *status, int grid, cudaStream_t st,
                             float *cand_g, uint64_t *rank_g, bool comb);
 
-// epi_peak.cu: tensor-pipe rate of the counting MMA (one CTA per SM,
+// epi_peak.cu: tensor-pipe rate of FP8 MMAs (one CTA per SM,
 // `stages` groups of four M128 N128 K32 FP8 MMAs; per-CTA cycles)
 size_t mma_rate_smem_bytes(int shape);
 cudaError_t launch_mma_rate(int shape, int64_t stages, unsigned long long *cycles, int32_t *status, int grid,

@@ -1,13 +1,13 @@
-// Rate of the tensor pipe for the counting path's MMA shapes.
+// Rate of the tensor pipe for FP8 MMAs.
 //
 // The paper has no counterpart: this is a measurement aid.  The roofline of
-// the tensor-core counting kernel is the rate at which one SM retires the
-// MMA that kernel issues: tcgen05.mma.kind::f8f6f4 M128 N128 K32 with E4M3
-// operands (shape 0, the separate-class variant) or M128 N256 K32 with E5M2
-// operands (shape 1, the combined-class variant), FP32 accumulation, both
-// operands in shared memory in the 128-byte swizzle.  One CTA per SM issues
-// that MMA back to back from one thread, accumulating 32 K steps into one of
-// two tensor-memory accumulators in turn (the counting kernel's pattern),
+// the tensor-core counting kernel is twice the rate at which one SM retires
+// these MMAs (its kind::mxf4 retires 16384 multiply-adds per SM clock, the FP8
+// kinds 8192, both measured): tcgen05.mma.kind::f8f6f4 M128 N128 K32 with E4M3
+// operands (shape 0) or M128 N256 K32 with E5M2 operands (shape 1), FP32
+// accumulation, both operands in shared memory in the 128-byte swizzle.  One
+// CTA per SM issues that MMA back to back from one thread, accumulating 32 K
+// steps into one of two tensor-memory accumulators in turn (as the counting kernel does),
 // with no other work on the SM; the operands are zero tiles (the rate does
 // not depend on the values).  Every CTA records the SM
 // cycles of its issue loop up to the completion of its last MMA; the host

@@ -16,7 +16,7 @@
 //   variant 2  binary MMA: mma.sync m16n8k256 with AND + POPC on the
 //              tensor cores (16 prefix rows x 4 last SNPs x 2 genotypes per
 //              instruction, 256 individuals deep).
-// The tensor-core FP8 0/1 GEMM (epi_tc.cu) is the fourth way and is timed by
+// The tensor-core 0/1 GEMM (epi_tc.cu) is the fourth way and is timed by
 // the search itself.  Each kernel folds every count into a checksum that
 // does not depend on the order of the work, and can also write every table.
 #include <cuda_runtime.h>
