@@ -919,12 +919,15 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
             st = ensure_b4(it.ds);
             if (st != EPI_OK) return st;
         }
-    // graph key: datasets, orders, sizes, path
+    // graph key: datasets, orders, sizes, path, and what each dataset's route
+    // depends on beside them (the autotuner's choices, memory for the operand):
+    // the places of the results follow from it
     std::vector<uint64_t> key;
     key.push_back((uint64_t)path | (ctx->tc_combined ? 1ull << 32 : 0));
     for (auto &it : items) {
         key.push_back(it.ds->id);
         key.push_back((uint64_t)it.k << 32 | (uint64_t)it.top_n);
+        key.push_back((uint64_t)it.comb_p << 2 | (uint64_t)it.tc << 1 | (uint64_t)it.alone);
     }
     char *dev = static_cast<char *>(ctx->batch_dev);
     char *host = static_cast<char *>(ctx->batch_host);

@@ -194,6 +194,28 @@ def test_fused_gradients(epi, ctx, rows, n_in, hidden):
     net.close()
 
 
+# the autotuner's choice moves a study between the batch's launches and a
+# search of its own: the same batch before and after
+def test_batch_after_new_choices(epi, tmp_path):
+    own = epi.Context(0)
+    sets = [epi.Dataset(own, *random_data(n, 300, seed=n)) for n in (60, 20, 50)]
+    orders = [4, 3, 4]
+    want = [epi.search(s, k, 20, path="popc") for s, k in zip(sets, orders)]
+    epi.autotune(sets[0], 4)
+    file = str(tmp_path / "tune.txt")
+    epi.tune_save(own, file)
+    with open(file) as f:
+        lines = [x.split() for x in f.read().splitlines() if x and x[0] != "#"]
+    for path in (2, 1, 2):
+        with open(file, "w") as f:
+            f.writelines(" ".join(x[:4] + [str(path)] + x[5:]) + "\n" for x in lines)
+        epi.tune_load(own, file)
+        for _ in range(2):
+            for a, b in zip(epi.search_batched(own, sets, orders, [20] * 3), want):
+                _same(a, b)
+    own.close()
+
+
 # orders 6-8 by histogram: items past a class's words, one individual in a
 # class, eight and sixteen items a thread, counts past the logarithms kept in
 # shared memory (1024), everyone in one cell, more samples than it takes
