@@ -14,7 +14,12 @@
 //     m MI = sum_i [ln own_i - ln n_i] + m ln m - m1 ln m1 - m0 ln m0,
 // with ln from a table in fixed point (2^-44), so the sum is exact in any
 // order and the score is rounded once, to FP32: its error is at most
-// 2^-24 MI + 2^-44.
+// 2^-24 MI + 2^-43 (the logarithms' roundings, at most two units an
+// individual).  Below an MI of 2^-19, where the second part would be the larger
+// (balanced or nearly constant genotypes; the margin of the exact top N needs
+// a relative bound, and an MI of zero has to score zero), the combination is
+// counted again and its cells scored in the cancellation-free form, in double
+// precision.
 //
 // What bounds it is shared memory: per individual one atomic add, a read and a
 // clear at scattered cells (about 3.5 wavefronts a warp) and two reads of the
@@ -106,7 +111,7 @@ struct State {
     int64_t rank;                    // of the combination (prefix, last)
     int32_t pre[kMaxOrderGpu];
     int32_t last, from;              // the prefix's first last SNP here; first changed place
-    int32_t list_len, nbuf, done, published;
+    int32_t list_len, nbuf, done, published, small;
     float thr;
 };
 
@@ -133,6 +138,26 @@ __device__ inline void flush(State &S, float *sc, uint64_t *rk, const Params &P)
         }
     }
     __syncthreads();
+}
+
+// MI of the block's table in double precision, without cancellation: the cells
+// shared out over the threads, the sums added in a fixed order.  Out of line,
+// so that its registers are not the counting loop's.
+__device__ __noinline__ double precise_mi(const uint32_t *tab, int cells, int64_t m1, int64_t m0, int64_t m,
+                                          long long *part)
+{
+    double x = 0.0;
+    for (int c = threadIdx.x; c < cells; c += blockDim.x) {
+        const uint32_t a = tab[c] >> 16, n = a + (tab[c] & 0xffffu);
+        x += mi_term_f64(a, n, m1, m);
+        x += mi_term_f64(n - a, n, m0, m);
+    }
+    for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = __double_as_longlong(x);
+    __syncthreads();
+    x = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); w++) x += __longlong_as_double(part[w]);
+    return x / (double)m;
 }
 
 template <int K, int kItems>
@@ -179,6 +204,7 @@ __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1)
     }
     const long long base = d.m * P.ln[d.m] - d.m1 * P.ln[d.m1] - d.m0 * P.ln[d.m0];
     const double scale = 1.0 / ((double)d.m * kLnScale);
+    const long long small = (long long)d.m << 25;   // an MI of 2^-19
     uint32_t c6[kItems], c7[kItems];   // byte offsets of the first K-2 and K-1 SNPs' cells, times 3
 #pragma unroll
     for (int i = 0; i < kItems; i++) c6[i] = c7[i] = 0;
@@ -209,6 +235,14 @@ __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1)
         const int j0 = S.last;
         const int nj = (int)min((int64_t)(d.n - j0), R_e - r0);
         geno(j0, g);
+        auto record = [&](float score, int jj) {
+            if (P.all_scores) P.all_scores[r0 + jj - (int64_t)P.rank_begin] = score;
+            if (score >= S.thr) {
+                const int pos = S.list_len + S.nbuf++;
+                sc[pos] = score;
+                rk[pos] = (uint64_t)(r0 + jj);
+            }
+        };
 #pragma unroll 1
         for (int jj = 0; jj < nj; jj++) {
             uint32_t at[kItems];
@@ -246,15 +280,25 @@ __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1)
             if (t == 0) {
                 long long sum = base;
                 for (int w = 0; w < warps; w++) sum += part[w];
-                const float score = sum > 0 ? (float)((double)sum * scale) : 0.0f;
-                if (P.all_scores) P.all_scores[r0 + jj - (int64_t)P.rank_begin] = score;
-                if (score >= S.thr) {
-                    const int pos = S.list_len + S.nbuf++;
-                    sc[pos] = score;
-                    rk[pos] = (uint64_t)(r0 + jj);
-                }
+                S.small = sum < small;
+                if (sum >= small) record((float)((double)sum * scale), jj);
             }
             __syncthreads();
+            if (S.small) {
+                uint32_t again[kWords];
+                geno(j0 + jj, again);
+#pragma unroll
+                for (int i = 0; i < kItems; i++) {
+                    at[i] = c7[i] + (again[i / 8] >> (4 * (i % 8)) & 12u);
+                    atomicAdd(reinterpret_cast<uint32_t *>(tab + at[i]), inc);
+                }
+                __syncthreads();
+                const double mi = precise_mi(reinterpret_cast<const uint32_t *>(tab), kCells, d.m1, d.m0, d.m, part);
+#pragma unroll
+                for (int i = 0; i < kItems; i++) *reinterpret_cast<uint32_t *>(tab + at[i]) = 0;
+                if (t == 0) record((float)mi, jj);
+                __syncthreads();
+            }
             if (S.nbuf == kBuffer || (!S.published && P.top_n > 0 && S.list_len + S.nbuf >= P.top_n)) {
                 flush(S, sc, rk, P);
                 if (t == 0 && S.list_len >= P.top_n) S.published = 1;

@@ -240,3 +240,34 @@ def test_high_orders_by_histogram(epi, ctx, k, n, m, m1, rare):
         check_topn(r.combs, r.mi, oc, om)
         assert (r.counts == tables[r.rank.astype(np.int64)]).all()
         assert (np.abs(r.mi_f32 - want[r.rank.astype(np.int64)]) <= F32_RTOL * r.mi + 1e-12).all()
+
+
+# controls that repeat the cases' genotypes `copies` times: every score is
+# zero, and rank order decides (for these sizes the fixed-point logarithms
+# leave a positive remainder)
+@pytest.mark.parametrize("k,n,cases,copies", [(6, 16, 70, 2), (7, 16, 70, 2), (8, 16, 42, 4)])
+def test_high_orders_without_association(epi, ctx, k, n, cases, copies):
+    half, _ = random_data(n, cases, seed=k)
+    geno = np.concatenate([half] * (1 + copies), axis=1)
+    pheno = (np.arange(geno.shape[1]) < cases).astype(np.uint8)
+    ds = epi.Dataset(ctx, geno, pheno)
+    r = epi.search(ds, k, 10, path="popc")
+    assert (r.mi == 0).all() and (r.mi_f32 == 0).all()
+    assert (r.rank == np.arange(10)).all()
+    assert float(epi.score_all(ds, k).abs().max()) == 0.0
+    ds.close()
+
+
+# one SNP with a single individual's difference between the classes, the
+# others constant: scores far below 2^-19 keep their relative accuracy
+@pytest.mark.parametrize("k,m", [(6, 3000), (7, 8000), (8, 8000), (8, 16000)])
+def test_high_orders_smallest_scores(epi, ctx, k, m):
+    geno = np.zeros((k + 1, m), np.uint8)
+    geno[3, :m // 4 + 1] = 1
+    geno[3, m // 2:m // 2 + m // 4] = 1
+    pheno = (np.arange(m) < m // 2).astype(np.uint8)
+    ds = epi.Dataset(ctx, geno, pheno)
+    r = epi.search(ds, k, k + 1, path="popc")
+    assert (r.mi[:k] > 0).all() and r.mi[k] == 0
+    assert (np.abs(r.mi_f32 - r.mi) <= F32_RTOL * r.mi).all()
+    ds.close()
