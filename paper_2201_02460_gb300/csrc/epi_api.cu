@@ -1381,7 +1381,7 @@ epi_status epi_score_all(epi_dataset *ds, int order, float *out_dev)
                                 reinterpret_cast<uint32_t *>(base + o_thr), reinterpret_cast<int32_t *>(base + o_lc),
                                 reinterpret_cast<int32_t *>(base + o_status), grid, total, ctx->stream,
                                 ctx->wait_limit_ns, comb_p));
-            ctx->launches += 3;
+            ctx->launches += 4;
             int32_t bits = 0;
             CK(cudaMemcpyAsync(&bits, base + o_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
             CK(cudaStreamSynchronize(ctx->stream));

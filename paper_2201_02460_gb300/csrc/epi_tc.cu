@@ -2037,7 +2037,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 // in shared memory as integers of 2^-46, so the sum is exact
                 // and the score's error is the two roundings to float (the
                 // popcount path's per-term series takes ten times the
-                // instructions: order 4, 200 x 2000, 177 ms)
+                // instructions: order 4, 200 x 2000, 177 ms); the scores too
+                // small for the table are made again (small_scores_kernel)
                 auto score_chunk = [&](int32_t jb, const uint32_t *cs, const uint32_t *cn) {
                     long long *w64 = reinterpret_cast<long long *>(wb);
                     const int pp = kPPW > 1 ? lane >> 2 : 0;
@@ -2383,6 +2384,58 @@ __global__ void tlog_kernel(int64_t m, long long *__restrict__ out)
 {
     for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c <= m; c += (int64_t)gridDim.x * blockDim.x)
         out[c] = c > 0 ? __double2ll_rn((double)c * log((double)c) * 70368744177664.0) : 0;   // 2^46
+}
+
+// The scores of a whole table of scores that are small beside the errors of
+// the sums of n ln n, made again in the cancellation-free form in double
+// precision.  Half a unit of 2^-46 for each entry and a last place of each
+// double-precision product add up to less than m ln m / 16 + 123 units, so
+// scores from 2^24 times that (an MI of 1e-7 at 3000 individuals) keep their
+// accuracy; below are combinations with hardly any association, or none,
+// whose score has to be zero.  A warp looks through 32 scores at a time and
+// takes a small one together, its lanes over the words; there are none in an
+// ordinary study, so what bounds it is one read of the scores (order 4, 200
+// SNPs: 259 MB).
+__host__ __device__ inline float small_score_limit(int64_t m)
+{
+    const double units = (double)m * log((double)m) / 16.0 + 123.0;
+    return (float)(units * 16777216.0 / 70368744177664.0 / (double)m);
+}
+
+__global__ void __launch_bounds__(256) small_scores_kernel(DevData d, int k, uint64_t total, float limit,
+                                                           float *__restrict__ scores)
+{
+    const int lane = threadIdx.x & 31;
+    const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+    int cells = 1;
+    for (int t = 0; t < k; t++) cells *= 3;
+    for (uint64_t r0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); r0 < total; r0 += step) {
+        uint32_t todo = __ballot_sync(0xffffffffu, r0 + lane < total && scores[r0 + lane] < limit);
+        for (; todo; todo &= todo - 1) {
+            const uint64_t r = r0 + __ffs(todo) - 1;
+            int32_t comb[kMaxOrderGpu];
+            unrank_lex(d.binom, d.n, k, r, comb);
+            double mine = 0.0;
+            for (int x0 = 0; x0 < cells; x0 += 32) {
+                uint32_t a = 0, b = 0;   // counts of cell x0 + lane
+                for (int x = x0; x < min(cells, x0 + 32); x++) {
+                    uint32_t ca = 0, cb = 0;
+                    for (int w = lane; w < d.Wt; w += 32) {
+                        uint32_t bits = 0xffffffffu;
+                        for (int q = k - 1, y = x; q >= 0; q--, y /= 3)
+                            bits &= d.masks[((int64_t)comb[q] * 3 + y % 3) * d.Wt + w];
+                        (w < d.W1 ? ca : cb) += __popc(bits);
+                    }
+                    ca = __reduce_add_sync(0xffffffffu, ca);
+                    cb = __reduce_add_sync(0xffffffffu, cb);
+                    if (lane == x - x0) { a = ca; b = cb; }
+                }
+                mine += mi_term_f64(a, a + b, d.m1, d.m) + mi_term_f64(b, a + b, d.m0, d.m);
+            }
+            for (int off = 16; off; off >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, off);
+            if (lane == 0) scores[r] = (float)(mine / (double)d.m);
+        }
+    }
 }
 
 // The producers' masks: the 256 individuals of a K stage of every SNP's three
@@ -2819,8 +2872,11 @@ cudaError_t launch_tc_scores(const DevData &d, int k, const unsigned char *b4, u
     P.wait_ns = wait_ns;
     cudaError_t e = launch_tc_item_cum(d, k, 0, total, item_cum, st, comb_p != 0);
     if (e == cudaSuccess) e = encode_map(&map, d, b4, comb_p != 0);
+    if (e == cudaSuccess) e = launch_kernel(map, P, k, grid, st, comb_p != 0);
     if (e != cudaSuccess) return e;
-    return launch_kernel(map, P, k, grid, st, comb_p != 0);
+    tc::small_scores_kernel<<<(unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)grid * 8), 256, 0, st>>>(
+        d, k, total, tc::small_score_limit(d.m), scores);
+    return cudaGetLastError();
 }
 
 size_t tc_ds_bytes() { return sizeof(tc::DsParams); }

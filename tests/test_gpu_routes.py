@@ -258,6 +258,29 @@ def test_high_orders_without_association(epi, ctx, k, n, cases, copies):
     ds.close()
 
 
+# the same at orders 3 and 4 (every score from the table of n ln n, which
+# leaves up to 19 of its units here), and one SNP whose classes differ by one
+# individual: scores far below the table's accuracy
+@pytest.mark.parametrize("k", [3, 4])
+@pytest.mark.parametrize("cases,copies", [(70, 2), (42, 4), (101, 1)])
+def test_score_tables_without_association(epi, ctx, k, cases, copies):
+    half, _ = random_data(9, cases, seed=k)
+    geno = np.concatenate([half] * (1 + copies), axis=1)
+    pheno = (np.arange(geno.shape[1]) < cases).astype(np.uint8)
+    ds = epi.Dataset(ctx, geno, pheno)
+    assert float(epi.score_all(ds, k).abs().max()) == 0.0
+    geno = np.zeros((9, 2990), np.uint8)
+    geno[3, :700] = 1
+    geno[3, 1495:2194] = 1
+    ds.close()
+    ds = epi.Dataset(ctx, geno, (np.arange(2990) < 1495).astype(np.uint8))
+    got = epi.score_all(ds, k).cpu().numpy()
+    want = np.array([epi.search(ds, k, 1, path="popc", rank_range=(r, r + 1)).mi[0] for r in range(math.comb(9, k))])
+    assert (want > 0).sum() == math.comb(8, k - 1)
+    assert (np.abs(got - want) <= F32_RTOL * want).all()
+    ds.close()
+
+
 # one SNP with a single individual's difference between the classes, the
 # others constant: scores far below 2^-19 keep their relative accuracy
 @pytest.mark.parametrize("k,m", [(6, 3000), (7, 8000), (8, 8000), (8, 16000)])
