@@ -422,6 +422,14 @@ def tc_executed_flops(d, k):
     return 2.0 * cols * 128 * kt
 
 
+def tc_pair_executed_flops(d, k):
+    """The same with pair tiles (orders 4-5 from 40 and 24 SNPs): 128 rows of
+    12 or 4 prefixes and four columns a pair, and the single counts' pass one
+    order lower; tile edges left out."""
+    kt = 128 * (-(-d.n_cases // 128) + -(-(d.n_samples - d.n_cases) // 128))
+    return 2.0 * math.comb(d.n_snps, k) * 128 / (12 if k == 4 else 4) * 4 * kt + tc_executed_flops(d, k - 1)
+
+
 def roofline(kind, d, k, kern_ms, peaks, tc_rate=None, hist=False):
     total = math.comb(d.n_snps, k)
     if kind == "tc":
@@ -430,7 +438,8 @@ def roofline(kind, d, k, kern_ms, peaks, tc_rate=None, hist=False):
         # columns of the last SNP, padded rows and K)
         flops = 2.0 * total * (3 ** k) * d.n_samples
         achieved = flops / (kern_ms / 1e3) / 1e12
-        executed = tc_executed_flops(d, k) / (kern_ms / 1e3) / 1e12
+        executed = (tc_pair_executed_flops(d, k) if k >= 4 and d.n_snps >= (40 if k == 4 else 24) else
+                    tc_executed_flops(d, k)) / (kern_ms / 1e3) / 1e12
         fp4_conv = FP4_OVER_BF16 * peaks["bf16"]
         comb = class_shift(d) != 0
         if tc_rate:

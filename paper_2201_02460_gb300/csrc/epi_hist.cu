@@ -23,9 +23,10 @@
 //
 // What bounds it is shared memory: per individual one atomic add, a read and a
 // clear at scattered cells (about 3.5 wavefronts a warp) and two reads of the
-// logarithms.  23 x 2048 at order 8, 490314 combinations: 2.35 ms, where the
+// logarithms.  23 x 2048 at order 8, 490314 combinations: 2.38 ms (shared-memory
+// data pipe 80 % of its peak; 2.35 without the recount of small scores), where the
 // bitwise kernel on prefix tables took 35 ms; 3.8 ms with 98 registers a
-// thread instead of 62 (two CTAs an SM instead of four) and a predicate per
+// thread instead of 64 (two CTAs an SM instead of four) and a predicate per
 // item for the places without an individual.
 //
 // GPU mapping: persistent CTAs with contiguous rank ranges, one table (4-byte
