@@ -499,7 +499,7 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
             CK(launch_tc_pair_search(d, p.k, ds->b4, ws, p.pool, thr, ls, lr, lc, status, p.grid, p.total, ctx->stream,
                                      reinterpret_cast<float *>(base + o_tcs), reinterpret_cast<uint64_t *>(base + o_tcr),
                                      dump, waits, ctx->wait_limit_ns, p.comb_p, p.top_n,
-                                     reinterpret_cast<uint32_t *>(base + o_hist), TcCollect{}));
+                                     reinterpret_cast<uint32_t *>(base + o_hist)));
             ctx->launches += 3;
         } else
         CK(launch_tc_search(d, p.k, ds->b4, ic, p.pool, thr, ls, lr, lc, status, p.grid,
@@ -1128,7 +1128,7 @@ namespace {
 
 // Ranks of every combination whose single-precision score is at least thr
 // (> 0), found by the tensor path, appended to cand in any order; *n_dev
-// counts them (more than cap: the pass gave up).  The dataset's operand and
+// counts them (more than cap: the pass ended there, with no error).  The dataset's operand and
 // the pass's buffers are in place when this returns; the work is queued.
 epi_status queue_collect(epi_dataset *ds, int order, uint64_t total, float thr, uint64_t *cand, uint64_t cap,
                          unsigned long long *n_dev, int32_t **status_out)
@@ -1290,7 +1290,7 @@ epi_status epi_search_threshold(epi_dataset *ds, int order, double threshold, in
             TCK(cudaStreamSynchronize(sm));
             done = nc <= cand_cap;
         }
-        if (done && bits != 0) {
+        if (bits != 0) {
             cleanup();
             return bits & ST_TIMEOUT ? fail(EPI_ETIMEOUT, "device wait expired")
                                      : fail(EPI_ECUDA, "device status 0x%x", bits);

@@ -117,7 +117,7 @@ cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *
                                   uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                                   int32_t *status, int grid, uint64_t total, cudaStream_t st, float *cand_g,
                                   uint64_t *rank_g, uint32_t *dump, unsigned long long *waits,
-                                  unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist, TcCollect collect);
+                                  unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist);
 // Every score of an order-3 or -4 dataset by rank (tlog: device [m + 1] work
 // space), where the shared memory suffices
 size_t tc_scores_smem_bytes(const DevData &d, bool comb);

@@ -181,7 +181,7 @@ struct Params {
     int32_t *status;
     float *scores;                // orders 3-4: every combination's score, by rank (nothing is kept)
     const long long *tlog;        // with scores: n ln n 2^46 for n = 0 .. m, rounded
-    TcCollect collect;            // ranks != NULL: every combination at or above its threshold instead of the best
+    TcCollect collect;            // of a collecting launch
     unsigned long long wait_ns;   // limit of the pipeline waits (0: kTimeoutNs)
     uint32_t *dump;            // optional: every table, [rank][2][3^k] (validation)
     unsigned long long *waits; // optional: [grid][8] cycles spent waiting, per role (tracing)
@@ -193,6 +193,9 @@ struct Params {
 // kTimeoutNs, so that no asynchronous copy or MMA is outstanding when the CTA
 // leaves.
 __shared__ unsigned long long g_wait_limit_ns;
+// The item at which every role ends, set where a collecting pass has found
+// more than the caller's array holds (none: ~0).
+__shared__ volatile uint32_t g_end_item;
 
 // Bounded wait for the phase of parity `parity`; false when it gave up (the
 // CTA-wide abort flag is then set).
@@ -208,6 +211,23 @@ __device__ __noinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile 
             *abort_flag = 1;
             return false;
         }
+    }
+}
+
+// The wait for an item's descriptor; in a collecting pass also false when the
+// pass ends at that item.
+template <bool COLLECT>
+__device__ __forceinline__ bool wait_desc(uint64_t *bar, uint32_t parity, volatile int *abort_flag, int64_t item)
+{
+    if constexpr (COLLECT) {
+        const uint64_t t0 = now_ns();
+        while (!mbar_try(bar, parity)) {
+            if (now_ns() - t0 > g_wait_limit_ns) *abort_flag = 1;
+            if (*abort_flag || g_end_item == (uint32_t)item) return false;
+        }
+        return true;
+    } else {
+        return mbar_wait(bar, parity, abort_flag);
     }
 }
 
@@ -244,15 +264,17 @@ __device__ __forceinline__ bool wait_fast(uint64_t *bar, uint32_t parity, volati
 
 // The issuing warp's wait, inline: a function call in its loop would keep
 // every value that lives across it out of the uniform registers the MMAs take
-// their operands from.
-__device__ __forceinline__ bool wait_inline(uint64_t *bar, uint32_t parity, volatile int *abort_flag, long long &acc)
+// their operands from.  In a collecting pass also false when it ends at `item`.
+template <bool COLLECT>
+__device__ __forceinline__ bool wait_inline(uint64_t *bar, uint32_t parity, volatile int *abort_flag, long long &acc,
+                                            uint32_t item)
 {
     const long long t0 = clock64();
     const uint64_t n0 = now_ns();
     bool ok = true;
     while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
         if (now_ns() - n0 > g_wait_limit_ns) *abort_flag = 1;
-        if (__any_sync(0xffffffffu, *abort_flag)) {
+        if (__any_sync(0xffffffffu, *abort_flag || (COLLECT && g_end_item == item))) {
             ok = false;
             break;
         }
@@ -928,7 +950,11 @@ __device__ __forceinline__ void last_snp_range(const DsParams &DS, const DevData
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) \
                  : "r"(taddr))
 
-template <int K, bool C, bool PAIR>
+// COLLECT: every combination that scores at least a threshold instead of the
+// best (a kernel of its own: its end in mid-pass, as branches of the search's
+// kernel, cost that 0.7 % at order 3, 2000 x 4000, and 1.2 % at order 5,
+// 93 x 2001)
+template <int K, bool C, bool PAIR, bool COLLECT>
 __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __grid_constant__ CUtensorMap tmap_b,
                                                                 const Params P)
 {
@@ -994,6 +1020,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
     // with the item's descriptor
     __shared__ uint32_t item_idesc[kDescDepth];
     __shared__ volatile int abort_flag;
+    __shared__ volatile int over_flag;               // COLLECT: more found than the caller's array holds
     __shared__ EpiState ES;
     __shared__ uint32_t hist_tmp[kEpiWarps + 1];
     // order 5: per-quadrant sums of the item's last SNPs, and their flags
@@ -1037,9 +1064,13 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         }
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
+        if constexpr (COLLECT) {
+            over_flag = 0;
+            g_end_item = ~0u;
+        }
         g_wait_limit_ns = P.wait_ns ? P.wait_ns : kTimeoutNs;
         ES.list_len = 0; ES.nbuf = 0; ES.stop = 0; ES.any = 0; ES.seen = 0;
-        ES.thr = ES.next_thr = P.collect.ranks ? P.collect.thr : -1.0f;
+        ES.thr = ES.next_thr = COLLECT ? P.collect.thr : -1.0f;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == kWarpMma) {
@@ -1136,9 +1167,19 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 }
             };
             fill_tile();
-            // item i's descriptor, and the operand row its N tile starts at
+            // item i's descriptor, and the operand row its N tile starts at.
+            // Once a collecting epilogue has found too many there is none:
+            // every role ends at this item, all stages before it taken (an
+            // abort instead would leave this warp's last loads to barriers
+            // that the producers no longer reach, two seconds a stage)
             int y_next = 0;
             auto write_desc = [&](int64_t i) -> bool {
+                if constexpr (COLLECT) {
+                    if (__any_sync(0xffffffffu, over_flag)) {
+                        g_end_item = (uint32_t)i;
+                        return false;
+                    }
+                }
                 const int dq = (int)(i % kDescDepth);
                 const uint32_t ud = (uint32_t)(i / kDescDepth);
                 if (!__all_sync(0xffffffffu, mbar_wait(&desc_empty[dq], (ud & 1) ^ 1, &abort_flag))) return false;
@@ -1256,7 +1297,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             const long long t_start = clock64();
             auto next_acc = [&](uint32_t &col) -> bool {
                 if (!__all_sync(0xffffffffu, mbar_test(&acc_empty[ab], aph ^ 1)) &&
-                    !wait_inline(&acc_empty[ab], aph ^ 1, &abort_flag, w_acc))
+                    !wait_inline<false>(&acc_empty[ab], aph ^ 1, &abort_flag, w_acc, 0))
                     return false;
                 tc_fence_after();
                 col = tb + (uint32_t)(ab * S::N);
@@ -1270,7 +1311,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                 bool ok = true;
                 for (int st = 0; st < u_nst; st++) {
                     if (!__all_sync(0xffffffffu, ready)) {
-                        ok = wait_inline(&full_ab[s], ph, &abort_flag, w_a);
+                        ok = wait_inline<COLLECT>(&full_ab[s], ph, &abort_flag, w_a, i);
                         if (!ok) break;
                     }
                     tc_fence_after();
@@ -1355,7 +1396,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             if (abort_flag) break;
             const int dq = (int)(i % kDescDepth);
             const uint32_t ud = (uint32_t)(i / kDescDepth);
-            if (!mbar_wait(&desc_full[dq], ud & 1, &abort_flag)) break;
+            if (!wait_desc<COLLECT>(&desc_full[dq], ud & 1, &abort_flag, i)) break;
             const Desc &D = desc[dq];
             // the row's SNP rows at stage 0; rows of no prefix read the zero
             // rows kept past the last SNP
@@ -1512,7 +1553,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             const uint32_t ud = (uint32_t)(i / kDescDepth);
             const int b = (int)(i & 1);
             const uint32_t ub = (uint32_t)(i >> 1);
-            bool ok = mbar_wait(&desc_full[dq], ud & 1, &abort_flag);
+            bool ok = wait_desc<COLLECT>(&desc_full[dq], ud & 1, &abort_flag, i);
             ok = ok && wait_fast(&acc_full[b], ub & 1, &abort_flag, w_epi);
             ok = ok && wait_fast(&tot_full[b], ub & 1, &abort_flag, w_epi);
             ok = __all_sync(0xffffffffu, ok);
@@ -1574,9 +1615,12 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             auto refresh = [&]() {
                 if (tid == 0) {
                     ES.next_thr = gthr > 0.0f ? fmaxf(ES.thr, gthr) : ES.thr;
-                    // more than the caller's array holds: give up
-                    if (P.collect.ranks && *(volatile unsigned long long *)P.collect.n > P.collect.cap) abort_flag = 1;
                     ES.stop = abort_flag;
+                    if constexpr (COLLECT) {
+                        // more than the caller's array holds: no further descriptors
+                        if (*(volatile unsigned long long *)P.collect.n > P.collect.cap) over_flag = 1;
+                        if (g_end_item == (uint32_t)i) ES.stop = 1;
+                    }
                 }
             };
             // one chunk's accumulators (queued): last SNPs j0 + kCS jcg ..
@@ -1637,15 +1681,15 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     for (int tt = 0; tt < km1; tt++) qs[tt] = D.snp[pt * km1 + tt];
                     uint64_t rank = DS.total - 1 - prefix_rank_sum<km1>(d, qs, K) - (uint64_t)(d.n - 1 - j);
                     if constexpr (PAIR) rank -= binom_at(d.binom, d.n, d.n - 1 - D.j1, 2);
-                    if (P.collect.ranks) {
+                    if constexpr (COLLECT) {
                         const unsigned long long at = atomicAdd(P.collect.n, 1ull);
                         if (at < P.collect.cap) P.collect.ranks[at] = rank;
-                        return;
+                    } else {
+                        const int slot = list_len + atomicAdd(&ES.nbuf, 1);
+                        if (DS.top_n > 0) atomicAdd(DS.hist + hist_bin(score), 1u);
+                        sc[slot] = score;
+                        rk[slot] = rank;
                     }
-                    const int slot = list_len + atomicAdd(&ES.nbuf, 1);
-                    if (DS.top_n > 0) atomicAdd(DS.hist + hist_bin(score), 1u);
-                    sc[slot] = score;
-                    rk[slot] = rank;
                 }
             };
             // the threshold of everything kept so far, by all CTAs
@@ -2746,20 +2790,24 @@ static void fill_launch(tc::Params &P, int k, int pool, float *list_score, uint6
 }
 
 static cudaError_t launch_kernel(const CUtensorMap &map, const tc::Params &P, int k, int grid, cudaStream_t st,
-                                 bool comb, bool pair = false)
+                                 bool comb, bool pair = false, bool collect = false)
 {
     const size_t smem = tc_smem_bytes(P.cand_p2, P.cand_score_g != nullptr, comb) +
                         (P.scores ? (size_t)(P.one.d.m + 1) * 8 : 0);
     using Kernel = void (*)(const CUtensorMap, const tc::Params);
-    static const Kernel kernels[2][4] = {
-        {tc::tc_search_kernel<2, false, false>, tc::tc_search_kernel<3, false, false>,
-         tc::tc_search_kernel<4, false, false>, tc::tc_search_kernel<5, false, false>},
-        {tc::tc_search_kernel<2, true, false>, tc::tc_search_kernel<3, true, false>,
-         tc::tc_search_kernel<4, true, false>, tc::tc_search_kernel<5, true, false>}};
+    static const Kernel kernels[2][2][4] = {
+        {{tc::tc_search_kernel<2, false, false, false>, tc::tc_search_kernel<3, false, false, false>,
+          tc::tc_search_kernel<4, false, false, false>, tc::tc_search_kernel<5, false, false, false>},
+         {tc::tc_search_kernel<2, true, false, false>, tc::tc_search_kernel<3, true, false, false>,
+          tc::tc_search_kernel<4, true, false, false>, tc::tc_search_kernel<5, true, false, false>}},
+        {{tc::tc_search_kernel<2, false, false, true>, tc::tc_search_kernel<3, false, false, true>,
+          tc::tc_search_kernel<4, false, false, true>, tc::tc_search_kernel<5, false, false, true>},
+         {tc::tc_search_kernel<2, true, false, true>, tc::tc_search_kernel<3, true, false, true>,
+          tc::tc_search_kernel<4, true, false, true>, tc::tc_search_kernel<5, true, false, true>}}};
     static const Kernel pair_kernels[2][2] = {
-        {tc::tc_search_kernel<4, false, true>, tc::tc_search_kernel<5, false, true>},
-        {tc::tc_search_kernel<4, true, true>, tc::tc_search_kernel<5, true, true>}};
-    const Kernel kern = pair ? pair_kernels[comb][k - 4] : kernels[comb][k - 2];
+        {tc::tc_search_kernel<4, false, true, false>, tc::tc_search_kernel<5, false, true, false>},
+        {tc::tc_search_kernel<4, true, true, false>, tc::tc_search_kernel<5, true, true, false>}};
+    const Kernel kern = pair ? pair_kernels[comb][k - 4] : kernels[collect][comb][k - 2];
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, tc::Roles::Threads, smem, st>>>(map, P);
@@ -2794,7 +2842,7 @@ cudaError_t launch_tc_search(const DevData &d, int k, const unsigned char *b4, u
     CUtensorMap map;
     e = encode_map(&map, d, b4, comb_p != 0);
     if (e != cudaSuccess) return e;
-    return launch_kernel(map, P, k, grid, st, comb_p != 0);
+    return launch_kernel(map, P, k, grid, st, comb_p != 0, false, collect.ranks != nullptr);
 }
 
 // The same search with pair tiles (whole range): ws holds tc_pair_bytes of
@@ -2803,7 +2851,7 @@ cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *
                                   uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                                   int32_t *status, int grid, uint64_t total, cudaStream_t st, float *cand_g,
                                   uint64_t *rank_g, uint32_t *dump, unsigned long long *waits,
-                                  unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist, TcCollect collect)
+                                  unsigned long long wait_ns, int comb_p, int top_n, uint32_t *hist)
 {
     const bool comb = comb_p != 0;
     const int kp = k - 2;                       // prefix SNPs: the tiles of an order-(k-1) search
@@ -2845,7 +2893,6 @@ cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *
         P.one.n_items += (host_binom(j, kp) + tc_ppt(k - 1) - 1) / tc_ppt(k - 1) * (uint64_t)tc::panel_ntiles(d.n, j, kj);
     fill_launch(P, k, pool, list_score, list_rank, list_count, status, dump, waits, cand_g, rank_g, comb, true);
     P.wait_ns = wait_ns;
-    P.collect = collect;
     e = encode_map(&map, d, ws.operand, comb, pair_operand_rows(d.n));
     if (e != cudaSuccess) return e;
     return launch_kernel(map, P, k, grid, st, comb, true);

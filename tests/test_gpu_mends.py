@@ -1,0 +1,55 @@
+"""Calls at the edges of a rule that once answered them slowly or unsafely:
+one test per rule."""
+from __future__ import annotations
+
+import math
+import time
+
+import pytest
+
+from tests.helpers import random_data
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def epi():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2201_02460_gb300 import epi as E
+    E.load()
+    return E
+
+
+@pytest.fixture(scope="module")
+def ctx(epi):
+    return epi.Context(0)
+
+
+# more combinations at or above a threshold than the collecting pass has room
+# for (2^20): it ends at an item that all its warps know, without waiting for
+# loads that nothing takes (a wait of two seconds a stage), and every score is
+# looked at instead
+@pytest.mark.parametrize("k,n,m", [(2, 1600, 200), (3, 200, 300), (4, 80, 130), (5, 50, 260)])
+@pytest.mark.parametrize("variant", ["auto", "separate"])
+def test_threshold_found_too_often(epi, ctx, k, n, m, variant):
+    ds = epi.Dataset(ctx, *random_data(n, m, seed=n))
+
+    def timed(chunk):
+        t = time.perf_counter()
+        r, found = epi.search_threshold(ds, k, 1e-9, 100, chunk=chunk, with_counts=False)
+        return r, found, time.perf_counter() - t
+
+    ctx.set_tc_variant(variant)
+    try:
+        want, n_want, t_want = timed(math.comb(n, k))
+        assert n_want > 1 << 20
+        for _ in range(2):
+            got, n_got, t_got = timed(0)
+            assert n_got == n_want
+            assert (got.rank == want.rank).all() and (got.mi == want.mi).all()
+            assert t_got < t_want + 1.5
+    finally:
+        ctx.set_tc_variant("auto")
+        ds.close()
