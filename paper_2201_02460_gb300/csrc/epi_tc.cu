@@ -1392,11 +1392,13 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         const int64_t stage_stride = 6 * (d.n + 1);
         uint64_t g = 0;                      // stages of the CTA so far (all groups)
         long long w_prod = 0, w_prod_acc = 0;
+        // (a warp's lanes leave together: one that left alone would be waited
+        // for at the next __syncwarp)
         for (int64_t i = 0; i < n_my; i++) {
-            if (abort_flag) break;
+            if (__any_sync(0xffffffffu, abort_flag)) break;
             const int dq = (int)(i % kDescDepth);
             const uint32_t ud = (uint32_t)(i / kDescDepth);
-            if (!wait_desc<COLLECT>(&desc_full[dq], ud & 1, &abort_flag, i)) break;
+            if (!__all_sync(0xffffffffu, wait_desc<COLLECT>(&desc_full[dq], ud & 1, &abort_flag, i))) break;
             const Desc &D = desc[dq];
             // the row's SNP rows at stage 0; rows of no prefix read the zero
             // rows kept past the last SNP
@@ -1476,11 +1478,10 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     int s2 = s + kGroups;
                     uint32_t ph2 = ph;
                     if (s2 >= kStages) { s2 -= kStages; ph2 ^= 1; }
-                    if (!wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_prod) ||
-                        (two && !wait_here(&empty_ab[s2], ph2 ^ 1, &abort_flag, w_prod))) {
-                        ok = false;
-                        break;
-                    }
+                    ok = wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_prod) &&
+                         (!two || wait_here(&empty_ab[s2], ph2 ^ 1, &abort_flag, w_prod));
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
                     produce(st, s, ring[u]);
                     if (two) produce(st + kGroups, s2, ring[u + 1]);
                     fetch(st + kGroups * kPf, ring[u]);
@@ -1501,7 +1502,7 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             g += (uint64_t)nst;
             const int b = (int)(i & 1);
             const uint32_t ub = (uint32_t)(i >> 1);
-            if (!wait_fast(&tot_empty[b], (ub & 1) ^ 1, &abort_flag, w_prod_acc)) break;
+            if (!__all_sync(0xffffffffu, wait_fast(&tot_empty[b], (ub & 1) ^ 1, &abort_flag, w_prod_acc))) break;
             tot[((b * 128 + r) * kGroups + grp) * 2 + 0] = t1;
             tot[((b * 128 + r) * kGroups + grp) * 2 + 1] = ta - t1;
             __syncwarp();
