@@ -250,6 +250,25 @@ __device__ __forceinline__ bool wait_here(uint64_t *bar, uint32_t parity, volati
     return ok;
 }
 
+// The same for a whole warp in step: the lanes' tests are voted on, so that
+// they go on, or give up, together.
+__device__ __forceinline__ bool wait_together(uint64_t *bar, uint32_t parity, volatile int *abort_flag, long long &acc)
+{
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    const long long c0 = clock64();
+    const uint64_t n0 = now_ns();
+    bool ok = true;
+    while (!__all_sync(0xffffffffu, mbar_try(bar, parity))) {
+        if (now_ns() - n0 > g_wait_limit_ns) *abort_flag = 1;
+        if (__any_sync(0xffffffffu, *abort_flag)) {
+            ok = false;
+            break;
+        }
+    }
+    acc += clock64() - c0;
+    return ok;
+}
+
 // Hot-path wait: one inline non-blocking test; the bounded out-of-line wait
 // (and the cycle accounting of the trace) only when the phase is not
 // complete yet, so the trace counts every cycle spent waiting.
@@ -1392,13 +1411,13 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
         const int64_t stage_stride = 6 * (d.n + 1);
         uint64_t g = 0;                      // stages of the CTA so far (all groups)
         long long w_prod = 0, w_prod_acc = 0;
-        // (a warp's lanes leave together: one that left alone would be waited
-        // for at the next __syncwarp)
+        // A warp's lanes leave together, by votes: one that left alone would be
+        // waited for at the next __syncwarp.
         for (int64_t i = 0; i < n_my; i++) {
-            if (__any_sync(0xffffffffu, abort_flag)) break;
             const int dq = (int)(i % kDescDepth);
             const uint32_t ud = (uint32_t)(i / kDescDepth);
-            if (!__all_sync(0xffffffffu, wait_desc<COLLECT>(&desc_full[dq], ud & 1, &abort_flag, i))) break;
+            const bool go = wait_desc<COLLECT>(&desc_full[dq], ud & 1, &abort_flag, i) && !abort_flag;
+            if (!__all_sync(0xffffffffu, go)) break;
             const Desc &D = desc[dq];
             // the row's SNP rows at stage 0; rows of no prefix read the zero
             // rows kept past the last SNP
@@ -1478,10 +1497,14 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
                     int s2 = s + kGroups;
                     uint32_t ph2 = ph;
                     if (s2 >= kStages) { s2 -= kStages; ph2 ^= 1; }
-                    ok = wait_here(&empty_ab[s], ph ^ 1, &abort_flag, w_prod) &&
-                         (!two || wait_here(&empty_ab[s2], ph2 ^ 1, &abort_flag, w_prod));
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
+                    // (one vote for both tests: a vote for each, or one after the
+                    // lanes' own waits, took 0.5 to 2 % more at order 4)
+                    if (!__all_sync(0xffffffffu, mbar_test(&empty_ab[s], ph ^ 1) &&
+                                                     (!two || mbar_test(&empty_ab[s2], ph2 ^ 1)))) {
+                        ok = wait_together(&empty_ab[s], ph ^ 1, &abort_flag, w_prod) &&
+                             (!two || wait_together(&empty_ab[s2], ph2 ^ 1, &abort_flag, w_prod));
+                        if (!ok) break;
+                    }
                     produce(st, s, ring[u]);
                     if (two) produce(st + kGroups, s2, ring[u + 1]);
                     fetch(st + kGroups * kPf, ring[u]);
@@ -1502,7 +1525,8 @@ __global__ void __launch_bounds__(Roles::Threads, 1) tc_search_kernel(const __gr
             g += (uint64_t)nst;
             const int b = (int)(i & 1);
             const uint32_t ub = (uint32_t)(i >> 1);
-            if (!__all_sync(0xffffffffu, wait_fast(&tot_empty[b], (ub & 1) ^ 1, &abort_flag, w_prod_acc))) break;
+            ok = ok && wait_fast(&tot_empty[b], (ub & 1) ^ 1, &abort_flag, w_prod_acc);
+            if (!__all_sync(0xffffffffu, ok)) break;
             tot[((b * 128 + r) * kGroups + grp) * 2 + 0] = t1;
             tot[((b * 128 + r) * kGroups + grp) * 2 + 1] = ta - t1;
             __syncwarp();
