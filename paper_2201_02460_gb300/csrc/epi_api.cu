@@ -633,7 +633,7 @@ struct BatchItem {
     int k = 0, top_n = 0, pool = 0, cells = 0;
     bool tc = false;
     int comb_p = 0;                // tensor path: class shift, 0 = separate classes
-    bool alone = false;            // pair tiles: a search of its own, after the batch's launches
+    bool alone = false;            // a search of its own, after the batch's launches (batch_alone)
     uint64_t total = 0;
     double cost = 0;
     int group = -1, cta_begin = 0, cta_count = 0;
@@ -655,6 +655,24 @@ struct BatchGroup {
 };
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) & ~(a - 1); }
+
+// Whether a study of a batch is searched by itself, with pair tiles, after the
+// batch's launches: where the time that pairs save exceeds what a search of
+// its own costs beyond a place in the batch (120 us: its launches wait for
+// each other and the host for it).  Plain tiles take 1.25 ns an item and
+// 128-individual chunk of the whole GPU, and 16 chunks' worth at least; pairs
+// save 0.3 of it at order 4 below 24 chunks, half above, two thirds at order
+// 5.  us a study, batches of 24, in the batch and alone:
+//   order 4   40 x 1000  117 and 215    75 x 1000  384 and 406    90 x 1000  646 and 573
+//             50 x 4000  259 and 281    60 x 4000  395 and 339    40 x 16000 393 and 315
+//   order 5   24 x  300  233 and 245    26 x  300  308 and 264    24 x 4000  577 and 332
+bool batch_alone(const DevData &d, int k, bool comb)
+{
+    if (!tc_pair_applies(d, k, comb)) return false;
+    const double chunks = d.Wt / 4;
+    const double plain_us = 1.25e-3 * (double)tc_item_count(d.n, k, comb) * std::max(chunks, 16.0);
+    return plain_us * (k == 5 ? 0.66 : chunks >= 24 ? 0.5 : 0.3) >= 120.0;
+}
 
 // Popcount launch shape for a group: residency first, then staged prefixes.
 bool plan_group_popc(const epi_ctx *ctx, BatchGroup &g)
@@ -828,7 +846,7 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         if (st != EPI_OK) return fail(st, "dataset %d: %s", i, epi_last_error());
         const DevData d = it.ds->dev();
         if (it.tc) it.comb_p = plan_comb_shift(it.ds);
-        it.alone = it.tc && tc_pair_applies(d, it.k, it.comb_p != 0);
+        it.alone = it.tc && batch_alone(d, it.k, it.comb_p != 0);
         // work estimate for the CTA split: a tensor-core item costs its
         // 128-individual chunks, but never less than its epilogue (about 32
         // chunks' worth)

@@ -74,3 +74,23 @@ def test_wait_limit_at_every_order(epi, k, n, m, variant):
     assert (got.rank == want.rank).all() and (got.mi == want.mi).all()
     ds.close()
     own.close()
+
+
+# studies of a batch that are searched by themselves are those whose pair
+# tiles save more than a search of its own costs: a replayed graph launches
+# nothing that the context counts, a search of its own does
+@pytest.mark.parametrize("k,n,m,alone", [(4, 45, 1000, False), (4, 48, 4000, False), (5, 24, 300, False),
+                                         (4, 100, 1000, True), (4, 60, 4000, True), (5, 30, 300, True)])
+def test_batch_searches_large_studies_alone(epi, k, n, m, alone):
+    own = epi.Context(0)
+    sets = [epi.Dataset(own, *random_data(n - i, m, seed=n + i)) for i in (0, 1)] + \
+        [epi.Dataset(own, *random_data(30, 200, seed=1))]
+    orders = [k, k, 3]
+    want = [epi.search(s, o, 20, path="popc") for s, o in zip(sets, orders)]
+    epi.search_batched(own, sets, orders, [20] * 3)
+    before = own.kernel_launches()
+    got = epi.search_batched(own, sets, orders, [20] * 3)
+    assert (own.kernel_launches() > before) == alone
+    for a, b in zip(got, want):
+        assert (a.rank == b.rank).all() and (a.mi == b.mi).all() and (a.counts == b.counts).all()
+    own.close()
