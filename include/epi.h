@@ -92,7 +92,9 @@ const char *epi_last_error(void);
 
 /* Context on CUDA device `device`; all work is queued on `cuda_stream` (a
  * cudaStream_t, NULL = the legacy default stream).  The context owns its
- * device scratch memory, allocated on first use and grown as needed.
+ * device scratch memory, allocated on first use and grown as needed.  Order-4
+ * and -5 searches take work space of up to 16 GiB beside it on the stream; up
+ * to 4 GiB of it stay with the context, more is freed behind the search.
  * epi_destroy may be called while datasets of the context are alive: the
  * context is then freed by the last epi_dataset_destroy, and no other call
  * may use it meanwhile. */

@@ -41,6 +41,8 @@ struct epi_ctx {
     unsigned long long *waits_dev = nullptr;   // own buffer: per-role wait cycles of a profiled TC search
     int waits_grid = 0;                        // CTAs recorded in waits_dev (0: nothing recorded)
     bool destroy_requested = false;
+    void *pair_space = nullptr;    // pair tiles' operand and single counts (at most kPairKeep bytes), stream-ordered
+    size_t pair_space_bytes = 0;
     void *result_host = nullptr;   // pinned staging of one search's results (at most kResultStaging bytes)
     size_t result_host_bytes = 0;
     // test controls (epi_set_wait_limit, epi_inject_alloc_failure)
@@ -137,7 +139,16 @@ bool injected_alloc_failure(epi_ctx *ctx)
 cudaError_t ctx_malloc(epi_ctx *ctx, void **p, size_t bytes)
 {
     if (injected_alloc_failure(ctx)) return cudaErrorMemoryAllocation;
-    const cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->pair_space) {
+        // the space kept for pair tiles first
+        cudaGetLastError();
+        cudaFreeAsync(ctx->pair_space, ctx->stream);
+        cudaStreamSynchronize(ctx->stream);
+        ctx->pair_space = nullptr;
+        ctx->pair_space_bytes = 0;
+        e = cudaMalloc(p, bytes);
+    }
     // a caller may go on without the memory: no launch check sees this error
     if (e == cudaErrorMemoryAllocation) cudaGetLastError();
     return e;
@@ -146,7 +157,9 @@ cudaError_t ctx_malloc(epi_ctx *ctx, void **p, size_t bytes)
 cudaError_t ctx_malloc_async(epi_ctx *ctx, void **p, size_t bytes, cudaStream_t st)
 {
     if (injected_alloc_failure(ctx)) return cudaErrorMemoryAllocation;
-    return cudaMallocAsync(p, bytes, st);
+    const cudaError_t e = cudaMallocAsync(p, bytes, st);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
 }
 
 int pow3i(int k)
@@ -182,6 +195,44 @@ epi_status ensure_scratch(epi_ctx *ctx, size_t bytes)
     want = (want + ((1u << 20) - 1)) & ~(size_t)((1u << 20) - 1);
     CK(ctx_malloc(ctx, &ctx->scratch, want));
     ctx->scratch_bytes = want;
+    return EPI_OK;
+}
+
+// Work space of one search's pair tiles on the context's stream, without a
+// host wait.  Up to kPairKeep (1.5 % of the memory) it stays with the context,
+// until another allocation fails; a larger one, of up to 16 GiB, is the
+// search's alone and freed on the stream behind it, so that the memory is the
+// program's again.  That takes 2 ms a GiB and search: order 4, 500 x 8192
+// (3.3 GiB) 423.4 ms kept and 427.2 freed, order 5, 120 x 1000 (1.9 GiB) 71.6
+// and 75.1.  Within a stream capture the allocation is the graph's.
+constexpr size_t kPairKeep = (size_t)4 << 30;
+struct PairSpace {
+    epi_ctx *ctx;
+    void *p = nullptr;
+    bool once = false;
+    explicit PairSpace(epi_ctx *c) : ctx(c) {}
+    ~PairSpace()
+    {
+        if (p && once) cudaFreeAsync(p, ctx->stream);
+    }
+};
+epi_status take_pair_space(epi_ctx *ctx, size_t bytes, PairSpace &out)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(ctx->stream, &cap));
+    out.once = bytes > kPairKeep || cap != cudaStreamCaptureStatusNone;
+    if (out.once) {
+        CK(ctx_malloc_async(ctx, &out.p, bytes, ctx->stream));
+        return EPI_OK;
+    }
+    if (ctx->pair_space_bytes < bytes) {
+        if (ctx->pair_space) cudaFreeAsync(ctx->pair_space, ctx->stream);
+        ctx->pair_space = nullptr;
+        ctx->pair_space_bytes = 0;
+        CK(ctx_malloc_async(ctx, &ctx->pair_space, bytes, ctx->stream));
+        ctx->pair_space_bytes = bytes;
+    }
+    out.p = ctx->pair_space;
     return EPI_OK;
 }
 
@@ -434,11 +485,13 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     const bool tc_cg = p.tc && (p.tc_pair || tc_smem_bytes(tc_cp2, false, p.comb_p != 0) > tc_smem_limit(ctx));
     const TcPairBytes pb = p.tc_pair ? tc_pair_bytes(ds->dev(), p.k, p.comb_p != 0) : TcPairBytes();
     const size_t o_pt = p.tc_pair ? a.take<char>(pb.tables) : 0;
-    const size_t o_po = p.tc_pair ? a.take<char>(pb.operand) : 0;
-    const size_t o_ps = p.tc_pair ? a.take<char>(pb.singles) : 0;
     const size_t o_tcs = tc_cg ? a.take<float>((size_t)p.grid * tc_cp2) : 0;
     const size_t o_tcr = tc_cg ? a.take<uint64_t>((size_t)p.grid * tc_cp2) : 0;
     epi_status st = ensure_scratch(ctx, a.off);
+    const size_t singles_at = (pb.operand + 255) & ~(size_t)255;
+    PairSpace pair_space(ctx);
+    if (st == EPI_OK && p.tc) st = ensure_b4(ds);
+    if (st == EPI_OK && p.tc_pair) st = take_pair_space(ctx, singles_at + pb.singles, pair_space);
     if (st == EPI_ENOMEM && p.tc_pair) {
         // no room for the pairs: the search without them
         SearchPlan q = p;
@@ -459,10 +512,6 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
     double *mi = reinterpret_cast<double *>(base + o_mi);
     int32_t *cb = reinterpret_cast<int32_t *>(base + o_cb);
     uint64_t *ic = reinterpret_cast<uint64_t *>(base + o_ic);
-    if (p.tc) {
-        st = ensure_b4(ds);
-        if (st != EPI_OK) return st;
-    }
     if (own) {
         own->head = base;
         own->results = base + o_res;
@@ -493,8 +542,8 @@ epi_status queue_search(epi_dataset *ds, const SearchPlan &p, int path, epi_resu
             ctx->waits_grid = p.grid;
         }
         if (p.tc_pair) {
-            const TcPairWork ws{reinterpret_cast<unsigned char *>(base + o_po),
-                                reinterpret_cast<unsigned char *>(base + o_ps),
+            const TcPairWork ws{static_cast<unsigned char *>(pair_space.p),
+                                static_cast<unsigned char *>(pair_space.p) + singles_at,
                                 reinterpret_cast<uint64_t *>(base + o_pt)};
             CK(launch_tc_pair_search(d, p.k, ds->b4, ws, p.pool, thr, ls, lr, lc, status, p.grid, p.total, ctx->stream,
                                      reinterpret_cast<float *>(base + o_tcs), reinterpret_cast<uint64_t *>(base + o_tcr),
@@ -1566,6 +1615,7 @@ static void free_ctx(epi_ctx *ctx)
         cudaStreamSynchronize(ctx->stream);
         cudaFree(ctx->scratch);
     }
+    if (ctx->pair_space) cudaFreeAsync(ctx->pair_space, ctx->stream);
     for (auto &pr : ctx->prof_events) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
     if (ctx->waits_dev) cudaFree(ctx->waits_dev);
     if (ctx->batch_exec) cudaGraphExecDestroy(ctx->batch_exec);

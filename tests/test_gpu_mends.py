@@ -94,3 +94,37 @@ def test_batch_searches_large_studies_alone(epi, k, n, m, alone):
     for a, b in zip(got, want):
         assert (a.rank == b.rank).all() and (a.mi == b.mi).all() and (a.counts == b.counts).all()
     own.close()
+
+
+# the work space of a large search with pair tiles (5.4 GiB here) is given back
+# behind it; a small one stays with the context
+def test_pair_space_is_given_back(epi):
+    import torch
+    own = epi.Context(0)
+    small = epi.Dataset(own, *random_data(60, 300, seed=1))
+    large = epi.Dataset(own, *random_data(160, 300, seed=2))
+    want = epi.search(large, 3, 10, path="tc")          # the operand and the scratch are there
+    epi.search(small, 5, 10)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    a = epi.search(large, 5, 10)
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 1 << 30
+    b = epi.search(large, 5, 10)
+    assert (a.rank == b.rank).all() and (a.mi == b.mi).all()
+    assert (epi.search(large, 3, 10, path="tc").rank == want.rank).all()
+    own.close()
+
+
+# a search that finds no room for pair tiles runs without them
+def test_no_room_for_pair_space(epi):
+    own = epi.Context(0)
+    ds = epi.Dataset(own, *random_data(60, 300, seed=1))
+    want = epi.search(ds, 4, 10, path="popc")
+    epi.search(ds, 3, 10, path="tc")
+    epi.search(ds, 4, 10, path="tc", rank_range=(0, 480000))   # the operand and the scratch are there
+    own.inject_alloc_failure(0)
+    got = epi.search(ds, 4, 10, path="tc")
+    own.inject_alloc_failure(-1)
+    assert (got.rank == want.rank).all() and (got.mi == want.mi).all()
+    own.close()
