@@ -412,12 +412,16 @@ epi_status ensure_b4(epi_dataset *ds)
 int plan_comb_shift(const epi_dataset *ds) { return ds->ctx->tc_combined ? tc_comb_shift(ds->dev()) : 0; }
 
 // choose_path, with the operand an automatic choice of the tensor path needs;
-// where that does not fit in memory, the popcount path.
+// where that does not fit in memory, or is not there yet while the stream is
+// being captured (it would be built only when the graph runs), the popcount
+// path.
 epi_status take_path(epi_dataset *ds, int k, int path, uint64_t rb, uint64_t re, uint64_t total, bool &tc)
 {
     epi_status st = choose_path(ds, k, path, rb, re, total, tc);
-    if (st == EPI_OK && tc && path == EPI_PATH_AUTO) {
-        st = ensure_b4(ds);
+    if (st == EPI_OK && tc && path == EPI_PATH_AUTO && !ds->b4) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(ds->ctx->stream, &cap));
+        st = cap == cudaStreamCaptureStatusNone ? ensure_b4(ds) : EPI_ENOMEM;
         if (st == EPI_ENOMEM) {
             tc = false;
             st = EPI_OK;

@@ -5,6 +5,7 @@ from __future__ import annotations
 import math
 import time
 
+import numpy as np
 import pytest
 
 from tests.helpers import random_data
@@ -128,3 +129,32 @@ def test_no_room_for_pair_space(epi):
     own.inject_alloc_failure(-1)
     assert (got.rank == want.rank).all() and (got.mi == want.mi).all()
     own.close()
+
+
+# a search captured into a graph, of a study that was never searched: order 2
+# chooses the tensor path from 100 SNPs, whose operand a capture cannot build
+def test_captured_search_of_a_new_study(epi):
+    import torch
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        own = epi.Context(0)
+        warm, ds = (epi.Dataset(own, *random_data(200, 400, seed=i)) for i in (1, 2))
+        out = torch.zeros(10 * epi.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        n_out = torch.zeros(1, dtype=torch.int32, device="cuda")
+        status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+        # the context's scratch is there
+        epi.search_async(warm, 2, 10, out, None, n_out, status, path="popc")
+        epi.search_async(warm, 2, 10, out, None, n_out, status)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            epi.search_async(ds, 2, 10, out, None, n_out, status)
+        want = epi.search(ds, 2, 10)
+        out.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        got = np.frombuffer(out.cpu().numpy().tobytes(), dtype=epi.RESULT_DTYPE)
+        assert int(status.item()) == 0 and int(n_out.item()) == 10
+        assert (got["rank"] == want.rank).all() and (got["mi"] == want.mi).all()
+        del graph
+        own.close()
