@@ -88,12 +88,16 @@ epi_status fail(epi_status s, const char *fmt, ...)
     return s;
 }
 
+// (a failed call's error is taken off the thread: the next launch's check
+// would report it again)
 #define CK(call)                                                                                   \
     do {                                                                                           \
         cudaError_t e_ = (call);                                                                   \
-        if (e_ != cudaSuccess)                                                                     \
+        if (e_ != cudaSuccess) {                                                                   \
+            cudaGetLastError();                                                                    \
             return fail(e_ == cudaErrorMemoryAllocation ? EPI_ENOMEM : EPI_ECUDA, "%s: %s (%s:%d)", \
                         #call, cudaGetErrorString(e_), __FILE__, __LINE__);                        \
+        }                                                                                          \
     } while (0)
 
 // Makes the context's device current for the scope of a call.
@@ -401,8 +405,12 @@ epi_status ensure_b4(epi_dataset *ds)
 {
     if (ds->b4) return EPI_OK;
     epi_ctx *ctx = ds->ctx;
-    CK(ctx_malloc(ctx, (void **)&ds->b4, tc_b4_bytes(ds->dev())));
-    CK(launch_build_b4(ds->dev(), ds->b4, ctx->num_sms, ctx->stream));
+    unsigned char *b4 = nullptr;
+    CK(ctx_malloc(ctx, (void **)&b4, tc_b4_bytes(ds->dev())));
+    const cudaError_t build_b4 = launch_build_b4(ds->dev(), b4, ctx->num_sms, ctx->stream);
+    if (build_b4 != cudaSuccess) cudaFree(b4);   // never an operand that was not built
+    CK(build_b4);
+    ds->b4 = b4;
     ctx->launches += 2;
     return EPI_OK;
 }

@@ -158,3 +158,30 @@ def test_captured_search_of_a_new_study(epi):
         assert (got["rank"] == want.rank).all() and (got["mi"] == want.mi).all()
         del graph
         own.close()
+
+
+# a search that a stream capture refuses (the tensor path's operand is not
+# there) leaves the study and the context as they were
+def test_search_after_a_refused_capture(epi):
+    import torch
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        own = epi.Context(0)
+        warm, ds = (epi.Dataset(own, *random_data(120, 400, seed=i)) for i in (1, 2))
+        want = epi.search(ds, 3, 10, path="popc")
+        out = torch.zeros(10 * epi.RESULT_DTYPE.itemsize, dtype=torch.uint8, device="cuda")
+        n_out = torch.zeros(1, dtype=torch.int32, device="cuda")
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        epi.search_async(warm, 3, 10, out, None, n_out, status)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        with pytest.raises(epi.EpiError):
+            epi.search_async(ds, 3, 10, out, None, n_out, status, path="tc")
+        with pytest.raises(RuntimeError):
+            graph.capture_end()
+        for _ in range(2):
+            got = epi.search(ds, 3, 10, path="tc")
+            assert (got.rank == want.rank).all() and (got.mi == want.mi).all() and (got.counts == want.counts).all()
+        del graph
+        own.close()
