@@ -438,14 +438,20 @@ epi_status take_path(epi_dataset *ds, int k, int path, uint64_t rb, uint64_t re,
     return st;
 }
 
+// The tensor path's variant and tiles for p's order and range.
+void plan_tc(const epi_dataset *ds, SearchPlan &p)
+{
+    p.grid = ds->ctx->num_sms;
+    p.comb_p = plan_comb_shift(ds);
+    p.tc_pair = p.rb == 0 && p.re == p.total && tc_pair_applies(ds->dev(), p.k, p.comb_p != 0);
+}
+
 epi_status make_plan(epi_dataset *ds, SearchPlan &p, int path)
 {
     epi_status st = take_path(ds, p.k, path, p.rb, p.re, p.total, p.tc);
     if (st != EPI_OK) return st;
     if (!p.tc) return plan_popc(ds, p);
-    p.grid = ds->ctx->num_sms;
-    p.comb_p = plan_comb_shift(ds);
-    p.tc_pair = p.rb == 0 && p.re == p.total && tc_pair_applies(ds->dev(), p.k, p.comb_p != 0);
+    plan_tc(ds, p);
     return EPI_OK;
 }
 
@@ -1092,8 +1098,7 @@ double time_pass(epi_dataset *ds, int k, bool tc, int R, int tile, int slots, ui
     p.k = k; p.top_n = 10; p.pool = initial_pool(10); p.rb = 0; p.re = tc ? total : r; p.total = tc ? total : r;
     p.tc = tc;
     if (tc) {
-        p.grid = ctx->num_sms;
-        p.comb_p = plan_comb_shift(ds);
+        plan_tc(ds, p);
     } else {
         p.tile = tile;
         p.slots = slots;

@@ -185,3 +185,23 @@ def test_search_after_a_refused_capture(epi):
             assert (got.rank == want.rank).all() and (got.mi == want.mi).all() and (got.counts == want.counts).all()
         del graph
         own.close()
+
+
+# the autotuner times the tensor path as searches run it, with pair tiles where
+# they apply (from 40 SNPs at order 4): its two passes then launch as many
+# kernels more than those of a study without them as two searches do
+def test_autotuner_times_pair_tiles(epi):
+    counts = []
+    for n in (39, 40):
+        own = epi.Context(0)
+        ds = epi.Dataset(own, *random_data(n, 300, seed=n))
+        epi.search(ds, 4, 10, path="tc")
+        start = own.kernel_launches()
+        epi.autotune(ds, 4)
+        tuned = own.kernel_launches()
+        epi.search(ds, 4, 10, path="tc")
+        counts.append((tuned - start, own.kernel_launches() - tuned))
+        own.close()
+    (tune39, search39), (tune40, search40) = counts
+    assert search40 > search39
+    assert tune40 - tune39 == 2 * (search40 - search39)
