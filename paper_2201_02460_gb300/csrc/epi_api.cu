@@ -1142,7 +1142,13 @@ epi_status epi_autotune(epi_dataset *ds, int order, int *out)
     DeviceGuard g(ctx->device);
     if (!g.ok) return fail(EPI_ECUDA, "cannot select device %d", ctx->device);
     // probe range: about 16 sub-tiles per resident CTA
-    const uint64_t r = std::min<uint64_t>(total, (uint64_t)ctx->num_sms * 8 * 512 * 16);
+    uint64_t r = std::min<uint64_t>(total, (uint64_t)ctx->num_sms * 8 * 512 * 16);
+    // orders 7-8: searches take the histogram kernel whatever the shape and
+    // batches keep their prefix tables elsewhere, so a sixteenth of the range
+    // has to do for the kernels on global prefix tables (order 8, 20 x 1000:
+    // the whole call took 90 ms with all of it; at order 6 the shapes timed are
+    // the batches')
+    if (order >= 7 && hist_applies(ds->dev(), order, initial_pool(10))) r = std::max<uint64_t>(1, r / 16);
     std::vector<int> Rs;
     for (int R : {1, 3, 9, 27})
         if (popc_row_group_ok(order, R)) Rs.push_back(R);

@@ -205,3 +205,22 @@ def test_autotuner_times_pair_tiles(epi):
     (tune39, search39), (tune40, search40) = counts
     assert search40 > search39
     assert tune40 - tune39 == 2 * (search40 - search39)
+
+
+# at orders 7-8 the autotuner's shapes are those of kernels that neither
+# searches nor batches take: it must not spend more on them than on a few
+# searches (a few shapes, two passes each)
+@pytest.mark.parametrize("k,n,m,times", [(7, 20, 1000, 17), (8, 20, 1000, 40)])
+def test_autotuner_at_high_orders(epi, k, n, m, times):
+    own = epi.Context(0)
+    ds = epi.Dataset(own, *random_data(n, m, seed=k))
+
+    def seconds(f):
+        f()
+        t = time.perf_counter()
+        f()
+        return time.perf_counter() - t
+
+    search = seconds(lambda: epi.search(ds, k, 100))
+    assert seconds(lambda: epi.autotune(ds, k)) < times * search
+    own.close()
