@@ -58,8 +58,7 @@ def test_threshold_found_too_often(epi, ctx, k, n, m, variant):
 
 # a pipeline wait that runs out ends the search with an error at every order
 # and variant, whichever role's wait it was, and the context stays usable
-@pytest.mark.parametrize("k,n,m", [(2, 300, 3000), (3, 90, 3000), (4, 39, 3000), (4, 60, 3000), (5, 23, 3000),
-                                   (5, 40, 3000)])
+@pytest.mark.parametrize("k,n,m", [(2, 300, 3000), (3, 90, 3000), (4, 60, 3000), (5, 23, 3000)])
 @pytest.mark.parametrize("variant", ["auto", "separate"])
 def test_wait_limit_at_every_order(epi, k, n, m, variant):
     own = epi.Context(0)
@@ -224,3 +223,16 @@ def test_autotuner_at_high_orders(epi, k, n, m, times):
     search = seconds(lambda: epi.search(ds, k, 100))
     assert seconds(lambda: epi.autotune(ds, k)) < times * search
     own.close()
+
+
+# a pass that writes every score launches its kernel alone: nothing selects the
+# best of the scores
+@pytest.mark.parametrize("k,n,m", [(1, 50, 300), (2, 40, 300), (5, 12, 200), (6, 12, 200)])
+def test_every_score_alone(epi, ctx, k, n, m):
+    ds = epi.Dataset(ctx, *random_data(n, m, seed=k))
+    before = ctx.kernel_launches()
+    scores = epi.score_all(ds, k).cpu().numpy()
+    assert ctx.kernel_launches() - before == (2 if k >= 6 else 1)
+    best = epi.search(ds, k, 10, path="popc")
+    assert (scores[best.rank.astype(np.int64)] == best.mi_f32).all()
+    ds.close()
