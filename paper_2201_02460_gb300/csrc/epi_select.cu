@@ -21,6 +21,12 @@ __host__ __device__ inline int merge_entries(int group, int cap, int pool)
     return next_pow2(e) + (pool < 2 ? 2 : pool);
 }
 
+// Entries up to which the last level of a merge sorts by counting, with work
+// that grows with their square (the k best of 2^20 floats in order, by counting
+// and by the bitonic sort: k = 600 171 and 170 us, 1000 198 and 175, 4096 943
+// and 243).
+constexpr int kCountSort = 512;
+
 // float bits in an order-preserving unsigned form
 __device__ __forceinline__ uint32_t order_bits(float f)
 {
@@ -32,8 +38,9 @@ __device__ __forceinline__ uint32_t order_bits(float f)
 // i at ls + i pitch with lc[i lstep] entries -- and keeps the best `pool` of
 // their entries: in place as list b group of the next level, or sorted in
 // out_* when this is the last level (one block).  The cut is found by a radix
-// select over the scores (four 8-bit passes), and the last level sorts by
-// counting, for each entry kept, the better ones; entries below the search's
+// select over the scores (four 8-bit passes), and the last level sorts few
+// entries by counting, for each, the better ones, and more of them by a bitonic
+// sort; entries below the search's
 // threshold are dropped on loading.  (One block that sorted 1024 entries at a
 // time took 124 us for 155 lists of 128, two levels of 4096-entry bitonic
 // sorts 2 x 45.)
@@ -131,7 +138,17 @@ __global__ void __launch_bounds__(1024) merge_level_kernel(float *__restrict__ l
         __syncthreads();
         L = pool;
     }
-    if (out_s) {
+    if (out_s && L > kCountSort) {
+        // (entries past the front are free: the kept ones lie behind them all)
+        if (ks != sc)
+            for (int i = threadIdx.x; i < L; i += blockDim.x) { sc[i] = ks[i]; rk[i] = kr[i]; }
+        const int p2 = next_pow2(L);
+        for (int i = L + threadIdx.x; i < p2; i += blockDim.x) { sc[i] = -INFINITY; rk[i] = ~0ull; }
+        __syncthreads();
+        block_sort_cands(sc, rk, p2);
+        for (int i = threadIdx.x; i < L; i += blockDim.x) { out_s[i] = sc[i]; out_r[i] = rk[i]; }
+        if (threadIdx.x == 0) *out_n = L;
+    } else if (out_s) {
         for (int i = threadIdx.x; i < L; i += blockDim.x) {
             const float v = ks[i];
             const uint64_t r = kr[i];

@@ -236,3 +236,25 @@ def test_every_score_alone(epi, ctx, k, n, m):
     best = epi.search(ds, k, 10, path="popc")
     assert (scores[best.rank.astype(np.int64)] == best.mi_f32).all()
     ds.close()
+
+
+# the last level of a merge sorts up to 512 entries by counting, more by a
+# bitonic sort: both sides, equal scores, and pools cut down by the selection
+@pytest.mark.parametrize("k", [1, 2, 511, 512, 513, 1000, 1025, 4096])
+@pytest.mark.parametrize("levels", [3, 100000])
+def test_sorted_topk(epi, ctx, k, levels):
+    import torch
+    rng = np.random.default_rng(k + levels)
+    x = (rng.integers(0, levels, 20000) / 16.0 - 1.0).astype(np.float32)
+    s, i = epi.topk(ctx, torch.from_numpy(x).cuda(), k)
+    want = np.lexsort((np.arange(len(x)), -x))[:k]
+    assert (np.asarray(i.cpu()).astype(np.int64) == want).all()
+    assert (s.cpu().numpy() == x[want]).all()
+
+
+@pytest.mark.parametrize("top_n", [400, 500, 700, 1024])
+def test_merge_of_large_pools(epi, ctx, top_n):
+    ds = epi.Dataset(ctx, *random_data(90, 300, seed=top_n))
+    a, b = epi.search(ds, 3, top_n, path="tc"), epi.search(ds, 3, top_n, path="popc")
+    assert len(a) == top_n and (a.rank == b.rank).all() and (a.mi == b.mi).all()
+    ds.close()
