@@ -1444,6 +1444,45 @@ epi_status epi_search_threshold(epi_dataset *ds, int order, double threshold, in
     return EPI_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// The scores of a whole table that are too small for the table of n ln n;
+// done is false where so many have to be counted again that the popcount path
+// should make the whole table (see small_score_limit).
+epi_status make_small_scores(epi_dataset *ds, int order, uint64_t total, float *scores, bool &done)
+{
+    epi_ctx *ctx = ds->ctx;
+    const uint64_t cap = std::min<uint64_t>(total / 4 + 1024, 1ull << 22);
+    Arena a;
+    const size_t o_n = a.take<unsigned long long>(2);
+    const size_t o_same = a.take<uint8_t>((size_t)ds->n);
+    const size_t o_list = a.take<uint64_t>((size_t)cap);
+    const epi_status st = ensure_scratch(ctx, a.off);
+    if (st != EPI_OK) return st;
+    char *base = static_cast<char *>(ctx->scratch);
+    unsigned long long *n_dev = reinterpret_cast<unsigned long long *>(base + o_n);
+    uint64_t *list = reinterpret_cast<uint64_t *>(base + o_list);
+    uint8_t *same = reinterpret_cast<uint8_t *>(base + o_same);
+    CK(cudaMemsetAsync(n_dev, 0, 16, ctx->stream));
+    CK(launch_list_small(ds->dev(), order, total, scores, same, list, cap, n_dev, ctx->num_sms, ctx->stream));
+    ctx->launches += 2;
+    unsigned long long n[2] = {};
+    CK(cudaMemcpyAsync(n, n_dev, 16, cudaMemcpyDeviceToHost, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
+    done = n[0] <= cap && n[1] <= (uint64_t)pow3i(order) * (total / 64 + 1024);
+    if (!done || !n[0]) return EPI_OK;
+    CK(launch_small_scores(ds->dev(), order, same, list, n[0], scores, ctx->num_sms, ctx->stream));
+    ctx->launches += 1;
+    CK(cudaStreamSynchronize(ctx->stream));
+    return EPI_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 epi_status epi_score_all(epi_dataset *ds, int order, float *out_dev)
 {
     uint64_t total = 0, re = UINT64_MAX;
@@ -1462,6 +1501,7 @@ epi_status epi_score_all(epi_dataset *ds, int order, float *out_dev)
         const int grid = ctx->num_sms;
         const size_t o_thr = a.take<uint32_t>(1);
         const size_t o_status = a.take<int32_t>(1);
+        const size_t o_small = a.take<unsigned long long>(1);
         const size_t o_lc = a.take<int32_t>((size_t)grid);
         const size_t o_ic = a.take<uint64_t>(2 * ((size_t)ds->n + 1));
         const size_t o_tl = a.take<long long>((size_t)ds->m + 1);
@@ -1469,21 +1509,28 @@ epi_status epi_score_all(epi_dataset *ds, int order, float *out_dev)
         if (st == EPI_OK) st = ensure_b4(ds);
         if (st == EPI_OK) {
             char *base = static_cast<char *>(ctx->scratch);
-            CK(cudaMemsetAsync(base, 0, 512, ctx->stream));
+            unsigned long long *small_dev = reinterpret_cast<unsigned long long *>(base + o_small);
+            CK(cudaMemsetAsync(base, 0, o_small + 8, ctx->stream));
             CK(launch_tc_scores(ds->dev(), order, ds->b4, reinterpret_cast<uint64_t *>(base + o_ic),
                                 reinterpret_cast<long long *>(base + o_tl), out_dev,
                                 reinterpret_cast<uint32_t *>(base + o_thr), reinterpret_cast<int32_t *>(base + o_lc),
                                 reinterpret_cast<int32_t *>(base + o_status), grid, total, ctx->stream,
-                                ctx->wait_limit_ns, comb_p));
+                                ctx->wait_limit_ns, comb_p, small_dev));
             ctx->launches += 4;
             int32_t bits = 0;
+            unsigned long long small = 0;
             CK(cudaMemcpyAsync(&bits, base + o_status, 4, cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaMemcpyAsync(&small, small_dev, 8, cudaMemcpyDeviceToHost, ctx->stream));
             CK(cudaStreamSynchronize(ctx->stream));
             if (bits & ST_TIMEOUT) return fail(EPI_ETIMEOUT, "device wait expired");
             if (bits) return fail(EPI_ECUDA, "device status 0x%x", bits);
-            return EPI_OK;
+            if (!small) return EPI_OK;
+            bool done = false;
+            st = make_small_scores(ds, order, total, out_dev, done);
+            if (st == EPI_OK && done) return EPI_OK;
         }
-        if (st != EPI_ENOMEM) return st;   // no room for the operand: the popcount path
+        // no room for the operand, or too many small scores: the popcount path
+        if (st != EPI_OK && st != EPI_ENOMEM) return st;
     }
     SearchPlan p;
     p.k = order; p.top_n = 1; p.pool = initial_pool(1); p.rb = 0; p.re = total; p.total = total;

@@ -123,7 +123,16 @@ cudaError_t launch_tc_pair_search(const DevData &d, int k, const unsigned char *
 size_t tc_scores_smem_bytes(const DevData &d, bool comb);
 cudaError_t launch_tc_scores(const DevData &d, int k, const unsigned char *b4, uint64_t *item_cum, long long *tlog,
                              float *scores, uint32_t *global_thr, int32_t *list_count, int32_t *status, int grid,
-                             uint64_t total, cudaStream_t st, unsigned long long wait_ns, int comb_p);
+                             uint64_t total, cudaStream_t st, unsigned long long wait_ns, int comb_p,
+                             unsigned long long *small);
+// Of the scores too small for that table (*small counted them, zeroed before):
+// those of SNPs with one genotype set to zero, the ranks of the others to list
+// (n[0] counts them, n[1] the cells of their tables, zeroed before; same: a byte
+// a SNP), and those made again
+cudaError_t launch_list_small(const DevData &d, int k, uint64_t total, float *scores, uint8_t *same, uint64_t *list,
+                              uint64_t cap, unsigned long long *n, int num_sms, cudaStream_t st);
+cudaError_t launch_small_scores(const DevData &d, int k, const uint8_t *same, const uint64_t *list, uint64_t n,
+                                float *scores, int num_sms, cudaStream_t st);
 constexpr int kTcWaitSlots = 8;
 // batched tensor-core launches: per-dataset descriptors and B-operand maps
 // (128-byte CUtensorMap, 64-byte aligned) live in device memory

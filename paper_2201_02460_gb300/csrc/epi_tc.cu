@@ -2461,49 +2461,119 @@ __global__ void tlog_kernel(int64_t m, long long *__restrict__ out)
 // double-precision product add up to less than m ln m / 16 + 123 units, so
 // scores from 2^24 times that (an MI of 1e-7 at 3000 individuals) keep their
 // accuracy; below are combinations with hardly any association, or none,
-// whose score has to be zero.  A warp looks through 32 scores at a time and
-// takes a small one together, its lanes over the words; there are none in an
-// ordinary study, so what bounds it is one read of the scores (order 4, 200
-// SNPs: 259 MB).
+// whose score has to be zero.  An ordinary study has none: one read of the
+// scores (order 4, 200 SNPs: 259 MB) counts them.  Where there are some, SNPs
+// with one genotype are left out of the combination (they do not change its
+// score): of none but such the score is zero, and the others go to a list, a
+// warp each with a table of 3^(SNPs left) cells.  Where those cells come to
+// more than a sixty-fourth of the whole table's, the popcount path makes the
+// table.  (Every second of 300 SNPs so, order 3 x 2000: 8.9 ms when each was
+// counted in full, 0.7 so; 100 SNPs with 0 to 2 carriers, order 4 x 2000: 17.4
+// and 4.3.)
 __host__ __device__ inline float small_score_limit(int64_t m)
 {
     const double units = (double)m * log((double)m) / 16.0 + 123.0;
     return (float)(units * 16777216.0 / 70368744177664.0 / (double)m);
 }
 
-__global__ void __launch_bounds__(256) small_scores_kernel(DevData d, int k, uint64_t total, float limit,
-                                                           float *__restrict__ scores)
+__global__ void __launch_bounds__(256) count_small_kernel(uint64_t total, float limit, const float *__restrict__ scores,
+                                                          unsigned long long *__restrict__ n)
+{
+    uint32_t c = 0;
+    for (uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; r < total; r += (uint64_t)gridDim.x * blockDim.x)
+        c += scores[r] < limit;
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(n, (unsigned long long)c);
+}
+
+// one warp per SNP: whether everyone has the same genotype
+__global__ void __launch_bounds__(256) one_genotype_kernel(DevData d, uint8_t *__restrict__ same)
+{
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s >= d.n) return;
+    uint32_t held = 0;
+    for (int w = threadIdx.x & 31; w < d.Wt; w += 32)
+        for (int g = 0; g < 3; g++) held |= d.masks[(s * 3 + g) * d.Wt + w] ? 1u << g : 0u;
+    held = __reduce_or_sync(0xffffffffu, held);
+    if ((threadIdx.x & 31) == 0) same[s] = __popc(held) == 1;
+}
+
+// the combination of rank r without its SNPs of one genotype; how many are left
+__device__ __forceinline__ int varying_snps(const DevData &d, int k, uint64_t r, const uint8_t *__restrict__ same,
+                                            int32_t *out)
+{
+    int32_t comb[kMaxOrderGpu];
+    unrank_lex(d.binom, d.n, k, r, comb);
+    int left = 0;
+    for (int t = 0; t < k; t++)
+        if (!same[comb[t]]) out[left++] = comb[t];
+    return left;
+}
+
+__global__ void __launch_bounds__(256) list_small_kernel(DevData d, int k, uint64_t total, float limit,
+                                                         const uint8_t *__restrict__ same, float *__restrict__ scores,
+                                                         uint64_t *__restrict__ list, uint64_t cap,
+                                                         unsigned long long *__restrict__ n)
 {
     const int lane = threadIdx.x & 31;
     const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
-    int cells = 1;
-    for (int t = 0; t < k; t++) cells *= 3;
     for (uint64_t r0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); r0 < total; r0 += step) {
-        uint32_t todo = __ballot_sync(0xffffffffu, r0 + lane < total && scores[r0 + lane] < limit);
-        for (; todo; todo &= todo - 1) {
-            const uint64_t r = r0 + __ffs(todo) - 1;
+        const uint64_t r = r0 + lane;
+        uint32_t cells = 0;                  // of this lane's table, where it is listed
+        if (r < total && scores[r] < limit) {
             int32_t comb[kMaxOrderGpu];
-            unrank_lex(d.binom, d.n, k, r, comb);
-            double mine = 0.0;
-            for (int x0 = 0; x0 < cells; x0 += 32) {
-                uint32_t a = 0, b = 0;   // counts of cell x0 + lane
-                for (int x = x0; x < min(cells, x0 + 32); x++) {
-                    uint32_t ca = 0, cb = 0;
-                    for (int w = lane; w < d.Wt; w += 32) {
-                        uint32_t bits = 0xffffffffu;
-                        for (int q = k - 1, y = x; q >= 0; q--, y /= 3)
-                            bits &= d.masks[((int64_t)comb[q] * 3 + y % 3) * d.Wt + w];
-                        (w < d.W1 ? ca : cb) += __popc(bits);
-                    }
-                    ca = __reduce_add_sync(0xffffffffu, ca);
-                    cb = __reduce_add_sync(0xffffffffu, cb);
-                    if (lane == x - x0) { a = ca; b = cb; }
-                }
-                mine += mi_term_f64(a, a + b, d.m1, d.m) + mi_term_f64(b, a + b, d.m0, d.m);
+            const int left = varying_snps(d, k, r, same, comb);
+            if (left) {
+                cells = 1;
+                for (int t = 0; t < left; t++) cells *= 3;
+            } else {
+                scores[r] = 0.0f;
             }
-            for (int off = 16; off; off >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, off);
-            if (lane == 0) scores[r] = (float)(mine / (double)d.m);
         }
+        const uint32_t mask = __ballot_sync(0xffffffffu, cells != 0);
+        if (!mask) continue;
+        const uint32_t all = __reduce_add_sync(0xffffffffu, cells);
+        unsigned long long at = 0;
+        if (lane == 0) {
+            at = atomicAdd(n, (unsigned long long)__popc(mask));
+            atomicAdd(n + 1, (unsigned long long)all);
+        }
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(mask & ((1u << lane) - 1u));
+        if (cells && at < cap) list[at] = r;
+    }
+}
+
+__global__ void __launch_bounds__(256) small_scores_kernel(DevData d, int k, const uint8_t *__restrict__ same,
+                                                           const uint64_t *__restrict__ list, uint64_t n,
+                                                           float *__restrict__ scores)
+{
+    const int lane = threadIdx.x & 31;
+    for (uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n;
+         i += ((uint64_t)gridDim.x * blockDim.x) >> 5) {
+        const uint64_t r = list[i];
+        int32_t comb[kMaxOrderGpu];
+        const int left = varying_snps(d, k, r, same, comb);
+        int cells = 1;
+        for (int t = 0; t < left; t++) cells *= 3;
+        double mine = 0.0;
+        for (int x0 = 0; x0 < cells; x0 += 32) {
+            uint32_t a = 0, b = 0;   // counts of cell x0 + lane
+            for (int x = x0; x < min(cells, x0 + 32); x++) {
+                uint32_t ca = 0, cb = 0;
+                for (int w = lane; w < d.Wt; w += 32) {
+                    uint32_t bits = 0xffffffffu;
+                    for (int q = left - 1, y = x; q >= 0; q--, y /= 3)
+                        bits &= d.masks[((int64_t)comb[q] * 3 + y % 3) * d.Wt + w];
+                    (w < d.W1 ? ca : cb) += __popc(bits);
+                }
+                ca = __reduce_add_sync(0xffffffffu, ca);
+                cb = __reduce_add_sync(0xffffffffu, cb);
+                if (lane == x - x0) { a = ca; b = cb; }
+            }
+            mine += mi_term_f64(a, a + b, d.m1, d.m) + mi_term_f64(b, a + b, d.m0, d.m);
+        }
+        for (int off = 16; off; off >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, off);
+        if (lane == 0) scores[r] = (float)(mine / (double)d.m);
     }
 }
 
@@ -2928,7 +2998,8 @@ size_t tc_scores_smem_bytes(const DevData &d, bool comb) { return tc_smem_bytes(
 
 cudaError_t launch_tc_scores(const DevData &d, int k, const unsigned char *b4, uint64_t *item_cum, long long *tlog,
                              float *scores, uint32_t *global_thr, int32_t *list_count, int32_t *status, int grid,
-                             uint64_t total, cudaStream_t st, unsigned long long wait_ns, int comb_p)
+                             uint64_t total, cudaStream_t st, unsigned long long wait_ns, int comb_p,
+                             unsigned long long *small)
 {
     tc::tlog_kernel<<<16, 256, 0, st>>>(d.m, tlog);
     tc::Params P;
@@ -2946,8 +3017,25 @@ cudaError_t launch_tc_scores(const DevData &d, int k, const unsigned char *b4, u
     if (e == cudaSuccess) e = encode_map(&map, d, b4, comb_p != 0);
     if (e == cudaSuccess) e = launch_kernel(map, P, k, grid, st, comb_p != 0);
     if (e != cudaSuccess) return e;
-    tc::small_scores_kernel<<<(unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)grid * 8), 256, 0, st>>>(
-        d, k, total, tc::small_score_limit(d.m), scores);
+    tc::count_small_kernel<<<(unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)grid * 8), 256, 0, st>>>(
+        total, tc::small_score_limit(d.m), scores, small);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_small(const DevData &d, int k, uint64_t total, float *scores, uint8_t *same, uint64_t *list,
+                              uint64_t cap, unsigned long long *n, int num_sms, cudaStream_t st)
+{
+    tc::one_genotype_kernel<<<(unsigned)((d.n + 7) / 8), 256, 0, st>>>(d, same);
+    tc::list_small_kernel<<<(unsigned)std::min<uint64_t>((total + 255) / 256, (uint64_t)num_sms * 8), 256, 0, st>>>(
+        d, k, total, tc::small_score_limit(d.m), same, scores, list, cap, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_small_scores(const DevData &d, int k, const uint8_t *same, const uint64_t *list, uint64_t n,
+                                float *scores, int num_sms, cudaStream_t st)
+{
+    tc::small_scores_kernel<<<(unsigned)std::min<uint64_t>((n + 7) / 8, (uint64_t)num_sms * 8), 256, 0, st>>>(
+        d, k, same, list, n, scores);
     return cudaGetLastError();
 }
 

@@ -2,13 +2,14 @@
 one test per rule."""
 from __future__ import annotations
 
+import itertools
 import math
 import time
 
 import numpy as np
 import pytest
 
-from tests.helpers import random_data
+from tests.helpers import F32_RTOL, random_data
 
 pytestmark = pytest.mark.gpu
 
@@ -258,3 +259,64 @@ def test_merge_of_large_pools(epi, ctx, top_n):
     a, b = epi.search(ds, 3, top_n, path="tc"), epi.search(ds, 3, top_n, path="popc")
     assert len(a) == top_n and (a.rank == b.rank).all() and (a.mi == b.mi).all()
     ds.close()
+
+
+def _copies(n, cases, copies, seed):
+    """Controls that repeat the cases: every score is zero."""
+    half, _ = random_data(n, cases, seed=seed)
+    geno = np.concatenate([half] * (1 + copies), axis=1)
+    return geno, (np.arange(geno.shape[1]) < cases).astype(np.uint8)
+
+
+# scores too small for the table of n ln n: all of SNPs with one genotype (zero
+# without a count), a few others (a list, without such SNPs), more cells in all
+# than those of 1024 tables and one in 64 (the popcount path)
+@pytest.mark.parametrize("k,n,kind", [(3, 60, "constant"), (4, 30, "constant"), (3, 40, "half"), (4, 22, "half"),
+                                      (3, 40, "balanced"), (4, 22, "balanced"), (4, 40, "balanced"),
+                                      (3, 19, "copies"), (3, 20, "copies"), (3, 60, "copies"), (4, 25, "copies")])
+def test_small_scores(epi, ctx, k, n, kind):
+    if kind == "copies":
+        geno, pheno = _copies(n, 70, 2, n)
+    elif kind == "balanced":
+        # two SNPs whose carriers are shared out evenly among constant ones and others
+        geno, pheno = random_data(n, 300, seed=n, m1=150)
+        geno[::2] = 1
+        cases, ctrls = np.nonzero(pheno == 1)[0], np.nonzero(pheno == 0)[0]
+        geno[0, cases[:1]] = geno[0, ctrls[:1]] = 2
+        geno[2, cases[5:8]] = geno[2, ctrls[9:12]] = 0
+    else:
+        geno, pheno = random_data(n, 300, seed=n)
+        geno[::2 if kind == "half" else 1] = np.arange(len(geno[::2 if kind == "half" else 1]))[:, None] % 3
+    ds = epi.Dataset(ctx, geno, pheno)
+    got = epi.score_all(ds, k).cpu().numpy().astype(np.float64)
+    combs = np.array(list(itertools.combinations(range(n), k)), dtype=np.uint32)
+    _, want = epi.score_tables(ds, k, epi.tables(ds, combs))
+    assert (np.abs(got - want) <= F32_RTOL * want + 1e-9 * (want > 0)).all()
+    assert (got[want == 0] == 0).all()
+    assert kind in ("half", "balanced") or (want == 0).all()
+    ds.close()
+
+
+# a table of nothing but such scores costs no more than a few of the popcount
+# path's (which finds the best of them by ranges of the ranks)
+@pytest.mark.parametrize("k,n,m", [(3, 250, 300), (4, 80, 300)])
+@pytest.mark.parametrize("kind", ["constant", "copies"])
+def test_small_scores_are_quick(epi, ctx, k, n, m, kind):
+    def seconds(ds, f):
+        f()
+        best = 1e9
+        for _ in range(3):
+            t = time.perf_counter()
+            f()
+            best = min(best, time.perf_counter() - t)
+        ds.close()
+        return best
+
+    plain = epi.Dataset(ctx, *random_data(n, m, seed=1))
+    usual = seconds(plain, lambda: epi.search_threshold(plain, k, 1e9, 1, chunk=math.comb(n, k)))
+    if kind == "copies":
+        geno, pheno = _copies(n, m // 3, 2, 1)
+    else:
+        geno, pheno = np.zeros((n, m), np.uint8), (np.arange(m) % 2).astype(np.uint8)
+    ds = epi.Dataset(ctx, geno, pheno)
+    assert seconds(ds, lambda: epi.score_all(ds, k)) < 2 * usual
