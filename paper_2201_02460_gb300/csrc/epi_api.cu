@@ -57,6 +57,7 @@ struct epi_dataset {
     int64_t n = 0, m = 0, m1 = 0, m0 = 0;
     int32_t W1 = 0, W0 = 0, Wt = 0;
     int32_t c1max = 0, c0max = 0;  // largest case / control count of a genotype-0 or -1 row
+    float top_share = 0.0f;        // of the commonest genotype, mean over the SNPs
     uint32_t *masks = nullptr;
     uint64_t *binom = nullptr;
     unsigned char *b4 = nullptr;   // tensor-core operand, built on first use
@@ -69,6 +70,7 @@ struct epi_dataset {
         d.masks = masks;
         d.binom = binom;
         d.c1max = c1max; d.c0max = c0max;
+        d.top_share = top_share;
         return d;
     }
 };
@@ -344,7 +346,8 @@ epi_status plan_popc(const epi_dataset *ds, SearchPlan &p, int R_req = 0)
         return fail(EPI_EUNSUPPORTED, "order %d with %lld samples: one prefix table does not fit in shared memory",
                     p.k, (long long)ds->m);
     // orders 6-8: by histogram wherever it takes the sample; 100 best, against
-    // the kernels over words it replaced (a table of k - 2 or k - 1 SNPs):
+    // the kernels over words it replaced (a table of k - 2 or k - 1 SNPs), at
+    // allele frequencies of 0.05-0.5 (rarer ones: see epi_hist.cu):
     //   order 6   14 x  200  0.30 and 0.86 ms    40 x  2048  17.9 and  30.1 ms
     //   order 7   12 x  300  0.47 and 1.31 ms    26 x  2048   3.8 and  17.8 ms
     //   order 7   22 x 6000   3.5 and 15.9 ms    20 x 16000   4.8 and  53.5 ms
@@ -1750,8 +1753,9 @@ epi_status epi_dataset_create(epi_ctx *ctx, const uint8_t *geno, const uint8_t *
     // 2 m int32 entries end on an 8-byte boundary
     int64_t *dm1 = reinterpret_cast<int64_t *>(case_idx + 2 * m);
     int32_t *dstatus = reinterpret_cast<int32_t *>(dm1 + 1);
-    // status word, then the largest row counts of the two classes
-    CK(cudaMemsetAsync(dstatus, 0, 12, st));
+    // status word, then the largest row counts of the two classes and the
+    // commonest genotypes' shares
+    CK(cudaMemsetAsync(dstatus, 0, 16, st));
     launch_scan_pheno(dpheno, m, case_idx, ctrl_idx, dm1, dstatus, st);
     CK(cudaGetLastError());
     int64_t m1 = 0;
@@ -1778,15 +1782,16 @@ epi_status epi_dataset_create(epi_ctx *ctx, const uint8_t *geno, const uint8_t *
         } else {
             launch_pack_masks(dgeno, n, m, case_idx, ctrl_idx, m1, ds->W1, ds->Wt, ds->masks, dstatus, ctx->num_sms, st);
             launch_binom(n, ds->binom, ctx->num_sms, st);
-            launch_count_max(ds->masks, n, ds->W1, ds->Wt, dstatus + 1, st);
+            launch_count_max(ds->masks, n, m, ds->W1, ds->Wt, dstatus + 1, st);
             ctx->launches += 4;
-            int32_t words[3] = {};
+            int32_t words[4] = {};
             cudaError_t e = cudaGetLastError();
-            if (e == cudaSuccess) e = cudaMemcpyAsync(words, dstatus, 12, cudaMemcpyDeviceToHost, st);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(words, dstatus, 16, cudaMemcpyDeviceToHost, st);
             if (e == cudaSuccess) e = cudaStreamSynchronize(st);
             hstatus = words[0];
             ds->c1max = words[1];
             ds->c0max = words[2];
+            ds->top_share = (float)((double)words[3] / (127.0 * (double)n));
             if (e != cudaSuccess) ret = fail(EPI_ECUDA, "packing failed: %s", cudaGetErrorString(e));
             else if (hstatus & ST_BAD_GENO) ret = fail(EPI_EINVAL, "genotype values must be 0, 1 or 2");
         }

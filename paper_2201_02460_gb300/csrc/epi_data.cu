@@ -125,32 +125,40 @@ void launch_pack_masks(const uint8_t *geno, int64_t n, int64_t m, const int32_t 
                                                        m1_check);
 }
 
-// One warp per genotype-0 or -1 row.
-__global__ void __launch_bounds__(256) count_max_kernel(const uint32_t *__restrict__ masks, int64_t n, int32_t W1,
-                                                        int32_t Wt, int32_t *__restrict__ out)
+// One warp per SNP.
+__global__ void __launch_bounds__(256) count_max_kernel(const uint32_t *__restrict__ masks, int64_t n, int64_t m,
+                                                        int32_t W1, int32_t Wt, int32_t *__restrict__ out)
 {
     const int lane = threadIdx.x & 31;
-    int32_t best1 = 0, best0 = 0;
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < 2 * n;
-         r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const uint32_t *row = masks + ((r >> 1) * 3 + (r & 1)) * Wt;
-        uint32_t c1 = 0, c0 = 0;
-        for (int w = lane; w < Wt; w += 32) {
-            const uint32_t c = __popc(row[w]);
-            if (w < W1) c1 += c;
-            else c0 += c;
+    int32_t best1 = 0, best0 = 0, share = 0;
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < n;
+         s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        int32_t top = 0, rest = (int32_t)m;
+        for (int g = 0; g < 2; g++) {
+            const uint32_t *row = masks + (s * 3 + g) * Wt;
+            uint32_t c1 = 0, c0 = 0;
+            for (int w = lane; w < Wt; w += 32) {
+                const uint32_t c = __popc(row[w]);
+                if (w < W1) c1 += c;
+                else c0 += c;
+            }
+            const int32_t a = (int32_t)__reduce_add_sync(0xffffffffu, c1), b = (int32_t)__reduce_add_sync(0xffffffffu, c0);
+            best1 = max(best1, a);
+            best0 = max(best0, b);
+            top = max(top, a + b);
+            rest -= a + b;
         }
-        best1 = max(best1, (int32_t)__reduce_add_sync(0xffffffffu, c1));
-        best0 = max(best0, (int32_t)__reduce_add_sync(0xffffffffu, c0));
+        share += (int32_t)((int64_t)max(top, rest) * 127 / m);
     }
     if (lane == 0 && best1) atomicMax(out, best1);
     if (lane == 0 && best0) atomicMax(out + 1, best0);
+    if (lane == 0) atomicAdd(out + 2, share);
 }
 
-void launch_count_max(const uint32_t *masks, int64_t n, int32_t W1, int32_t Wt, int32_t *out, cudaStream_t st)
+void launch_count_max(const uint32_t *masks, int64_t n, int64_t m, int32_t W1, int32_t Wt, int32_t *out, cudaStream_t st)
 {
-    const int64_t blocks = (2 * n + 7) / 8;
-    count_max_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, st>>>(masks, n, W1, Wt, out);
+    const int64_t blocks = (n + 7) / 8;
+    count_max_kernel<<<(unsigned)(blocks < 1216 ? blocks : 1216), 256, 0, st>>>(masks, n, m, W1, Wt, out);
 }
 
 void launch_binom(int64_t n, uint64_t *tab, int num_sms, cudaStream_t st)

@@ -29,6 +29,17 @@
 // thread instead of 64 (two CTAs an SM instead of four) and a predicate per
 // item for the places without an individual.
 //
+// Rare variants put most individuals into one cell, and an atomic add takes the
+// lanes of one cell in turn: order 6, 40 x 2048, 18.7 ms at allele frequencies
+// of 0.05-0.5, 29.7 at 0.01-0.05 and 34.6 at 0.001-0.01 (the bitwise kernel 30
+// at all of them).  Studies whose commonest cell is expected to hold
+// kCrowdShare of the individuals run a kernel whose warps look, prefix by
+// prefix, for a cell that half of their lanes share, and add that crowd once:
+// 18.6 and 15.9 ms.  The look costs the others 1 to 3 %, hence the two
+// kernels; they meet at a share of 0.3 to 0.4 (frequencies 0.02-0.15: order 6
+// 23.7 plain and 22.5, order 7, 26 x 2048, 4.38 and 4.48, order 8, 23 x 2048,
+// 3.78 and 3.89; 0.01-0.1: 26.6 and 21.1, 4.83 and 4.52, 4.12 and 4.08).
+//
 // GPU mapping: persistent CTAs with contiguous rank ranges, one table (4-byte
 // cells, cases in the upper half) a CTA and as many CTAs as fit.  A thread
 // keeps its kItems individuals' cell of the first K-1 and K-2 SNPs in
@@ -46,6 +57,8 @@ namespace hist {
 
 constexpr int kLogShared = 1024;    // ln table entries in shared memory
 constexpr int kBuffer = 192;        // candidates between sorts
+constexpr double kCrowdShare = 0.33;
+constexpr int kCrowd = 16;          // individuals of a warp that make a crowd
 constexpr double kLnScale = 17592186044416.0;   // 2^44
 
 __host__ __device__ constexpr int cells_of(int k) { return k <= 0 ? 1 : 3 * cells_of(k - 1); }
@@ -161,7 +174,7 @@ __device__ __noinline__ double precise_mi(const uint32_t *tab, int cells, int64_
     return x / (double)m;
 }
 
-template <int K, int kItems>
+template <int K, int kItems, bool CROWDS>
 __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1) hist_kernel(Params P)
 {
     constexpr int kWords = kItems / 8;
@@ -232,6 +245,15 @@ __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1)
 #pragma unroll
         for (int i = 0; i < kItems; i++)
             c7[i] = valid >> i & 1u ? 3 * (c6[i] + (g[i / 8] >> (4 * (i % 8)) & 12u)) : spare;
+        // a cell of the prefix that kCrowd of the warp's first items share: lane
+        // 0's or (low bit set) lane 13's
+        uint32_t crowd = ~0u;
+        if constexpr (CROWDS) {
+            const uint32_t a = __shfl_sync(0xffffffffu, c7[0], 0), b = __shfl_sync(0xffffffffu, c7[0], 13);
+            const int na = __popc(__ballot_sync(0xffffffffu, c7[0] == a));
+            const int nb = __popc(__ballot_sync(0xffffffffu, c7[0] == b));
+            if (max(na, nb) >= kCrowd) crowd = na >= nb ? a : b | 1u;
+        }
         const int64_t r0 = S.rank;
         const int j0 = S.last;
         const int nj = (int)min((int64_t)(d.n - j0), R_e - r0);
@@ -248,9 +270,20 @@ __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1)
         for (int jj = 0; jj < nj; jj++) {
             uint32_t at[kItems];
 #pragma unroll
-            for (int i = 0; i < kItems; i++) {
-                at[i] = c7[i] + (g[i / 8] >> (4 * (i % 8)) & 12u);
-                atomicAdd(reinterpret_cast<uint32_t *>(tab + at[i]), inc);
+            for (int i = 0; i < kItems; i++) at[i] = c7[i] + (g[i / 8] >> (4 * (i % 8)) & 12u);
+            if (!CROWDS || crowd == ~0u) {
+#pragma unroll
+                for (int i = 0; i < kItems; i++) atomicAdd(reinterpret_cast<uint32_t *>(tab + at[i]), inc);
+            } else {
+                // the crowd's cell once for the warp
+                const uint32_t its = (crowd & ~1u) + (__shfl_sync(0xffffffffu, g[0], crowd & 1u ? 13 : 0) & 12u);
+                uint32_t many = 0;
+#pragma unroll
+                for (int i = 0; i < kItems; i++) {
+                    many += __popc(__ballot_sync(0xffffffffu, at[i] == its));
+                    if (at[i] != its) atomicAdd(reinterpret_cast<uint32_t *>(tab + at[i]), inc);
+                }
+                if (lane == 0) atomicAdd(reinterpret_cast<uint32_t *>(tab + its), inc * many);
             }
             if (jj + 1 < nj) geno(j0 + jj + 1, g);
             __syncthreads();
@@ -327,6 +360,10 @@ __global__ void __launch_bounds__(kItems == 8 ? 512 : 1024, kItems == 8 ? 2 : 1)
     if (t == 0) P.list_count[blockIdx.x] = S.list_len;
 }
 
+// Whether a study's commonest cell is expected to hold kCrowdShare of the
+// individuals.
+static bool crowds(const DevData &d, int k) { return pow((double)d.top_share, k) >= kCrowdShare; }
+
 // Warps of a CTA: those of cases, then those of controls; and items a thread,
 // 8 while that is at most 16 warps.
 static int class_warps(int32_t words, int items) { return (words + items - 1) / items; }
@@ -334,17 +371,16 @@ static int warps_of(const DevData &d, int items) { return class_warps(d.W1, item
 static int items_of(const DevData &d) { return warps_of(d, 8) <= 16 ? 8 : 16; }
 static int threads_of(const DevData &d) { return 32 * warps_of(d, items_of(d)); }
 
-static const void *kernel_of(int k, int items)
+static const void *kernel_of(const DevData &d, int k)
 {
-    switch (k * 100 + items) {
-    case 608: return (const void *)hist_kernel<6, 8>;
-    case 616: return (const void *)hist_kernel<6, 16>;
-    case 708: return (const void *)hist_kernel<7, 8>;
-    case 716: return (const void *)hist_kernel<7, 16>;
-    case 808: return (const void *)hist_kernel<8, 8>;
-    case 816: return (const void *)hist_kernel<8, 16>;
-    default: return nullptr;
-    }
+    static const void *const kernels[3][2][2] = {
+        {{(const void *)hist_kernel<6, 8, false>, (const void *)hist_kernel<6, 8, true>},
+         {(const void *)hist_kernel<6, 16, false>, (const void *)hist_kernel<6, 16, true>}},
+        {{(const void *)hist_kernel<7, 8, false>, (const void *)hist_kernel<7, 8, true>},
+         {(const void *)hist_kernel<7, 16, false>, (const void *)hist_kernel<7, 16, true>}},
+        {{(const void *)hist_kernel<8, 8, false>, (const void *)hist_kernel<8, 8, true>},
+         {(const void *)hist_kernel<8, 16, false>, (const void *)hist_kernel<8, 16, true>}}};
+    return k >= 6 && k <= 8 ? kernels[k - 6][items_of(d) == 16][crowds(d, k)] : nullptr;
 }
 
 }  // namespace hist
@@ -375,7 +411,7 @@ size_t hist_geno_words(const DevData &d)
 
 int hist_grid(int num_sms, const DevData &d, int k, int pool)
 {
-    const void *kern = hist::kernel_of(k, hist::items_of(d));
+    const void *kern = hist::kernel_of(d, k);
     const size_t smem = hist_smem_bytes(k, pool);
     int occ = 0;
     if (!kern || cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
@@ -404,7 +440,7 @@ cudaError_t launch_hist_search(const DevData &d, int k, uint64_t rank_begin, uin
     p.list_count = list_count;
     p.all_scores = all_scores;
     const int items = hist::items_of(d), threads = hist::threads_of(d);
-    const void *kern = hist::kernel_of(k, items);
+    const void *kern = hist::kernel_of(d, k);
     if (!kern) return cudaErrorInvalidValue;
     const size_t smem = hist_smem_bytes(k, pool);
     const int64_t total = std::max<int64_t>((int64_t)hist_geno_words(d), d.m + 1);

@@ -30,9 +30,10 @@ void launch_scan_pheno(const uint8_t *pheno, int64_t m, int32_t *case_idx, int32
 void launch_pack_masks(const uint8_t *geno, int64_t n, int64_t m, const int32_t *case_idx, const int32_t *ctrl_idx,
                        int64_t m1, int32_t W1, int32_t Wt, uint32_t *masks, int32_t *status, int num_sms,
                        cudaStream_t st, const int64_t *m1_check = nullptr);
-// largest case (out[0]) and control (out[1]) count of a genotype-0 or -1 row
+// largest case (out[0]) and control (out[1]) count of a genotype-0 or -1 row;
+// the shares of the SNPs' commonest genotypes in 127ths, added up (out[2])
 // (out zeroed before)
-void launch_count_max(const uint32_t *masks, int64_t n, int32_t W1, int32_t Wt, int32_t *out, cudaStream_t st);
+void launch_count_max(const uint32_t *masks, int64_t n, int64_t m, int32_t W1, int32_t Wt, int32_t *out, cudaStream_t st);
 void launch_binom(int64_t n, uint64_t *tab, int num_sms, cudaStream_t st);
 
 // epi_popc.cu

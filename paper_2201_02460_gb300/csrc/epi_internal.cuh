@@ -38,6 +38,7 @@ struct DevData {
     const uint32_t *masks;       // [n][3][Wt]
     const uint64_t *binom;       // [9][n+1]
     int32_t c1max = 0, c0max = 0;   // largest case / control count of a genotype-0 or -1 row
+    float top_share = 0.0f;         // of the commonest genotype, mean over the SNPs (rounded down)
 };
 
 __host__ __device__ inline uint64_t binom_at(const uint64_t *tab, int64_t n, int64_t a, int b)

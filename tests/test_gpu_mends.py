@@ -320,3 +320,19 @@ def test_small_scores_are_quick(epi, ctx, k, n, m, kind):
         geno, pheno = np.zeros((n, m), np.uint8), (np.arange(m) % 2).astype(np.uint8)
     ds = epi.Dataset(ctx, geno, pheno)
     assert seconds(ds, lambda: epi.score_all(ds, k)) < 2 * usual
+
+
+# rare variants put most individuals into one cell of an order-6 table: the
+# search must not take much longer than on common ones
+def test_high_order_rare_variants(epi, ctx):
+    times = []
+    for p in ((0.05, 0.5), (0.001, 0.01)):
+        ds = epi.Dataset(ctx, *random_data(36, 2048, seed=3, m1=1024, p_levels=p))
+        best = 1e9
+        for _ in range(3):
+            t = time.perf_counter()
+            epi.search(ds, 6, 20)
+            best = min(best, time.perf_counter() - t)
+        times.append(best)
+        ds.close()
+    assert times[1] < 1.3 * times[0]
