@@ -544,16 +544,22 @@ struct FusedParts {
     __host__ __device__ int total() const { return loss() + 1; }
 };
 
+// a row tile's inputs in shared memory, read four at a time
+struct alignas(16) InputTile {
+    float x[kFusedRows][kFusedIn];
+};
+static_assert(alignof(InputTile) >= alignof(float4) && kFusedIn % 4 == 0, "rows of the tile are read as float4");
+
 // normalised BF16 inputs of a row tile, as floats, padded to 32 columns
 __device__ __forceinline__ void stage_inputs(const float *__restrict__ X, int64_t r0, int64_t rows, int in,
-                                             const float *__restrict__ norm, float (*xs)[kFusedIn])
+                                             const float *__restrict__ norm, InputTile &xs)
 {
 #pragma unroll 4
     for (int e = threadIdx.x; e < kFusedRows * kFusedIn; e += blockDim.x) {
         const int r = e / kFusedIn, f = e - r * kFusedIn;
         const int fc = min(f, in - 1);
         const float v = (X[min(r0 + r, rows - 1) * in + fc] - norm[fc]) * norm[in + fc];
-        xs[r][f] = f < in && r0 + r < rows ? __bfloat162float(__float2bfloat16(v)) : 0.0f;
+        xs.x[r][f] = f < in && r0 + r < rows ? __bfloat162float(__float2bfloat16(v)) : 0.0f;
     }
 }
 
@@ -582,7 +588,7 @@ __global__ void __launch_bounds__(256) fused_layer1_kernel(const float *__restri
                                                            const float *__restrict__ b1, __nv_bfloat16 *__restrict__ H1,
                                                            __nv_bfloat16 *__restrict__ H1t, int64_t ldt)
 {
-    __shared__ float xs[kFusedRows][kFusedIn];
+    __shared__ InputTile xs;
     const int j = threadIdx.x;
     float w[kFusedIn];
 #pragma unroll
@@ -598,7 +604,7 @@ __global__ void __launch_bounds__(256) fused_layer1_kernel(const float *__restri
             float z = 0.0f;
 #pragma unroll
             for (int f = 0; f < kFusedIn; f += 4) {
-                const float4 x = *reinterpret_cast<const float4 *>(&xs[r][f]);
+                const float4 x = *reinterpret_cast<const float4 *>(&xs.x[r][f]);
                 z = fmaf(x.x, w[f], z);
                 z = fmaf(x.y, w[f + 1], z);
                 z = fmaf(x.z, w[f + 2], z);
@@ -690,7 +696,7 @@ __global__ void __launch_bounds__(256) fused_grad1_kernel(const float *__restric
                                                           const float *__restrict__ norm, float *__restrict__ part,
                                                           FusedParts at)
 {
-    __shared__ float xs[kFusedRows][kFusedIn];
+    __shared__ InputTile xs;
     const int j = threadIdx.x;
     float acc[kFusedIn], db1 = 0.0f;
 #pragma unroll
@@ -719,7 +725,7 @@ __global__ void __launch_bounds__(256) fused_grad1_kernel(const float *__restric
             db1 += dz;
 #pragma unroll
             for (int f = 0; f < kFusedIn; f += 4) {
-                const float4 x = *reinterpret_cast<const float4 *>(&xs[r][f]);
+                const float4 x = *reinterpret_cast<const float4 *>(&xs.x[r][f]);
                 acc[f] = fmaf(dz, x.x, acc[f]);
                 acc[f + 1] = fmaf(dz, x.y, acc[f + 1]);
                 acc[f + 2] = fmaf(dz, x.z, acc[f + 2]);
