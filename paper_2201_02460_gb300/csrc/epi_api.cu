@@ -707,7 +707,8 @@ struct BatchItem {
     int k = 0, top_n = 0, pool = 0, cells = 0;
     bool tc = false;
     int comb_p = 0;                // tensor path: class shift, 0 = separate classes
-    bool alone = false;            // a search of its own, after the batch's launches (batch_alone)
+    bool alone = false;            // a search of its own, with pair tiles, after the batch's launches
+    double saves = 0;              // what pair tiles save it, us
     uint64_t total = 0;
     double cost = 0;
     int group = -1, cta_begin = 0, cta_count = 0;
@@ -730,23 +731,29 @@ struct BatchGroup {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) & ~(a - 1); }
 
-// Whether a study of a batch is searched by itself, with pair tiles, after the
-// batch's launches: where the time that pairs save exceeds what a search of
-// its own costs beyond a place in the batch (120 us: its launches wait for
-// each other and the host for it).  Plain tiles take 1.25 ns an item and
-// 128-individual chunk of the whole GPU, and 16 chunks' worth at least; pairs
-// save 0.3 of it at order 4 below 24 chunks, half above, two thirds at order
-// 5.  us a study, batches of 24, in the batch and alone:
-//   order 4   40 x 1000  117 and 215    75 x 1000  384 and 406    90 x 1000  646 and 573
-//             50 x 4000  259 and 281    60 x 4000  395 and 339    40 x 16000 393 and 315
-//   order 5   24 x  300  233 and 245    26 x  300  308 and 264    24 x 4000  577 and 332
-bool batch_alone(const DevData &d, int k, bool comb)
+// What pair tiles save a study of orders 4-5, in us.  In batches of 24 studies
+// alike, plain tiles take about 20 ns of the whole GPU an item while the four
+// ring stages hold its whole K range (8 chunks of 128 individuals), 22 and 0.87
+// a chunk above; pairs save 0.3 of it, half above 8 chunks, two thirds at
+// order 5.
+double pair_saving_us(const DevData &d, int k, bool comb)
 {
-    if (!tc_pair_applies(d, k, comb)) return false;
     const double chunks = d.Wt / 4;
-    const double plain_us = 1.25e-3 * (double)tc_item_count(d.n, k, comb) * std::max(chunks, 16.0);
-    return plain_us * (k == 5 ? 0.66 : chunks >= 24 ? 0.5 : 0.3) >= 120.0;
+    const double plain_ns = (double)tc_item_count(d.n, k, comb) * (chunks <= 8 ? 20.0 : 22.0 + 0.87 * chunks);
+    return 1e-3 * plain_ns * (k == 5 ? 0.66 : chunks <= 8 ? 0.3 : 0.5);
 }
+
+// Studies that take pair tiles are searched by themselves after the batch's
+// launches, at the price of launches that wait for each other and of the host's
+// wait: about 120 us a study more than in the batch.  Where kBatchSmall or more
+// of them save less than kBatchSaving, those stay in the batch with plain tiles
+// (us a study, in a batch of 24 and alone: order 4, 46 x 1000 132 and 225, 60 x
+// 1000 217 and 278, 75 x 1000 384 and 406, 60 x 1875 325 and 291, 40 x 4000 169
+// and 231, 50 x 4000 259 and 281).  A few of them do not: their launch waits for
+// its slowest study, and plain tiles are slower by themselves (60 x 1875: 563
+// and 311 us; in drawn batches of mixed sizes it took up to a tenth more).
+constexpr int kBatchSmall = 8;
+constexpr double kBatchSaving = 50.0;
 
 // Popcount launch shape for a group: residency first, then staged prefixes.
 bool plan_group_popc(const epi_ctx *ctx, BatchGroup &g)
@@ -920,13 +927,18 @@ extern "C" epi_status epi_search_batched(epi_ctx *ctx, epi_dataset *const *dss, 
         if (st != EPI_OK) return fail(st, "dataset %d: %s", i, epi_last_error());
         const DevData d = it.ds->dev();
         if (it.tc) it.comb_p = plan_comb_shift(it.ds);
-        it.alone = it.tc && batch_alone(d, it.k, it.comb_p != 0);
+        it.alone = it.tc && tc_pair_applies(d, it.k, it.comb_p != 0);
+        if (it.alone) it.saves = pair_saving_us(d, it.k, it.comb_p != 0);
         // work estimate for the CTA split: a tensor-core item costs its
         // 128-individual chunks, but never less than its epilogue (about 32
         // chunks' worth)
         it.cost = it.tc ? (double)tc_item_count(d.n, it.k, it.comb_p != 0) * (double)std::max(d.Wt / 4, 32)
                         : (double)total * (double)(it.cells / 3) * (double)d.Wt;
     }
+    const auto stays = [](const BatchItem &it) { return it.alone && it.saves < kBatchSaving; };
+    if (std::count_if(items.begin(), items.end(), stays) >= kBatchSmall)
+        for (auto &it : items)
+            if (stays(it)) it.alone = false;
     // one group per (path, order, tensor variant)
     std::vector<BatchGroup> groups;
     for (int i = 0; i < n_ds; i++) {

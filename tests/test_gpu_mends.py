@@ -78,21 +78,24 @@ def test_wait_limit_at_every_order(epi, k, n, m, variant):
     own.close()
 
 
-# studies of a batch that are searched by themselves are those whose pair
-# tiles save more than a search of its own costs: a replayed graph launches
-# nothing that the context counts, a search of its own does
-@pytest.mark.parametrize("k,n,m,alone", [(4, 45, 1000, False), (4, 48, 4000, False), (5, 24, 300, False),
-                                         (4, 100, 1000, True), (4, 60, 4000, True), (5, 30, 300, True)])
-def test_batch_searches_large_studies_alone(epi, k, n, m, alone):
+# studies with pair tiles are searched by themselves, except where eight or more
+# of a batch save little by them: a replayed graph launches nothing that the
+# context counts, a search of its own does
+@pytest.mark.parametrize("k,n,m,count,alone", [(4, 45, 1000, 8, 0), (4, 45, 1000, 7, 7), (4, 60, 900, 9, 0),
+                                               (4, 45, 4000, 8, 8), (4, 100, 1000, 8, 8), (5, 26, 300, 8, 8)])
+def test_batch_searches_studies_alone(epi, k, n, m, count, alone):
     own = epi.Context(0)
-    sets = [epi.Dataset(own, *random_data(n - i, m, seed=n + i)) for i in (0, 1)] + \
-        [epi.Dataset(own, *random_data(30, 200, seed=1))]
-    orders = [k, k, 3]
+    sets = [epi.Dataset(own, *random_data(n, m, seed=n + i)) for i in range(count)]
+    sets.append(epi.Dataset(own, *random_data(30, 200, seed=1)))
+    orders = [k] * count + [3]
     want = [epi.search(s, o, 20, path="popc") for s, o in zip(sets, orders)]
-    epi.search_batched(own, sets, orders, [20] * 3)
+    epi.search_batched(own, sets, orders, [20] * len(sets))
     before = own.kernel_launches()
-    got = epi.search_batched(own, sets, orders, [20] * 3)
-    assert (own.kernel_launches() > before) == alone
+    epi.search(sets[0], k, 20, path="tc")
+    each = own.kernel_launches() - before
+    before = own.kernel_launches()
+    got = epi.search_batched(own, sets, orders, [20] * len(sets))
+    assert own.kernel_launches() - before == alone * each
     for a, b in zip(got, want):
         assert (a.rank == b.rank).all() and (a.mi == b.mi).all() and (a.counts == b.counts).all()
     own.close()
