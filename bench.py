@@ -38,7 +38,8 @@ DEFAULT_WORKLOAD = "order3_2000snp_4000"
 POPC_PER_SM_CLK = 16
 N_SMS = 152
 SM_MAX_MHZ = 2070.0
-# FP8 dense rate = 2 x BF16 dense (nominal 4.5 vs 2.25 PFLOP/s)
+# dense rate of the FP4 kinds by instruction shape: K = 64 an instruction, 32 with
+# FP8, 16 with BF16
 FP4_OVER_BF16 = 4.0
 
 
@@ -444,8 +445,8 @@ def roofline(kind, d, k, kern_ms, peaks, tc_rate=None, hist=False):
         comb = class_shift(d) != 0
         if tc_rate:
             # twice the measured rate of the FP8 MMA, at the maximum SM clock
-            # (kind::mxf4 retires 16384 multiply-adds per SM clock where the
-            # FP8 kinds retire 8192, both measured)
+            # (kind::mxf4 has K = 64 an instruction where the FP8 kinds have
+            # 32; its own rate is not measured)
             r = tc_rate[1]
             peak = 2 * 2.0 * r["mac_per_clk_sm"] * N_SMS * SM_MAX_MHZ * 1e6 / 1e12
             note = (f"peak = 2 x the measured FP8 tcgen05.mma rate, {r['mac_per_clk_sm']:.0f} "

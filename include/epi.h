@@ -462,8 +462,8 @@ epi_status epi_inject_alloc_failure(epi_ctx *ctx, int64_t after);
 epi_status epi_set_tc_variant(epi_ctx *ctx, int variant);
 
 /* Rate of the tensor pipe for FP8 MMAs (tcgen05.mma kind::f8f6f4, operands in
- * shared memory, FP32 accumulation; the FP4 MMAs of the counting path retire
- * twice the multiply-adds per clock):
+ * shared memory, FP32 accumulation; the FP4 MMAs of the counting path have
+ * twice the K an instruction):
  * shape 0 = M128 N128 K32 with E4M3 operands,
  * shape 1 = M128 N256 K32 with E5M2 operands;
  * EPI_EINVAL for other shapes.  One CTA per SM issues `stages` (32..2^32)

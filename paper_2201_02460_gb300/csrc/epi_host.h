@@ -49,7 +49,6 @@ cudaError_t launch_popc_search(const DevData &d, int k, int R, uint64_t rank_beg
                                int pool, int slots, int cand_p2, uint32_t *global_thr, float *list_score,
                                uint64_t *list_rank, int32_t *list_count, int grid, size_t smem, cudaStream_t st,
                                float *all_scores = nullptr, uint32_t *pre_global = nullptr);
-// batched: one launch over several datasets of order k (descriptors in device memory)
 // epi_hist.cu (geno: hist_geno_words words, ln: m + 1 entries, both filled by the launch)
 bool hist_applies(const DevData &d, int k, int pool);
 size_t hist_geno_words(const DevData &d);
@@ -58,6 +57,8 @@ cudaError_t launch_hist_search(const DevData &d, int k, uint64_t rank_begin, uin
                                uint32_t *global_thr, float *list_score, uint64_t *list_rank, int32_t *list_count,
                                int grid, float *all_scores, uint32_t *geno, long long *ln, cudaStream_t st);
 
+// batched popcount path: one launch over several datasets of order k
+// (descriptors in device memory)
 size_t popc_ds_bytes();
 void popc_fill_ds(void *dst, const DevData &d, uint64_t rank_begin, uint64_t rank_end, int cta_begin, int cta_count,
                   uint32_t *global_thr);

@@ -2,8 +2,8 @@
 //
 // The paper has no counterpart: this is a measurement aid.  The roofline of
 // the tensor-core counting kernel is twice the rate at which one SM retires
-// these MMAs (its kind::mxf4 retires 16384 multiply-adds per SM clock, the FP8
-// kinds 8192, both measured): tcgen05.mma.kind::f8f6f4 M128 N128 K32 with E4M3
+// these MMAs (8192 multiply-adds per SM clock; the counting kernel's kind::mxf4
+// has K = 64 an instruction where these have 32): tcgen05.mma.kind::f8f6f4 M128 N128 K32 with E4M3
 // operands (shape 0) or M128 N256 K32 with E5M2 operands (shape 1), FP32
 // accumulation, both operands in shared memory in the 128-byte swizzle.  One
 // CTA per SM issues that MMA back to back from one thread, accumulating 32 K

@@ -6,10 +6,9 @@
 // with A[(p, x')] the genotype-table row x' of prefix p (Section 2.1) and
 // B[(j, g)] row g of SNP j, summed separately over the case and the control
 // individuals.  Both operands hold 0/1 patterns as FP4 E2M1 nibbles
-// (kind::mxf4: K = 64 per MMA, twice the FP8 kinds' rate, measured 16384
-// multiply-adds per SM clock, and half their operand bytes) and the MMA
-// accumulates in FP32 in tensor memory.  Because the product sums over K, any
-// fixed permutation of the individuals inside a K step, applied to both
+// (kind::mxf4: K = 64 per MMA, twice that of the FP8 kinds, and half their
+// operand bytes) and the MMA accumulates in FP32 in tensor memory.  Because
+// the product sums over K, any fixed permutation of the individuals inside a K step, applied to both
 // operands, leaves the counts unchanged, and the two operands may carry
 // different weights per K position as long as their product is constant:
 //   * 32-bit word i (of 4) of the 16 bytes of a mask word holds, in nibble b,

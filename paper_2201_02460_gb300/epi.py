@@ -270,7 +270,7 @@ class Context:
     def tc_rate(self, stages: int = 1 << 19, shape: int = 0) -> dict:
         """Rate of the tensor pipe for an FP8 MMA (shape 0: E4M3 M128 N128
         K32; shape 1: E5M2 M128 N256 K32; the counting path's FP4 MMAs
-        retire twice the multiply-adds), measured with one CTA
+        have K = 64), measured with one CTA
         per SM issuing it back to back."""
         out = np.zeros(4, dtype=np.float64)
         _check(load().epi_tc_rate(self._h, int(shape), int(stages), _np_ptr(out)))
