@@ -1704,7 +1704,7 @@ static void free_ctx(epi_ctx *ctx)
         cudaStreamSynchronize(ctx->stream);
         cudaFree(ctx->scratch);
     }
-    if (ctx->pair_space) cudaFreeAsync(ctx->pair_space, ctx->stream);
+    if (ctx->pair_space) cudaFree(ctx->pair_space);   // (the stream may be gone)
     for (auto &pr : ctx->prof_events) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
     if (ctx->waits_dev) cudaFree(ctx->waits_dev);
     if (ctx->batch_exec) cudaGraphExecDestroy(ctx->batch_exec);
